@@ -36,22 +36,23 @@ constexpr int kExitBT = 8;      // samples per exit CTA (one LayerNorm per warp)
 constexpr int kExitCT = 128;    // classes per exit CTA
 constexpr int kExitThreads = 256;
 
-constexpr int kPlanThreads = 1024;
+constexpr int kPlanThreads = 256;
+constexpr int kPlanTile = 32;   // samples per tile of the plan kernel (one warp each)
 constexpr int kImageThreads = 512;
 constexpr int kImageWarps = kImageThreads / 32;
 
 // Workspace layout (bytes from the workspace base; every block 256-aligned).
-// The slot map and the plan come first, so their offsets depend on max_batch
+// The plan's counts and the plan come first, so their offsets depend on max_batch
 // only; the exit counters and partial softmax sums follow, then the logits tiles of
 // the general exit kernel (heads of more than kExitClMaxTiles class tiles only: its
 // CTAs cannot wait for one another, so the last CTA of a sample tile copies the rows
 // of the samples that exit from there).
 constexpr int kExitClMaxTiles = 8;   // class tiles of the cluster exit kernel (portable cluster size)
 struct WsLayout {
-    size_t slot;       // int[max_batch]: output sample of every input sample
+    size_t slot;       // int[max_batch]: output rows of every input sample (the plan's counts)
     size_t plan;       // int[4]: batch valid, survivor count
     size_t counters;   // int[n_btile + 1], zero between calls
-    size_t partials;   // float2[n_btile * kExitBT * n_ctile]
+    size_t partials;   // float2[n_btile * kExitBT * n_ctile]; after the exit check the plan's tile totals
     size_t lg;         // float[n_btile * kExitBT][classes] (empty for heads of <= kExitClMaxTiles tiles)
     size_t total;
 };

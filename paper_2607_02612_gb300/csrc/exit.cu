@@ -4,13 +4,13 @@
 // LayerNorm and GELU(W1 u + b1) rounded to the dtype; the second reads those rows densely,
 // without LayerNorm, and ends in the softmax maximum and the exit rule.
 //
-// Two kernels.  The cluster kernel (heads of at most 8 class tiles) is described below.
+// Three kernels.  The cluster kernels (heads of at most 8 class tiles; few samples, or many) are
+// described below.
 // The general one: grid (class tiles of kExitCT) x (sample tiles of kExitBT).  Every CTA computes
 // the LayerNorm of its samples' CLS rows, one logits tile (bf16: the weight tile by TMA and one
 // tcgen05 product D[128 classes][16 samples] in tensor memory; f32: FFMA) and a partial softmax
 // (tile max and sum of exponentials) per sample.  The last CTA of a sample tile to finish
-// (atomic counter, no waiting) merges the partials into c and the exit mask; the
-// last sample tile to finish runs the compaction plan for the fused stage.
+// (atomic counter, no waiting) merges the partials into c and the exit mask.
 #include <cooperative_groups.h>
 
 #include "launch.h"
@@ -64,8 +64,10 @@ constexpr size_t kExitClBudget = 112 * 1024;   // the cluster kernel's dynamic s
 // the general kernel's bound: two CTAs per SM with its larger static shared memory
 constexpr size_t kExitTcBudget = 110 * 1024;
 
-// Instruction descriptor of D[128][16] (float32) += A[128][16] B[16][16]^T, A and B bf16, K-major.
-constexpr uint32_t kExitIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(16 >> 3) << 17) | (8u << 24);
+// Instruction descriptor of D[128][N] (float32) += A[128][16] B[N][16]^T, A and B bf16, K-major.
+__host__ __device__ constexpr uint32_t exit_idesc(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | (8u << 24);
+}
 
 // The general kernel's bf16 shared memory, offsets from a 1024-byte aligned base: the u tile
 // (u_tc_off; 16 rows, rows 8..15 zero) | the weight ring (w_stages TMA stages, the whole tile when
@@ -82,19 +84,19 @@ struct ExitTcSmem {
     static __host__ __device__ size_t w_off(int dim) { return u_bytes(dim); }
     static __host__ __device__ size_t bias_off(int dim) { return w_off(dim) + (size_t)w_stages(dim) * kExitWStage; }
     static __host__ __device__ size_t total(int dim) {
-        const size_t t = bias_off(dim) + kExitCT * sizeof(float);
-        const size_t plan = plan_smem_bytes(kExitThreads);   // run_plan reuses the buffer from its start
-        return (t > plan ? t : plan) + 1024;
+        return bias_off(dim) + kExitCT * sizeof(float) + 1024;
     }
 };
 
-// D[128 classes][16 samples] = W_tile u^T on tcgen05, by one thread: per 64-dim K-block, wait
+// D[128 classes][NB rows] = W_tile u^T on tcgen05, by one thread (u: K-blocks of [NB rows][128
+// bytes]): per 64-dim K-block, wait
 // for its weight stage (stages 0..nws-1 already issued), four MMAs (K = 16; fewer in a short
 // last block), commit; when the tile is not resident, the stage of the block before is
 // refilled by TMA once its MMAs completed (one block late, so that the wait overlaps the
 // products just issued).  Every wait is bounded; after a failure the copies and products in
 // flight are waited for (bounded) and FUSION_DEV_TIMEOUT is raised.  Returns whether D is
 // complete.
+template <int NB>
 __device__ __forceinline__ bool exit_tc_product(const CUtensorMap *wmap, uint32_t tmem, uint32_t ub, uint32_t wr,
                                                 int dim, int nws, int c0, unsigned long long *wbar,
                                                 unsigned long long *wempty, unsigned long long *wdone, int *status) {
@@ -110,10 +112,10 @@ __device__ __forceinline__ bool exit_tc_product(const CUtensorMap *wmap, uint32_
             break;
         }
         waited = kc + 1;
-        const uint32_t a0 = wr + (uint32_t)st * kExitWStage, b0 = ub + (uint32_t)kc * 2048u;
+        const uint32_t a0 = wr + (uint32_t)st * kExitWStage, b0 = ub + (uint32_t)kc * (NB * 128u);
         const int kw = min(64, dim - kc * 64);
         for (int k = 0; k * 16 < kw; ++k)
-            umma_bf16(tmem, sw128_desc(a0 + k * 32), sw128_desc(b0 + k * 32), kExitIdesc, (kc | k) ? 1u : 0u);
+            umma_bf16(tmem, sw128_desc(a0 + k * 32), sw128_desc(b0 + k * 32), exit_idesc(NB), (kc | k) ? 1u : 0u);
         umma_commit(smem_addr(&wempty[st]));
         issued = kc + 1;
         const int kp = kc - 1;   // the block before; its stage next holds block kp + nws
@@ -149,9 +151,7 @@ struct ExitSmem {
     static __host__ __device__ int u_stride(int dim) { return dim + 16 / EB; }   // row bytes = 16 (mod 32)
     static __host__ __device__ size_t u_bytes(int dim) { return ((size_t)16 * u_stride(dim) * EB + 15) / 16 * 16; }
     static __host__ __device__ size_t total(int dim) {
-        size_t t = u_bytes(dim) + 2 * w_stage + kExitCT * sizeof(float);
-        const size_t plan = plan_smem_bytes(kExitThreads);
-        return t > plan ? t : plan;
+        return u_bytes(dim) + 2 * w_stage + kExitCT * sizeof(float);
     }
 };
 
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
             const uint32_t tmem = tmem_base;
             const int nws = TS::w_stages(dim);
             if (tid == 0)
-                s_wfail = exit_tc_product(&wmap, tmem, smem_addr(base), smem_addr(w_region), dim, nws, c0, wbar,
+                s_wfail = exit_tc_product<16>(&wmap, tmem, smem_addr(base), smem_addr(w_region), dim, nws, c0, wbar,
                                           wempty, &wdone, p.status)
                               ? 0
                               : 1;
@@ -690,18 +690,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
     }
     if (tid == 0) p.counters[bt] = 0;
 
-    // ---- the last sample tile runs the plan ------------------------------------------
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) s_last = (atomicAdd(&p.counters[p.n_btile], 1) == p.n_btile - 1);
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    if (tid == 0) {
-        p.counters[p.n_btile] = 0;
-        if (Bdev < 0 && !p.do_plan) raise_status(p.status, FUSION_DEV_BAD_BATCH);
-    }
-    if (p.do_plan) run_plan(p.plan, reinterpret_cast<int *>(sm));
+    if (tid == 0 && bt == 0 && Bdev < 0 && !p.plan_follows) raise_status(p.status, FUSION_DEV_BAD_BATCH);
 }
 
 __device__ __forceinline__ float to_float(float v) { return v; }
@@ -714,10 +703,11 @@ __device__ __forceinline__ float to_float(__nv_bfloat16 v) { return __bfloat162f
 // sum and sum of squares in float-float, var = E[x^2] - mean^2) and stores the normalised
 // row into the shared memory of every CTA of the cluster; each CTA then computes its logits
 // tile and partial softmax, sends (max, sum of exponentials) to the sample's owner, and the
-// owner merges them.  bf16: the head's weight tile arrives by TMA from the kernel's start
+// owner merges them.  For batches whose tiles fit one wave (k_exit_rows takes the larger ones).
+// bf16: the head's weight tile arrives by TMA from the kernel's start
 // (all of it when it fits, else a ring), and the logits tile is one tcgen05 product
 // D[128 classes][16 samples] in tensor memory; float32: cp.async stages and FFMA.  No global
-// atomics unless the plan kernel's work runs here (batches above the fused-plan bound).
+// atomics.
 // ---------------------------------------------------------------------------
 
 template <typename T>
@@ -758,9 +748,7 @@ struct ExitClSmem {
     static __host__ __device__ size_t red_off(int dim) { return part_off(dim) + (size_t)BT * 8 * sizeof(float2); }
     static __host__ __device__ size_t flag_off(int dim) { return red_off(dim) + (size_t)(kExitThreads / 32) * 8 * sizeof(float); }
     static __host__ __device__ size_t total(int dim) {
-        const size_t t = flag_off(dim) + (size_t)BT * sizeof(int);
-        const size_t plan = w_off(dim) + plan_smem_bytes(kExitThreads);   // run_plan reuses the W stages
-        return (t > plan ? t : plan) + (kTc ? 1024 : 0);
+        return flag_off(dim) + (size_t)BT * sizeof(int) + (kTc ? 1024 : 0);
     }
 };
 
@@ -973,7 +961,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
             // ---- D[128 classes][16 samples] = W_tile u^T on tcgen05 (exit_tc_product) ----------
             const uint32_t tmem = tmem_base;
             if (tid == 0)
-                s_wfail = exit_tc_product(&wmap, tmem, smem_addr(base), smem_addr(w_region), dim, L::w_stages(dim), c0,
+                s_wfail = exit_tc_product<16>(&wmap, tmem, smem_addr(base), smem_addr(w_region), dim, L::w_stages(dim), c0,
                                           wbar, wempty, &wdone, p.status)
                               ? 0
                               : 1;
@@ -1056,28 +1044,401 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
             for (int col = lane; col < kExitCT; col += 32)
                 if (c0 + col < C) p.logits[(size_t)sw * C + c0 + col] = lg_s[slw * kExitCT + col];
     }
-    if (!p.do_plan) {
-        if (Bdev < 0 && bt == 0 && rank == 0 && tid == 0) raise_status(p.status, FUSION_DEV_BAD_BATCH);
-        return;
+    if (Bdev < 0 && bt == 0 && rank == 0 && tid == 0) raise_status(p.status, FUSION_DEV_BAD_BATCH);
+}
+
+// ---------------------------------------------------------------------------
+// The exit check of many samples: clusters as above, of BT samples (16, 32 or 64) and n_ctile CTAs,
+// so that a weight tile is read once per BT samples and the product has BT columns.  Bound by the
+// chain of latencies of one CTA.  The CLS rows land in the u tile itself and are normalised in place,
+// LPR lanes per row (all the CTA's rows at once), so BT rows and the weight ring leave room for two
+// CTAs per SM; the softmax takes eight lanes per sample, the same way.  float32: FFMA, warp -> BT / 4
+// samples x 64 classes, a lane two classes (24 shared-memory wavefronts per 128 FFMA at BT = 64; one
+// sample x 128 classes per warp, as k_exit_cl has it, takes 17 per 16).
+// Measured, tiles of 8 before -> now (cold caches): 8192 samples x 100 classes, d = 384, with the plan,
+// float32 173 -> 45 us and bf16 129 -> 30 us; 512 samples x 1000 classes, d = 768, bf16 34 -> 24 us.
+// ---------------------------------------------------------------------------
+template <typename T, int BT>
+struct ExitRowsSmem {
+    static constexpr int EB = Elem<T>::kBytes;
+    static constexpr bool kTc = EB == 2;
+    static constexpr int KC = 32;               // float32: dims per cp.async weight stage
+    static constexpr int kF32Stages = 3;
+    static constexpr int w_stride = KC + 4;     // floats; rows 16 bytes apart modulo 128: conflict-free
+    static constexpr uint32_t w_stage = kTc ? kExitWStage : kExitCT * w_stride * 4u;
+    static constexpr int lg_stride = kExitCT + 8;   // floats: the four samples of a warp 8 banks apart
+    // u tile (bf16: K-blocks of [BT rows][128 bytes], swizzled; float32: [BT][dim + 4]) | weight ring (the
+    // logits tile [BT][lg_stride] afterwards) | bias | partials [BT][8] | rows, counts and bits [BT]
+    static __host__ __device__ size_t u_bytes(int dim) {
+        return kTc ? (size_t)((dim + 63) / 64) * BT * 128 : (size_t)BT * (dim + 4) * 4;
     }
-    // ---- the last cluster to finish runs the plan (batches above the fused-plan bound) ----
-    __threadfence();
-    cl.sync();   // this cluster's exit masks are written
-    __shared__ int s_last;
-    if (tid == 0) {
-        s_last = 0;
-        if (rank == 0) {
-            __threadfence();
-            s_last = (atomicAdd(&p.counters[p.n_btile], 1) == p.n_btile - 1);
+    static __host__ __device__ size_t rest(int dim) {
+        return u_bytes(dim) + kExitCT * sizeof(float) + (size_t)BT * (8 * sizeof(float2) + 3 * sizeof(int)) + (kTc ? 1024 : 0);
+    }
+    static __host__ __device__ int w_stages(int dim) {
+        if (!kTc) return kF32Stages;
+        const int nk = (dim + 63) / 64;
+        int st = rest(dim) + 2 * (size_t)w_stage <= kExitClBudget ? (int)((kExitClBudget - rest(dim)) / w_stage) : 2;
+        st = st < kExitClMaxW ? st : kExitClMaxW;
+        return nk < st ? nk : st;
+    }
+    static __host__ __device__ size_t ring_bytes(int dim) {
+        const size_t r = (size_t)w_stages(dim) * w_stage, lg = (size_t)BT * lg_stride * sizeof(float);
+        return r > lg ? r : lg;
+    }
+    static __host__ __device__ size_t bias_off(int dim) { return u_bytes(dim) + ring_bytes(dim); }
+    static __host__ __device__ size_t part_off(int dim) { return bias_off(dim) + kExitCT * sizeof(float); }
+    static __host__ __device__ size_t row_off(int dim) { return part_off(dim) + (size_t)BT * 8 * sizeof(float2); }
+    static __host__ __device__ size_t total(int dim) {
+        return row_off(dim) + (size_t)BT * 3 * sizeof(int) + (kTc ? 1024 : 0);
+    }
+};
+
+// KC dims of the float32 weight tile from k0 (one commit group; zeros past the head).
+template <typename S>
+__device__ __forceinline__ void issue_w_rows(const ExitParams &p, float *dst, int c0, int k0, int dim, int C) {
+    constexpr int wch = S::KC / 4;
+    for (int it = threadIdx.x; it < kExitCT * wch; it += kExitThreads) {
+        const int row = it / wch, c = it - row * wch;
+        float *d = dst + row * S::w_stride + c * 4;
+        if (c0 + row < C && k0 + c * 4 < dim)
+            cp_async16(d, reinterpret_cast<const float *>(p.head.weight) + (size_t)(c0 + row) * dim + k0 + c * 4);
+        else
+            *reinterpret_cast<uint4 *>(d) = make_uint4(0, 0, 0, 0);
+    }
+    cp_async_commit();
+}
+
+template <typename T, int BT>
+__global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_constant__ CUtensorMap wmap, ExitParams p) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ __align__(8) unsigned long long wbar[kExitClMaxW], wempty[kExitClMaxW], wdone;
+    __shared__ int s_wfail, s_last;
+    __shared__ uint32_t tmem_base;
+    using L = ExitRowsSmem<T, BT>;
+    constexpr int CH = Elem<T>::kPerChunk;
+    constexpr bool kBf16 = L::kTc;
+    constexpr int kWarps = kExitThreads / 32;
+    constexpr uint32_t kCols = BT < 32 ? 32 : BT;     // tensor-memory columns of D
+    cg::cluster_group cl = cg::this_cluster();
+    const int ncl = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int dim = p.dim, nchunk = dim / CH;
+    unsigned char *base = kBf16 ? reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(sm) + 1023) &
+                                                                    ~uintptr_t(1023))
+                                : sm;
+    auto uchunk = [&](int r, int c) -> unsigned char * {   // chunk c of row r of the u tile
+        return kBf16 ? base + (uint32_t)(c >> 3) * (BT * 128u) + (uint32_t)r * 128u + ((uint32_t)((c & 7) ^ (r & 7)) << 4)
+                     : base + ((size_t)r * (dim + 4) + c * 4) * 4;
+    };
+    unsigned char *ring = base + L::u_bytes(dim);
+    float *lg_s = reinterpret_cast<float *>(ring);   // [BT][kExitCT], after the product
+    float *bias_s = reinterpret_cast<float *>(base + L::bias_off(dim));
+    float2 *part_s = reinterpret_cast<float2 *>(base + L::part_off(dim));
+    int *row_s = reinterpret_cast<int *>(base + L::row_off(dim));   // CLS row of each sample, -1: none
+    int *cnt_s = row_s + BT;     // the plan's counts: rows if the sample continues, then -1 where it exits
+    int *bits_s = cnt_s + BT;    // and its status bits
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int ct = blockIdx.x, bt = blockIdx.y;
+    const int s0 = bt * BT, c0 = ct * kExitCT;
+    const int C = p.head.classes;
+    const int Bdev = device_batch(p.in);
+    const int B = Bdev < 0 ? 0 : Bdev;
+    const bool active = s0 < B;   // uniform over the cluster (same sample tile)
+
+    if (tid == 0) s_wfail = 0;
+    if (active) {
+        if constexpr (kBf16) {
+            if (warp == 0) {
+                asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                                 smem_addr(&tmem_base)),
+                             "r"(kCols)
+                             : "memory");
+                asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+            }
+            if (tid == 32) {
+                const int nws = L::w_stages(dim);
+                for (int q = 0; q < nws; ++q) {
+                    mbar_init(smem_addr(&wbar[q]), 1);
+                    mbar_init(smem_addr(&wempty[q]), 1);
+                }
+                mbar_init(smem_addr(&wdone), 1);
+                asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+                for (int q = 0; q < nws; ++q) {
+                    mbar_expect_tx(smem_addr(&wbar[q]), kExitWStage);
+                    tma_load_2d(smem_addr(ring + (size_t)q * kExitWStage), &wmap, q * 64, c0, smem_addr(&wbar[q]));
+                }
+            }
+        } else {
+            for (int q = 0; q < L::kF32Stages; ++q)
+                issue_w_rows<L>(p, reinterpret_cast<float *>(ring + q * L::w_stage), c0, q * L::KC, dim, C);
+        }
+        for (int k = tid; k < BT; k += kExitThreads) {
+            int row = -1, n = -1, bits = 0;
+            if (s0 + k < B) {
+                row = p.in.offsets[s0 + k];
+                if (row < 0 || row >= p.in.max_rows) {
+                    row = -1;
+                    raise_status(p.status, FUSION_DEV_BAD_OFFSETS);
+                }
+                if (p.do_plan && rank == 0) n = plan_count(p.plan, s0 + k, bits);
+            }
+            row_s[k] = row;
+            cnt_s[k] = n;
+            bits_s[k] = bits;
+        }
+        for (int c = tid; c < kExitCT; c += kExitThreads) bias_s[c] = c0 + c < C ? p.head.bias[c0 + c] : 0.0f;
+    }
+    // every CTA of the cluster runs before any remote shared-memory store (and row_s is complete)
+    cl.sync();
+    if (active) {
+        // ---- this CTA's rows (samples rank, rank + ncl, ... of the tile) into the u tile ------------
+        const int nr = (BT - rank + ncl - 1) / ncl;
+        for (int j = warp; j < nr; j += kWarps) {
+            const int sl = rank + j * ncl, row = row_s[sl];
+            const T *src = reinterpret_cast<const T *>(p.x) + (long long)row * dim;
+            for (int c = lane; c < nchunk; c += 32) {
+                if (row >= 0)
+                    cp_async16(uchunk(sl, c), src + c * CH);
+                else
+                    *reinterpret_cast<uint4 *>(uchunk(sl, c)) = make_uint4(0, 0, 0, 0);
+            }
+        }
+        cp_async_commit();
+        const F2 rdim = f2_recip((float)dim);
+        // lanes per row: a power of two, 4 (64 rows) .. 32 (8 rows or fewer)
+        int lpr = 32;
+        while (lpr > 4 && lpr * nr > kExitThreads) lpr >>= 1;
+        cp_async_wait_all();
+        __syncthreads();
+        // ---- LayerNorm in place, lpr lanes per row: one pass of sum and sum of squares ---------------
+        for (int j0 = 0; j0 < nr; j0 += kExitThreads / lpr) {
+            const int j = j0 + tid / lpr, l = tid & (lpr - 1);
+            const int sl = rank + j * ncl;
+            const bool ok = j < nr && row_s[sl] >= 0;
+            float s1 = 0.0f, c1 = 0.0f, s2 = 0.0f, c2 = 0.0f, l2 = 0.0f;
+            if (ok) {
+#pragma unroll 1
+                for (int c = l; c < nchunk; c += lpr) {
+                    float f[CH];
+                    chunk_to_f(*reinterpret_cast<const uint4 *>(uchunk(sl, c)), f);
+#pragma unroll
+                    for (int e = 0; e < CH; ++e) {
+                        neu_add(s1, c1, f[e]);
+                        const F2 sq = two_prod(f[e], f[e]);
+                        neu_add(s2, c2, sq.hi);
+                        l2 = __fadd_rn(l2, sq.lo);
+                    }
+                }
+            }
+            F2 a1 = two_sum(s1, c1), a2 = f2_add_f(two_sum(s2, c2), l2);
+#pragma unroll 1
+            for (int m = lpr >> 1; m >= 1; m >>= 1) {
+                a1 = f2_add(a1, f2_shfl_xor(a1, m));
+                a2 = f2_add(a2, f2_shfl_xor(a2, m));
+            }
+            if (!ok) continue;   // no barrier and no shuffle below
+            const F2 mean = f2_mul(a1, rdim);
+            const F2 ex2 = f2_mul(a2, rdim);
+            const F2 m2 = f2_mul(mean, mean);
+            F2 var = f2_add(ex2, {-m2.hi, -m2.lo});
+            if (var.hi < 0.0f) var = {0.0f, 0.0f};
+            const F2 rstd = f2_rsqrt(f2_add_f(var, p.head.eps));
+            if (l == 0 && !(isfinite(mean.hi) && isfinite(var.hi))) raise_status(p.status, FUSION_DEV_NONFINITE);
+#pragma unroll 1
+            for (int c = l; c < nchunk; c += lpr) {
+                uint4 *dst = reinterpret_cast<uint4 *>(uchunk(sl, c));
+                float f[CH], gf[CH], bf[CH];
+                chunk_to_f(*dst, f);
+                chunk_to_f(ldg16(reinterpret_cast<const T *>(p.head.gamma) + c * CH), gf);
+                chunk_to_f(ldg16(reinterpret_cast<const T *>(p.head.beta) + c * CH), bf);
+                uint32_t w4[4];
+                if constexpr (kBf16) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        w4[e] = (uint32_t)ln_out_bf16(f[2 * e], mean, rstd, gf[2 * e], bf[2 * e]) |
+                                ((uint32_t)ln_out_bf16(f[2 * e + 1], mean, rstd, gf[2 * e + 1], bf[2 * e + 1]) << 16);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) w4[e] = __float_as_uint(ln_out_f32(f[e], mean, rstd, gf[e], bf[e]));
+                }
+                const uint4 o = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+                *dst = o;
+                for (int r = 1; r < ncl; ++r) *cl.map_shared_rank(dst, rank + r < ncl ? rank + r : rank + r - ncl) = o;
+            }
+        }
+        // rows past the batch (or malformed): zero in the other CTAs too
+        for (int j = warp; ncl > 1 && j < nr; j += kWarps) {
+            const int sl = rank + j * ncl;
+            if (row_s[sl] >= 0) continue;
+            for (int c = lane; c < nchunk; c += 32)
+                for (int r = 0; r < ncl; ++r)
+                    *cl.map_shared_rank(reinterpret_cast<uint4 *>(uchunk(sl, c)), r) = make_uint4(0, 0, 0, 0);
         }
     }
+    // bf16: the u tile, written by the generic proxy here and in the other CTAs, is read by the
+    // tensor core (async proxy) after the barrier
+    if constexpr (kBf16) asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
+    cl.sync();   // all LayerNorm rows are in every CTA's shared memory
+
+    if (active) {
+        if constexpr (kBf16) {
+            const uint32_t tmem = tmem_base;
+            if (tid == 32)
+                s_wfail = exit_tc_product<BT>(&wmap, tmem, smem_addr(base), smem_addr(ring), dim, L::w_stages(dim), c0,
+                                              wbar, wempty, &wdone, p.status)
+                              ? 0
+                              : 1;
+            __syncthreads();
+            // the product is done: a programmatic dependent may start its prologue now
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (s_wfail == 0) {   // D's lanes are classes; warps w and w + 4 share a quadrant's columns
+                const int cls = (warp & 3) * 32 + lane;
+                for (int n0 = (warp >> 2) * 16; n0 < BT; n0 += 32) {
+                    uint32_t v[16];
+                    tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)n0, v);
+#pragma unroll
+                    for (int n = 0; n < 16; ++n)
+                        lg_s[(n0 + n) * L::lg_stride + cls] = c0 + cls < C ? __uint_as_float(v[n]) + bias_s[cls] : -INFINITY;
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncthreads();
+            if (warp == 0)
+                asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
+        } else {
+            constexpr int SP = BT / 4;   // samples of this warp
+            const int sg = (warp >> 1) * SP, cb = (warp & 1) * 64;
+            float acc[SP][2];
+#pragma unroll
+            for (int i = 0; i < SP; ++i) acc[i][0] = acc[i][1] = 0.0f;
+            const int n_k = (dim + L::KC - 1) / L::KC;
+            for (int kc = 0; kc < n_k; ++kc) {
+                asm volatile("cp.async.wait_group %0;\n" ::"n"(L::kF32Stages - 1) : "memory");
+                __syncthreads();
+                unsigned char *stage = ring + (kc % L::kF32Stages) * L::w_stage;
+                const float *ws = reinterpret_cast<const float *>(stage) + (cb + lane) * L::w_stride;
+                const float *ur = reinterpret_cast<const float *>(base) + (size_t)sg * (dim + 4) + kc * L::KC;
+                const int kw = min(L::KC, dim - kc * L::KC);   // a multiple of 16
+                for (int k0 = 0; k0 < kw; k0 += 16) {   // partial sums of 16 dims, as k_exit_cl
+                    float t[SP][2];
+#pragma unroll
+                    for (int i = 0; i < SP; ++i) t[i][0] = t[i][1] = 0.0f;
+#pragma unroll
+                    for (int kk = k0; kk < k0 + 16; kk += 4) {
+                        const float4 w0 = *reinterpret_cast<const float4 *>(ws + kk);
+                        const float4 w1 = *reinterpret_cast<const float4 *>(ws + 32 * L::w_stride + kk);
+#pragma unroll
+                        for (int i = 0; i < SP; ++i) {
+                            const float4 u = *reinterpret_cast<const float4 *>(ur + (size_t)i * (dim + 4) + kk);
+                            t[i][0] = fmaf(u.x, w0.x, t[i][0]);
+                            t[i][1] = fmaf(u.x, w1.x, t[i][1]);
+                            t[i][0] = fmaf(u.y, w0.y, t[i][0]);
+                            t[i][1] = fmaf(u.y, w1.y, t[i][1]);
+                            t[i][0] = fmaf(u.z, w0.z, t[i][0]);
+                            t[i][1] = fmaf(u.z, w1.z, t[i][1]);
+                            t[i][0] = fmaf(u.w, w0.w, t[i][0]);
+                            t[i][1] = fmaf(u.w, w1.w, t[i][1]);
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < SP; ++i) {
+                        acc[i][0] += t[i][0];
+                        acc[i][1] += t[i][1];
+                    }
+                }
+                __syncthreads();   // everyone is done with this stage
+                if (kc + L::kF32Stages < n_k)
+                    issue_w_rows<L>(p, reinterpret_cast<float *>(stage), c0, (kc + L::kF32Stages) * L::KC, dim, C);
+                else
+                    cp_async_commit();   // an empty group keeps the count
+            }
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#pragma unroll
+            for (int i = 0; i < SP; ++i)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const int col = cb + 32 * q + lane;
+                    lg_s[(sg + i) * L::lg_stride + col] = c0 + col < C ? acc[i][q] + bias_s[col] : -INFINITY;
+                }
+            __syncthreads();
+        }
+    }
+    // partial softmax of this class tile, eight lanes per sample; to every CTA of the cluster (a
+    // tile whose product timed out sends z = -1: no decision)
+    const bool failed = s_wfail != 0;
+    const int l8 = lane & 7;
+    for (int k = tid >> 3; active && k < BT; k += kExitThreads / 8) {   // uniform per warp
+        const float *l = lg_s + k * L::lg_stride + l8;
+        float m = -INFINITY, z = 0.0f;
+#pragma unroll
+        for (int q = 0; q < kExitCT; q += 8) m = fmaxf(m, l[q]);
+#pragma unroll
+        for (int o = 4; o >= 1; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+#pragma unroll
+        for (int q = 0; q < kExitCT; q += 8)
+            if (l[q] != -INFINITY) z += expf(l[q] - m);
+#pragma unroll
+        for (int o = 4; o >= 1; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
+        if (l8 < ncl)
+            *cl.map_shared_rank(part_s + k * 8 + rank, l8) = failed ? make_float2(0.0f, -1.0f) : make_float2(m, z);
+    }
+    cl.sync();   // every CTA holds every partial of the tile's samples
+    // every CTA merges the partials in the same order; the owner writes the decision, every CTA its
+    // logits tile of the samples that exit
+    for (int k = tid >> 3; active && k < BT; k += kExitThreads / 8) {
+        const int sw = s0 + k;
+        const float2 pz = l8 < ncl ? part_s[k * 8 + l8] : make_float2(-INFINITY, 0.0f);
+        float m = pz.x, bad = pz.y < 0.0f ? 1.0f : 0.0f;
+#pragma unroll
+        for (int o = 4; o >= 1; o >>= 1) {
+            m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+            bad = fmaxf(bad, __shfl_xor_sync(0xFFFFFFFFu, bad, o));
+        }
+        float z = l8 < ncl ? pz.y * expf(pz.x - m) : 0.0f;
+#pragma unroll
+        for (int o = 4; o >= 1; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
+        if (bad != 0.0f || sw >= B) continue;   // a product timed out (status raised): no decision
+        const float c = 1.0f / z;   // max_k softmax = exp(l_max - l_max) / sum
+        const bool ex = c >= p.head.tau;
+        if (l8 == 0) {
+            if (ex) {
+                cnt_s[k] = -1;
+                bits_s[k] &= ~kPlanRhoNonfinite;
+            }
+            if (k % ncl == rank) {
+                p.exit_mask[sw] = ex ? 1 : 0;
+                if (p.max_prob) p.max_prob[sw] = c;
+                if (!isfinite(m)) raise_status(p.status, FUSION_DEV_NONFINITE);
+            }
+        }
+        if (ex && p.logits)   // logits only for the samples that exit
+#pragma unroll
+            for (int q = 0; q < kExitCT; q += 8)
+                if (c0 + l8 + q < C) p.logits[(size_t)sw * C + c0 + l8 + q] = lg_s[k * L::lg_stride + l8 + q];
+    }
+    if (rank != 0) return;   // no CTA reads another's shared memory any more
+    if (!p.do_plan) {
+        if (Bdev < 0 && bt == 0 && tid == 0) raise_status(p.status, FUSION_DEV_BAD_BATCH);
+        return;
+    }
+    // ---- the plan: this tile's counts and totals, then the last tile's scan of all totals ----------
+    __syncthreads();   // the counts are complete
+    if (active && warp == 0) {
+        const int k0 = min(lane, BT - 1), k1 = min(lane + 32, BT - 1);
+        const int c[2] = {cnt_s[k0], cnt_s[k1]};
+        plan_tile(p.plan, bt, B, c, bits_s[k0] | bits_s[k1]);
+        __threadfence();
+    }
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(p.plan.counter, 1) == p.n_btile - 1;
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    if (tid == 0) p.counters[p.n_btile] = 0;
-    run_plan(p.plan, reinterpret_cast<int *>(w_region));
+    if (tid == 0) *p.plan.counter = 0;
+    plan_scan(p.plan, Bdev);
 }
-
 }  // namespace
 
 size_t exit_smem_bytes(int dtype, int dim) {
@@ -1153,12 +1514,77 @@ cudaError_t launch_exit_cluster(const ExitParams &p, cudaStream_t s) {
     return cudaLaunchKernelEx(&cfg, k_exit_cl<T>, wmap, q);
 }
 
+namespace {
+template <typename T, int BT>
+cudaError_t launch_exit_rows(const ExitParams &p, cudaStream_t s) {
+    CUtensorMap wmap;
+    cudaError_t e = head_weight_map(sizeof(T) == 2 ? FUSION_BF16 : FUSION_F32, p, &wmap);
+    if (e != cudaSuccess) return e;
+    const size_t smem = ExitRowsSmem<T, BT>::total(p.dim);
+    e = cudaFuncSetAttribute(k_exit_rows<T, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    ExitParams q = p;   // at least one tile: with max_batch == 0 the kernel still runs the plan
+    q.n_btile = ceil_div(p.in.max_batch > 0 ? p.in.max_batch : 1, BT);
+    q.lg_tmp = nullptr;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(q.n_ctile, q.n_btile);
+    cfg.blockDim = dim3(kExitThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = p.n_ctile;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_exit_rows<T, BT>, wmap, q);
+}
+
+size_t exit_rows_smem(int dtype, int bt, int dim) {
+    if (dtype == FUSION_BF16)
+        return bt == 16 ? ExitRowsSmem<__nv_bfloat16, 16>::total(dim)
+                        : bt == 32 ? ExitRowsSmem<__nv_bfloat16, 32>::total(dim) : ExitRowsSmem<__nv_bfloat16, 64>::total(dim);
+    return bt == 16 ? ExitRowsSmem<float, 16>::total(dim)
+                    : bt == 32 ? ExitRowsSmem<float, 32>::total(dim) : ExitRowsSmem<float, 64>::total(dim);
+}
+
+// The linear head's samples per cluster: 8 (k_exit_cl, several warps per LayerNorm row) while the
+// class tiles of all sample tiles fit one wave of two CTAs per SM, else the smallest of 16, 32 and 64
+// (k_exit_rows, one warp per row) whose tiles do, 64 for the largest batches: a larger tile reads the
+// weights for more samples (8192 samples x 100 classes at d = 384 read them 1024 times in tiles of 8),
+// a smaller one has more CTAs to spread.  The plan's tiles are at least 32.  0: the general kernel.
+int exit_samples_per_tile(int dtype, const ExitParams &p, bool plan) {
+    if (!(p.n_ctile <= kExitClMaxTiles && p.in_mode == 0 && !p.skip_ln && p.out_mode == 0)) return 0;
+    constexpr int kSms = 152;
+    const long long B = p.in.max_batch > 0 ? p.in.max_batch : 1;
+    if (!plan && (long long)p.n_ctile * ((B + 7) / 8) <= 2 * kSms) return 8;
+    int best = 0;
+    for (int bt = plan ? 32 : 16; bt <= 64; bt *= 2) {
+        const size_t smem = exit_rows_smem(dtype, bt, p.dim);
+        if (smem > 226 * 1024) break;
+        best = bt;
+        const int per_sm = smem <= kExitClBudget ? 2 : 1;
+        if ((long long)p.n_ctile * ((B + bt - 1) / bt) <= (long long)per_sm * kSms) break;
+    }
+    return best;
+}
+}  // namespace
+
+int exit_plan_tile(int dtype, const ExitParams &p) { return exit_samples_per_tile(dtype, p, true); }
+
 cudaError_t launch_exit(int dtype, const ExitParams &p, cudaStream_t s) {
     // the class tiles of a sample tile as one cluster (portable size: at most 8 tiles,
     // 1024 classes); larger heads take the kernel with a global last-CTA merge
-    if (p.n_ctile <= kExitClMaxTiles && p.in_mode == 0 && !p.skip_ln && p.out_mode == 0)
-        return dtype == FUSION_BF16 ? launch_exit_cluster<__nv_bfloat16>(p, s) : launch_exit_cluster<float>(p, s);
-    return dtype == FUSION_BF16 ? launch_exit_general<__nv_bfloat16>(p, s, false) : launch_exit_general<float>(p, s, false);
+    const bool b16 = dtype == FUSION_BF16;
+    switch (exit_samples_per_tile(dtype, p, p.do_plan)) {
+    case 8: return b16 ? launch_exit_cluster<__nv_bfloat16>(p, s) : launch_exit_cluster<float>(p, s);
+    case 16: return b16 ? launch_exit_rows<__nv_bfloat16, 16>(p, s) : launch_exit_rows<float, 16>(p, s);
+    case 32: return b16 ? launch_exit_rows<__nv_bfloat16, 32>(p, s) : launch_exit_rows<float, 32>(p, s);
+    case 64: return b16 ? launch_exit_rows<__nv_bfloat16, 64>(p, s) : launch_exit_rows<float, 64>(p, s);
+    default: break;
+    }
+    return b16 ? launch_exit_general<__nv_bfloat16>(p, s, false) : launch_exit_general<float>(p, s, false);
 }
 
 // The general kernel as a programmatic dependent launch: its CTAs may start as the previous
@@ -1169,15 +1595,38 @@ cudaError_t launch_exit_pdl(int dtype, const ExitParams &p, cudaStream_t s) {
 }
 
 namespace {
+// The plan alone: a warp per tile of kPlanTile samples, the last block scans the tiles.
 __global__ void __launch_bounds__(kPlanThreads) k_plan(PlanArgs a) {
-    extern __shared__ int plan_sm[];
-    run_plan(a, plan_sm);
+    __shared__ int s_last;
+    const int lane = threadIdx.x & 31, t = blockIdx.x * (kPlanThreads / 32) + (threadIdx.x >> 5);
+    const int B = device_batch(a.in);
+    if (t * kPlanTile < B) {
+        const int i = t * kPlanTile + lane;
+        int bits = 0, c = -1;
+        if (i < B) {
+            const int n = plan_count(a, i, bits);
+            if (a.exit_mask && a.exit_mask[i] != 0)
+                bits &= ~kPlanRhoNonfinite;
+            else
+                c = n;
+        }
+        const int cc[2] = {c, -1};
+        plan_tile(a, t, B, cc, bits);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(a.counter, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x == 0) *a.counter = 0;
+    plan_scan(a, B);
 }
 }  // namespace
 
 cudaError_t launch_plan(const PlanArgs &a, cudaStream_t s) {
-    const size_t smem = plan_smem_bytes(kPlanThreads);
-    k_plan<<<1, kPlanThreads, smem, s>>>(a);
+    const int tiles = ceil_div(a.in.max_batch > 0 ? a.in.max_batch : 1, kPlanTile);
+    k_plan<<<ceil_div(tiles, kPlanThreads / 32), kPlanThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -56,7 +56,7 @@ Head dev(const fusion_exit_head &h) {
 }
 
 struct Ws {
-    int *slot;
+    int *cnt;
     int *plan;
     int *counters;
     float2 *partials;
@@ -69,6 +69,15 @@ Ws carve(void *ws, int32_t max_batch, int32_t classes) {
     return Ws{reinterpret_cast<int *>(b + L.slot), reinterpret_cast<int *>(b + L.plan),
               reinterpret_cast<int *>(b + L.counters), reinterpret_cast<float2 *>(b + L.partials),
               L.total > L.lg ? reinterpret_cast<float *>(b + L.lg) : nullptr};
+}
+
+// The plan's scratch for batches above the fused plan's bound.
+void plan_scratch(PlanArgs &pa, const Ws &w, int32_t max_batch) {
+    pa.cnt = w.cnt;
+    pa.plan = w.plan;
+    pa.agg = reinterpret_cast<int4 *>(w.partials);
+    pa.counter = w.counters + ceil_div(max_batch > 0 ? max_batch : 1, kExitBT);
+    pa.pt = kPlanTile;
 }
 
 int cuda_rc(cudaError_t e) { return e == cudaSuccess ? FUSION_OK : FUSION_ERR_CUDA; }
@@ -109,8 +118,7 @@ void record(cudaEvent_t e, cudaStream_t s) {
 
 ImageParams image_params(const fusion_ragged &in, const void *x, int32_t dim, const void *keys,
                          int32_t key_dim, const float *sizes, const float *scores, const int32_t *r,
-                         const float *rho, int do_merge, int do_prune, const Ws &w,
-                         const int32_t *offsets_out, void *x_out, float *sizes_out, float *scores_out,
+                         const float *rho, int do_merge, int do_prune, void *x_out, float *sizes_out, float *scores_out,
                          int32_t *keep_idx, int32_t *dst_map, int32_t *a_match, int32_t *status,
                          const ImageGeometry &G) {
     ImageParams p{};
@@ -127,9 +135,6 @@ ImageParams image_params(const fusion_ragged &in, const void *x, int32_t dim, co
     p.do_merge = do_merge;
     p.do_prune = do_prune;
     p.need_match = a_match != nullptr;
-    p.slot = w.slot;
-    p.plan = w.plan;
-    p.offsets_out = offsets_out;
     p.x_out = x_out;
     p.sizes_out = sizes_out;
     p.scores_out = scores_out;
@@ -233,13 +238,12 @@ int fusion_merge(int dtype, fusion_ragged in, const void *x, int32_t dim, const 
     pa.merge = 1;
     pa.r = r;
     pa.offsets_out = offsets_out;
-    pa.slot = w.slot;
-    pa.plan = w.plan;
+    plan_scratch(pa, w, in.max_batch);
     pa.status = dev_status;
     record(ev.start, s);
     if (!fuse_plan(in)) FZ_TRY(cuda_rc(launch_plan(pa, s)));
     record(ev.mid, s);
-    ImageParams p = image_params(in, x, dim, keys, key_dim, sizes, scores, r, nullptr, 1, 0, w, offsets_out,
+    ImageParams p = image_params(in, x, dim, keys, key_dim, sizes, scores, r, nullptr, 1, 0,
                                  x_out, sizes_out, scores_out, keep_idx, dst_map, a_match, dev_status, G);
     p.fused_plan = fuse_plan(in);
     p.plan_args = pa;
@@ -301,14 +305,13 @@ int fusion_prune(int dtype, fusion_ragged in, const void *x, int32_t dim, const 
     pa.prune = 1;
     pa.rho = rho;
     pa.offsets_out = offsets_out;
-    pa.slot = w.slot;
-    pa.plan = w.plan;
+    plan_scratch(pa, w, in.max_batch);
     pa.status = dev_status;
     const ProfileEvents ev = take_profile();
     record(ev.start, s);
     if (!fuse_plan(in)) FZ_TRY(cuda_rc(launch_plan(pa, s)));
     record(ev.mid, s);
-    ImageParams p = image_params(in, x, dim, nullptr, dim, sizes, scores, nullptr, rho, 0, 1, w, offsets_out,
+    ImageParams p = image_params(in, x, dim, nullptr, dim, sizes, scores, nullptr, rho, 0, 1,
                                  x_out, sizes_out, scores_out, keep_idx, nullptr, nullptr, dev_status, G);
     p.fused_plan = fuse_plan(in);
     p.plan_args = pa;
@@ -340,14 +343,13 @@ int fusion_compact(int dtype, fusion_ragged in, const void *x, int32_t dim, cons
     pa.offsets_out = offsets_out;
     pa.ids_out = ids_out;
     pa.batch_out = batch_out;
-    pa.slot = w.slot;
-    pa.plan = w.plan;
+    plan_scratch(pa, w, in.max_batch);
     pa.status = dev_status;
     const ProfileEvents ev = take_profile();
     record(ev.start, s);
     if (!fuse_plan(in)) FZ_TRY(cuda_rc(launch_plan(pa, s)));
     record(ev.mid, s);
-    ImageParams p = image_params(in, x, dim, nullptr, dim, sizes, scores, nullptr, nullptr, 0, 0, w, offsets_out,
+    ImageParams p = image_params(in, x, dim, nullptr, dim, sizes, scores, nullptr, nullptr, 0, 0,
                                  x_out, sizes_out, scores_out, keep_idx, nullptr, nullptr, dev_status, G);
     p.fused_plan = fuse_plan(in);
     p.plan_args = pa;
@@ -639,8 +641,7 @@ int stage_impl(int dtype, int flags, const fusion_ragged &in, const void *x, int
     pa.offsets_out = offsets_out;
     pa.ids_out = ids_out;
     pa.batch_out = batch_out;
-    pa.slot = w.slot;
-    pa.plan = w.plan;
+    plan_scratch(pa, w, in.max_batch);
     pa.status = dev_status;
     if (do_exit && mlp && do_merge) {
         // The MLP head reads the merged tokens (Sec. III-B): merge into the workspace, the exit
@@ -660,7 +661,7 @@ int stage_impl(int dtype, int flags, const fusion_ragged &in, const void *x, int
         pm.ids_out = nullptr;
         pm.batch_out = nullptr;
         if (!fuse_plan(in)) FZ_TRY(cuda_rc(launch_plan(pm, s)));
-        ImageParams q = image_params(in, x, dim, keys, key_dim, sizes, scores, r, nullptr, 1, 0, w, offs_m, x_m, sizes_m,
+        ImageParams q = image_params(in, x, dim, keys, key_dim, sizes, scores, r, nullptr, 1, 0, x_m, sizes_m,
                                      scores_m, keep_m, nullptr, a_match, dev_status, G);
         q.fused_plan = fuse_plan(in);
         q.plan_args = pm;
@@ -676,8 +677,8 @@ int stage_impl(int dtype, int flags, const fusion_ragged &in, const void *x, int
         if (!fuse_plan(in)) FZ_TRY(cuda_rc(launch_plan(pc, s)));
         const ImageGeometry G2 = image_geometry(dtype, in.max_tokens, dim, 0);
         if (!G2.ok) return FUSION_ERR_SHAPE;
-        ImageParams c = image_params(in_m, x_m, dim, nullptr, dim, sizes_m, scores_m, nullptr, rho, 0, do_prune, w,
-                                     offsets_out, x_out, sizes_out, scores_out, keep_idx, nullptr, nullptr, dev_status, G2);
+        ImageParams c = image_params(in_m, x_m, dim, nullptr, dim, sizes_m, scores_m, nullptr, rho, 0, do_prune,
+                                     x_out, sizes_out, scores_out, keep_idx, nullptr, nullptr, dev_status, G2);
         c.keep_map = keep_m;
         c.fused_plan = fuse_plan(in);
         c.plan_args = pc;
@@ -704,16 +705,20 @@ int stage_impl(int dtype, int flags, const fusion_ragged &in, const void *x, int
         e.lg_tmp = logits ? w.lg : nullptr;
         e.n_ctile = ceil_div(head.classes, kExitCT);
         e.n_btile = ceil_div(in.max_batch > 0 ? in.max_batch : 1, kExitBT);
-        e.do_plan = !fuse_plan(in);
-        e.plan = pa;
         e.status = dev_status;
+        const int pt = fuse_plan(in) ? 0 : exit_plan_tile(dtype, e);
+        if (pt > 0) pa.pt = pt;
+        e.do_plan = pt > 0;
+        e.plan = pa;
+        e.plan_follows = !fuse_plan(in) && pt == 0;
         FZ_TRY(cuda_rc(launch_exit(dtype, e, s)));
+        if (!fuse_plan(in) && pt == 0) FZ_TRY(cuda_rc(launch_plan(pa, s)));
     } else if (!fuse_plan(in)) {
         FZ_TRY(cuda_rc(launch_plan(pa, s)));
     }
     record(ev.mid, s);
     ImageParams p = image_params(in, x, dim, do_merge ? keys : nullptr, key_dim, sizes, scores, r, rho, do_merge,
-                                 do_prune, w, offsets_out, x_out, sizes_out, scores_out, keep_idx, nullptr, a_match,
+                                 do_prune, x_out, sizes_out, scores_out, keep_idx, nullptr, a_match,
                                  dev_status, G);
     p.fused_plan = fuse_plan(in);
     p.plan_args = pa;

@@ -24,8 +24,9 @@ struct ExitParams {
                      // no logits are requested or the cluster kernel runs
     int n_ctile;
     int n_btile;
-    int do_plan;     // run the compaction plan in the last CTA
+    int do_plan;     // the compaction plan runs here (k_exit_rows: its tiles, then the last cluster's scan)
     PlanArgs plan;
+    int plan_follows;   // a plan kernel runs after this one (and reports a bad batch count)
     int *status;
     // the layers of an MLP exit head (zero for the linear head of the ragged CLS rows)
     int in_mode;     // 0: CLS rows of the ragged batch x; 1: dense rows x[s] of [B, dim]; 2: dense float32 rows u_in[s]
@@ -36,6 +37,9 @@ struct ExitParams {
     void *hidden_out;    // [max_batch, classes] for out_mode 1
 };
 cudaError_t launch_exit(int dtype, const ExitParams &p, cudaStream_t s);
+// Samples per plan tile of the kernel that launch_exit picks for a call with do_plan, or 0 when that
+// kernel cannot run the plan (the caller then launches the plan kernel after it).
+int exit_plan_tile(int dtype, const ExitParams &p);
 size_t exit_smem_bytes(int dtype, int dim);
 
 // ---- merge router with profile scaling ----------------------------------------------
@@ -116,9 +120,6 @@ struct ImageParams {
     int do_merge;
     int do_prune;
     int need_match;      // compute matches even when no token merges (a_match requested)
-    const int *slot;     // workspace: output sample of every input sample (-1: gone)
-    const int *plan;     // workspace: plan[0] = batch valid
-    const int *offsets_out;
     void *x_out;
     float *sizes_out;
     float *scores_out;
@@ -129,8 +130,8 @@ struct ImageParams {
     int *dst_map;
     int *a_match;
     int *status;
-    // fused_plan: no plan kernel ran; every CTA derives its sample's slot and output
-    // offset from plan_args (which also receives the plan's outputs)
+    // fused_plan: no plan kernel ran; every CTA derives its sample's place in the output from
+    // the whole batch (which also writes the plan's outputs); otherwise from the plan's tiles
     int fused_plan;
     PlanArgs plan_args;
     // staging geometry, fixed by the host from max_tokens and the key width

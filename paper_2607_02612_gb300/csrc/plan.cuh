@@ -19,123 +19,120 @@ struct PlanArgs {
     int *offsets_out;          // [max_batch + 1]
     int *ids_out;              // [max_batch] or NULL
     int *batch_out;            // device scalar or NULL
-    int *slot;                 // workspace [max_batch]: output sample of every input sample, -1 if gone
-    int *plan;                 // workspace [4]: ok flag, survivor count
+    // batches above the fused plan's bound (scratch in the workspace):
+    int *cnt;                  // [max_batch]: output rows of every input sample, -1 if gone
+    int4 *agg;                 // [tiles of pt samples]: survivors and rows before the tile (x, y)
+    int *plan;                 // [4]: ok flag, survivor count
+    int *counter;              // zero between calls
+    int pt;                    // samples per tile (32 or 64)
     int *status;
 };
 
-// Samples staged in shared memory per round of the plan.
-constexpr int kPlanChunk = 2048;
+constexpr int kPlanRhoNonfinite = 1 << 30;   // a continuing sample's keep ratio is NaN or infinite
 
-// Shared memory run_plan needs for a block of nt threads: per round the chunk's offsets, ids,
-// counts and flags, then the block scan's scratch.
-__host__ __device__ inline size_t plan_smem_bytes(int nt) {
-    return (size_t)(3 * kPlanChunk + 1 + 2 * nt + 40) * sizeof(int) + kPlanChunk;
+// The plan of a batch above the fused plan's bound, in tiles of pt samples.  plan_tile, one warp:
+// a tile's output counts and its totals.  plan_scan, one block once every tile is done: the totals
+// become exclusive prefixes, and the batch-level outputs are written.  The per-sample kernel adds
+// the prefix inside its tile itself (sample_info), so no serial pass over the samples remains:
+// one block over 8192 samples took about 20 us, the tiles run beside one another in the kernel that
+// makes the exit decisions and the scan of 128 totals takes about 2.
+//
+// plan_count: the output rows of sample i if it continues (its merge and prune counts are inputs of
+// the call, so a kernel can take them before it knows who continues), 0 with `bits` set when its
+// offsets or id are malformed.
+__device__ __forceinline__ int plan_count(const PlanArgs &a, int i, int &bits) {
+    const int o0 = a.in.offsets[i], o1 = a.in.offsets[i + 1];
+    const int id = a.in.ids ? a.in.ids[i] : i;
+    const int N = o1 - o0;
+    const bool ok = o0 >= 0 && N >= 1 && N <= a.in.max_tokens && (long long)o1 <= a.in.max_rows;
+    const bool id_ok = id >= 0 && id < a.in.max_batch;
+    if (!ok) bits |= FUSION_DEV_BAD_OFFSETS;
+    if (!id_ok) bits |= FUSION_DEV_BAD_IDS;
+    if (!ok || !id_ok) return 0;
+    int c = N;
+    if (a.merge) c -= merge_count(a.r[id], N - 1);
+    if (a.prune) {
+        bool f = false;
+        c = 1 + keep_count(a.rho[id], c - 1, f);
+        if (f) bits |= kPlanRhoNonfinite;
+    }
+    return c;
 }
 
-// Run by ONE thread block (any size, multiple of 32) with plan_smem_bytes(blockDim.x) of shared
-// memory at `smem`.  The batch is taken in rounds of kPlanChunk samples: the round's offsets,
-// ids and exit flags are staged in shared memory with every load in flight at once, then the
-// merge counts and keep ratios by id; each thread sums a contiguous segment of the round, the
-// segment totals are scanned, and each thread writes its segment's slots, offsets and ids.
-__device__ inline void run_plan(const PlanArgs &a, int *smem) {
-    const int nt = blockDim.x;
-    int *o_s = smem;                          // [kPlanChunk + 1] offsets of the round
-    int *id_s = o_s + kPlanChunk + 1;         // [kPlanChunk] ids
-    int *cnt_s = id_s + kPlanChunk;           // [kPlanChunk] output counts (0 when the sample is gone)
-    int *flags = cnt_s + kPlanChunk;          // [nt] segment survivor counts, then their scan
-    int *cnts = flags + nt;                   // [nt] segment row counts, then their scan
-    int *tmp = cnts + nt;                     // 40 ints
-    unsigned char *sv_s = reinterpret_cast<unsigned char *>(tmp + 40);   // [kPlanChunk] survives
-    __shared__ int s_bad, s_nonfinite;
-    const int t = threadIdx.x;
-    if (t == 0) {
-        s_bad = 0;
-        s_nonfinite = 0;
+// Tile t of the plan by one warp: lane and lane + 32 bring their samples' counts (-1: gone, or
+// beyond the batch count B) and bits.
+__device__ __forceinline__ void plan_tile(const PlanArgs &a, int t, int B, const int (&c)[2], int bits) {
+    const int lane = threadIdx.x & 31;
+    int surv = 0, rows = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int k = lane + 32 * h, i = t * a.pt + k;
+        if (k >= a.pt || i >= B) continue;
+        a.cnt[i] = c[h];
+        if (c[h] >= 0) {
+            ++surv;
+            rows += c[h];
+        }
     }
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) {
+        surv += __shfl_xor_sync(0xFFFFFFFFu, surv, m);
+        rows += __shfl_xor_sync(0xFFFFFFFFu, rows, m);
+        bits |= __shfl_xor_sync(0xFFFFFFFFu, bits, m);
+    }
+    if (lane == 0) a.agg[t] = make_int4(surv, rows, bits, 0);
+}
+
+// Run by one block (any size, a multiple of 32); B: the device batch count, -1 when out of range.
+__device__ inline void plan_scan(const PlanArgs &a, int B) {
+    __shared__ int wsum[2][32], s_bad;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
+    if (t == 0) s_bad = 0;
     __syncthreads();
-
-    int B = device_batch(a.in);
-    if (B < 0) {
-        if (t == 0) {
-            raise_status(a.status, FUSION_DEV_BAD_BATCH);
-            a.plan[0] = 0;
-            a.plan[1] = 0;
-            a.offsets_out[0] = 0;
-            if (a.batch_out) *a.batch_out = 0;
-        }
-        return;
-    }
-
-    int base_s = 0;   // survivors so far
-    int base_r = 0;   // output rows so far
-    for (int c0 = 0; c0 < B; c0 += kPlanChunk) {
-        const int n = min(kPlanChunk, B - c0);
-        for (int k = t; k <= n; k += nt) o_s[k] = a.in.offsets[c0 + k];
-        for (int k = t; k < n; k += nt) {
-            id_s[k] = a.in.ids ? a.in.ids[c0 + k] : c0 + k;
-            sv_s[k] = (a.exit_mask == nullptr || __ldcg(a.exit_mask + c0 + k) == 0) ? 1 : 0;
-        }
-        __syncthreads();
-        for (int k = t; k < n; k += nt) {
-            const int o0 = o_s[k], o1 = o_s[k + 1];
-            const int N = o1 - o0;
-            const bool ok = o0 >= 0 && N >= 1 && N <= a.in.max_tokens && (long long)o1 <= a.in.max_rows;
-            const int id = id_s[k];
-            const bool id_ok = id >= 0 && id < a.in.max_batch;
-            if (!ok) atomicOr(&s_bad, FUSION_DEV_BAD_OFFSETS);
-            if (!id_ok) atomicOr(&s_bad, FUSION_DEV_BAD_IDS);
-            int cnt = 0;
-            if (ok && id_ok && sv_s[k]) {
-                int nn = N;
-                if (a.merge) nn -= merge_count(a.r[id], N - 1);
-                if (a.prune) {
-                    bool nf = false;
-                    nn = 1 + keep_count(a.rho[id], nn - 1, nf);
-                    if (nf) s_nonfinite = 1;
-                }
-                cnt = nn;
-            }
-            cnt_s[k] = cnt;
-        }
-        __syncthreads();
-        // contiguous segments of the round, one per thread
-        const int seg = (n + nt - 1) / nt;
-        const int k0 = min(n, t * seg), k1 = min(n, k0 + seg);
-        int ss = 0, rr = 0;
-        for (int k = k0; k < k1; ++k) {
-            ss += sv_s[k];
-            rr += cnt_s[k];
-        }
-        flags[t] = ss;
-        cnts[t] = rr;
-        __syncthreads();
-        const int tot_s = block_scan_excl(flags, nt, tmp);
-        const int tot_r = block_scan_excl(cnts, nt, tmp);
-        int js = base_s + flags[t], jr = base_r + cnts[t];
-        for (int k = k0; k < k1; ++k) {
-            const int i = c0 + k;
-            if (sv_s[k]) {
-                a.slot[i] = js;
-                a.offsets_out[js] = jr;
-                if (a.ids_out) a.ids_out[js] = id_s[k];
-                ++js;
-                jr += cnt_s[k];
-            } else {
-                a.slot[i] = -1;
+    const int tiles = B > 0 ? (B + a.pt - 1) / a.pt : 0;
+    int base_s = 0, base_r = 0;
+    for (int t0 = 0; t0 < tiles; t0 += blockDim.x) {
+        int4 v = make_int4(0, 0, 0, 0);
+        if (t0 + t < tiles) v = __ldcg(a.agg + t0 + t);
+        if (v.z) atomicOr(&s_bad, v.z);
+        int is = v.x, ir = v.y;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int ys = __shfl_up_sync(0xFFFFFFFFu, is, o), yr = __shfl_up_sync(0xFFFFFFFFu, ir, o);
+            if (lane >= o) {
+                is += ys;
+                ir += yr;
             }
         }
-        base_s += tot_s;
-        base_r += tot_r;
-        __syncthreads();   // the staging arrays are reused by the next round
+        if (lane == 31) {
+            wsum[0][w] = is;
+            wsum[1][w] = ir;
+        }
+        __syncthreads();
+        int ps = base_s, pr = base_r, ts = 0, tr = 0;
+        for (int k = 0; k < nw; ++k) {
+            if (k < w) {
+                ps += wsum[0][k];
+                pr += wsum[1][k];
+            }
+            ts += wsum[0][k];
+            tr += wsum[1][k];
+        }
+        if (t0 + t < tiles) a.agg[t0 + t] = make_int4(ps + is - v.x, pr + ir - v.y, 0, 0);
+        base_s += ts;
+        base_r += tr;
+        __syncthreads();   // wsum is reused by the next round
     }
     if (t == 0) {
-        a.offsets_out[base_s] = base_r;
-        if (a.batch_out) *a.batch_out = base_s;
-        a.plan[0] = s_bad ? 0 : 1;
-        a.plan[1] = base_s;
-        if (s_bad) raise_status(a.status, s_bad);
-        if (s_nonfinite) raise_status(a.status, FUSION_DEV_NONFINITE);
+        const int bits = s_bad & ~kPlanRhoNonfinite;
+        const bool bad = B < 0 || bits != 0;
+        a.offsets_out[bad ? 0 : base_s] = bad ? 0 : base_r;
+        if (a.batch_out) *a.batch_out = bad ? 0 : base_s;
+        a.plan[0] = bad ? 0 : 1;
+        a.plan[1] = bad ? 0 : base_s;
+        if (B < 0) raise_status(a.status, FUSION_DEV_BAD_BATCH);
+        if (bits) raise_status(a.status, bits);
+        if (s_bad & kPlanRhoNonfinite) raise_status(a.status, FUSION_DEV_NONFINITE);
     }
 }
 

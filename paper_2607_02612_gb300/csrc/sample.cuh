@@ -101,28 +101,45 @@ struct SampleInfo {
     bool decide;   // the merge decisions are needed (something merges, or matches are requested)
 };
 
-// The input sample this CTA handles; false when there is nothing to do (beyond the
-// device batch count, an invalid call, or a sample that exited).
+// The input sample this CTA handles, from the plan kernel's tiles (plan.cuh); false when there is
+// nothing to do (beyond the device batch count, an invalid call, or a sample that exited).
 // The grid has one CTA per possible sample (i < max_batch), so every load of the first
-// group is in bounds whatever the device batch count says; they issue together, and the
-// second group (which needs the output slot and the original id) follows.
+// group is in bounds whatever the device batch count says (counts beyond it are whatever
+// an earlier call left, and are not used); they issue together.  Every warp adds the tile's counts
+// before the sample itself; thread 0 writes the sample's place in the output batch.
 __device__ __forceinline__ bool sample_info(const ImageParams &p, int i, SampleInfo &s) {
+    const PlanArgs &a = p.plan_args;
+    const int lane = threadIdx.x & 31;
     const int bval = p.in.batch ? *p.in.batch : p.in.max_batch;
-    const int valid = p.plan[0];
-    const int j = p.slot[i];
+    const int valid = a.plan[0];
+    const int t = i / a.pt, t0 = t * a.pt, own = i - t0;
+    const int4 base = a.agg[t];
+    const int c0 = t0 + lane < p.in.max_batch ? a.cnt[t0 + lane] : -1;
+    const int c1 = (a.pt > 32 && t0 + 32 + lane < p.in.max_batch) ? a.cnt[t0 + 32 + lane] : -1;
     const int o0 = p.in.offsets[i], o1 = p.in.offsets[i + 1];
     const int id = p.in.ids ? p.in.ids[i] : i;
-    if (bval < 0 || bval > p.in.max_batch || i >= bval || valid == 0 || j < 0) return false;
+    if (bval < 0 || bval > p.in.max_batch || i >= bval || valid == 0) return false;
+    const int cnt = __shfl_sync(0xFFFFFFFFu, own < 32 ? c0 : c1, own & 31);
+    if (cnt < 0) return false;
+    const bool b0 = lane < own && c0 >= 0, b1 = lane + 32 < own && c1 >= 0;
+    int rows = (b0 ? c0 : 0) + (b1 ? c1 : 0);
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) rows += __shfl_xor_sync(0xFFFFFFFFu, rows, m);
+    const int j = base.x + __popc(__ballot_sync(0xFFFFFFFFu, b0)) + __popc(__ballot_sync(0xFFFFFFFFu, b1));
     s.start = o0;
     s.N = o1 - o0;
-    s.out_start = p.offsets_out[j];
-    s.out_n = p.offsets_out[j + 1] - s.out_start;
+    s.out_start = base.y + rows;
+    s.out_n = cnt;
     s.id = id;
     s.P = s.N - 1;
     s.nA = s.P / 2;
     s.nB = (s.P + 1) / 2;
     s.r_eff = p.do_merge ? merge_count(p.r[s.id], s.P) : 0;
     s.decide = p.do_merge && s.nA > 0 && (s.r_eff > 0 || p.need_match);
+    if (threadIdx.x == 0) {
+        a.offsets_out[j] = s.out_start;
+        if (a.ids_out) a.ids_out[j] = id;
+    }
     return true;
 }
 

@@ -1,0 +1,124 @@
+"""Batches beyond one wave of CTAs (GPU only): the exit check in tiles of 16, 32 and 64 samples, the
+compaction plan in tiles, and the per-sample kernels that read it, against the oracle."""
+import os
+import sys
+
+import numpy as np
+import pytest
+import torch
+
+sys.path.insert(0, os.path.dirname(os.path.abspath(__file__)))
+
+import oracle  # noqa: E402
+import parity as P  # noqa: E402
+import paper_2607_02612_gb300 as fz  # noqa: E402
+from paper_2607_02612_gb300 import runner  # noqa: E402
+from test_gpu_edges import make_batch, make_head, run_stage_and_compare  # noqa: E402
+from workloads import StageSpec  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def gap_tau(b, head, share):
+    """tau in the widest gap near the upper `share` of the oracle's confidences: no decision at it."""
+    c = np.sort(oracle.exit_check(b.dtype, b.offsets, b.x, head)["max_prob"])[::-1]
+    k = max(1, int(share * len(c)))
+    at = range(max(1, k - 4), min(len(c), k + 5))
+    k = max(at, key=lambda j: c[j - 1] - c[j])
+    return float(np.float32(0.5 * (float(c[k - 1]) + float(c[k]))))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("batch,classes,dim", [
+    (2433, 10, 16),       # 16-sample tiles, a short last K-block
+    (2440, 128, 80),      # a whole class tile
+    (9729, 100, 384),     # 64-sample tiles of one class tile, a ragged last tile
+    (313, 1000, 384),     # 16-sample tiles, clusters of 8, a short last class tile
+    (641, 257, 1024),     # the widest rows, three class tiles
+])
+def test_exit_check_many_samples(dtype, batch, classes, dim):
+    b = make_batch(np.full(batch, 1), dim, dtype, seed=batch)
+    head = make_head(dim, classes, dtype, 0.5, scale=3.0 / np.sqrt(dim))
+    head.tau = gap_tau(b, head, 0.3)
+    f = runner.Fusion(batch, classes)
+    g = P.to_host(f.exit_check(P.device_batch(b), runner.head_tensors(head, dtype)), dtype)
+    assert int(f.status.item()) == 0
+    rep = P.Report()
+    P.compare_exit(rep, dtype, np.arange(batch), g["exit_mask"], g["logits"], g["max_prob"],
+                   oracle.exit_check(dtype, b.offsets, b.x, head))
+    rep.check()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("batch,classes,merge,prune", [
+    (1025, 20, True, True), (1025, 1100, True, False), (2500, 20, True, True), (4300, 0, True, True),
+    (1060, 0, False, True), (2500, 20, False, False)])
+def test_stage_with_tiled_plan(dtype, batch, classes, merge, prune):
+    """Batches above the fused plan's bound: the plan after either exit kernel, or alone."""
+    rng = np.random.default_rng(batch)
+    b = make_batch(rng.integers(1, 24, batch), 64, dtype, seed=batch, sizes="u1to4")
+    head = None
+    if classes:
+        head = make_head(64, classes, dtype, 0.5, scale=0.4)
+        head.tau = gap_tau(b, head, 0.4)
+    r = rng.integers(0, 12, batch).astype(np.int32) if merge else None
+    rho = rng.uniform(0.2, 1.0, batch).astype(np.float32) if prune else None
+    run_stage_and_compare(b, StageSpec(merge, head is not None, prune, r=r, rho=rho, head=head),
+                          f"B={batch} C={classes}")
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("count,classes", [(0, 20), (1, 20), (37, 20), (1088, 20), (37, 0)])
+def test_tiled_plan_device_count(dtype, count, classes):
+    """A device batch count below the host bound, with ids: only its samples are planned."""
+    batch = 1100
+    rng = np.random.default_rng(count)
+    b = make_batch(rng.integers(1, 20, batch), 64, dtype, seed=7)
+    db = P.device_batch(b)
+    db.batch = torch.tensor([count], dtype=torch.int32, device="cuda")
+    ids = rng.permutation(batch).astype(np.int32)
+    db.ids = torch.from_numpy(ids).cuda()
+    head = make_head(64, 20, dtype, 0.5, scale=0.4)
+    head.tau = gap_tau(b, head, 0.4)
+    r = rng.integers(0, 9, batch).astype(np.int32)
+    rho = rng.uniform(0.2, 1.0, batch).astype(np.float32)
+    f = runner.Fusion(batch, 20)
+    flags = 7 if classes else 5
+    o = f.stage(db, flags, torch.from_numpy(r).cuda(), torch.from_numpy(rho).cuda(),
+                runner.head_tensors(head, dtype) if classes else None)
+    torch.cuda.synchronize()
+    assert int(f.status.item()) == 0
+    nb = int(o["batch"][0])
+    if count == 0:
+        assert nb == 0 and int(o["offsets"][0]) == 0
+        return
+    sub = make_batch(np.diff(b.offsets)[:count], 64, dtype)
+    t = int(b.offsets[count])
+    sub.x, sub.keys, sub.sizes, sub.scores = b.x[:t], b.x[:t], b.sizes[:t], b.scores[:t]
+    ref = oracle.stage(sub, StageSpec(True, bool(classes), True, r=r[ids[:count]], rho=rho[ids[:count]],
+                                      head=head if classes else None))
+    assert nb == ref["n_out"]
+    np.testing.assert_array_equal(o["offsets"][:nb + 1].cpu().numpy(), ref["offsets"])
+    np.testing.assert_array_equal(o["ids"][:nb].cpu().numpy(), ids[ref["ids"]])
+    rows = int(ref["offsets"][-1])
+    np.testing.assert_array_equal(o["keep_idx"][:rows].cpu().numpy(), ref["keep_idx"])
+
+
+def test_tiled_plan_rejects_malformed_offsets():
+    """One bad sample among many: the status bit, an empty output batch, no token row written."""
+    b = make_batch(np.full(1200, 8), 64, "bf16", seed=3)
+    db = P.device_batch(b)
+    offs = db.offsets.clone()
+    offs[700] = int(offs[699]) - 1
+    db.offsets = offs
+    f = runner.Fusion(1200, 20)
+    head = runner.head_tensors(make_head(64, 20, "bf16", 0.5), "bf16")
+    for flags in (5, 7):
+        f.status.zero_()
+        o = f.stage_outputs(db, 7, head)
+        o["x"].fill_(7)
+        f.stage(db, flags, torch.full((1200,), 2, dtype=torch.int32, device="cuda"),
+                torch.full((1200,), 0.5, device="cuda"), head, out=o)
+        torch.cuda.synchronize()
+        assert int(f.status.item()) & fz.FUSION_DEV_BAD_OFFSETS
+        assert int(o["batch"][0]) == 0 and int(o["offsets"][0]) == 0 and torch.all(o["x"] == 7)
