@@ -167,6 +167,10 @@ cudaError_t launch_sample_kernel(int dtype, const ImageParams &p, const ImageGeo
     if (p.do_merge) {
         const TcGeometry T = image_tc_geometry(dtype, p.in.max_tokens, p.kdim, p.dim, p.in.max_rows, 1, kTcSmemBudgetKb);
         if (T.ok) return launch_image_tc(p, T, s, pdl);
+        if (dtype == FUSION_F32) {   // the general kernel for samples whose stages do not fit
+            const F32Geometry F = image_f32_geometry(p);
+            if (F.ok) return launch_image_f32(p, F, s);
+        }
     }
     return launch_image(dtype, p, G.smem, s);
 }

@@ -1,5 +1,7 @@
 // Per-sample merge (Sec. III-C) -> prune (Sec. III-E) -> gather into the
-// compacted output batch.  One CTA per input sample; a sample that exited (or is
+// compacted output batch, for whatever the float32 merge kernel (image_f32.cu) and the tcgen05 one
+// (image_tc.cu) do not take: pruning or compaction without merging, bf16 keys whose width is not a
+// multiple of 64, the longest float32 samples.  One CTA per input sample; a sample that exited (or is
 // beyond the device batch count) returns at once.
 //
 // Merge decisions.  The keys of half A (even positions) and half B (odd

@@ -1,0 +1,319 @@
+// Per-sample merge -> prune -> gather for float32 tokens: the similarity on FFMA with the key dims
+// streamed through two cp.async stages, so that several CTAs share an SM (large batches of small
+// samples), and clusters of CTAs per sample (small batches of long ones).
+//
+// A cluster of CL CTAs owns a sample.  Each takes a run of 16-row strips of half A against all of half
+// B: warp tiles of 16 x 16 (a thread 2 rows x 4 columns, 6 shared-memory wavefronts per 32 FFMA), the
+// accumulators in registers over the whole key width.  The row maxima go to every CTA of the cluster,
+// each repeats the decisions (they are short), rank 0 writes the index outputs and every CTA a range of
+// columns of the token rows.
+//
+// Sums are formed as the general kernel (image.cu) forms them, bit for bit: dot products in partial
+// sums of 16 dims, squared norms per block of `kc` dims with chunk c of a block in lane c % 32.
+//
+// Bound by the chain of latencies of one sample (loads, FFMA, decisions, gather) and, with enough
+// samples, by FFMA and L2.  The general kernel keeps a whole sample in shared memory (98 KB for 65
+// tokens of 384: two CTAs per SM) and gives 16 x 32 strips to warps, of which 65 tokens have two.
+// Measured, general kernel -> this one: 3277 of 8192 samples of 65 tokens, d = 384, continuing: 606 -> 269
+// us (and 69 -> 39 us for the 210 that the fourth stage of that chain keeps); 8 samples of 197 tokens,
+// keys of their own, clusters of 8: 101 -> 55 us.  All with cold caches.
+#include <cooperative_groups.h>
+
+#include "sample.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace fz {
+namespace {
+
+__host__ __device__ inline uint32_t stage_row(int kd) { return (uint32_t)(kd + 4) * 4u; }   // bytes; 16 (mod 32): 8 rows conflict-free
+
+// NT threads; TPW warp tiles held in registers per pass; NP > 0: squared norms summed from the stages,
+// NP rows per 16 threads (kd = 64, one norm block), else read again from global memory (L2).
+template <int NT, int TPW, int NP>
+__global__ void __launch_bounds__(NT, NT == 128 ? 5 : 2) k_merge_f32(ImageParams p, F32Geometry g) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    constexpr int kW = NT / 32;
+    const int CL = g.cluster;
+    const int rank = CL > 1 ? (int)(blockIdx.x % (unsigned)CL) : 0;
+    SampleInfo s;
+    if (!sample_begin<NT>(p, CL > 1 ? blockIdx.x / CL : blockIdx.x, s)) return;   // the same in every CTA of the cluster
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int kdim = p.kdim, kd = g.kd;
+    const uint32_t rs = stage_row(kd);
+    // this CTA's strips of half A
+    const int strips = (s.nA + 15) / 16, per = (strips + CL - 1) / CL;
+    const int a0 = min(s.nA, rank * per * 16), na = min(s.nA, a0 + per * 16) - a0;
+    const uint32_t stage_bytes = (uint32_t)(g.rows_a + g.rows_b) * rs;
+    unsigned char *const st0 = sm;
+    MetaPtrs m(sm, meta_layout(p.in.max_tokens, 2 * (size_t)stage_bytes));
+    const float *keys = reinterpret_cast<const float *>(p.keys);
+
+    const int n_stage = (kdim + kd - 1) / kd;
+    const int rows = na + s.nB;
+    // stage q: dims [q kd, ..) of the CTA's A rows, then of all B rows
+    auto issue = [&](int q) {
+        unsigned char *dst = st0 + (q & 1) * stage_bytes;
+        const int nch = min(kd, kdim - q * kd) / 4;
+        int row = tid / nch, c = tid - row * nch;
+        const int rstep = NT / nch, cstep = NT - rstep * nch;
+        while (row < rows) {
+            const bool isA = row < na;
+            const int tok = isA ? a0 + row : row - na;
+            const long long grow = s.start + (isA ? 2 + 2 * tok : 1 + 2 * tok);
+            cp_async16(dst + (uint32_t)(isA ? row : g.rows_a + tok) * rs + c * 16, keys + grow * kdim + q * kd + c * 4);
+            row += rstep;
+            c += cstep;
+            if (c >= nch) {
+                c -= nch;
+                ++row;
+            }
+        }
+        cp_async_commit();
+    };
+    const int MT = (na + 15) / 16, NG = (s.nB + 15) / 16, tiles = MT * NG;
+    const int n_pass = (tiles + kW * TPW - 1) / (kW * TPW);
+    const bool sim = s.decide && na > 0;
+    if (sim) {
+        issue(0);
+        if (n_stage > 1) issue(1);
+        else cp_async_commit();
+    }
+    meta_init<NT>(p, s, m);
+    __syncthreads();
+    if (s.decide) {
+        const int g8 = lane >> 2, t4 = lane & 3;
+        float nlo[NP > 0 ? NP : 1], nhi[NP > 0 ? NP : 1];
+#pragma unroll
+        for (int k = 0; k < (NP > 0 ? NP : 1); ++k) nlo[k] = nhi[k] = 0.0f;
+        for (int pass = 0; sim && pass < n_pass; ++pass) {
+            if (pass > 0) {
+                issue(0);
+                if (n_stage > 1) issue(1);
+                else cp_async_commit();
+            }
+            float acc[TPW][2][4];
+#pragma unroll
+            for (int w = 0; w < TPW; ++w)
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[w][i][e] = 0.0f;
+            for (int q = 0; q < n_stage; ++q) {
+                asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+                __syncthreads();
+                const unsigned char *st = st0 + (q & 1) * stage_bytes;
+                const int kw = min(kd, kdim - q * kd);   // a multiple of 16
+#pragma unroll
+                for (int w = 0; w < TPW; ++w) {
+                    const int tile = (pass * TPW + w) * kW + warp;
+                    if (tile >= tiles) continue;
+                    const int mt = tile / NG, ng = tile - mt * NG;
+                    // rows past the halves read stale or unwritten shared memory inside the stage: their
+                    // products are never used
+                    const unsigned char *ra = st + (uint32_t)(mt * 16 + g8) * rs;
+                    const unsigned char *rb = st + (uint32_t)(g.rows_a + ng * 16 + t4) * rs;
+#pragma unroll 1
+                    for (int k0 = 0; k0 < kw; k0 += 16) {
+                        float t[2][4] = {};
+#pragma unroll
+                        for (int kk = 0; kk < 16; kk += 4) {
+                            const uint32_t o = (uint32_t)(k0 + kk) * 4;
+                            const float4 va = *reinterpret_cast<const float4 *>(ra + o);
+                            const float4 vb = *reinterpret_cast<const float4 *>(ra + 8 * rs + o);
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const float4 b = *reinterpret_cast<const float4 *>(rb + (uint32_t)(4 * e) * rs + o);
+                                t[0][e] = fmaf(va.x, b.x, t[0][e]);
+                                t[1][e] = fmaf(vb.x, b.x, t[1][e]);
+                                t[0][e] = fmaf(va.y, b.y, t[0][e]);
+                                t[1][e] = fmaf(vb.y, b.y, t[1][e]);
+                                t[0][e] = fmaf(va.z, b.z, t[0][e]);
+                                t[1][e] = fmaf(vb.z, b.z, t[1][e]);
+                                t[0][e] = fmaf(va.w, b.w, t[0][e]);
+                                t[1][e] = fmaf(vb.w, b.w, t[1][e]);
+                            }
+                        }
+#pragma unroll
+                        for (int i = 0; i < 2; ++i)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) acc[w][i][e] += t[i][e];
+                    }
+                }
+                if constexpr (NP > 0) {   // chunk c = 16 q + l of the row: lane c % 32 of the general kernel's sum
+                    const int l = tid & 15, r0 = tid >> 4;
+                    if (l * 4 < kw) {
+#pragma unroll
+                        for (int k = 0; k < NP; ++k) {
+                            const int row = r0 + k * (NT / 16);
+                            if (row >= rows) continue;
+                            const float4 f = *reinterpret_cast<const float4 *>(
+                                st + (uint32_t)(row < na ? row : g.rows_a + row - na) * rs + l * 16);
+                            float v = (q & 1) ? nhi[k] : nlo[k];
+                            v = fmaf(f.x, f.x, v);
+                            v = fmaf(f.y, f.y, v);
+                            v = fmaf(f.z, f.z, v);
+                            v = fmaf(f.w, f.w, v);
+                            if (q & 1) nhi[k] = v;
+                            else nlo[k] = v;
+                        }
+                    }
+                }
+                __syncthreads();   // everyone is done with this stage
+                if (q + 2 < n_stage) issue(q + 2);
+                else cp_async_commit();   // an empty group keeps the count
+            }
+            if (pass == 0) {
+                // inverse norms of the CTA's A rows and of the B rows
+                auto put = [&](int row, float v) {
+                    if (!isfinite(v)) raise_status(p.status, FUSION_DEV_NONFINITE);
+                    const float inv = 1.0f / fmaxf(sqrtf(v), 1e-12f);
+                    if (row < na) m.inv_a[a0 + row] = inv;
+                    else m.inv_b[row - na] = inv;
+                };
+                if constexpr (NP > 0) {
+#pragma unroll
+                    for (int k = 0; k < NP; ++k) {
+                        float v = nlo[k] + nhi[k];
+#pragma unroll
+                        for (int o = 8; o >= 1; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+                        const int row = (tid >> 4) + k * (NT / 16);
+                        if ((tid & 15) == 0 && row < rows) put(row, v);
+                    }
+                } else {
+                    for (int row = warp; row < rows; row += kW) {
+                        const int tok = row < na ? a0 + row : row - na;
+                        const float *src = keys + (long long)(s.start + (row < na ? 2 + 2 * tok : 1 + 2 * tok)) * kdim;
+                        float v = 0.0f;
+                        for (int k0 = 0; k0 < kdim; k0 += p.kc) {
+                            const int nch = min(p.kc, kdim - k0) / 4;
+                            float sq = 0.0f;
+#pragma unroll 4
+                            for (int c = lane; c < nch; c += 32) {
+                                const float4 f = __ldg(reinterpret_cast<const float4 *>(src + k0) + c);
+                                sq = fmaf(f.x, f.x, sq);
+                                sq = fmaf(f.y, f.y, sq);
+                                sq = fmaf(f.z, f.z, sq);
+                                sq = fmaf(f.w, f.w, sq);
+                            }
+#pragma unroll
+                            for (int o = 16; o >= 1; o >>= 1) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, o);
+                            v += sq;
+                        }
+                        if (lane == 0) put(row, v);
+                    }
+                }
+                __syncthreads();
+            }
+            // cosine and row maximum with the lowest column on ties
+#pragma unroll
+            for (int w = 0; w < TPW; ++w) {
+                const int tile = (pass * TPW + w) * kW + warp;
+                if (tile >= tiles) continue;
+                const int mt = tile / NG, ng = tile - mt * NG;
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int row = mt * 16 + g8 + 8 * i;
+                    unsigned long long bk = 0ull;
+                    if (row < na) {
+                        const float ia = m.inv_a[a0 + row];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int col = ng * 16 + t4 + 4 * e;
+                            if (col < s.nB) {
+                                const unsigned long long k = rank_key((acc[w][i][e] * ia) * m.inv_b[col], col);
+                                bk = k > bk ? k : bk;
+                            }
+                        }
+                    }
+                    unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, bk, 1);
+                    bk = o > bk ? o : bk;
+                    o = __shfl_xor_sync(0xFFFFFFFFu, bk, 2);
+                    bk = o > bk ? o : bk;
+                    if (t4 == 0 && row < na) atomicMax(m.best + a0 + row, bk);
+                }
+            }
+        }
+        __syncthreads();
+        if (CL > 1) {   // this CTA's row maxima to the others
+            cg::cluster_group cl = cg::this_cluster();
+            cl.sync();   // every CTA has initialised its maxima
+            for (int t = tid; t < na * (CL - 1); t += NT) {
+                const int k = t / na, a = a0 + t - k * na;
+                *cl.map_shared_rank(m.best + a, k < rank ? k : k + 1) = m.best[a];
+            }
+            cl.sync();   // all maxima here; no CTA reads another's shared memory after this
+        }
+        select_top_r<NT>(s, m);
+    }
+    const GlobalLoader<float> ld{reinterpret_cast<const float *>(p.x), (long long)s.start, p.dim};
+    if (!finish_decide<NT>(p, s, m)) return;
+    if (rank == 0) write_index_outputs<NT>(p, s, m);
+    const int w = p.dim / 4;
+    write_rows<float, NT>(p, s, m, ld, w * rank / CL, w * (rank + 1) / CL);
+}
+
+template <int NT, int TPW, int NP>
+cudaError_t launch(const ImageParams &p, const F32Geometry &g, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(k_merge_f32<NT, TPW, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_merge_f32<NT, TPW, NP>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)p.in.max_batch * (unsigned)g.cluster);
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = g.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = g.cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = g.cluster > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_merge_f32<NT, TPW, NP>, p, g);
+}
+
+constexpr int kSmallTokens = 65;   // four 16 x 16 tiles: four warps, one tile each
+
+}  // namespace
+
+F32Geometry image_f32_geometry(const ImageParams &p) {
+    F32Geometry g{};
+    const int nA = (p.in.max_tokens - 1) / 2, nB = p.in.max_tokens / 2;
+    const bool small = p.in.max_tokens <= kSmallTokens;
+    const int strips = ceil_div(nA > 0 ? nA : 1, 16);
+    // the most CTAs per sample (portable cluster sizes) that one wave of two CTAs per SM holds, while
+    // every CTA has a strip; a gate may stop a single CTA, which a cluster cannot
+    g.cluster = 1;
+    while (!p.gate && g.cluster < 8 && g.cluster * 2 <= strips + 1 &&
+           (long long)p.in.max_batch * g.cluster * 2 <= 2 * 152)
+        g.cluster *= 2;
+    g.rows_a = ceil_div(strips, g.cluster) * 16;
+    g.rows_b = ceil_div(nB > 0 ? nB : 1, 16) * 16;
+    auto need = [&](int kd) {
+        return meta_layout(p.in.max_tokens, 2 * (size_t)(g.rows_a + g.rows_b) * stage_row(kd)).total;
+    };
+    g.small = small;
+    for (size_t budget : {(size_t)110 * 1024, (size_t)224 * 1024})   // two CTAs per SM where 16 dims allow it
+        for (int kd = 64; kd >= 16; kd /= 2)
+            if (need(kd) <= budget) {
+                g.kd = kd;
+                g.smem = need(kd);
+                g.ok = 1;
+                return g;
+            }
+    return g;
+}
+
+cudaError_t launch_image_f32(const ImageParams &p, const F32Geometry &g, cudaStream_t s) {
+    if (p.in.max_batch == 0) return cudaSuccess;
+    if (g.small && g.cluster == 1) {
+        // rows of both halves: at most 64, 8 per 16 threads; one norm block of whole 64-dim stages' lanes
+        if (p.kc == p.kdim && g.kd == 64) return launch<128, 1, 8>(p, g, s);
+        return launch<128, 1, 0>(p, g, s);
+    }
+    return launch<256, 8, 0>(p, g, s);
+}
+
+}  // namespace fz

@@ -150,6 +150,18 @@ struct ImageGeometry {
 ImageGeometry image_geometry(int dtype, int max_tokens, int kdim, int do_merge);
 cudaError_t launch_image(int dtype, const ImageParams &p, size_t smem, cudaStream_t s);
 
+// ---- float32 merges with streamed keys (image_f32.cu) ----------------------------
+struct F32Geometry {
+    int ok;
+    int small;           // at most four 16 x 16 similarity tiles: CTAs of 128 threads
+    int cluster;         // CTAs per sample
+    int kd;              // key dims per stage
+    int rows_a, rows_b;  // rows of a stage: the CTA's share of half A, all of half B (multiples of 16)
+    size_t smem;
+};
+F32Geometry image_f32_geometry(const ImageParams &p);
+cudaError_t launch_image_f32(const ImageParams &p, const F32Geometry &g, cudaStream_t s);
+
 // ---- per-sample kernel on TMA + tcgen05 (bf16, |A|, |B| <= 128, key width % 64 == 0) ----
 struct TcGeometry {
     int ok;

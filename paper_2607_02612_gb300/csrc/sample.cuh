@@ -788,7 +788,7 @@ template <typename T, int NT, typename Loader>
 __device__ void write_rows(const ImageParams &p, const SampleInfo &s, MetaPtrs &m, const Loader &load, int c_lo,
                            int c_hi) {
     constexpr int CH = Elem<T>::kPerChunk;
-    constexpr int kGatherU = kGatherChunks / NT;
+    constexpr int kGatherU = NT <= 128 ? 8 : kGatherChunks / NT;   // several CTAs of 128 threads share an SM
     const int tid = threadIdx.x;
     const int out_n = s.out_n;
     const int dim = p.dim, w = c_hi - c_lo;

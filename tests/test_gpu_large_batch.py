@@ -122,3 +122,20 @@ def test_tiled_plan_rejects_malformed_offsets():
         torch.cuda.synchronize()
         assert int(f.status.item()) & fz.FUSION_DEV_BAD_OFFSETS
         assert int(o["batch"][0]) == 0 and int(o["offsets"][0]) == 0 and torch.all(o["x"] == 7)
+
+
+@pytest.mark.parametrize("counts,dim,keys,kdim", [
+    ([65, 64, 33, 34, 17, 3, 2, 1] * 2, 384, "alias", None),     # one wave, clusters; tile edges
+    ([65, 64, 33, 34, 17, 3, 2, 1] * 50, 80, "alias", None),     # 400 samples: small CTAs, a short stage
+    ([66, 40, 5] * 120, 64, "separate", 48),                     # just past the small kernel
+    ([197, 98, 1, 130], 384, "separate", 400),                   # clusters of 8, two norm blocks
+    ([197, 196] * 60, 32, "alias", None),                        # clusters of 2
+    ([129, 128, 113] * 110, 16, "alias", None),                  # one CTA per sample, several tiles per warp
+    ([577, 300], 1024, "alias", None),                           # long samples, narrow stages
+    ([650, 1], 64, "separate", 96)])
+def test_float32_merge_tiles(counts, dim, keys, kdim):
+    b = make_batch(counts, dim, "f32", seed=len(counts), keys=keys, kdim=kdim, sizes="u1to4")
+    rng = np.random.default_rng(1)
+    r = np.minimum(rng.integers(0, 40, len(counts)), np.asarray(counts) // 2).astype(np.int32)
+    rho = rng.uniform(0.3, 1.0, len(counts)).astype(np.float32)
+    run_stage_and_compare(b, StageSpec(True, False, True, r=r, rho=rho), f"{counts[:4]} x {len(counts)}")
