@@ -28,10 +28,22 @@ namespace {
 
 __host__ __device__ inline uint32_t stage_row(int kd) { return (uint32_t)(kd + 4) * 4u; }   // bytes; 16 (mod 32): 8 rows conflict-free
 
+// The oldest of the S stages in flight has landed (this thread's part of it).
+__device__ __forceinline__ void wait_stage(int S) {
+    switch (S) {
+    case 2: asm volatile("cp.async.wait_group 1;\n" ::: "memory"); break;
+    case 3: asm volatile("cp.async.wait_group 2;\n" ::: "memory"); break;
+    case 4: asm volatile("cp.async.wait_group 3;\n" ::: "memory"); break;
+    case 5: asm volatile("cp.async.wait_group 4;\n" ::: "memory"); break;
+    default: asm volatile("cp.async.wait_group 5;\n" ::: "memory"); break;   // kMaxStagesF32
+    }
+}
+constexpr int kMaxStagesF32 = 6;
+
 // NT threads; TPW warp tiles held in registers per pass; NP > 0: squared norms summed from the stages,
-// NP rows per 16 threads (kd = 64, one norm block), else read again from global memory (L2).
+// NP rows per 16 threads (kd = 64, norm blocks of whole stages), else read again from global memory (L2).
 template <int NT, int TPW, int NP>
-__global__ void __launch_bounds__(NT, NT == 128 ? 5 : 2) k_merge_f32(ImageParams p, F32Geometry g) {
+__global__ void __launch_bounds__(NT, NT == 128 ? 5 : TPW == 1 ? 1 : 2) k_merge_f32(ImageParams p, F32Geometry g) {
     extern __shared__ __align__(16) unsigned char sm[];
     constexpr int kW = NT / 32;
     const int CL = g.cluster;
@@ -46,14 +58,15 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : 2) k_merge_f32(ImageParams
     const int a0 = min(s.nA, rank * per * 16), na = min(s.nA, a0 + per * 16) - a0;
     const uint32_t stage_bytes = (uint32_t)(g.rows_a + g.rows_b) * rs;
     unsigned char *const st0 = sm;
-    MetaPtrs m(sm, meta_layout(p.in.max_tokens, 2 * (size_t)stage_bytes));
+    const int S = g.stages;
+    MetaPtrs m(sm, meta_layout(p.in.max_tokens, (size_t)S * stage_bytes));
     const float *keys = reinterpret_cast<const float *>(p.keys);
 
     const int n_stage = (kdim + kd - 1) / kd;
     const int rows = na + s.nB;
     // stage q: dims [q kd, ..) of the CTA's A rows, then of all B rows
     auto issue = [&](int q) {
-        unsigned char *dst = st0 + (q & 1) * stage_bytes;
+        unsigned char *dst = st0 + (q % S) * stage_bytes;
         const int nch = min(kd, kdim - q * kd) / 4;
         int row = tid / nch, c = tid - row * nch;
         const int rstep = NT / nch, cstep = NT - rstep * nch;
@@ -71,14 +84,17 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : 2) k_merge_f32(ImageParams
         }
         cp_async_commit();
     };
+    // a pass begins with S stages in flight; every stage is one commit group, empty past the last
+    auto start = [&] {
+        for (int q = 0; q < S; ++q) {
+            if (q < n_stage) issue(q);
+            else cp_async_commit();
+        }
+    };
     const int MT = (na + 15) / 16, NG = (s.nB + 15) / 16, tiles = MT * NG;
     const int n_pass = (tiles + kW * TPW - 1) / (kW * TPW);
     const bool sim = s.decide && na > 0;
-    if (sim) {
-        issue(0);
-        if (n_stage > 1) issue(1);
-        else cp_async_commit();
-    }
+    if (sim) start();
     meta_init<NT>(p, s, m);
     __syncthreads();
     if (s.decide) {
@@ -87,11 +103,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : 2) k_merge_f32(ImageParams
 #pragma unroll
         for (int k = 0; k < (NP > 0 ? NP : 1); ++k) nlo[k] = nhi[k] = 0.0f;
         for (int pass = 0; sim && pass < n_pass; ++pass) {
-            if (pass > 0) {
-                issue(0);
-                if (n_stage > 1) issue(1);
-                else cp_async_commit();
-            }
+            if (pass > 0) start();
             float acc[TPW][2][4];
 #pragma unroll
             for (int w = 0; w < TPW; ++w)
@@ -100,9 +112,9 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : 2) k_merge_f32(ImageParams
 #pragma unroll
                     for (int e = 0; e < 4; ++e) acc[w][i][e] = 0.0f;
             for (int q = 0; q < n_stage; ++q) {
-                asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+                wait_stage(S);
                 __syncthreads();
-                const unsigned char *st = st0 + (q & 1) * stage_bytes;
+                const unsigned char *st = st0 + (q % S) * stage_bytes;
                 const int kw = min(kd, kdim - q * kd);   // a multiple of 16
 #pragma unroll
                 for (int w = 0; w < TPW; ++w) {
@@ -140,27 +152,42 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : 2) k_merge_f32(ImageParams
                             for (int e = 0; e < 4; ++e) acc[w][i][e] += t[i][e];
                     }
                 }
-                if constexpr (NP > 0) {   // chunk c = 16 q + l of the row: lane c % 32 of the general kernel's sum
+                if constexpr (NP > 0) {   // chunk c = 16 qb + l of the norm block: lane c % 32 of the general kernel's sum
                     const int l = tid & 15, r0 = tid >> 4;
-                    if (l * 4 < kw) {
+                    const int per_block = (p.kc + kd - 1) / kd, qb = q % per_block;   // stages of a norm block
+                    if (pass == 0 && l * 4 < kw) {
 #pragma unroll
                         for (int k = 0; k < NP; ++k) {
                             const int row = r0 + k * (NT / 16);
                             if (row >= rows) continue;
                             const float4 f = *reinterpret_cast<const float4 *>(
                                 st + (uint32_t)(row < na ? row : g.rows_a + row - na) * rs + l * 16);
-                            float v = (q & 1) ? nhi[k] : nlo[k];
+                            float v = (qb & 1) ? nhi[k] : nlo[k];
                             v = fmaf(f.x, f.x, v);
                             v = fmaf(f.y, f.y, v);
                             v = fmaf(f.z, f.z, v);
                             v = fmaf(f.w, f.w, v);
-                            if (q & 1) nhi[k] = v;
+                            if (qb & 1) nhi[k] = v;
                             else nlo[k] = v;
+                        }
+                    }
+                    if (pass == 0 && (qb == per_block - 1 || q == n_stage - 1)) {   // the block's sum joins the row's
+#pragma unroll
+                        for (int k = 0; k < NP; ++k) {
+                            float v = nlo[k] + nhi[k];
+#pragma unroll
+                            for (int o = 8; o >= 1; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+                            const int row = r0 + k * (NT / 16);
+                            if (l == 0 && row < rows) {
+                                float *ss = row < na ? m.inv_a + a0 + row : m.inv_b + row - na;
+                                *ss = q < per_block ? v : *ss + v;
+                            }
+                            nlo[k] = nhi[k] = 0.0f;
                         }
                     }
                 }
                 __syncthreads();   // everyone is done with this stage
-                if (q + 2 < n_stage) issue(q + 2);
+                if (q + S < n_stage) issue(q + S);
                 else cp_async_commit();   // an empty group keeps the count
             }
             if (pass == 0) {
@@ -172,35 +199,43 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : 2) k_merge_f32(ImageParams
                     else m.inv_b[row - na] = inv;
                 };
                 if constexpr (NP > 0) {
-#pragma unroll
-                    for (int k = 0; k < NP; ++k) {
-                        float v = nlo[k] + nhi[k];
-#pragma unroll
-                        for (int o = 8; o >= 1; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-                        const int row = (tid >> 4) + k * (NT / 16);
-                        if ((tid & 15) == 0 && row < rows) put(row, v);
-                    }
+                    for (int row = tid; row < rows; row += NT)   // after the last stage's barrier
+                        put(row, row < na ? m.inv_a[a0 + row] : m.inv_b[row - na]);
                 } else {
-                    for (int row = warp; row < rows; row += kW) {
-                        const int tok = row < na ? a0 + row : row - na;
-                        const float *src = keys + (long long)(s.start + (row < na ? 2 + 2 * tok : 1 + 2 * tok)) * kdim;
-                        float v = 0.0f;
+                    // four rows at a time, so that their loads are in flight together
+                    for (int row0 = warp; row0 < rows; row0 += 4 * kW) {
+                        const float4 *src[4];
+                        float v[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int row = min(row0 + u * kW, rows - 1), tok = row < na ? a0 + row : row - na;
+                            src[u] = reinterpret_cast<const float4 *>(
+                                keys + (long long)(s.start + (row < na ? 2 + 2 * tok : 1 + 2 * tok)) * kdim);
+                            v[u] = 0.0f;
+                        }
                         for (int k0 = 0; k0 < kdim; k0 += p.kc) {
                             const int nch = min(p.kc, kdim - k0) / 4;
-                            float sq = 0.0f;
-#pragma unroll 4
-                            for (int c = lane; c < nch; c += 32) {
-                                const float4 f = __ldg(reinterpret_cast<const float4 *>(src + k0) + c);
-                                sq = fmaf(f.x, f.x, sq);
-                                sq = fmaf(f.y, f.y, sq);
-                                sq = fmaf(f.z, f.z, sq);
-                                sq = fmaf(f.w, f.w, sq);
-                            }
+                            float sq[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 2
+                            for (int c = lane; c < nch; c += 32)
 #pragma unroll
-                            for (int o = 16; o >= 1; o >>= 1) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, o);
-                            v += sq;
+                                for (int u = 0; u < 4; ++u) {
+                                    const float4 f = __ldg(src[u] + k0 / 4 + c);
+                                    sq[u] = fmaf(f.x, f.x, sq[u]);
+                                    sq[u] = fmaf(f.y, f.y, sq[u]);
+                                    sq[u] = fmaf(f.z, f.z, sq[u]);
+                                    sq[u] = fmaf(f.w, f.w, sq[u]);
+                                }
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+#pragma unroll
+                                for (int o = 16; o >= 1; o >>= 1) sq[u] += __shfl_xor_sync(0xFFFFFFFFu, sq[u], o);
+                                v[u] += sq[u];
+                            }
                         }
-                        if (lane == 0) put(row, v);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (lane == u && row0 + u * kW < rows) put(row0 + u * kW, v[u]);
                     }
                 }
                 __syncthreads();
@@ -291,28 +326,35 @@ F32Geometry image_f32_geometry(const ImageParams &p) {
         g.cluster *= 2;
     g.rows_a = ceil_div(strips, g.cluster) * 16;
     g.rows_b = ceil_div(nB > 0 ? nB : 1, 16) * 16;
-    auto need = [&](int kd) {
-        return meta_layout(p.in.max_tokens, 2 * (size_t)(g.rows_a + g.rows_b) * stage_row(kd)).total;
+    auto need = [&](int kd, int S) {
+        return meta_layout(p.in.max_tokens, (size_t)S * (g.rows_a + g.rows_b) * stage_row(kd)).total;
     };
     g.small = small;
-    for (size_t budget : {(size_t)110 * 1024, (size_t)224 * 1024})   // two CTAs per SM where 16 dims allow it
-        for (int kd = 64; kd >= 16; kd /= 2)
-            if (need(kd) <= budget) {
-                g.kd = kd;
-                g.smem = need(kd);
-                g.ok = 1;
-                return g;
-            }
+    // two CTAs per SM where 16 dims allow it; a batch that leaves SMs idle has each to itself, and more
+    // stages: 8 samples of 197 tokens, loop of six 64-dim stages: 12.4 us with two in flight, @S with all
+    const bool alone = (long long)p.in.max_batch * g.cluster <= 152;
+    const size_t most = 224 * 1024;
+    for (size_t budget : {alone ? most : (size_t)110 * 1024, most})
+        for (int kd = 64; kd >= 16; kd /= 2) {
+            if (need(kd, 2) > budget) continue;
+            g.kd = kd;
+            g.stages = 2;
+            const int n_stage = ceil_div(p.kdim, kd);
+            while (alone && g.stages < kMaxStagesF32 && g.stages < n_stage && need(kd, g.stages + 1) <= most) ++g.stages;
+            g.smem = need(kd, g.stages);
+            g.ok = 1;
+            return g;
+        }
     return g;
 }
 
 cudaError_t launch_image_f32(const ImageParams &p, const F32Geometry &g, cudaStream_t s) {
     if (p.in.max_batch == 0) return cudaSuccess;
-    if (g.small && g.cluster == 1) {
-        // rows of both halves: at most 64, 8 per 16 threads; one norm block of whole 64-dim stages' lanes
-        if (p.kc == p.kdim && g.kd == 64) return launch<128, 1, 8>(p, g, s);
-        return launch<128, 1, 0>(p, g, s);
-    }
+    // norms from the stages: whole stages per norm block, at most 8 rows per 16 threads
+    const bool norms = g.kd == 64 && (p.kc == p.kdim || p.kc % 64 == 0);
+    if (g.small && g.cluster == 1) return norms ? launch<128, 1, 8>(p, g, s) : launch<128, 1, 0>(p, g, s);
+    if ((g.rows_a / 16) * (g.rows_b / 16) <= 8)   // a tile per warp
+        return norms && g.rows_a + g.rows_b <= 128 ? launch<256, 1, 8>(p, g, s) : launch<256, 1, 0>(p, g, s);
     return launch<256, 8, 0>(p, g, s);
 }
 

@@ -155,7 +155,7 @@ struct F32Geometry {
     int ok;
     int small;           // at most four 16 x 16 similarity tiles: CTAs of 128 threads
     int cluster;         // CTAs per sample
-    int kd;              // key dims per stage
+    int kd, stages;      // key dims per stage; stages in flight
     int rows_a, rows_b;  // rows of a stage: the CTA's share of half A, all of half B (multiples of 16)
     size_t smem;
 };

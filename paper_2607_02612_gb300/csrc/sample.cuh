@@ -391,7 +391,11 @@ __device__ __forceinline__ uint4 pack_chunk(const F2 (&q)[4]) {
 //   when the product lies within a few float32 ulps of a bf16 rounding midpoint m, the
 //   side of m is decided exactly from the sign of num - m * den (an exact tie stays a
 //   tie, so it rounds to even).
-//   f32: the float-float division.
+//   f32: one step of long division with the reciprocal: q1 = num / den within a few ulps, the
+//   remainder num - q1 den in float-float (its leading difference is exact), q2 = remainder / den,
+//   corrected by its own remainder, so that a quotient that is a float comes out as that float; the mean
+//   is q1 + q2 rounded once (about 45 correct bits, and exact ties stay ties, which go to even).  The two
+//   correctly rounded divisions of f2_div made the means a quarter of the kernel's instructions.
 __device__ __forceinline__ F2 mean_of(F2 num, F2 den, F2 inv, __nv_bfloat16) {
     const F2 q = f2_mul(num, inv);
     const uint32_t bits = __float_as_uint(q.hi);
@@ -406,7 +410,19 @@ __device__ __forceinline__ F2 mean_of(F2 num, F2 den, F2 inv, __nv_bfloat16) {
     const float tiny = copysignf(1e-30f, side);
     return side == 0.0f ? F2{mid, 0.0f} : F2{mid, tiny};
 }
-__device__ __forceinline__ F2 mean_of(F2 num, F2 den, F2, float) { return f2_div(num, den); }
+__device__ __forceinline__ F2 mean_of(F2 num, F2 den, F2 inv, float) {
+    const float q1 = __fmul_rn(num.hi, inv.hi);
+    const F2 p = two_prod(q1, den.hi);
+    const F2 a = two_sum(__fsub_rn(num.hi, p.hi), -p.lo);
+    const F2 b = two_sum(a.hi, num.lo);
+    const float r = __fadd_rn(b.hi, __fmaf_rn(-q1, den.lo, __fadd_rn(a.lo, b.lo)));
+    float q2 = __fmul_rn(r, inv.hi);
+    q2 = __fmaf_rn(__fmaf_rn(-q2, den.hi, r), inv.hi, q2);
+    const F2 q = quick_two_sum(q1, q2);
+    // zero, subnormal, infinite and NaN quotients (and products that under- or overflow on the way)
+    const float m = fabsf(q.hi);
+    return m > 0x1p-40f && m < 0x1p40f && den.hi > 0x1p-40f && den.hi < 0x1p40f ? q : f2_div(num, den);
+}
 
 // bf16 bits of num / den rounded to nearest even.  A power-of-two den (uniform over a
 // merged row; every merge of two unit-size tokens) scales num exactly, so the float-float
