@@ -4,26 +4,32 @@
 // row m of the sample:
 //   out[m, h] = sum_j softmax_j(q_m . k_j / sqrt(dh) + log s_j) v_j.
 //
-// One CTA of 256 threads per (head, sample), dh = 64, bf16.  Samples of at most 256 tokens
-// (calls whose max_tokens is at most 256) keep the whole sample in shared memory (k_attn_tc);
-// longer samples, up to 1024 tokens, stream key blocks (k_attn_tc_long, below).
-// TMA brings the sample's query tiles of 128 rows, its K rows and its V rows (one 128-byte
-// row of 64 dims each, 128-byte swizzle) from the packed qkv matrix.  Q and K are K-major
-// operands; V, rows of keys with the dims contiguous, is the MN-major B operand of the second
-// product as it lies (8-key swizzle atoms 1024 bytes apart); its rows past the sample are
-// zeroed once it has landed.  Per query tile t: S_t = Q_t K^T (M = 128, N = tokens
-// rounded up to 16, K = 64) accumulates in tensor-memory columns [0, N);
-// warp w and warp w + 4 share the rows of lane quadrant w, each taking half of the columns
-// (maxima and sums meet in shared memory): logits scaled by log2(e) / sqrt(dh) plus
-// log2(s_j), masked past the sample, shifted by max_j S scale + max_j log2 s_j (an upper bound of
-// the row maximum within log2(max s / min s), so sizes within a factor 2^100 of each other keep
-// every probability a normal float), exp2 (ex2.approx), the row sum, and the
-// unnormalised probabilities P_t as bf16 pairs written back over S's first columns; O_t = P_t V
-// (M = 128, N = 64, K = tokens rounded up to 16, A = P from tensor memory) accumulates in
-// columns [128, 192); the epilogue divides each row by its sum and stores bf16.  P is rounded to
-// bf16 (the operand type of the second product); the sum is taken before that.  Without a P
-// buffer a CTA needs Q, K and V only (84 KB for 197 tokens) and 256 tensor-memory columns, so
-// two CTAs share an SM; the query tiles of a sample run one after the other.
+// One CTA per (pair of query tiles, head, sample), dh = 64, bf16; a query tile is 128 rows and has a
+// warpgroup of its own, one thread per row.  One more warp per tile issues its tensor-core products; the
+// query tiles and blocks of 64 keys (K and V rows) come by TMA through a ring of four stages (128-byte
+// swizzle; Q and K are K-major operands; V, rows of keys with the dims contiguous, is the MN-major B
+// operand of the second product as it lies).  Per tile and key block: S = Q K^T (M = 128, N = keys
+// rounded up to 16) into tensor-memory columns [0, 64) of the tile; the thread of a row reads it, forms
+// P = 2^(S scale + log2 s_j - m) (ex2.approx), adds its float32 sum and writes P as bf16 over S's first 32
+// columns; O += P V (A = P from tensor memory) accumulates in columns [64, 128), and the next block's S
+// follows it in the same issue order, so one barrier per block tells the warpgroup that its S is
+// ready and its O complete.
+//
+// The shift is m = max_j S scale + max_j log2 s_j over the blocks so far (an upper bound of the row
+// maximum within log2(max s / min s), so sizes within a factor 2^100 of each other keep every probability a
+// normal float); where it grows, the warp rescales its rows of O and their sums.  P is rounded to bf16
+// (the operand type of the second product), the sum is taken before that; the row's largest
+// probabilities end as 2^0, exact in bf16 (letting the shift lag, to rescale rarely, raised the error
+// against 64 bits at 577 tokens from 2.2e-3 to 2.3e-3).
+//
+// What bounds it: the softmax's instructions (about six issue slots per logit and row of 32) and, for short
+// samples, the way to the first product (metadata, barriers, loads: 5 of 15 thousand cycles at 197
+// tokens); two CTAs (four warpgroups) per SM hide each other's waits for the products.  The forms before
+// it, one CTA per (head, sample) with block-wide barriers between load, product, softmax and product,
+// idled in them, and samples past 256 tokens formed S twice (a pass for the maximum).  256 samples of
+// 100 to 197 tokens x 6 heads: 62 -> 43 us; 128 of 577 x 16 heads: 769 -> 317 us (0.55 PFLOP/s).
+// Measured and not taken: halves of 32 keys with two S buffers (495 us at 577 tokens: twice the barriers),
+// a first pass for the maximum with two S buffers (440), the shift allowed to lag by 2^8 (309).
 //
 // Every wait on an mbarrier is bounded; on a timeout the CTA raises FUSION_DEV_TIMEOUT, skips
 // its outputs, waits (bounded) for the operations it started and frees its tensor memory.
@@ -33,11 +39,13 @@
 namespace fz {
 namespace {
 
-constexpr int kAttnThreads = 256;
 constexpr int kAttnDh = 64;
-constexpr int kAttnMaxN = 256;
-constexpr uint32_t kQTileBytes = 128 * 128;   // 128 rows x one K-block of 64 bf16
-constexpr uint32_t kAttnTmemCols = 256;       // S (<= 256 columns); P over its first half; O at 128
+constexpr int kAttnMaxN = FUSION_ATTN_MAX_TOKENS;
+constexpr uint32_t kQTileBytes = 128 * 128;   // 128 rows x 64 bf16
+constexpr int kKeyBlock = 64;
+constexpr uint32_t kKeyBytes = kKeyBlock * 128;   // 64 key rows (K or V)
+constexpr int kStages = 4;      // K and V blocks in flight, at most
+constexpr uint32_t kTileCols = 128;           // tensor-memory columns of a query tile: S (P over it), O at 64
 
 __device__ __forceinline__ float ex2(float x) {   // 2^x, one MUFU instruction (2^-inf = 0)
     float y;
@@ -51,30 +59,10 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-// max of m and the 16 values of a tensor-memory chunk: a tree of three-source maxima (8
-// instructions, 3 deep, against 16 in a chain)
-__device__ __forceinline__ float max16(float m, const uint32_t (&v)[16]) {
-    const float a = max3(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]));
-    const float b = max3(__uint_as_float(v[3]), __uint_as_float(v[4]), __uint_as_float(v[5]));
-    const float c = max3(__uint_as_float(v[6]), __uint_as_float(v[7]), __uint_as_float(v[8]));
-    const float d = max3(__uint_as_float(v[9]), __uint_as_float(v[10]), __uint_as_float(v[11]));
-    const float e = max3(__uint_as_float(v[12]), __uint_as_float(v[13]), __uint_as_float(v[14]));
-    return max3(m, max3(a, b, c), max3(d, e, __uint_as_float(v[15])));
-}
-
 struct AttnMaps {
-    CUtensorMap b32, b8;   // qkv rows, boxes of 64 dims x 32 / 8 rows, 128-byte swizzle
+    CUtensorMap b128, b64, b32, b8;   // qkv rows, boxes of 64 dims x 128 / 64 / 32 / 8 rows, 128-byte swizzle
 };
 
-// The two warps that share lane quadrant w (warps w and w + 4) meet at named barrier 1 + w.
-__device__ __forceinline__ void pair_sync(int warp) {
-    switch (warp & 3) {   // literal ids: the kernel reserves barriers 0..4 only
-    case 0: asm volatile("bar.sync 1, 64;" ::: "memory"); break;
-    case 1: asm volatile("bar.sync 2, 64;" ::: "memory"); break;
-    case 2: asm volatile("bar.sync 3, 64;" ::: "memory"); break;
-    default: asm volatile("bar.sync 4, 64;" ::: "memory"); break;
-    }
-}
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]),
                  "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
@@ -89,539 +77,427 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, u
         : "memory");
 }
 
-__global__ void __launch_bounds__(kAttnThreads, 2)
-    k_attn_tc(const __grid_constant__ AttnMaps maps, AttnParams p) {
+
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t *r) {   // no wait: tmem_ld_wait
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
+        "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// Stages of the K and V rings: all of the call's blocks, up to four.
+__host__ __device__ inline int attn_stages(int max_tokens) {
+    const int nb = (max_tokens + kKeyBlock - 1) / kKeyBlock;
+    return nb < kStages ? nb : kStages;
+}
+// Position in a ring of n stages: the stage, and the parity of its current use.
+struct RingPos {
+    int st = 0;
+    uint32_t par = 0;
+    __device__ __forceinline__ void next(int n) {
+        if (++st == n) {
+            st = 0;
+            par ^= 1u;
+        }
+    }
+};
+
+__device__ __forceinline__ bool elect_one() {   // true in one lane of the (converged) warp
+    uint32_t p;
+    asm volatile("{ .reg .pred p; elect.sync _|p, 0xffffffff; selp.u32 %0, 1, 0, p; }" : "=r"(p));
+    return p != 0;
+}
+
+// mbar_wait by a whole warp, with one outcome.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
+    return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity));
+}
+
+// q: query tiles; k, v: key / value blocks landed; s: a tile's S complete (and its O up to the block
+// before); free: a stage's products done (each tile's); p: a tile's S replaced by P
+struct AttnBars {
+    unsigned long long q[2], drain[2], k[kStages], v[kStages], s[2], free[kStages], p[2];
+};
+
+// The softmax of one block for one row: S (64 logits in v) -> P over S's first columns; returns the sum
+// of the probabilities as an (even, odd) pair.  kSized: log2 sizes from lz, else all zero.
+template <bool kSized>
+__device__ __forceinline__ float2 block_probs(const uint32_t (&v)[64], uint32_t taddr, const float *lz, float m) {
+    constexpr float kScale2 = 0.18033688011112042f;   // log2(e) / sqrt(64)
+    float2 sum = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        uint32_t pk[8];
+#pragma unroll
+        for (int e = 0; e < 16; e += 2) {
+            const int j = 16 * c + e;
+            const float2 sv = make_float2(__uint_as_float(v[j]), __uint_as_float(v[j + 1]));
+            float2 x;
+            if constexpr (kSized)
+                x = __fadd2_rn(__ffma2_rn(sv, make_float2(kScale2, kScale2), *reinterpret_cast<const float2 *>(lz + j)),
+                               make_float2(-m, -m));
+            else
+                x = __ffma2_rn(sv, make_float2(kScale2, kScale2), make_float2(-m, -m));
+            const float2 pr = make_float2(ex2(x.x), ex2(x.y));
+            sum = __fadd2_rn(sum, pr);
+            const __nv_bfloat162 b2 = __floats2bfloat162_rn(pr.x, pr.y);
+            pk[e >> 1] = *reinterpret_cast<const uint32_t *>(&b2);
+        }
+        tmem_st8(taddr + 8u * c, pk);
+    }
+    return sum;
+}
+
+// NWG: query tiles (warpgroups) per CTA.
+template <int NWG>
+__global__ void __launch_bounds__(NWG * 160, NWG == 2 ? 2 : 3)
+    k_attn_tc(const __grid_constant__ AttnMaps maps, AttnParams p, int n_part) {
     extern __shared__ unsigned char sm_raw[];
     unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) & ~uintptr_t(1023));
-    // bar_ld: query tile 0 and K (the first product's operands); bar_ld2: V and the other query tiles
-    __shared__ __align__(8) unsigned long long bar_ld, bar_ld2, bar_s, bar_o;
+    __shared__ __align__(8) AttnBars bar;
     __shared__ uint32_t tmem_base;
-    __shared__ int s_fail, s_issued;   // s_issued: operations started (for the drain on a timeout)
+    __shared__ int s_fail, s_kv;             // s_kv: key blocks whose loads were issued
+    __shared__ float red_max[NWG * 4], red_min[NWG * 4];
     __shared__ __align__(16) float lsz[kAttnMaxN];   // log2 of the key sizes
-    __shared__ float red[2][128];      // the two column halves' row maxima, then row sums
-    __shared__ float s_lszmax;         // max_j log2 s_j
 
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int h = blockIdx.x, i = blockIdx.y;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (warp == NWG * 4 && lane < 4)   // the descriptors travel while the sample's metadata loads
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.b128 + lane)) : "memory");
+    const int part = blockIdx.x % n_part, h = blockIdx.x / n_part, i = blockIdx.y;
     const int B = device_batch(p.in);
     if (B < 0) {
-        if (h == 0 && i == 0 && tid == 0) raise_status(p.status, FUSION_DEV_BAD_BATCH);
+        if (blockIdx.x == 0 && i == 0 && tid == 0) raise_status(p.status, FUSION_DEV_BAD_BATCH);
         return;
     }
     if (i >= B) return;
     const int o0 = p.in.offsets[i], n = p.in.offsets[i + 1] - o0;
     if (o0 < 0 || n < 1 || n > p.in.max_tokens || n > kAttnMaxN || (long long)o0 + n > p.in.max_rows) {
-        if (h == 0 && tid == 0) raise_status(p.status, FUSION_DEV_BAD_OFFSETS);
+        if (blockIdx.x == 0 && tid == 0) raise_status(p.status, FUSION_DEV_BAD_OFFSETS);
         return;
     }
+    const int row0 = part * NWG * 128;            // this CTA's first query row
+    if (row0 >= n) return;
+    const int nw = min(NWG, (n - row0 + 127) >> 7);   // its query tiles
     const int H = p.heads;
-    const int npad = (n + 15) & ~15;              // keys rounded up to the MMA granularity
-    const int T = (n + 127) >> 7;                 // query tiles
-    unsigned char *Q = sm;                        // T tiles of 128 rows
-    unsigned char *Kr = sm + (size_t)T * kQTileBytes;
-    unsigned char *Vr = Kr + (size_t)npad * 128;  // V rows (MN-major B operand)
+    const int nb = (n + kKeyBlock - 1) / kKeyBlock;
+    unsigned char *Q = sm, *Kr = sm + NWG * kQTileBytes;
+    const int ns = attn_stages(p.in.max_tokens);
+    unsigned char *Vr = Kr + ns * kKeyBytes;
 
-    if (warp == 0) {
+    // (values that a whole warp shares, through shuffles, and elected lanes: the compiler then keeps the
+    // copies' and products' operands in uniform registers; a product took 100 cycles to issue from a lane
+    // picked by its index, 40 this way)
+    const int n_u = __shfl_sync(0xFFFFFFFFu, n, 0), o0_u = __shfl_sync(0xFFFFFFFFu, o0, 0);
+    auto rows = [&](unsigned char *dst, int x, int y0, int cnt, unsigned long long *b) {   // cnt: multiple of 8
+        mbar_expect_tx(smem_addr(b), (uint32_t)cnt * 128u);
+        if (cnt == 128) return tma_load_2d(smem_addr(dst), &maps.b128, x, y0, smem_addr(b));
+        int r = 0;
+        for (; r + 64 <= cnt; r += 64) tma_load_2d(smem_addr(dst + r * 128), &maps.b64, x, y0 + r, smem_addr(b));
+        for (; r + 32 <= cnt; r += 32) tma_load_2d(smem_addr(dst + r * 128), &maps.b32, x, y0 + r, smem_addr(b));
+        for (; r < cnt; r += 8) tma_load_2d(smem_addr(dst + r * 128), &maps.b8, x, y0 + r, smem_addr(b));
+    };
+    auto block_rows = [&](int j) { return (min(kKeyBlock, n_u - j * kKeyBlock) + 7) & ~7; };
+    auto load_k = [&](int j, int st) {
+        rows(Kr + st * kKeyBytes, (H + h) * kAttnDh, o0_u + j * kKeyBlock, block_rows(j), &bar.k[st]);
+    };
+    auto load_v = [&](int j, int st) {
+        rows(Vr + st * kKeyBytes, (2 * H + h) * kAttnDh, o0_u + j * kKeyBlock, block_rows(j), &bar.v[st]);
+    };
+    auto load_q = [&](int w) {
+        rows(Q + w * kQTileBytes, h * kAttnDh, o0_u + row0 + 128 * w, (min(128, n_u - row0 - 128 * w) + 7) & ~7, &bar.q[w]);
+    };
+    if (warp == NWG * 4) {   // the barriers, one per lane
+        if (lane < (int)(sizeof(AttnBars) / 8))
+            mbar_init(smem_addr(&bar.q[0] + lane), lane < 6 + 2 * kStages ? 1 : lane < 6 + 3 * kStages ? nw : 128);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if (lane == 0) {
+            s_fail = 0;
+            s_kv = min(nb, ns);
+        }
+        __syncwarp();
+    }
+    if (warp == NWG * 4) {   // the first blocks at once (the second issuing warp allocates meanwhile)
+        const int n0 = min((n_u + kKeyBlock - 1) / kKeyBlock, ns);
+        if (elect_one()) {
+            for (int j = 0; j < n0; ++j) {
+                load_k(j, j);
+                for (int w = 0; j == 0 && w < nw; ++w) load_q(w);
+                load_v(j, j);
+            }
+        }
+        __syncwarp();
+    }
+    if (warp == NWG * 5 - 1) {   // the last of the issuing warps
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_base)),
-                     "r"(kAttnTmemCols)
+                     "r"(NWG * kTileCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    if (tid == 0) {
-        s_fail = 0;
-        s_issued = 0;
-        mbar_init(smem_addr(&bar_ld), 1);
-        mbar_init(smem_addr(&bar_ld2), 1);
-        mbar_init(smem_addr(&bar_s), 1);
-        mbar_init(smem_addr(&bar_o), 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncthreads();
-
-    // ---- loads: the query tiles, K and V by TMA (rows rounded up to 8); query tile 0 and K on
-    // ---- bar_ld (the first product starts once they landed), V and the other tiles on bar_ld2 --
-    if (tid == 0) {
-        const int rk = (n + 7) & ~7;
-        auto qrows = [&](int t) { return (min(128, n - 128 * t) + 7) & ~7; };
-        uint32_t bytes2 = (uint32_t)rk * 128u;
-        for (int t = 1; t < T; ++t) bytes2 += (uint32_t)qrows(t) * 128u;
-        mbar_expect_tx(smem_addr(&bar_ld), (uint32_t)(rk + qrows(0)) * 128u);
-        mbar_expect_tx(smem_addr(&bar_ld2), bytes2);
-        auto rows = [&](unsigned char *dst, int x, int y0, int cnt, unsigned long long *bar) {   // cnt: multiple of 8
-            int r = 0;
-            for (; r + 32 <= cnt; r += 32) tma_load_2d(smem_addr(dst + r * 128), &maps.b32, x, y0 + r, smem_addr(bar));
-            for (; r < cnt; r += 8) tma_load_2d(smem_addr(dst + r * 128), &maps.b8, x, y0 + r, smem_addr(bar));
-        };
-        rows(Q, h * kAttnDh, o0, qrows(0), &bar_ld);
-        rows(Kr, (H + h) * kAttnDh, o0, rk, &bar_ld);
-        rows(Vr, (2 * H + h) * kAttnDh, o0, rk, &bar_ld2);
-        for (int t = 1; t < T; ++t) rows(Q + (size_t)t * kQTileBytes, h * kAttnDh, o0 + 128 * t, qrows(t), &bar_ld2);
-        s_issued = 1;
-    }
-    for (int j = tid; j < npad; j += kAttnThreads)
-        lsz[j] = j < n ? (p.sizes ? log2f(p.sizes[o0 + j]) : 0.0f) : 0.0f;
-    if (tid == 0 && !mbar_wait(smem_addr(&bar_ld), 0)) s_fail = 1;
-    __syncthreads();
-    if (warp == 0) {   // max_j log2 s_j over the sample
-        float lm = -INFINITY;
-        for (int j = threadIdx.x; j < n; j += 32) lm = fmaxf(lm, lsz[j]);
+    if (warp < NWG * 4) {   // log2 of the key sizes meanwhile, four loads of a thread in flight
+        float lmax = -INFINITY, lmin = INFINITY;
+        for (int j0 = tid; j0 < nb * kKeyBlock; j0 += NWG * 512) {
+            float sz[4];
 #pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) lm = fmaxf(lm, __shfl_xor_sync(0xFFFFFFFFu, lm, o));
-        if (threadIdx.x == 0) s_lszmax = lm;
-    }
-    __syncthreads();
-
-    const uint32_t tmem = tmem_base;
-    const int half = warp >> 2;                 // column half of the row
-    const int r = tid & 127;                    // row of the tile = tensor-memory lane
-    const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const int nch = npad >> 4;                  // 16-column chunks of S
-    const int cA = (nch + 1) >> 1;              // chunks [0, cA) to half 0, [cA, nch) to half 1
-    const int c_lo = half ? cA : 0, c_hi = half ? nch : cA;
-    constexpr float kScale2 = 0.18033688011112042f;   // log2(e) / sqrt(64)
-    const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(npad >> 3) << 17) | (8u << 24);
-    // B = V as it lies: MN-major (bit 16), 8-key swizzle atoms 1024 bytes apart
-    const uint32_t idesc_o =
-        (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(kAttnDh >> 3) << 17) | (8u << 24);
-
-    bool stop = s_fail != 0;   // read between two barriers: the same in every thread
-    for (int t = 0; t < T && !stop; ++t) {
-        // ---- S = Q_t K^T into columns [0, npad) ---------------------------------------------
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int k = 0; k < 4; ++k) {
+                const int j = j0 + k * NWG * 128;
+                sz[k] = j < n && p.sizes ? p.sizes[o0 + j] : 1.0f;
+            }
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                umma_bf16(tmem, sw128_desc(smem_addr(Q + (size_t)t * kQTileBytes) + k * 32), sw128_desc(smem_addr(Kr) + k * 32),
-                          idesc_s, k ? 1u : 0u);
-            umma_commit(smem_addr(&bar_s));
-            s_issued = 2 + 2 * t;
-        }
-        if (!mbar_wait(smem_addr(&bar_s), (uint32_t)t & 1u)) atomicOr(&s_fail, 2);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const bool rows_here = 128 * t + 32 * (warp & 3) < n;   // warp-uniform: a warp of rows past the sample idles
-        // ---- the softmax shift: max_j S * scale + max_j log2 s_j, an upper bound of the row's largest
-        // ---- logit by at most log2(max s / min s) (the result does not depend on the shift) -------
-        float mx = -INFINITY;
-        if (rows_here) {
-            for (int c = c_lo; c < c_hi; ++c) {
-                uint32_t v[16];
-                tmem_ld16(lane_addr + (uint32_t)(16 * c), v);
-                if (16 * c + 16 <= n) {
-                    mx = max16(mx, v);
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        if (16 * c + e < n) mx = fmaxf(mx, __uint_as_float(v[e]));
+            for (int k = 0; k < 4; ++k) {
+                const int j = j0 + k * NWG * 128;
+                if (j >= nb * kKeyBlock) break;
+                const float l = log2f(sz[k]);   // 0 past the sample
+                lsz[j] = l;
+                if (j < n) {
+                    lmax = fmaxf(lmax, l);
+                    lmin = fminf(lmin, l);
                 }
             }
         }
-        red[half][r] = mx;
-        pair_sync(warp);
-        mx = fmaf(fmaxf(red[0][r], red[1][r]), kScale2, s_lszmax);
-        // ---- P = 2^(logit - max) as bf16 pairs, and the row sum; P goes over S's first columns once
-        // ---- every S column of the row has been read (the other half reads some of them) ----------
-        float2 lsum2 = make_float2(0.0f, 0.0f);   // even and odd columns (packed float32 pairs)
-        uint32_t pk[8][8];   // this half's chunks, at most 8
-        if (rows_here) {
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int c = c_lo + q;
-                if (c < c_hi) {
-                    uint32_t v[16];
-                    tmem_ld16(lane_addr + (uint32_t)(16 * c), v);
-                    float pr[16];
-#pragma unroll
-                    for (int e = 0; e < 16; e += 2) {   // fma then subtract, two columns per instruction
-                        const float2 x = __fadd2_rn(
-                            __ffma2_rn(make_float2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])),
-                                       make_float2(kScale2, kScale2), *reinterpret_cast<const float2 *>(&lsz[16 * c + e])),
-                            make_float2(-mx, -mx));
-                        pr[e] = ex2(x.x);
-                        pr[e + 1] = ex2(x.y);
-                    }
-                    if (16 * c + 16 > n) {
-#pragma unroll
-                        for (int e = 0; e < 16; ++e)
-                            if (16 * c + e >= n) pr[e] = 0.0f;
-                    }
-#pragma unroll
-                    for (int e = 0; e < 16; e += 2) {
-                        lsum2 = __fadd2_rn(lsum2, make_float2(pr[e], pr[e + 1]));
-                        const __nv_bfloat162 b2 = __floats2bfloat162_rn(pr[e], pr[e + 1]);
-                        pk[q][e >> 1] = *reinterpret_cast<const uint32_t *>(&b2);
-                    }
-                }
-            }
+        for (int o = 16; o >= 1; o >>= 1) {
+            lmax = fmaxf(lmax, __shfl_xor_sync(0xFFFFFFFFu, lmax, o));
+            lmin = fminf(lmin, __shfl_xor_sync(0xFFFFFFFFu, lmin, o));
         }
-        pair_sync(warp);   // every S column of these rows read; both halves' maxima read
-        if (rows_here) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (c_lo + q < c_hi) tmem_st8(lane_addr + (uint32_t)(8 * (c_lo + q)), pk[q]);
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        if (lane == 0) {
+            red_max[warp] = lmax;
+            red_min[warp] = lmin;
         }
-        red[half][r] = lsum2.x + lsum2.y;
-        if (t == 0) {
-            // V and the other query tiles: landed while this tile's softmax ran; V rows n .. npad-1
-            // (another sample's rows or stale memory) read as zero in P V
-            if (tid == 0 && !mbar_wait(smem_addr(&bar_ld2), 0)) atomicOr(&s_fail, 8);
-            __syncthreads();
-            if (s_fail == 0)
-                for (int c = tid; c < (npad - n) * 8; c += kAttnThreads)
-                    reinterpret_cast<uint4 *>(Vr + (size_t)n * 128)[c] = make_uint4(0u, 0u, 0u, 0u);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
-        }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();   // all of P stored before the second product
-        const float lsum = red[0][r] + red[1][r];
-        // ---- O = P V into columns [128, 192) ---------------------------------------------------
-        const bool ok_s = s_fail == 0;   // the S waits' outcome, after the barrier above
-        if (tid == 0 && ok_s) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            for (int kk = 0; kk < npad / 16; ++kk)
-                umma_bf16_ts(tmem + 128u, tmem + 8u * kk, sw128_desc(smem_addr(Vr) + kk * 2048u), idesc_o, kk ? 1u : 0u);
-            umma_commit(smem_addr(&bar_o));
-            s_issued = 3 + 2 * t;
-        }
-        if (ok_s && !mbar_wait(smem_addr(&bar_o), (uint32_t)t & 1u)) atomicOr(&s_fail, 4);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        // ---- epilogue: this half's 32 dims of O / row sum -> bf16 -------------------------------
-        if (rows_here) {
-            uint32_t o[32];
-            tmem_ld16(lane_addr + 128u + 32u * half, *reinterpret_cast<uint32_t(*)[16]>(o));
-            tmem_ld16(lane_addr + 144u + 32u * half, *reinterpret_cast<uint32_t(*)[16]>(o + 16));
-            const int m = 128 * t + r;
-            if (m < n && s_fail == 0) {
-                const float inv = 1.0f / lsum;
-                uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(p.out) +
-                                                       (size_t)(o0 + m) * H * kAttnDh + (size_t)h * kAttnDh + 32 * half);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    uint32_t w[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float2 y = __fmul2_rn(
-                            make_float2(__uint_as_float(o[8 * c + 2 * e]), __uint_as_float(o[8 * c + 2 * e + 1])),
-                            make_float2(inv, inv));
-                        const __nv_bfloat162 b2 = __floats2bfloat162_rn(y.x, y.y);
-                        w[e] = *reinterpret_cast<const uint32_t *>(&b2);
-                    }
-                    dst[c] = make_uint4(w[0], w[1], w[2], w[3]);
-                }
-            }
-        }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();   // O read and the sums consumed before the next tile's S overwrites them
-        stop = s_fail != 0;
-        __syncthreads();   // nobody writes s_fail again before every thread has read it
-    }
-    if (tid == 0 && s_fail != 0) {   // let everything this CTA started finish before it leaves
-        raise_status(p.status, FUSION_DEV_TIMEOUT);
-        mbar_wait(smem_addr(&bar_ld), 0);
-        mbar_wait(smem_addr(&bar_ld2), 0);
-        const int k = s_issued;   // 2 + 2t: S of tile t issued; 3 + 2t: also its O
-        if (k >= 2) mbar_wait(smem_addr(&bar_s), (uint32_t)((k - 2) >> 1) & 1u);
-        if (k >= 3 && (k & 1)) mbar_wait(smem_addr(&bar_o), (uint32_t)((k - 3) >> 1) & 1u);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kAttnTmemCols) : "memory");
-}
-
-// ---------------------------------------------------------------------------
-// Samples of 257 .. 1024 tokens.  The keys come in blocks of 128 (K, and V for the second
-// pass), double-buffered by TMA one step ahead; per query tile a first pass over the key blocks
-// takes the softmax shift (max_j S scale + max_j log2 s_j, as above) and a second pass forms P
-// over S's first columns and accumulates O = P V over the key blocks in columns [128, 192).
-// Q tiles are double-buffered too; every step waits for the previous step's products, so a
-// buffer is refilled only once nothing reads it.
-// ---------------------------------------------------------------------------
-constexpr int kLongMaxN = 1024;
-constexpr uint32_t kKvBytes = 128 * 128;   // a block of 128 key rows (K or V)
-
-__global__ void __launch_bounds__(kAttnThreads, 2)
-    k_attn_tc_long(const __grid_constant__ AttnMaps maps, AttnParams p) {
-    extern __shared__ unsigned char sm_raw[];
-    unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ __align__(8) unsigned long long bar_ld[2], bar_s, bar_o;
-    __shared__ uint32_t tmem_base;
-    __shared__ int s_fail, s_ld, s_ns, s_no;   // steps whose loads were issued; products S and O issued
-    __shared__ __align__(16) float lsz[kLongMaxN];
-    __shared__ float red[2][128];
-    __shared__ float s_lszmax;
-
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int h = blockIdx.x, i = blockIdx.y;
-    const int B = device_batch(p.in);
-    if (B < 0) {
-        if (h == 0 && i == 0 && tid == 0) raise_status(p.status, FUSION_DEV_BAD_BATCH);
-        return;
-    }
-    if (i >= B) return;
-    const int o0 = p.in.offsets[i], n = p.in.offsets[i + 1] - o0;
-    if (o0 < 0 || n < 1 || n > p.in.max_tokens || n > kLongMaxN || (long long)o0 + n > p.in.max_rows) {
-        if (h == 0 && tid == 0) raise_status(p.status, FUSION_DEV_BAD_OFFSETS);
-        return;
-    }
-    const int H = p.heads;
-    const int T = (n + 127) >> 7;          // query tiles
-    const int nkv = (n + 127) >> 7;        // key blocks
-    const int steps = T * 2 * nkv;         // (tile, pass, block) in that order
-    unsigned char *Qb = sm;                                 // [2] query tiles
-    unsigned char *Kb = sm + 2 * kQTileBytes;               // [2] key blocks
-    unsigned char *Vb = Kb + 2 * kKvBytes;                  // [2] value blocks
-
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_base)),
-                     "r"(kAttnTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    // the loads of step k into buffer k & 1: the key block, the value block in the second pass,
-    // the query tile at a tile's first step
-    auto issue = [&](int k) {
-        const int t = k / (2 * nkv), pass = (k / nkv) & 1, kb = k % nkv;
-        const int buf = k & 1;
-        const int rows_k = min(128, n - 128 * kb), rk = (rows_k + 7) & ~7;
-        const bool q = pass == 0 && kb == 0;
-        const int rq = (min(128, n - 128 * t) + 7) & ~7;
-        uint32_t bytes = (uint32_t)rk * 128u * (pass ? 2u : 1u) + (q ? (uint32_t)rq * 128u : 0u);
-        const uint32_t bar = smem_addr(&bar_ld[buf]);
-        mbar_expect_tx(bar, bytes);
-        auto rows = [&](unsigned char *dst, int x, int y0, int cnt) {
-            int r = 0;
-            for (; r + 32 <= cnt; r += 32) tma_load_2d(smem_addr(dst + r * 128), &maps.b32, x, y0 + r, bar);
-            for (; r < cnt; r += 8) tma_load_2d(smem_addr(dst + r * 128), &maps.b8, x, y0 + r, bar);
-        };
-        rows(Kb + buf * kKvBytes, (H + h) * kAttnDh, o0 + 128 * kb, rk);
-        if (pass) rows(Vb + buf * kKvBytes, (2 * H + h) * kAttnDh, o0 + 128 * kb, rk);
-        if (q) rows(Qb + (t & 1) * kQTileBytes, h * kAttnDh, o0 + 128 * t, rq);
-    };
-    if (tid == 0) {
-        s_fail = 0;
-        s_ns = s_no = 0;
-        mbar_init(smem_addr(&bar_ld[0]), 1);
-        mbar_init(smem_addr(&bar_ld[1]), 1);
-        mbar_init(smem_addr(&bar_s), 1);
-        mbar_init(smem_addr(&bar_o), 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        issue(0);
-        s_ld = 1;
-    }
-    for (int j = tid; j < n; j += kAttnThreads) lsz[j] = p.sizes ? log2f(p.sizes[o0 + j]) : 0.0f;
-    __syncthreads();
-    if (warp == 0) {
-        float lm = -INFINITY;
-        for (int j = threadIdx.x; j < n; j += 32) lm = fmaxf(lm, lsz[j]);
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) lm = fmaxf(lm, __shfl_xor_sync(0xFFFFFFFFu, lm, o));
-        if (threadIdx.x == 0) s_lszmax = lm;
-    }
-    __syncthreads();
-
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base;
-    const int half = warp >> 2;
-    const int r = tid & 127;
-    const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    constexpr float kScale2 = 0.18033688011112042f;   // log2(e) / sqrt(64)
-    const uint32_t idesc_o =
-        (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(kAttnDh >> 3) << 17) | (8u << 24);
-    float mraw = -INFINITY, mx = 0.0f;
-    float2 lsum2 = make_float2(0.0f, 0.0f);   // even and odd columns (packed float32 pairs)
-    bool stop = false;
-    for (int k = 0; k < steps && !stop; ++k) {
-        const int t = k / (2 * nkv), pass = (k / nkv) & 1, kb = k % nkv;
-        const int buf = k & 1;
-        const int rows_k = min(128, n - 128 * kb), npadb = (rows_k + 15) & ~15;
-        const bool rows_here = 128 * t + 32 * (warp & 3) < n;   // warp-uniform
-        const int nch = npadb >> 4, cA = (nch + 1) >> 1;
-        const int c_lo = half ? cA : 0, c_hi = half ? nch : cA;
-        // ---- this step's blocks landed; the next step's loads go out -------------------------
-        if (tid == 0) {
-            if (!mbar_wait(smem_addr(&bar_ld[buf]), (uint32_t)(k >> 1) & 1u)) {
-                s_fail = 1;
-            } else if (k + 1 < steps) {
-                issue(k + 1);
-                s_ld = k + 2;
+
+    if (warp >= NWG * 4 && warp - NWG * 4 < nw) {
+        // ---- products of tile w ----------------------------------------------------------------------
+        // S of block 0; then per block O += P V, followed by the next block's S
+        const int w = __shfl_sync(0xFFFFFFFFu, warp, 0) - NWG * 4;
+        const int nb_u = (n_u + kKeyBlock - 1) / kKeyBlock;
+        const uint32_t d = __shfl_sync(0xFFFFFFFFu, tmem, 0) + w * kTileCols;
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);
+        const uint64_t qd = sw128_desc(smem_addr(Q + w * kQTileBytes));
+        const uint64_t kd0 = sw128_desc(smem_addr(Kr)), vd0 = sw128_desc(smem_addr(Vr));   // (in 16-byte units)
+        auto keys_of = [&](int j) { return (min(kKeyBlock, n_u - j * kKeyBlock) + 15) & ~15; };   // the MMA granularity
+        auto s_product = [&](int j, int st, uint32_t dst) {
+            const uint64_t kd = kd0 + (uint32_t)st * (kKeyBytes >> 4);
+            const uint32_t id = idesc | ((uint32_t)(keys_of(j) >> 3) << 17);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) umma_bf16(dst, qd + 2u * k, kd + 2u * k, id, k ? 1u : 0u);
+        };
+        bool ok = warp_wait(smem_addr(&bar.q[w]), 0);
+        RingPos kp, vp, rf;   // stages of block j + 1's K, of block j's V, and of the block to refill next
+        int next = min(nb_u, ns);
+        for (int j = -1; ok && j < nb_u; ++j) {
+            const int cnt = min(kKeyBlock, n_u - j * kKeyBlock), np = (cnt + 15) & ~15;
+            if (j >= 0) {
+                ok = warp_wait(smem_addr(&bar.v[vp.st]), vp.par);
+                if (ok && cnt < np) {
+                    // V rows past the sample (another sample's rows or stale memory) read as zero in P V (both
+                    // tiles' warps write these zeros)
+                    for (int c = lane; c < (np - cnt) * 8; c += 32)
+                        reinterpret_cast<uint4 *>(Vr + vp.st * kKeyBytes + (size_t)cnt * 128)[c] = make_uint4(0u, 0u, 0u, 0u);
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
+                    __syncwarp();
+                }
             }
+            if (ok && j + 1 < nb_u) ok = warp_wait(smem_addr(&bar.k[kp.st]), kp.par);
+            if (ok && j >= 0) ok = warp_wait(smem_addr(&bar.p[w]), (uint32_t)j & 1u);
+            if (elect_one() && ok) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (j >= 0) {
+                    // B = V as it lies: MN-major (bit 16), 8-key swizzle atoms 1024 bytes apart
+                    const uint64_t vd = vd0 + (uint32_t)vp.st * (kKeyBytes >> 4);
+                    const uint32_t id = idesc | (1u << 16) | ((uint32_t)(kAttnDh >> 3) << 17);
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        if (kk * 16 < np) umma_bf16_ts(d + 64u, d + 8u * kk, vd + 128u * kk, id, (j | kk) ? 1u : 0u);
+                }
+                if (j + 1 < nb_u) s_product(j + 1, kp.st, d);
+                umma_commit(smem_addr(&bar.s[w]));
+                if (j >= 0) umma_commit(smem_addr(&bar.free[vp.st]));   // this block's K and V are read
+                // the last tile's lane refills the stage of the block before (both tiles are past it, or nearly)
+                if (w == nw - 1 && j >= 1 && next < nb_u) {
+                    ok = mbar_wait(smem_addr(&bar.free[rf.st]), rf.par);
+                    if (ok) {
+                        load_k(next, rf.st);
+                        load_v(next, rf.st);
+                        rf.next(ns);
+                        s_kv = ++next;
+                    }
+                }
+            }
+            ok = __all_sync(0xFFFFFFFFu, ok);
+            if (j + 1 < nb_u) kp.next(ns);
+            if (j >= 0) vp.next(ns);
         }
-        __syncthreads();
-        if (s_fail & 1) break;   // uniform: bit 1 is written only before the barrier above
-        if (pass == 1 && rows_k < npadb)   // value rows past the sample read as zero in P V
-            for (int c = tid; c < (npadb - rows_k) * 8; c += kAttnThreads)
-                reinterpret_cast<uint4 *>(Vb + buf * kKvBytes + (size_t)rows_k * 128)[c] = make_uint4(0u, 0u, 0u, 0u);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        // ---- S = Q_t K_kb^T --------------------------------------------------------------------
-        if (tid == 0) {
+        if (!ok) atomicOr(&s_fail, 2);
+    } else if (warp < nw * 4) {
+        // ---- softmax: one thread per query row ---------------------------------------------------
+        const int w = warp >> 2, r = tid & 127;
+        const bool here = row0 + 128 * w + 32 * (warp & 3) < n;   // warp-uniform: a warp of rows past the sample idles
+        const uint32_t taddr = tmem + w * kTileCols + ((uint32_t)((warp & 3) * 32) << 16);
+        float lszmax = red_max[0], lszmin = red_min[0];
+#pragma unroll
+        for (int k = 1; k < NWG * 4; ++k) {
+            lszmax = fmaxf(lszmax, red_max[k]);
+            lszmin = fminf(lszmin, red_min[k]);
+        }
+        const bool sized = lszmax != 0.0f || lszmin != 0.0f;
+        constexpr float kScale2 = 0.18033688011112042f;   // log2(e) / sqrt(64)
+        float m = 0.0f, mraw = -INFINITY;        // the shift; the largest S so far
+        float2 lsum = make_float2(0.0f, 0.0f);   // even and odd keys
+        bool ok = true;
+        for (int j = 0; ok && j < nb; ++j) {
+            ok = warp_wait(smem_addr(&bar.s[w]), (uint32_t)j & 1u);   // S of block j, and O up to the block before
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(npadb >> 3) << 17) | (8u << 24);
+            if (ok && here) {
+                const int cnt = n - j * kKeyBlock;
+                uint32_t v[64];
+                tmem_ld32(taddr, v);
+                tmem_ld32(taddr + 32u, v + 32);
+                tmem_ld_wait();
+                if (cnt < kKeyBlock) {   // keys past the sample: probability 2^-inf = 0
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                umma_bf16(tmem, sw128_desc(smem_addr(Qb + (t & 1) * kQTileBytes) + kk * 32),
-                          sw128_desc(smem_addr(Kb + buf * kKvBytes) + kk * 32), idesc_s, kk ? 1u : 0u);
-            umma_commit(smem_addr(&bar_s));
-            s_ns = s_ns + 1;
-        }
-        if (!mbar_wait(smem_addr(&bar_s), (uint32_t)k & 1u)) atomicOr(&s_fail, 2);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (pass == 0) {
-            // ---- first pass: running maximum of S over this half's columns ---------------------
-            if (rows_here) {
-                for (int c = c_lo; c < c_hi; ++c) {
-                    uint32_t v[16];
-                    tmem_ld16(lane_addr + (uint32_t)(16 * c), v);
-                    if (16 * c + 16 <= rows_k) {
-                        mraw = max16(mraw, v);
-                    } else {
+                    for (int e = 0; e < 64; ++e) v[e] = e < cnt ? v[e] : 0xFF800000u;
+                }
+                float a[4] = {mraw, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-                        for (int e = 0; e < 16; ++e)
-                            if (16 * c + e < rows_k) mraw = fmaxf(mraw, __uint_as_float(v[e]));
+                for (int e = 0; e < 64; e += 8)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        a[q] = max3(a[q], __uint_as_float(v[e + 2 * q]), __uint_as_float(v[e + 2 * q + 1]));
+                const float mx = fmaxf(max3(a[0], a[1], a[2]), a[3]);
+                const float mn = fmaf(mx, kScale2, lszmax), f = ex2(m - mn);   // the shift follows the largest S
+                const bool grows = j > 0 && __any_sync(0xFFFFFFFFu, mx > mraw);
+                m = mn;
+                mraw = mx;
+                const float2 ps = sized ? block_probs<true>(v, taddr, lsz + j * kKeyBlock, m)
+                                        : block_probs<false>(v, taddr, nullptr, m);
+                if (grows) {   // and the rows of O and their sums follow the shift (after P: S's registers are free)
+                    lsum = __fmul2_rn(lsum, make_float2(f, f));
+                    uint32_t o[64];
+                    tmem_ld32(taddr + 64u, o);
+                    tmem_ld32(taddr + 96u, o + 32);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 64; e += 8) {
+                        uint32_t o8[8];
+#pragma unroll
+                        for (int q = 0; q < 8; q += 2) {
+                            const float2 y = __fmul2_rn(make_float2(__uint_as_float(o[e + q]), __uint_as_float(o[e + q + 1])),
+                                                        make_float2(f, f));
+                            o8[q] = __float_as_uint(y.x);
+                            o8[q + 1] = __float_as_uint(y.y);
+                        }
+                        tmem_st8(taddr + 64u + e, o8);
                     }
                 }
-            }
-            if (kb == nkv - 1) {   // the tile's shift from both halves
-                red[half][r] = mraw;
-                pair_sync(warp);
-                mx = fmaf(fmaxf(red[0][r], red[1][r]), kScale2, s_lszmax);
-                pair_sync(warp);
-            }
-        } else {
-            // ---- second pass: P over S's first columns, then O += P V_kb ----------------------
-            uint32_t pk[4][8];   // this half's chunks, at most 4
-            if (rows_here) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int c = c_lo + q;
-                    if (c < c_hi) {
-                        uint32_t v[16];
-                        tmem_ld16(lane_addr + (uint32_t)(16 * c), v);
-                        float pr[16];
-#pragma unroll
-                        for (int e = 0; e < 16; e += 2) {   // fma then subtract, two columns per instruction
-                            const float2 x = __fadd2_rn(
-                                __ffma2_rn(make_float2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])),
-                                           make_float2(kScale2, kScale2),
-                                           *reinterpret_cast<const float2 *>(&lsz[128 * kb + 16 * c + e])),
-                                make_float2(-mx, -mx));
-                            pr[e] = 16 * c + e < rows_k ? ex2(x.x) : 0.0f;
-                            pr[e + 1] = 16 * c + e + 1 < rows_k ? ex2(x.y) : 0.0f;
-                        }
-#pragma unroll
-                        for (int e = 0; e < 16; e += 2) {
-                            lsum2 = __fadd2_rn(lsum2, make_float2(pr[e], pr[e + 1]));
-                            const __nv_bfloat162 b2 = __floats2bfloat162_rn(pr[e], pr[e + 1]);
-                            pk[q][e >> 1] = *reinterpret_cast<const uint32_t *>(&b2);
-                        }
-                    }
-                }
-            }
-            pair_sync(warp);   // every S column of these rows read
-            if (rows_here) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (c_lo + q < c_hi) tmem_st8(lane_addr + (uint32_t)(8 * (c_lo + q)), pk[q]);
-                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                lsum = __fadd2_rn(lsum, ps);
+                tmem_st_wait();
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncthreads();
-            const bool ok_s = s_fail == 0;
-            if (tid == 0 && ok_s) {
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                for (int kk = 0; kk < npadb / 16; ++kk)
-                    umma_bf16_ts(tmem + 128u, tmem + 8u * kk, sw128_desc(smem_addr(Vb + buf * kKvBytes) + kk * 2048u),
-                                 idesc_o, (kb | kk) ? 1u : 0u);
-                umma_commit(smem_addr(&bar_o));
-                s_no = s_no + 1;
-            }
-            if (ok_s && !mbar_wait(smem_addr(&bar_o), (uint32_t)(t * nkv + kb) & 1u)) atomicOr(&s_fail, 4);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (kb == nkv - 1) {
-                // ---- the tile's epilogue: O / row sum -> bf16 --------------------------------------
-                red[half][r] = lsum2.x + lsum2.y;
-                __syncthreads();
-                const float l = red[0][r] + red[1][r];
-                if (rows_here && s_fail == 0) {
-                    uint32_t o[32];
-                    tmem_ld16(lane_addr + 128u + 32u * half, *reinterpret_cast<uint32_t(*)[16]>(o));
-                    tmem_ld16(lane_addr + 144u + 32u * half, *reinterpret_cast<uint32_t(*)[16]>(o + 16));
-                    const int m = 128 * t + r;
-                    if (m < n) {
-                        const float inv = 1.0f / l;
-                        uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(p.out) +
-                                                               (size_t)(o0 + m) * H * kAttnDh + (size_t)h * kAttnDh +
-                                                               32 * half);
+            mbar_arrive(smem_addr(&bar.p[w]));
+        }
+        if (ok) ok = warp_wait(smem_addr(&bar.s[w]), (uint32_t)nb & 1u);   // the last block's O
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (!ok) atomicOr(&s_fail, 4);
+        if (ok && here) {
+            // ---- O / row sum -> bf16, through the tile's Q rows (read by now), eight lanes per row ----
+            uint32_t o[64];
+            tmem_ld32(taddr + 64u, o);
+            tmem_ld32(taddr + 96u, o + 32);
+            tmem_ld_wait();
+            const float inv = 1.0f / (lsum.x + lsum.y);
+            unsigned char *qt = Q + w * kQTileBytes;
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            uint32_t w[4];
+            for (int c = 0; c < 8; ++c) {
+                uint32_t q4[4];
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float2 y = __fmul2_rn(
-                                    make_float2(__uint_as_float(o[8 * c + 2 * e]), __uint_as_float(o[8 * c + 2 * e + 1])),
-                                    make_float2(inv, inv));
-                                const __nv_bfloat162 b2 = __floats2bfloat162_rn(y.x, y.y);
-                                w[e] = *reinterpret_cast<const uint32_t *>(&b2);
-                            }
-                            dst[c] = make_uint4(w[0], w[1], w[2], w[3]);
-                        }
-                    }
+                for (int e = 0; e < 4; ++e) {
+                    const float2 y = __fmul2_rn(
+                        make_float2(__uint_as_float(o[8 * c + 2 * e]), __uint_as_float(o[8 * c + 2 * e + 1])),
+                        make_float2(inv, inv));
+                    const __nv_bfloat162 b2 = __floats2bfloat162_rn(y.x, y.y);
+                    q4[e] = *reinterpret_cast<const uint32_t *>(&b2);
                 }
-                mraw = -INFINITY;
-                lsum2 = make_float2(0.0f, 0.0f);
+                *reinterpret_cast<uint4 *>(qt + r * 128 + ((c ^ (r & 7)) << 4)) = make_uint4(q4[0], q4[1], q4[2], q4[3]);
+            }
+            __syncwarp();
+            __nv_bfloat16 *out = reinterpret_cast<__nv_bfloat16 *>(p.out) + (size_t)h * kAttnDh;
+            const int rw = 32 * (warp & 3) + (lane >> 3), c = lane & 7;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int rr = rw + 4 * k, mrow = row0 + 128 * w + rr;
+                if (mrow < n)
+                    *reinterpret_cast<uint4 *>(out + (size_t)(o0 + mrow) * H * kAttnDh + c * 8) =
+                        *reinterpret_cast<const uint4 *>(qt + rr * 128 + ((c ^ (rr & 7)) << 4));
             }
         }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();   // S, P and O read before the next step's products overwrite them
-        stop = s_fail != 0;
-        __syncthreads();
-    }
-    if (tid == 0 && s_fail != 0) {   // let everything this CTA started finish before it leaves
-        raise_status(p.status, FUSION_DEV_TIMEOUT);
-        for (int b = 0; b < 2; ++b) {
-            const int last = s_ld - 1 - ((s_ld - 1 - b) & 1);   // the last step issued into buffer b
-            if (last >= 0) mbar_wait(smem_addr(&bar_ld[b]), (uint32_t)(last >> 1) & 1u);
-        }
-        if (s_ns > 0) mbar_wait(smem_addr(&bar_s), (uint32_t)(s_ns - 1) & 1u);
-        if (s_no > 0) mbar_wait(smem_addr(&bar_o), (uint32_t)(s_no - 1) & 1u);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kAttnTmemCols) : "memory");
+    if (s_fail != 0 && warp == NWG * 4) {   // let everything this CTA started finish before it leaves
+        if (lane == 0) {
+            raise_status(p.status, FUSION_DEV_TIMEOUT);
+            for (int j = max(0, s_kv - ns); j < s_kv; ++j) {
+                (void)mbar_wait(smem_addr(&bar.k[j % ns]), (uint32_t)(j / ns) & 1u);
+                (void)mbar_wait(smem_addr(&bar.v[j % ns]), (uint32_t)(j / ns) & 1u);
+            }
+            for (int w = 0; w < nw; ++w) (void)mbar_wait(smem_addr(&bar.q[w]), 0);
+        }
+        __syncwarp();
+    }
+    if (s_fail != 0) {   // uniform: each issuing thread drains its own products
+        if (warp >= NWG * 4 && warp - NWG * 4 < nw && lane == 0) {
+            umma_commit(smem_addr(&bar.drain[warp - NWG * 4]));
+            (void)mbar_wait(smem_addr(&bar.drain[warp - NWG * 4]), 0);
+        }
+        __syncthreads();
+    }
+    if (warp == NWG * 5 - 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NWG * kTileCols) : "memory");
+}
+
+template <int NWG>
+cudaError_t launch_tiles(const AttnMaps &maps, const AttnParams &p, cudaStream_t s) {
+    const int n_part = ceil_div(p.in.max_tokens, NWG * 128);
+    const size_t smem = 1024 + (size_t)NWG * kQTileBytes + 2 * (size_t)attn_stages(p.in.max_tokens) * kKeyBytes;
+    cudaError_t e = cudaFuncSetAttribute(k_attn_tc<NWG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_attn_tc<NWG>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) return e;
+    k_attn_tc<NWG><<<dim3((unsigned)(p.heads * n_part), (unsigned)p.in.max_batch), NWG * 160, smem, s>>>(maps, p, n_part);
+    return cudaGetLastError();
 }
 
 }  // namespace
-
-size_t attn_smem_bytes(int max_tokens) {
-    if (max_tokens > kAttnMaxN) return 1024u + 2u * kQTileBytes + 4u * kKvBytes;   // two Q tiles, two K and V blocks
-    const int npad = (max_tokens + 15) & ~15, T = (max_tokens + 127) >> 7;
-    return 1024u + (size_t)T * kQTileBytes + 2u * (size_t)npad * 128u;   // alignment, Q tiles, K, V
-}
 
 cudaError_t launch_attention(const AttnParams &p, cudaStream_t s) {
     if (p.in.max_batch == 0 || p.heads == 0) return cudaSuccess;
     EncodeTiledFn enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
-    const size_t smem = attn_smem_bytes(p.in.max_tokens);
     AttnMaps maps;
-    for (int b = 0; b < 2; ++b) {
+    CUtensorMap *dst[4] = {&maps.b128, &maps.b64, &maps.b32, &maps.b8};
+    for (int b = 0; b < 4; ++b) {
         cuuint64_t dims[2] = {(cuuint64_t)3 * p.heads * kAttnDh, (cuuint64_t)p.in.max_rows};
         cuuint64_t strides[1] = {(cuuint64_t)3 * p.heads * kAttnDh * 2};
-        cuuint32_t box[2] = {64, b == 0 ? 32u : 8u};
+        cuuint32_t box[2] = {64, b == 0 ? 128u : b == 1 ? 64u : b == 2 ? 32u : 8u};
         cuuint32_t estr[2] = {1, 1};
-        if (enc(b == 0 ? &maps.b32 : &maps.b8, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(p.qkv), dims,
+        if (enc(dst[b], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(p.qkv), dims,
                 strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                 CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
-    auto kern = p.in.max_tokens > kAttnMaxN ? k_attn_tc_long : k_attn_tc;   // whole samples resident, or key blocks
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<dim3((unsigned)p.heads, (unsigned)p.in.max_batch), kAttnThreads, smem, s>>>(maps, p);
-    return cudaGetLastError();
+    // one query tile per CTA where the call's samples have one
+    return p.in.max_tokens <= 128 ? launch_tiles<1>(maps, p, s) : launch_tiles<2>(maps, p, s);
 }
 
 }  // namespace fz

@@ -77,7 +77,6 @@ struct AttnParams {
     void *out;             // [max_rows, heads, 64] bf16
     int *status;
 };
-size_t attn_smem_bytes(int max_tokens);
 cudaError_t launch_attention(const AttnParams &p, cudaStream_t s);
 
 // ---- pruning router: linear token scores ------------------------------------------------
