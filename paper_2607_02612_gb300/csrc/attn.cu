@@ -108,12 +108,6 @@ struct RingPos {
     }
 };
 
-__device__ __forceinline__ bool elect_one() {   // true in one lane of the (converged) warp
-    uint32_t p;
-    asm volatile("{ .reg .pred p; elect.sync _|p, 0xffffffff; selp.u32 %0, 1, 0, p; }" : "=r"(p));
-    return p != 0;
-}
-
 // mbar_wait by a whole warp, with one outcome.
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
     return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity));

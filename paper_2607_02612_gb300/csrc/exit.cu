@@ -1371,14 +1371,15 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
     const int l8 = lane & 7;
     for (int k = tid >> 3; active && k < BT; k += kExitThreads / 8) {   // uniform per warp
         const float *l = lg_s + k * L::lg_stride + l8;
-        float m = -INFINITY, z = 0.0f;
+        float m = -INFINITY, zq[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int q = 0; q < kExitCT; q += 8) m = fmaxf(m, l[q]);
 #pragma unroll
         for (int o = 4; o >= 1; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
 #pragma unroll
         for (int q = 0; q < kExitCT; q += 8)
-            if (l[q] != -INFINITY) z += expf(l[q] - m);
+            if (l[q] != -INFINITY) zq[(q >> 3) & 3] += expf(l[q] - m);
+        float z = (zq[0] + zq[1]) + (zq[2] + zq[3]);
 #pragma unroll
         for (int o = 4; o >= 1; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
         if (l8 < ncl)

@@ -165,7 +165,8 @@ bool fuse_plan(const fusion_ragged &in) { return in.max_batch >= 1 && in.max_bat
 cudaError_t launch_sample_kernel(int dtype, const ImageParams &p, const ImageGeometry &G, cudaStream_t s,
                                  bool pdl = false) {
     if (p.do_merge) {
-        const TcGeometry T = image_tc_geometry(dtype, p.in.max_tokens, p.kdim, p.dim, p.in.max_rows, 1, kTcSmemBudgetKb);
+        const TcGeometry T = image_tc_geometry(dtype, p.in.max_tokens, p.kdim, p.dim, p.in.max_rows, 1, kTcSmemBudgetKb,
+                                               p.in.max_batch);
         if (T.ok) return launch_image_tc(p, T, s, pdl);
         if (dtype == FUSION_F32) {   // the general kernel for samples whose stages do not fit
             const F32Geometry F = image_f32_geometry(p);

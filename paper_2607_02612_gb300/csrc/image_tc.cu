@@ -31,6 +31,7 @@ namespace fz {
 namespace {
 
 constexpr int kTcThreads = 256;
+constexpr int kSms = 152;
 constexpr int kMaxStages = 16;
 
 struct TcMaps {
@@ -123,11 +124,12 @@ __device__ __forceinline__ void issue_box(const TcMaps &maps, const Ring &R, int
 // Every barrier a ring can use, from one thread at kernel entry: the fence that publishes the
 // initialisation waits for the thread's outstanding memory operations, so it runs before the
 // thread has issued any.
+template <int NT>
 __device__ __forceinline__ void ring_barriers_init(unsigned long long *bar_full, unsigned long long *bar_empty,
                                                    unsigned long long *bar_done) {
     for (int st = 0; st < kMaxStages; ++st) {
         mbar_init(smem_addr(&bar_full[st]), 1);
-        mbar_init(smem_addr(&bar_empty[st]), 1 + kTcThreads / 32);
+        mbar_init(smem_addr(&bar_empty[st]), 1 + NT / 32);
     }
     mbar_init(smem_addr(bar_done), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -168,24 +170,27 @@ __device__ __forceinline__ void group_start(const TcMaps &maps, const Ring &R, i
 }
 // The sample's token sizes and scores and its CLS row into shared memory (cp.async, one
 // group; waited for in meta_init_rest).
+template <int NT>
 __device__ __forceinline__ void prefetch_own(const ImageParams &p, int start, int N, const MetaPtrs &m, uint4 *cls) {
-    for (int pos = threadIdx.x; pos < N; pos += kTcThreads) {
+    for (int pos = threadIdx.x; pos < N; pos += NT) {
         cp_async4(&m.tsize[pos], p.sizes + start + pos);
         if (p.scores) cp_async4(&m.tscore[pos], p.scores + start + pos);
     }
     const uint4 *row = reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(p.x) + (long long)start * p.dim);
-    for (int c = threadIdx.x; c < p.dim / 8; c += kTcThreads) cp_async16(&cls[c], row + c);
+    for (int c = threadIdx.x; c < p.dim / 8; c += NT) cp_async16(&cls[c], row + c);
     cp_async_commit();
 }
 
-__global__ void __launch_bounds__(kTcThreads, 2)
+// NT 256: two CTAs per SM; 128 (large batches of samples of at most 129 tokens): four.
+template <int NT>
+__global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
     k_image_tc(const __grid_constant__ TcMaps maps, ImageParams p, TcGeometry g) {
     extern __shared__ unsigned char sm_raw[];
     unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) & ~uintptr_t(1023));
     __shared__ __align__(8) unsigned long long bar_full[kMaxStages], bar_empty[kMaxStages], bar_done;
     __shared__ uint32_t tmem_base;
     __shared__ int s_fail;
-    __shared__ unsigned long long half_best[kTcThreads / 2];
+    __shared__ unsigned long long half_best[NT == 256 ? 128 : 1];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // Tensor memory first: an SM admits another CTA of a kernel that allocates tensor
@@ -203,7 +208,7 @@ __global__ void __launch_bounds__(kTcThreads, 2)
     }
     // the ring's barriers, before this thread issues any memory operation (warp 0 issues the
     // tokens' loads after a CTA barrier: the fused plan's, or the one below)
-    if (tid == 36) ring_barriers_init(bar_full, bar_empty, &bar_done);
+    if (tid == 36) ring_barriers_init<NT>(bar_full, bar_empty, &bar_done);
     if (g.grouped && (tid == 38 || tid == 39))
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tid == 38 ? &maps.ge : &maps.go)) : "memory");
     if (tid == 0) s_fail = 0;   // visible after the barriers below, before any other write
@@ -215,7 +220,7 @@ __global__ void __launch_bounds__(kTcThreads, 2)
     // kernel's end; the exit mask is read after `griddepcontrol.wait` (without a programmatic
     // predecessor the wait returns at once)
     SampleInfo s;
-    if (!sample_begin<kTcThreads>(p, blockIdx.x, s, true)) {   // uniform over the CTA
+    if (!sample_begin<NT>(p, blockIdx.x, s, true)) {   // uniform over the CTA
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         if (warp == 0)
@@ -237,7 +242,7 @@ __global__ void __launch_bounds__(kTcThreads, 2)
 
     // the sample's sizes, scores and CLS row first (a few KB that would otherwise queue behind the
     // bulk loads), then its tokens: the grouped layout or the ring's first stages (warp 0)
-    prefetch_own(p, s.start, s.N, m, cls);
+    prefetch_own<NT>(p, s.start, s.N, m, cls);
     const bool grouped = g.grouped && S >= nkb;   // the layout of this sample (uniform)
     const uint32_t gstride = (uint32_t)nkb * 1024u;
     unsigned char *gB = sm + (size_t)(R.rowsA >> 3) * gstride;   // grouped layout: half B
@@ -247,7 +252,7 @@ __global__ void __launch_bounds__(kTcThreads, 2)
         else
             ring_start(maps, R, s.start, s.nA, s.nB, nkb, sm, bar_full);
     }
-    meta_init_rest<kTcThreads>(p, s, m);
+    meta_init_rest<NT>(p, s, m);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -260,15 +265,16 @@ __global__ void __launch_bounds__(kTcThreads, 2)
         // Squared row norms: for a sample that stays resident, after all stages landed with
         // kT threads per row; otherwise one thread per row, K-block by K-block as the ring turns.
         const bool resident = S >= nkb;
-        const bool isA = tid < 128;
-        const int row = isA ? tid : tid - 128;
+        const int splitA = NT == 256 ? 128 : s.nA;   // 128 threads: nA + nB <= 128
+        const bool isA = tid < splitA;
+        const int row = isA ? tid : tid - splitA;
         const bool has_row = !resident && row < (isA ? s.nA : s.nB);
         float ss = 0.0f, sc = 0.0f;
         bool ok = true;
         if (grouped) {   // everything behind one barrier; all products at once
             if (!mbar_wait(smem_addr(&bar_full[0]), 0u)) {
                 ok = false;
-            } else if (tid == 32) {
+            } else if (warp == 1 && elect_one()) {
                 const uint32_t a0 = smem_addr(sm), b0 = smem_addr(gB);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 for (int kb = 0; kb < nkb; ++kb)
@@ -286,7 +292,7 @@ __global__ void __launch_bounds__(kTcThreads, 2)
                 ok = false;
                 break;
             }
-            if (tid == 32) {
+            if (warp == 1 && elect_one()) {
                 const uint32_t a0 = smem_addr(regA + (size_t)st * kbs), b0 = smem_addr(regB + (size_t)st * kbs);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
@@ -318,7 +324,7 @@ __global__ void __launch_bounds__(kTcThreads, 2)
             // kT threads per row (the largest power of two up to 8 that fits), each taking
             // every kT-th chunk of the row; the partial sums meet by shuffles
             const int R = s.nA + s.nB;
-            const int kT = R <= 32 ? 8 : R <= 64 ? 4 : R <= 128 ? 2 : 1;
+            const int kT = R <= NT / 8 ? 8 : R <= NT / 4 ? 4 : R <= NT / 2 ? 2 : 1;
             const int r = tid / kT, part = tid % kT;
             if (r < R) {
                 const bool rA = r < s.nA;
@@ -358,7 +364,7 @@ __global__ void __launch_bounds__(kTcThreads, 2)
             // epilogue: thread -> A row (tid % 128); the two warpgroups take the low / high columns
             const int wg = tid >> 7;
             const int r = tid & 127;
-            const int half_cols = ((npad / 16 + 1) / 2) * 16;
+            const int half_cols = NT == 256 ? ((npad / 16 + 1) / 2) * 16 : npad;
             const int c_lo = wg ? half_cols : 0, c_hi = wg ? npad : half_cols;
             const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
             const float ia = r < s.nA ? m.inv_a[r] : 0.0f;
@@ -382,17 +388,21 @@ __global__ void __launch_bounds__(kTcThreads, 2)
                 }
             }
             const unsigned long long bk = (r < s.nA && bi >= 0) ? rank_key(bv, bi) : 0ull;
-            if (wg == 1) half_best[r] = bk;
-            __syncthreads();
-            if (wg == 0 && r < s.nA) {
-                const unsigned long long o = half_best[r];
-                m.best[r] = o > bk ? o : bk;
+            if constexpr (NT == 256) {
+                if (wg == 1) half_best[r] = bk;
+                __syncthreads();
+                if (wg == 0 && r < s.nA) {
+                    const unsigned long long o = half_best[r];
+                    m.best[r] = o > bk ? o : bk;
+                }
+            } else if (r < s.nA) {
+                m.best[r] = bk;
             }
         } else {
             if (tid == 0) raise_status(p.status, FUSION_DEV_TIMEOUT);
         }
         __syncthreads();
-        if (s_fail == 0) select_top_r<kTcThreads>(s, m);
+        if (s_fail == 0) select_top_r<NT>(s, m);
     }
 
     if (s_fail == 0) {
@@ -406,7 +416,7 @@ __global__ void __launch_bounds__(kTcThreads, 2)
             ld.G = grouped ? gstride : 1024u;
             ld.K = grouped ? 1024u : kbs;
         }
-        finish_sample<__nv_bfloat16, kTcThreads>(p, s, m, ld);
+        finish_sample<__nv_bfloat16, NT>(p, s, m, ld);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -720,7 +730,7 @@ TcGeometry tiled_geometry(int max_tokens, int kdim) {
 }  // namespace
 
 TcGeometry image_tc_geometry(int dtype, int max_tokens, int kdim, int dim, long long max_rows, int do_merge,
-                             int stage_budget_kb) {
+                             int stage_budget_kb, int max_batch) {
     TcGeometry g{};
     if (dtype != FUSION_BF16 || !do_merge || kdim % 64 != 0 || max_rows < 2) return g;
     const int nAmax = (max_tokens - 1) / 2, nBmax = max_tokens / 2;
@@ -735,6 +745,32 @@ TcGeometry image_tc_geometry(int dtype, int max_tokens, int kdim, int dim, long 
     // the largest read from a stage base: 128 A rows, or half A and npad B rows
     const size_t npad_max = (size_t)((nBmax + 15) & ~15);
     const size_t reach = std::max<size_t>(16384, g.kb_a + npad_max * 128);
+    // More samples than two CTAs per SM hold, each with at most 128 rows: CTAs of 128 threads with
+    // four K-block stages, as many per SM as fit (the samples' chains of latencies overlap; a sample that does
+    // not stay in shared memory is gathered from L2).  8192 samples of 9 to 65 tokens, d = 384, four stages
+    // that keep 40 % each, per-sample kernels 452 -> 318 us; at 304 samples a CTA of 256 threads finishes its
+    // sample sooner and every sample has one at once.
+    if (max_batch > 2 * kSms && max_tokens <= 129) {
+        auto small = [&](int S) {
+            const size_t meta_base = (size_t)S * per_stage;
+            return std::max(meta_layout(max_tokens, meta_base).total + (size_t)dim * 2, (size_t)(S - 1) * per_stage + reach);
+        };
+        const int S = std::min(g.n_kb, 4);
+        for (int per_sm = 4; per_sm >= 3; --per_sm) {
+            // 228 KB per SM, 1 KB of it reserved per CTA, 1 KB of alignment slack and the static arrays
+            if (small(S) + 1024 + 1536 + 1024 > (size_t)228 * 1024 / per_sm) continue;
+            g.threads = 128;
+            g.stages = S;
+            g.stage_region = (uint32_t)(S * per_stage);
+            g.meta_base = g.stage_region;
+            g.cls_base = (uint32_t)meta_layout(max_tokens, g.meta_base).total;
+            g.usable = (uint32_t)small(S);
+            g.smem = g.usable + 1024;
+            g.ok = 1;
+            return g;
+        }
+    }
+    g.threads = 256;
     size_t budget = (size_t)stage_budget_kb * 1024;
     if (budget > 227 * 1024 - 4096) budget = 227 * 1024 - 4096;   // room for static shared memory
     // usable bytes for S stages at max_tokens: the ring, the metadata, the CLS row (dim bf16)
@@ -795,7 +831,7 @@ cudaError_t launch_image_tc(const ImageParams &p, const TcGeometry &g, cudaStrea
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
-    auto kernel = g.tiled ? k_image_tc_tiled : k_image_tc;
+    auto kernel = g.tiled ? k_image_tc_tiled : g.threads == 128 ? k_image_tc<128> : k_image_tc<256>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
     if (e != cudaSuccess) return e;
     // the largest shared-memory carveout, so that both CTAs of an SM are resident from the start
@@ -803,7 +839,7 @@ cudaError_t launch_image_tc(const ImageParams &p, const TcGeometry &g, cudaStrea
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(p.in.max_batch);
-    cfg.blockDim = dim3(kTcThreads);
+    cfg.blockDim = dim3(g.tiled ? kTcThreads : g.threads);
     cfg.dynamicSmemBytes = g.smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];

@@ -165,6 +165,7 @@ cudaError_t launch_image_f32(const ImageParams &p, const F32Geometry &g, cudaStr
 struct TcGeometry {
     int ok;
     int tiled;         // halves beyond one tile: k_image_tc_tiled (M-tiles of 128 A rows, one CTA per SM)
+    int threads;       // of k_image_tc
     int grouped;       // samples that fit in shared memory load in 8-row groups of all K-blocks (one 3-D box
                        // per group) instead of through the ring
     int n_kb;          // key K-blocks of 64 dims
@@ -178,7 +179,7 @@ struct TcGeometry {
     size_t smem;                     // dynamic shared memory bytes (usable + 1 KB alignment slack)
 };
 TcGeometry image_tc_geometry(int dtype, int max_tokens, int kdim, int dim, long long max_rows, int do_merge,
-                             int stage_budget_kb);
+                             int stage_budget_kb, int max_batch);
 // pdl: launched as a programmatic dependent of the kernel before it on the stream (the exit
 // check of a fused stage); the kernel waits for that grid before it reads any input
 cudaError_t launch_image_tc(const ImageParams &p, const TcGeometry &g, cudaStream_t s, bool pdl = false);

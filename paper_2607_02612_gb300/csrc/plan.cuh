@@ -33,7 +33,7 @@ constexpr int kPlanRhoNonfinite = 1 << 30;   // a continuing sample's keep ratio
 // The plan of a batch above the fused plan's bound, in tiles of pt samples.  plan_tile, one warp:
 // a tile's output counts and its totals.  plan_scan, one block once every tile is done: the totals
 // become exclusive prefixes, and the batch-level outputs are written.  The per-sample kernel adds
-// the prefix inside its tile itself (sample_info), so no serial pass over the samples remains:
+// the prefix inside its tile itself (sample_live), so no serial pass over the samples remains:
 // one block over 8192 samples took about 20 us, the tiles run beside one another in the kernel that
 // makes the exit decisions and the scan of 128 totals takes about 2.
 //

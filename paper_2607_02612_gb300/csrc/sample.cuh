@@ -101,31 +101,44 @@ struct SampleInfo {
     bool decide;   // the merge decisions are needed (something merges, or matches are requested)
 };
 
-// The input sample this CTA handles, from the plan kernel's tiles (plan.cuh); false when there is
-// nothing to do (beyond the device batch count, an invalid call, or a sample that exited).
-// The grid has one CTA per possible sample (i < max_batch), so every load of the first
-// group is in bounds whatever the device batch count says (counts beyond it are whatever
-// an earlier call left, and are not used); they issue together.  Every warp adds the tile's counts
-// before the sample itself; thread 0 writes the sample's place in the output batch.
-__device__ __forceinline__ bool sample_info(const ImageParams &p, int i, SampleInfo &s) {
+// The j-th sample that continues, from the plan's tiles (plan.cuh); false when there is none, or when
+// the call is invalid.  Every warp finds the tile that holds it (the last one with at most j survivors
+// before it) among 32 pivots and then inside a pivot's tiles, and the sample in the tile by its counts.
+// Thread 0 writes the sample's place in the output batch.  Uniform over the CTA; no barrier.
+__device__ __forceinline__ bool sample_live(const ImageParams &p, int j, SampleInfo &s) {
     const PlanArgs &a = p.plan_args;
     const int lane = threadIdx.x & 31;
     const int bval = p.in.batch ? *p.in.batch : p.in.max_batch;
-    const int valid = a.plan[0];
-    const int t = i / a.pt, t0 = t * a.pt, own = i - t0;
+    const int valid = a.plan[0], n_live = a.plan[1];
+    const int all = (p.in.max_batch + a.pt - 1) / a.pt, step = (all + 31) / 32;
+    const int pv = lane * step < all ? a.agg[lane * step].x : 0;   // in bounds; beyond the batch it is not used
+    if (bval < 0 || bval > p.in.max_batch || valid == 0 || j >= n_live) return false;
+    const int tiles = (bval + a.pt - 1) / a.pt;
+    // (survivor counts before a tile never decrease, so the tiles with at most j form a prefix)
+    int t = (__popc(__ballot_sync(0xFFFFFFFFu, lane * step < tiles && pv <= j)) - 1) * step;
+    const int t_end = min(tiles, t + step);
+    for (int t0 = t + 1; t0 < t_end; t0 += 32) {
+        const int c = __popc(__ballot_sync(0xFFFFFFFFu, t0 + lane < t_end && a.agg[min(t0 + lane, t_end - 1)].x <= j));
+        t += c;
+        if (c < 32) break;
+    }
+    const int t0 = t * a.pt;
     const int4 base = a.agg[t];
-    const int c0 = t0 + lane < p.in.max_batch ? a.cnt[t0 + lane] : -1;
-    const int c1 = (a.pt > 32 && t0 + 32 + lane < p.in.max_batch) ? a.cnt[t0 + 32 + lane] : -1;
-    const int o0 = p.in.offsets[i], o1 = p.in.offsets[i + 1];
-    const int id = p.in.ids ? p.in.ids[i] : i;
-    if (bval < 0 || bval > p.in.max_batch || i >= bval || valid == 0) return false;
-    const int cnt = __shfl_sync(0xFFFFFFFFu, own < 32 ? c0 : c1, own & 31);
-    if (cnt < 0) return false;
-    const bool b0 = lane < own && c0 >= 0, b1 = lane + 32 < own && c1 >= 0;
-    int rows = (b0 ? c0 : 0) + (b1 ? c1 : 0);
+    const int c0 = t0 + lane < bval ? a.cnt[t0 + lane] : -1;
+    const int c1 = (a.pt > 32 && t0 + 32 + lane < bval) ? a.cnt[t0 + 32 + lane] : -1;
+    const unsigned m0 = __ballot_sync(0xFFFFFFFFu, c0 >= 0), m1 = __ballot_sync(0xFFFFFFFFu, c1 >= 0);
+    const int want = j - base.x, n0 = __popc(m0);   // the want-th set bit of (m1, m0)
+    const unsigned lt = (1u << lane) - 1u;
+    const bool h0 = c0 >= 0 && __popc(m0 & lt) == want, h1 = c1 >= 0 && n0 + __popc(m1 & lt) == want;
+    const unsigned f0 = __ballot_sync(0xFFFFFFFFu, h0), f1 = __ballot_sync(0xFFFFFFFFu, h1);
+    if (!(f0 | f1)) return false;   // cannot happen for a consistent plan
+    const int own = f0 ? __ffs(f0) - 1 : 32 + __ffs(f1) - 1, i = t0 + own;
+    const int cnt = __shfl_sync(0xFFFFFFFFu, f0 ? c0 : c1, own & 31);
+    int rows = (lane < own && c0 >= 0 ? c0 : 0) + (lane + 32 < own && c1 >= 0 ? c1 : 0);
 #pragma unroll
     for (int m = 16; m >= 1; m >>= 1) rows += __shfl_xor_sync(0xFFFFFFFFu, rows, m);
-    const int j = base.x + __popc(__ballot_sync(0xFFFFFFFFu, b0)) + __popc(__ballot_sync(0xFFFFFFFFu, b1));
+    const int o0 = p.in.offsets[i], o1 = p.in.offsets[i + 1];
+    const int id = p.in.ids ? p.in.ids[i] : i;
     s.start = o0;
     s.N = o1 - o0;
     s.out_start = base.y + rows;
@@ -291,8 +304,8 @@ __device__ __forceinline__ bool gate_open(const int *gate, unsigned spins) {
     return s_open != 0;
 }
 
-// Either the fused plan or the plan kernel's results, once the launch gate (if any) is open;
-// a CTA whose gate wait gives up raises FUSION_DEV_TIMEOUT and writes nothing.
+// Either the fused plan (i: the input sample) or the plan kernel's results (i: the i-th sample that
+// continues), once the launch gate (if any) is open; a CTA whose gate wait gives up raises FUSION_DEV_TIMEOUT and writes nothing.
 template <int NT>
 // dep_wait: see sample_plan; without the fused plan the wait comes first (the plan's results may be
 // the predecessor's output).
@@ -302,7 +315,7 @@ __device__ __forceinline__ bool sample_begin(const ImageParams &p, int i, Sample
         return false;
     }
     if (dep_wait && !p.fused_plan) asm volatile("griddepcontrol.wait;" ::: "memory");
-    return p.fused_plan ? sample_plan<NT>(p, i, s, dep_wait) : sample_info(p, i, s);
+    return p.fused_plan ? sample_plan<NT>(p, i, s, dep_wait) : sample_live(p, i, s);
 }
 
 template <int NT>

@@ -139,3 +139,16 @@ def test_float32_merge_tiles(counts, dim, keys, kdim):
     r = np.minimum(rng.integers(0, 40, len(counts)), np.asarray(counts) // 2).astype(np.int32)
     rho = rng.uniform(0.3, 1.0, len(counts)).astype(np.float32)
     run_stage_and_compare(b, StageSpec(True, False, True, r=r, rho=rho), f"{counts[:4]} x {len(counts)}")
+
+
+@pytest.mark.parametrize("counts,dim,keys,kdim", [
+    ([65, 64, 33, 17, 3, 2, 1] * 45, 384, "alias", None),       # 315 samples: four stages, some stay resident
+    ([129, 128, 97, 9] * 77, 192, "separate", 128),             # the longest samples of the small CTAs
+    ([130, 65] * 153, 64, "alias", None),                       # one token past them
+    ([33, 1] * 520, 1024, "alias", None)])                      # with the tiled plan, wide rows
+def test_bf16_merge_small_ctas(counts, dim, keys, kdim):
+    b = make_batch(counts, dim, "bf16", seed=len(counts), keys=keys, kdim=kdim, sizes="u1to4")
+    rng = np.random.default_rng(2)
+    r = np.minimum(rng.integers(0, 40, len(counts)), np.asarray(counts) // 2).astype(np.int32)
+    rho = rng.uniform(0.3, 1.0, len(counts)).astype(np.float32)
+    run_stage_and_compare(b, StageSpec(True, False, True, r=r, rho=rho), f"{counts[:4]} x {len(counts)}")
