@@ -36,6 +36,7 @@ constexpr int kMaxStages = 16;
 
 struct TcMaps {
     CUtensorMap e32, o32, e8, o8;   // even / odd rows, boxes of 32 / 8 rows x 64 dims
+    CUtensorMap e256, o256, e128, o128;   // the same with 256 / 128 rows (k_image_tc_tiled)
     // even / odd rows seen as (64 dims, row, K-block) with the K-block stride 128 B: a box of
     // 8 rows x all K-blocks lands as [K-block][8 rows][128 B], one 1 KB swizzle atom per K-block
     CUtensorMap ge, go;
@@ -427,7 +428,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
 
 // ---------------------------------------------------------------------------
 // Samples whose halves exceed one tile (|A| or |B| above 128; ViT-L/16 at 384: 288 x 288 x
-// 1024): one CTA per SM, tensor memory of 256 or 512 columns.  Half A is taken in M-tiles of
+// 1024): one CTA of 512 threads per SM, tensor memory of 256 or 512 columns.  Half A is taken in M-tiles of
 // 128 rows; half B in N-blocks of at most 256 columns, all of them held in tensor memory at once.
 // For every M-tile the K-blocks of (that tile's A rows, all B rows) stream by TMA through the
 // ring (stage q = M-tile q / n_kb, K-block q % n_kb); the B rows are loaded again for every
@@ -436,15 +437,16 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
 // norms: A rows of each tile and, during the first tile, the B rows, one thread per row.
 // ---------------------------------------------------------------------------
 constexpr int kTiledMaxStages = 8;
+constexpr int kTiledThreads = 512;
 
-__global__ void __launch_bounds__(kTcThreads, 1)
+__global__ void __launch_bounds__(kTiledThreads, 1)
     k_image_tc_tiled(const __grid_constant__ TcMaps maps, ImageParams p, TcGeometry g) {
     extern __shared__ unsigned char sm_raw[];
     unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) & ~uintptr_t(1023));
     __shared__ __align__(8) unsigned long long bar_full[kTiledMaxStages], bar_empty[kTiledMaxStages], bar_done, bar_drain;
     __shared__ uint32_t tmem_base;
     __shared__ int s_fail;
-    __shared__ unsigned long long half_best[kTcThreads / 2];
+    __shared__ unsigned long long part_best[kTiledThreads];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (warp == 0) {
@@ -459,7 +461,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");   // as in k_image_tc: the exit check's grid first
     SampleInfo s;
-    if (!sample_begin<kTcThreads>(p, blockIdx.x, s)) {
+    if (!sample_begin<kTiledThreads>(p, blockIdx.x, s)) {
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         if (warp == 0)
@@ -485,7 +487,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const bool oddA = (s.start + 2) & 1, oddB = (s.start + 1) & 1;
     // boxes of stage q: the A rows of its M-tile (32-row boxes, then 8-row boxes), then all B rows
     auto tile_rows = [&](int mt) { return min(128, s.nA - mt * 128); };
-    auto nboxes = [&](int n) { return (n >> 5) + (((n & 31) + 7) >> 3); };
+    // 256- and 128-row boxes while they fit, then 32, then 8: a copy costs its issuing thread about 200
+    // cycles, and 32-row boxes alone (13 per stage at 288 x 288) held the ring to 1.75 us per stage
+    auto nboxes = [&](int n) { return (n >> 8) + ((n >> 7) & 1) + ((n >> 5) & 3) + (((n & 31) + 7) >> 3); };
     auto stage_tx = [&](int mt) { return (uint32_t)(((tile_rows(mt) + 7) & ~7) + rowsB) * 128u; };
     auto issue_box = [&](int q, int b) {
         const int st = q % S, mt = q / nkb, kb = q - mt * nkb;
@@ -494,11 +498,23 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         const bool half = b >= nbA;   // B rows
         const int qq = half ? b - nbA : b;
         const int n = half ? s.nB : nA_t;
-        const int n32 = n >> 5;
-        const bool big = qq < n32;
-        const int row0 = big ? qq * 32 : n32 * 32 + (qq - n32) * 8;
         const bool odd = half ? oddB : oddA;
-        const CUtensorMap *map = big ? (odd ? &maps.o32 : &maps.e32) : (odd ? &maps.o8 : &maps.e8);
+        const int n256 = n >> 8, n128 = (n >> 7) & 1, n32 = (n >> 5) & 3;
+        int row0, u = qq;
+        const CUtensorMap *map;
+        if (u < n256) {
+            row0 = u * 256;
+            map = odd ? &maps.o256 : &maps.e256;
+        } else if ((u -= n256) < n128) {
+            row0 = n256 * 256;
+            map = odd ? &maps.o128 : &maps.e128;
+        } else if ((u -= n128) < n32) {
+            row0 = (n >> 7) * 128 + u * 32;
+            map = odd ? &maps.o32 : &maps.e32;
+        } else {
+            row0 = (n >> 5) * 32 + (u - n32) * 8;
+            map = odd ? &maps.o8 : &maps.e8;
+        }
         unsigned char *base = sm + (size_t)st * kbs + (half ? aBytes : 0u);
         tma_load_2d(smem_addr(base + (size_t)row0 * 128), map, kb * 64, (half ? yB : yA0 + mt * 128) + row0,
                     smem_addr(&bar_full[st]));
@@ -511,13 +527,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     };
 
     MetaPtrs m(sm, meta_layout(p.in.max_tokens, g.meta_base));
-    meta_prefetch<kTcThreads>(p, s, m);
+    meta_prefetch<kTiledThreads>(p, s, m);
     if (warp == 0) {
         if (lane == 0) s_fail = 0;
         if (dec) {
             if (lane < S) {
                 mbar_init(smem_addr(&bar_full[lane]), 1);
-                mbar_init(smem_addr(&bar_empty[lane]), 1 + kTcThreads / 32);
+                mbar_init(smem_addr(&bar_empty[lane]), 1 + kTiledThreads / 32);
             }
             if (lane == 31) mbar_init(smem_addr(&bar_done), 1);
             if (lane == 30) mbar_init(smem_addr(&bar_drain), 1);
@@ -533,20 +549,22 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
         }
     }
-    meta_init_rest<kTcThreads>(p, s, m);
+    meta_init_rest<kTiledThreads>(p, s, m);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
     if (dec) {
         const uint32_t tmem = tmem_base;
+        constexpr int kBRows = 2;   // B rows per thread: at most 512 over 384 threads
+        static_assert(kBRows * (kTiledThreads - 128) >= FUSION_MAX_TOKENS / 2, "B rows");
         bool ok = true;
         for (int mt = 0; mt < nM && ok; ++mt) {
             const int nA_t = tile_rows(mt);
             // norms: thread t < 128 owns A row t of this tile; during tile 0 threads 128.. own the
-            // B rows 128 apart
+            // B rows, kTiledThreads - 128 apart
             float ssA = 0.0f, scA = 0.0f;
-            float ssB[4] = {0.0f, 0.0f, 0.0f, 0.0f}, scB[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            float ssB[kBRows] = {}, scB[kBRows] = {};
             for (int kb = 0; kb < nkb; ++kb) {
                 const int q = mt * nkb + kb;
                 const int st = q % S;
@@ -556,7 +574,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     break;
                 }
                 const unsigned char *stA = sm + (size_t)st * kbs, *stB = stA + aBytes;
-                if (tid == 32) {
+                if (warp == 1 && elect_one()) {
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     for (int nb = 0; nb < nNB; ++nb) {
                         const int ncols = min(256, npad - nb * 256);
@@ -580,8 +598,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     }
                 } else if (mt == 0) {
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int br = tid - 128 + u * 128;
+                    for (int u = 0; u < kBRows; ++u) {
+                        const int br = tid - 128 + u * (kTiledThreads - 128);
                         if (br < s.nB) {
                             const unsigned char *rb = stB + br * 128;
 #pragma unroll
@@ -593,12 +611,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_addr(&bar_empty[st]));
-                if (tid == 0 && q + S < nq) {   // refill this stage (possibly with the next tile's K-block)
-                    if (!mbar_wait(smem_addr(&bar_empty[st]), par)) {
-                        ok = false;
-                        break;
-                    }
-                    produce(q + S);
+                if (warp == 0 && q + S < nq) {   // refill this stage (possibly with the next tile's K-block)
+                    ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_addr(&bar_empty[st]), par));
+                    if (!ok) break;
+                    if (elect_one()) produce(q + S);
+                    __syncwarp();
                     ++issued;
                 }
             }
@@ -610,8 +627,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             if (mt == 0 && tid >= 128) {
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int br = tid - 128 + u * 128;
+                for (int u = 0; u < kBRows; ++u) {
+                    const int br = tid - 128 + u * (kTiledThreads - 128);
                     if (br < s.nB) {
                         const float sq = __fadd_rn(ssB[u], scB[u]);
                         if (!isfinite(sq)) raise_status(p.status, FUSION_DEV_NONFINITE);
@@ -628,10 +645,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 ok = false;
                 break;
             }
-            // epilogue of the tile: thread -> A row (tid % 128); the warpgroups split the columns
+            // epilogue of the tile: thread -> A row (tid % 128); the four warpgroups split the columns
             const int wg = tid >> 7, r = tid & 127;
-            const int half_cols = ((npad / 16 + 1) / 2) * 16;
-            const int c_lo = wg ? half_cols : 0, c_hi = wg ? npad : half_cols;
+            const int part_cols = ((npad / 16 + 3) / 4) * 16;
+            const int c_lo = min(npad, wg * part_cols), c_hi = min(npad, c_lo + part_cols);
             const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
             const int arow = mt * 128 + r;
             const float ia = r < nA_t ? m.inv_a[arow] : 0.0f;
@@ -653,15 +670,17 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 }
             }
             const unsigned long long bk = (r < nA_t && bi >= 0) ? rank_key(bv, bi) : 0ull;
-            if (wg == 1) half_best[r] = bk;
+            part_best[tid] = bk;
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncthreads();   // the next tile's products overwrite the accumulators after this
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (wg == 0 && r < nA_t) {
-                const unsigned long long o = half_best[r];
-                m.best[arow] = o > bk ? o : bk;
+                unsigned long long o = bk;
+#pragma unroll
+                for (int k = 1; k < 4; ++k) o = part_best[k * 128 + r] > o ? part_best[k * 128 + r] : o;
+                m.best[arow] = o;
             }
-            __syncthreads();   // half_best is reused by the next tile
+            __syncthreads();   // part_best is reused by the next tile
         }
         if (s_fail != 0) {
             // a wait gave up: let the copies and products in flight land (bounded) before the
@@ -676,13 +695,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 (void)mbar_wait(smem_addr(&bar_drain), 0u);
             }
         } else {
-            select_top_r<kTcThreads>(s, m);
+            select_top_r<kTiledThreads>(s, m);
         }
         __syncthreads();
     }
     if (s_fail == 0) {
         const GlobalLoader<__nv_bfloat16> gl{reinterpret_cast<const __nv_bfloat16 *>(p.x), (long long)s.start, p.dim};
-        finish_sample<__nv_bfloat16, kTcThreads>(p, s, m, gl);
+        finish_sample<__nv_bfloat16, kTiledThreads>(p, s, m, gl);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -807,13 +826,15 @@ cudaError_t launch_image_tc(const ImageParams &p, const TcGeometry &g, cudaStrea
     TcMaps maps{};
     const cuuint64_t rows_even = (cuuint64_t)((p.in.max_rows + 1) / 2), rows_odd = (cuuint64_t)(p.in.max_rows / 2);
     const char *keys = reinterpret_cast<const char *>(p.keys);
-    for (int i = 0; i < 4; ++i) {
-        const int odd = i & 1, box_rows = i < 2 ? 32 : 8;
+    CUtensorMap *const dsts[8] = {&maps.e32, &maps.o32, &maps.e8, &maps.o8, &maps.e256, &maps.o256, &maps.e128, &maps.o128};
+    for (int i = 0; i < (g.tiled ? 8 : 4); ++i) {
+        constexpr int kBox[4] = {32, 8, 256, 128};
+        const int odd = i & 1, box_rows = kBox[i >> 1];
         cuuint64_t dims[2] = {(cuuint64_t)p.kdim, odd ? rows_odd : rows_even};
         cuuint64_t strides[1] = {(cuuint64_t)p.kdim * 2 * 2};   // every other row
         cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
         cuuint32_t estr[2] = {1, 1};
-        CUtensorMap *dst = i == 0 ? &maps.e32 : i == 1 ? &maps.o32 : i == 2 ? &maps.e8 : &maps.o8;
+        CUtensorMap *dst = dsts[i];
         void *base = const_cast<char *>(keys + (odd ? (size_t)p.kdim * 2 : 0));
         if (enc(dst, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -839,7 +860,7 @@ cudaError_t launch_image_tc(const ImageParams &p, const TcGeometry &g, cudaStrea
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(p.in.max_batch);
-    cfg.blockDim = dim3(g.tiled ? kTcThreads : g.threads);
+    cfg.blockDim = dim3(g.tiled ? kTiledThreads : g.threads);
     cfg.dynamicSmemBytes = g.smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
