@@ -30,7 +30,6 @@
 namespace fz {
 namespace {
 
-constexpr int kTcThreads = 256;
 constexpr int kSms = 152;
 constexpr int kMaxStages = 16;
 
@@ -428,13 +427,16 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
 
 // ---------------------------------------------------------------------------
 // Samples whose halves exceed one tile (|A| or |B| above 128; ViT-L/16 at 384: 288 x 288 x
-// 1024): one CTA of 512 threads per SM, tensor memory of 256 or 512 columns.  Half A is taken in M-tiles of
-// 128 rows; half B in N-blocks of at most 256 columns, all of them held in tensor memory at once.
-// For every M-tile the K-blocks of (that tile's A rows, all B rows) stream by TMA through the
-// ring (stage q = M-tile q / n_kb, K-block q % n_kb); the B rows are loaded again for every
-// M-tile (from L2 after the first).  The tile's products accumulate over its K-blocks, its
-// epilogue keeps each A row's best column, and the next tile reuses the accumulators.  Row
-// norms: A rows of each tile and, during the first tile, the B rows, one thread per row.
+// 1024): one CTA of 512 threads per SM, 512 tensor-memory columns.  Half A lies in M-tiles of 128
+// rows (up to four), half B in passes of at most 512 / M-tiles columns (a multiple of 16, at most 256), so
+// that the accumulators of all M-tiles of a pass fit tensor memory.  Per pass the K-blocks of (all A
+// rows, the pass's B rows) stream by TMA through the ring (stage q = pass q / n_kb, K-block q % n_kb); the
+// epilogue keeps each A row's best column over the passes.  Row norms, one thread per row: A during
+// the first pass, a pass's B rows during it.
+//
+// Bound by DRAM while it streams: A is read once per pass and B once.  One pass per M-tile, which reads
+// B once per M-tile (three times at 288 x 288, the second and third mostly from DRAM: a wave's first
+// tiles are larger than L2), took 58 us for the three tiles of 128 samples; the whole call takes 15 us less in this order (159 -> 144).
 // ---------------------------------------------------------------------------
 constexpr int kTiledMaxStages = 8;
 constexpr int kTiledThreads = 512;
@@ -472,32 +474,33 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
     const bool dec = s.decide;
     const int nkb = g.n_kb;
     int issued = 0;   // stages issued (thread 0's count; warp 0 issues the first ones)
-    const int nM = (s.nA + 127) >> 7;               // M-tiles of half A
-    const int rowsB = (s.nB + 7) & ~7;
+    const int nM = max(1, (s.nA + 127) >> 7);       // M-tiles of half A
+    const int rowsA = (s.nA + 7) & ~7;
     const int npad = (s.nB + 15) & ~15;             // columns of the product
-    const int nNB = (npad + 255) >> 8;              // N-blocks of at most 256 columns
-    // stage: [128 A rows][rowsB B rows] x 128 B; an MMA reads 128 A rows and up to npad B rows
-    const uint32_t aBytes = 128u * 128u;
-    const uint32_t kbs = aBytes + (uint32_t)rowsB * 128u;
-    const uint32_t reach = aBytes + (uint32_t)npad * 128u;
-    const int nq = nM * nkb;
+    const int nblk = min(256, g.tmem_cols / nM & ~15);   // columns of a pass and M-tile
+    const int nP = (npad + nblk - 1) / nblk;
+    // stage: [A rows][a pass's B rows] x 128 B; an MMA reads 128 A rows from a tile's start, and up to a
+    // pass's columns of B rows
+    const uint32_t aBytes = (uint32_t)rowsA * 128u;
+    const uint32_t kbs = aBytes + (uint32_t)min(nblk, (s.nB + 7) & ~7) * 128u;
+    const uint32_t reach = max((uint32_t)nM * 16384u, aBytes + (uint32_t)min(nblk, npad) * 128u);
+    const int nq = nP * nkb;
     int S = min(min(nq, kTiledMaxStages), (int)(g.stage_region / kbs));
     while (S > 1 && (uint32_t)(S - 1) * kbs + reach > g.usable) --S;
     const int yB = (s.start + 1) >> 1, yA0 = (s.start + 2) >> 1;
     const bool oddA = (s.start + 2) & 1, oddB = (s.start + 1) & 1;
-    // boxes of stage q: the A rows of its M-tile (32-row boxes, then 8-row boxes), then all B rows
-    auto tile_rows = [&](int mt) { return min(128, s.nA - mt * 128); };
+    // boxes of stage q: the A rows, then the B rows of its pass
+    auto pass_rows = [&](int ps) { return min(nblk, s.nB - ps * nblk); };
     // 256- and 128-row boxes while they fit, then 32, then 8: a copy costs its issuing thread about 200
     // cycles, and 32-row boxes alone (13 per stage at 288 x 288) held the ring to 1.75 us per stage
     auto nboxes = [&](int n) { return (n >> 8) + ((n >> 7) & 1) + ((n >> 5) & 3) + (((n & 31) + 7) >> 3); };
-    auto stage_tx = [&](int mt) { return (uint32_t)(((tile_rows(mt) + 7) & ~7) + rowsB) * 128u; };
+    auto stage_tx = [&](int ps) { return (uint32_t)(rowsA + ((pass_rows(ps) + 7) & ~7)) * 128u; };
     auto issue_box = [&](int q, int b) {
-        const int st = q % S, mt = q / nkb, kb = q - mt * nkb;
-        const int nA_t = tile_rows(mt);
-        const int nbA = nboxes(nA_t);
+        const int st = q % S, ps = q / nkb, kb = q - ps * nkb;
+        const int nbA = nboxes(s.nA);
         const bool half = b >= nbA;   // B rows
         const int qq = half ? b - nbA : b;
-        const int n = half ? s.nB : nA_t;
+        const int n = half ? pass_rows(ps) : s.nA;
         const bool odd = half ? oddB : oddA;
         const int n256 = n >> 8, n128 = (n >> 7) & 1, n32 = (n >> 5) & 3;
         int row0, u = qq;
@@ -516,10 +519,10 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
             map = odd ? &maps.o8 : &maps.e8;
         }
         unsigned char *base = sm + (size_t)st * kbs + (half ? aBytes : 0u);
-        tma_load_2d(smem_addr(base + (size_t)row0 * 128), map, kb * 64, (half ? yB : yA0 + mt * 128) + row0,
+        tma_load_2d(smem_addr(base + (size_t)row0 * 128), map, kb * 64, (half ? yB + ps * nblk : yA0) + row0,
                     smem_addr(&bar_full[st]));
     };
-    auto boxes_of = [&](int q) { return nboxes(tile_rows(q / nkb)) + nboxes(s.nB); };
+    auto boxes_of = [&](int q) { return nboxes(s.nA) + nboxes(pass_rows(q / nkb)); };
     auto produce = [&](int q) {
         mbar_expect_tx(smem_addr(&bar_full[q % S]), stage_tx(q / nkb));
         const int nb = boxes_of(q);
@@ -556,17 +559,16 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
 
     if (dec) {
         const uint32_t tmem = tmem_base;
-        constexpr int kBRows = 2;   // B rows per thread: at most 512 over 384 threads
-        static_assert(kBRows * (kTiledThreads - 128) >= FUSION_MAX_TOKENS / 2, "B rows");
+        // norms: a thread takes the rows tid, tid + 512 of (all A rows, this pass's B rows); |A| + nblk < 1024
+        constexpr int kRows = 2;
         bool ok = true;
-        for (int mt = 0; mt < nM && ok; ++mt) {
-            const int nA_t = tile_rows(mt);
-            // norms: thread t < 128 owns A row t of this tile; during tile 0 threads 128.. own the
-            // B rows, kTiledThreads - 128 apart
-            float ssA = 0.0f, scA = 0.0f;
-            float ssB[kBRows] = {}, scB[kBRows] = {};
+        for (int a = tid; a < s.nA; a += kTiledThreads) m.best[a] = 0ull;   // (each row's threads meet at barriers below)
+        for (int ps = 0; ps < nP && ok; ++ps) {
+            const int nB_p = pass_rows(ps), cols = (nB_p + 15) & ~15;
+            const int nrA = ps == 0 ? s.nA : 0, nr = nrA + nB_p;
+            float ss[kRows] = {}, sc[kRows] = {};
             for (int kb = 0; kb < nkb; ++kb) {
-                const int q = mt * nkb + kb;
+                const int q = ps * nkb + kb;
                 const int st = q % S;
                 const uint32_t par = (uint32_t)(q / S) & 1u;
                 if (!mbar_wait(smem_addr(&bar_full[st]), par)) {
@@ -576,42 +578,32 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
                 const unsigned char *stA = sm + (size_t)st * kbs, *stB = stA + aBytes;
                 if (warp == 1 && elect_one()) {
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    for (int nb = 0; nb < nNB; ++nb) {
-                        const int ncols = min(256, npad - nb * 256);
-                        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(ncols >> 3) << 17) |
-                                               (8u << 24);
-                        const uint32_t a0 = smem_addr(stA), b0 = smem_addr(stB + (size_t)nb * 256 * 128);
+                    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(cols >> 3) << 17) | (8u << 24);
+                    for (int mt = 0; mt < nM; ++mt) {
+                        const uint32_t a0 = smem_addr(stA + (size_t)mt * 16384), b0 = smem_addr(stB);
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            umma_bf16(tmem + (uint32_t)(nb * 256), sw128_desc(a0 + k * 32), sw128_desc(b0 + k * 32),
-                                      idesc, (kb | k) ? 1u : 0u);
+                            umma_bf16(tmem + (uint32_t)(mt * nblk), sw128_desc(a0 + k * 32), sw128_desc(b0 + k * 32), idesc,
+                                      (kb | k) ? 1u : 0u);
                     }
                     umma_commit(smem_addr(&bar_empty[st]));
                     if (kb == nkb - 1) umma_commit(smem_addr(&bar_done));
                 }
-                if (tid < 128) {
-                    if (tid < nA_t) {
-                        const unsigned char *rb = stA + tid * 128;
+#pragma unroll
+                for (int u = 0; u < kRows; ++u) {
+                    const int r = tid + u * kTiledThreads;
+                    if (r < nr) {
+                        const bool isA = r < nrA;
+                        const int rr = isA ? r : r - nrA;
+                        const unsigned char *rb = (isA ? stA : stB) + rr * 128;
 #pragma unroll
                         for (int j = 0; j < 8; ++j)
-                            neumaier_add(ssA, scA, chunk_sq(*reinterpret_cast<const uint4 *>(rb + ((j ^ (tid & 7)) << 4))));
-                    }
-                } else if (mt == 0) {
-#pragma unroll
-                    for (int u = 0; u < kBRows; ++u) {
-                        const int br = tid - 128 + u * (kTiledThreads - 128);
-                        if (br < s.nB) {
-                            const unsigned char *rb = stB + br * 128;
-#pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                neumaier_add(ssB[u], scB[u],
-                                             chunk_sq(*reinterpret_cast<const uint4 *>(rb + ((j ^ (br & 7)) << 4))));
-                        }
+                            neumaier_add(ss[u], sc[u], chunk_sq(*reinterpret_cast<const uint4 *>(rb + ((j ^ (rr & 7)) << 4))));
                     }
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_addr(&bar_empty[st]));
-                if (warp == 0 && q + S < nq) {   // refill this stage (possibly with the next tile's K-block)
+                if (warp == 0 && q + S < nq) {   // refill this stage (possibly with the next pass's K-block)
                     ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_addr(&bar_empty[st]), par));
                     if (!ok) break;
                     if (elect_one()) produce(q + S);
@@ -620,24 +612,21 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
                 }
             }
             if (!ok) atomicOr(&s_fail, 1);
-            if (tid < nA_t) {
-                const float sq = __fadd_rn(ssA, scA);
-                if (!isfinite(sq)) raise_status(p.status, FUSION_DEV_NONFINITE);
-                m.inv_a[mt * 128 + tid] = 1.0f / fmaxf(sqrtf(sq), 1e-12f);
-            }
-            if (mt == 0 && tid >= 128) {
 #pragma unroll
-                for (int u = 0; u < kBRows; ++u) {
-                    const int br = tid - 128 + u * (kTiledThreads - 128);
-                    if (br < s.nB) {
-                        const float sq = __fadd_rn(ssB[u], scB[u]);
-                        if (!isfinite(sq)) raise_status(p.status, FUSION_DEV_NONFINITE);
-                        m.inv_b[br] = 1.0f / fmaxf(sqrtf(sq), 1e-12f);
-                    }
+            for (int u = 0; u < kRows; ++u) {
+                const int r = tid + u * kTiledThreads;
+                if (r < nr) {
+                    const float sq = __fadd_rn(ss[u], sc[u]);
+                    if (!isfinite(sq)) raise_status(p.status, FUSION_DEV_NONFINITE);
+                    const float inv = 1.0f / fmaxf(sqrtf(sq), 1e-12f);
+                    if (r < nrA)
+                        m.inv_a[r] = inv;
+                    else
+                        m.inv_b[ps * nblk + r - nrA] = inv;
                 }
             }
             __syncthreads();
-            const bool mma_ok = s_fail == 0 && mbar_wait(smem_addr(&bar_done), (uint32_t)mt & 1u);
+            const bool mma_ok = s_fail == 0 && mbar_wait(smem_addr(&bar_done), (uint32_t)ps & 1u);
             if (!mma_ok) atomicOr(&s_fail, 2);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             __syncthreads();
@@ -645,42 +634,45 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
                 ok = false;
                 break;
             }
-            // epilogue of the tile: thread -> A row (tid % 128); the four warpgroups split the columns
+            // epilogue of the pass, M-tile by M-tile: thread -> A row (tid % 128); the four warpgroups split
+            // the columns
             const int wg = tid >> 7, r = tid & 127;
-            const int part_cols = ((npad / 16 + 3) / 4) * 16;
-            const int c_lo = min(npad, wg * part_cols), c_hi = min(npad, c_lo + part_cols);
-            const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-            const int arow = mt * 128 + r;
-            const float ia = r < nA_t ? m.inv_a[arow] : 0.0f;
-            float bv = -INFINITY;   // as in k_image_tc: strict comparison over rising columns
-            int bi = -1;
-            for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
-                uint32_t v[16];
-                tmem_ld16(lane_addr + (uint32_t)c0, v);
+            const int part_cols = ((cols / 16 + 3) / 4) * 16;
+            const int c_lo = min(cols, wg * part_cols), c_hi = min(cols, c_lo + part_cols);
+            for (int mt = 0; mt < nM; ++mt) {
+                const uint32_t lane_addr = tmem + (uint32_t)(mt * nblk) + ((uint32_t)((warp & 3) * 32) << 16);
+                const int arow = mt * 128 + r;
+                const float ia = arow < s.nA ? m.inv_a[arow] : 0.0f;
+                float bv = -INFINITY;   // as in k_image_tc: strict comparison over rising columns
+                int bi = -1;
+                for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+                    uint32_t v[16];
+                    tmem_ld16(lane_addr + (uint32_t)c0, v);
 #pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const int col = c0 + e;
-                    if (col < s.nB) {
-                        const float cs = (__uint_as_float(v[e]) * ia) * m.inv_b[col];
-                        if (cs > bv || bi < 0) {
-                            bv = cs;
-                            bi = col;
+                    for (int e = 0; e < 16; ++e) {
+                        const int col = ps * nblk + c0 + e;
+                        if (c0 + e < nB_p) {
+                            const float cs = (__uint_as_float(v[e]) * ia) * m.inv_b[col];
+                            if (cs > bv || bi < 0) {
+                                bv = cs;
+                                bi = col;
+                            }
                         }
                     }
                 }
-            }
-            const unsigned long long bk = (r < nA_t && bi >= 0) ? rank_key(bv, bi) : 0ull;
-            part_best[tid] = bk;
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncthreads();   // the next tile's products overwrite the accumulators after this
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (wg == 0 && r < nA_t) {
-                unsigned long long o = bk;
+                part_best[tid] = (arow < s.nA && bi >= 0) ? rank_key(bv, bi) : 0ull;
+                __syncthreads();
+                if (wg == 0 && arow < s.nA) {   // (the larger key: the lower column among equal values)
+                    unsigned long long o = m.best[arow];
 #pragma unroll
-                for (int k = 1; k < 4; ++k) o = part_best[k * 128 + r] > o ? part_best[k * 128 + r] : o;
-                m.best[arow] = o;
+                    for (int k = 0; k < 4; ++k) o = part_best[k * 128 + r] > o ? part_best[k * 128 + r] : o;
+                    m.best[arow] = o;
+                }
+                __syncthreads();   // part_best is reused
             }
-            __syncthreads();   // part_best is reused by the next tile
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncthreads();   // the next pass's products overwrite the accumulators after this
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
         if (s_fail != 0) {
             // a wait gave up: let the copies and products in flight land (bounded) before the
@@ -718,30 +710,32 @@ int ceil8(int v) { return (v + 7) & ~7; }
 }  // namespace
 
 namespace {
-// Geometry of k_image_tc_tiled: one CTA per SM, a ring of [128 A rows | all B rows] stages.
+// Geometry of k_image_tc_tiled: one CTA per SM, a ring of [all A rows | a pass's B rows] stages.
 TcGeometry tiled_geometry(int max_tokens, int kdim) {
     TcGeometry g{};
-    const int nBmax = max_tokens / 2;
+    const int nAmax = (max_tokens - 1) / 2, nBmax = max_tokens / 2;
     const int npad_max = (nBmax + 15) & ~15;
     g.tiled = 1;
     g.n_kb = kdim / 64;
-    g.tmem_cols = npad_max <= 256 ? 256 : 512;
-    g.kb_a = 128u * 128u;
-    g.kb_b = (uint32_t)ceil8(nBmax) * 128u;
-    const size_t per_stage = g.kb_a + g.kb_b;
-    const size_t reach = g.kb_a + (size_t)npad_max * 128;
-    const size_t budget = 227 * 1024 - 4096;   // room for static shared memory
-    auto need = [&](int S) {
-        const size_t meta_base = (size_t)S * per_stage + 2048;
-        return std::max(meta_layout(max_tokens, meta_base).total, (size_t)(S - 1) * per_stage + reach);
-    };
-    int S = kTiledMaxStages;
-    while (S > 2 && need(S) + 1024 > budget) --S;
-    if (need(S) + 1024 > budget) return TcGeometry{};
-    g.stages = S;
-    g.stage_region = (uint32_t)(S * per_stage);
-    g.meta_base = (uint32_t)(S * per_stage + 2048);
-    g.usable = (uint32_t)need(S);
+    g.tmem_cols = 512;
+    // the largest stage and the furthest read from its start over all samples of at most max_tokens: with
+    // one M-tile less a pass has more columns
+    size_t per_stage = 0, reach = 0;
+    for (int nM = 1; nM <= (nAmax + 127) / 128; ++nM) {
+        const int nblk = std::min(256, 512 / nM & ~15);
+        const size_t a = (size_t)ceil8(std::min(nAmax, nM * 128)) * 128;
+        per_stage = std::max(per_stage, a + (size_t)std::min(nblk, ceil8(nBmax)) * 128);
+        reach = std::max({reach, (size_t)nM * 16384, a + (size_t)std::min(nblk, npad_max) * 128});
+    }
+    // one CTA per SM: all of its shared memory, the metadata at the end; at least two stages (shorter
+    // samples of the call have more, from their own sizes)
+    const size_t usable = (227 * 1024 - 6144 - 1024) / 1024 * 1024;   // static shared memory, alignment
+    const size_t meta = meta_layout(max_tokens, 0).total;
+    if (2 * per_stage + 2048 + meta > usable || per_stage + reach > usable) return TcGeometry{};
+    g.meta_base = (uint32_t)((usable - meta) / 16 * 16);
+    g.stage_region = g.meta_base - 2048;
+    g.stages = (int)(g.stage_region / per_stage);
+    g.usable = (uint32_t)usable;
     g.smem = g.usable + 1024;
     g.ok = 1;
     return g;

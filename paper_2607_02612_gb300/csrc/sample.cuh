@@ -30,8 +30,10 @@ __host__ __device__ inline Meta meta_layout(int nmax, size_t base) {
     Meta L;
     size_t off = (base + 15) / 16 * 16;
     L.best = off;   off += sizeof(unsigned long long) * nA;
-    L.rk = off;     off += sizeof(unsigned long long) * nA;
+    off = (off + 15) / 16 * 16;   // rk and pk are read four values at a time
+    L.rk = off;     off += (sizeof(unsigned long long) * nA + 15) / 16 * 16;
     L.pk = off;     off += sizeof(unsigned long long) * nmax;
+    off = (off + 15) / 16 * 16;
     L.inv_a = off;  off += sizeof(float) * nA;
     L.inv_b = off;  off += sizeof(float) * nB;
     L.match = off;  off += sizeof(int) * nA;
@@ -361,6 +363,23 @@ __device__ __forceinline__ void meta_init_rest(const ImageParams &p, const Sampl
     cp_async_wait_all();
 }
 
+// Rank of entry `self` (value v >= 1) among v[0..n): the entries of larger value, and those of equal value
+// at a lower index.  Four values per shared-memory load (v 16-byte aligned): one load per value kept
+// the loop on the load pipe.  Entries n .. of the last group must be 0.
+__device__ __forceinline__ int rank_of(const uint32_t *vals, int n, int self, uint32_t v) {
+    const uint4 *v4 = reinterpret_cast<const uint4 *>(vals);
+    const int own = self >> 2, groups = (n + 3) >> 2;
+    int rank = 0;
+#pragma unroll 4
+    for (int q = 0; q < groups; ++q) {   // a lower index also counts at equal value: larger than v - 1
+        const uint4 x = v4[q];
+        const uint32_t t = q < own ? v - 1u : v;
+        rank += (x.x > t ? 1 : 0) + (x.y > t ? 1 : 0) + (x.z > t ? 1 : 0) + (x.w > t ? 1 : 0);
+    }
+    for (int q = own * 4; q < self; ++q) rank += vals[q] == v ? 1 : 0;   // the own group's lower indices
+    return rank;
+}
+
 // best[a] holds the packed (similarity, lowest B index) maximum of every A row.  Writes
 // match[a] and, when tokens merge, sel[a] for the r_eff A tokens of largest similarity
 // (lowest position on ties) and mkey[rank] = (match[a] << kKeyShift) | a for each of them.
@@ -372,17 +391,11 @@ __device__ __forceinline__ void select_top_r(const SampleInfo &s, MetaPtrs &m) {
     if (s.r_eff > 0) {
         // the ordered similarity of every A row (the high half of its key)
         uint32_t *rv = reinterpret_cast<uint32_t *>(m.rk);
-        for (int a = tid; a < s.nA; a += NT) rv[a] = (uint32_t)(m.best[a] >> 32);
+        // (at least 1, a NaN of all ones apart, which joins the lowest: zeros pad the last group of four)
+        for (int a = tid; a < ((s.nA + 3) & ~3); a += NT) rv[a] = a < s.nA ? max((uint32_t)(m.best[a] >> 32), 1u) : 0u;
         __syncthreads();
         for (int a = tid; a < s.nA; a += NT) {
-            // rank of a: the rows of larger similarity, and the rows of equal similarity at a
-            // lower position (32-bit comparisons in two ranges instead of 64-bit keys)
-            const uint32_t va = rv[a];
-            int rank = 0;
-#pragma unroll 8
-            for (int q = 0; q < a; ++q) rank += rv[q] >= va ? 1 : 0;
-#pragma unroll 8
-            for (int q = a + 1; q < s.nA; ++q) rank += rv[q] > va ? 1 : 0;
+            const int rank = rank_of(rv, s.nA, a, rv[a]);
             m.sel[a] = rank < s.r_eff ? 1 : 0;
             if (rank < s.r_eff) m.mkey[rank] = (m.match[a] << kKeyShift) | a;
         }
@@ -744,21 +757,16 @@ __device__ bool finish_decide(const ImageParams &p, const SampleInfo &s, MetaPtr
         // the ordered merged score of every candidate; 0 marks a non-candidate (CLS or merged
         // away), below every candidate's value (ordered values of floats are >= 1)
         uint32_t *pv = reinterpret_cast<uint32_t *>(m.pk);
-        for (int pos = tid; pos < N; pos += NT) pv[pos] = (pos > 0 && m.mflag[pos]) ? ordered_bits(m.mscore[pos]) : 0u;
+        for (int pos = tid; pos < ((N + 3) & ~3); pos += NT)
+            pv[pos] = (pos > 0 && pos < N && m.mflag[pos]) ? max(ordered_bits(m.mscore[pos]), 1u) : 0u;
         __syncthreads();
         for (int pos = tid; pos < N; pos += NT) {
             int keep = 0;
             if (pos == 0) {
                 keep = 1;
             } else if (m.mflag[pos]) {
-                // rank: candidates of larger score, and of equal score at a lower position
-                const uint32_t vp = pv[pos];
-                int rank = 0;
-#pragma unroll 8
-                for (int q = 1; q < pos; ++q) rank += pv[q] >= vp ? 1 : 0;
-#pragma unroll 8
-                for (int q = pos + 1; q < N; ++q) rank += pv[q] > vp ? 1 : 0;
-                keep = rank < k ? 1 : 0;
+                // (CLS and merged-away tokens are 0, below every candidate)
+                keep = rank_of(pv, N, pos, pv[pos]) < k ? 1 : 0;
             }
             m.kflag[pos] = keep;
             m.opos[pos] = keep;

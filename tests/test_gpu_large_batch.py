@@ -152,3 +152,17 @@ def test_bf16_merge_small_ctas(counts, dim, keys, kdim):
     r = np.minimum(rng.integers(0, 40, len(counts)), np.asarray(counts) // 2).astype(np.int32)
     rho = rng.uniform(0.3, 1.0, len(counts)).astype(np.float32)
     run_stage_and_compare(b, StageSpec(True, False, True, r=r, rho=rho), f"{counts[:4]} x {len(counts)}")
+
+
+@pytest.mark.parametrize("counts,dim", [
+    ([258, 257, 259, 300, 17, 1], 128),      # one pass, two M-tiles; short samples in the same call
+    ([513, 514, 512, 258], 64),              # two M-tiles of 128 rows exactly, one row over, three
+    ([577, 640, 641, 130], 192),             # three M-tiles: passes of 160 columns, the last ones ragged
+    ([769, 770, 771, 300], 64),              # four M-tiles: passes of 128
+    ([900, 860], 128), ([1024, 3], 64)])     # the longest samples, and those the general kernel takes
+def test_bf16_merge_long_samples(counts, dim):
+    b = make_batch(counts, dim, "bf16", seed=len(counts), sizes="u1to4")
+    rng = np.random.default_rng(3)
+    r = np.minimum(rng.integers(20, 200, len(counts)), np.asarray(counts) // 2).astype(np.int32)
+    rho = rng.uniform(0.3, 1.0, len(counts)).astype(np.float32)
+    run_stage_and_compare(b, StageSpec(True, False, True, r=r, rho=rho), f"{counts}")
