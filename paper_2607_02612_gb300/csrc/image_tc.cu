@@ -35,7 +35,8 @@ constexpr int kMaxStages = 16;
 
 struct TcMaps {
     CUtensorMap e32, o32, e8, o8;   // even / odd rows, boxes of 32 / 8 rows x 64 dims
-    CUtensorMap e256, o256, e128, o128;   // the same with 256 / 128 rows (k_image_tc_tiled)
+    // larger boxes: 256 / 128 rows (k_image_tc_tiled); a whole half of max_tokens / 64 rows (k_image_tc)
+    CUtensorMap e256, o256, e128, o128;
     // even / odd rows seen as (64 dims, row, K-block) with the K-block stride 128 B: a box of
     // 8 rows x all K-blocks lands as [K-block][8 rows][128 B], one 1 KB swizzle atom per K-block
     CUtensorMap ge, go;
@@ -89,6 +90,11 @@ struct Ring {
     int S, rowsA, rowsB, npad, nbA, per_kb;
     uint32_t kbs;
 };
+// The boxes of n rows: one of `full` rows where that is n rounded up to 8 (the longest samples of a call,
+// all of a uniform one), else 64, 32 and 8 rows.  A copy costs its issuing thread about 200 cycles.
+__device__ __forceinline__ int box_count(int n, int full) {
+    return ((n + 7) & ~7) == full ? 1 : (n >> 6) + ((n >> 5) & 1) + (((n & 31) + 7) >> 3);
+}
 __device__ __forceinline__ Ring ring_for(int nA, int nB, int nkb, const TcGeometry &g) {
     Ring R;
     R.rowsA = (nA + 7) & ~7;
@@ -101,22 +107,33 @@ __device__ __forceinline__ Ring ring_for(int nA, int nB, int nkb, const TcGeomet
     int S = min(min(nkb, kMaxStages), (int)(g.stage_region / R.kbs));
     while (S > 1 && (uint32_t)(S - 1) * R.kbs + reach > g.usable) --S;
     R.S = S;
-    R.nbA = (nA >> 5) + (((nA & 31) + 7) >> 3);
-    R.per_kb = R.nbA + (nB >> 5) + (((nB & 31) + 7) >> 3);
+    R.nbA = box_count(nA, g.full_rows);
+    R.per_kb = R.nbA + box_count(nB, g.full_rows);
     return R;
 }
 // Box b of K-block kb of the sample whose rows start at `start` (half A: positions 2, 4, ...,
 // half B: 1, 3, ..., each contiguous in the even or odd row view).
-__device__ __forceinline__ void issue_box(const TcMaps &maps, const Ring &R, int start, int nA, int nB,
-                                          unsigned char *sm, unsigned long long *bar_full, int kb, int b) {
+__device__ __forceinline__ void issue_box(const TcMaps &maps, const Ring &R, const TcGeometry &g, int start, int nA,
+                                          int nB, unsigned char *sm, unsigned long long *bar_full, int kb, int b) {
     const int st = kb % R.S;
     const int half = b >= R.nbA ? 1 : 0;
-    const int q = half ? b - R.nbA : b;
-    const int n32 = (half ? nB : nA) >> 5;
-    const bool big = q < n32;
-    const int row0 = big ? q * 32 : n32 * 32 + (q - n32) * 8;
+    const int q = half ? b - R.nbA : b, n = half ? nB : nA;
     const bool odd = half ? ((start + 1) & 1) : ((start + 2) & 1);
-    const CUtensorMap *map = big ? (odd ? &maps.o32 : &maps.e32) : (odd ? &maps.o8 : &maps.e8);
+    const int n64 = n >> 6, n32 = (n >> 5) & 1;
+    int row0 = 0;
+    const CUtensorMap *map;
+    if (((n + 7) & ~7) == g.full_rows) {
+        map = odd ? &maps.o256 : &maps.e256;
+    } else if (q < n64) {
+        row0 = q * 64;
+        map = odd ? &maps.o128 : &maps.e128;
+    } else if (q - n64 < n32) {
+        row0 = n64 * 64;
+        map = odd ? &maps.o32 : &maps.e32;
+    } else {
+        row0 = (n >> 5) * 32 + (q - n64 - n32) * 8;
+        map = odd ? &maps.o8 : &maps.e8;
+    }
     const int y = half ? (start + 1) >> 1 : (start + 2) >> 1;
     const uint32_t dst = smem_addr(sm + (half ? (size_t)R.rowsA * 128 : (size_t)0) + (size_t)st * R.kbs + (size_t)row0 * 128);
     tma_load_2d(dst, map, kb * 64, y + row0, smem_addr(&bar_full[st]));
@@ -137,14 +154,14 @@ __device__ __forceinline__ void ring_barriers_init(unsigned long long *bar_full,
 }
 // From the 32 lanes of one warp, once the barriers are initialised and that is visible to the
 // warp: the first min(S, nkb) K-blocks.
-__device__ __forceinline__ void ring_start(const TcMaps &maps, const Ring &R, int start, int nA, int nB, int nkb,
+__device__ __forceinline__ void ring_start(const TcMaps &maps, const Ring &R, const TcGeometry &g, int start, int nA, int nB, int nkb,
                                            unsigned char *sm, unsigned long long *bar_full) {
     const int lane = threadIdx.x & 31;
     __syncwarp();
     const int S0 = min(R.S, nkb);
     if (lane < S0) mbar_expect_tx(smem_addr(&bar_full[lane]), R.kbs);
     for (int t = lane; t < S0 * R.per_kb; t += 32)
-        issue_box(maps, R, start, nA, nB, sm, bar_full, t / R.per_kb, t % R.per_kb);
+        issue_box(maps, R, g, start, nA, nB, sm, bar_full, t / R.per_kb, t % R.per_kb);
 }
 // A sample that fits in shared memory, grouped: half A in 8-row groups g at g * nkb KB, each
 // group [K-block][8 rows][128 B], half B after it the same way, all behind bar_full[0]; one box
@@ -237,7 +254,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
     unsigned char *regB = sm + (size_t)R.rowsA * 128;  // stage st, half B: regB + st * kbs (ring layout)
     auto produce = [&](int kb) {   // a whole K-block from one thread
         mbar_expect_tx(smem_addr(&bar_full[kb % S]), kbs);
-        for (int b = 0; b < R.per_kb; ++b) issue_box(maps, R, s.start, s.nA, s.nB, sm, bar_full, kb, b);
+        for (int b = 0; b < R.per_kb; ++b) issue_box(maps, R, g, s.start, s.nA, s.nB, sm, bar_full, kb, b);
     };
 
     // the sample's sizes, scores and CLS row first (a few KB that would otherwise queue behind the
@@ -250,7 +267,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
         if (grouped)
             group_start(maps, R, s.start, nkb, sm, bar_full);
         else
-            ring_start(maps, R, s.start, s.nA, s.nB, nkb, sm, bar_full);
+            ring_start(maps, R, g, s.start, s.nA, s.nB, nkb, sm, bar_full);
     }
     meta_init_rest<NT>(p, s, m);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -309,12 +326,11 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_addr(&bar_empty[st]));
-            if (tid == 0 && kb + S < nkb) {   // refill this stage once everyone is done with it
-                if (!mbar_wait(smem_addr(&bar_empty[st]), par)) {
-                    ok = false;
-                    break;
-                }
-                produce(kb + S);
+            if (warp == 0 && kb + S < nkb) {   // refill this stage once everyone is done with it
+                ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_addr(&bar_empty[st]), par));
+                if (!ok) break;
+                if (elect_one()) produce(kb + S);
+                __syncwarp();
             }
         }
         if (!ok) atomicOr(&s_fail, 1);
@@ -749,6 +765,7 @@ TcGeometry image_tc_geometry(int dtype, int max_tokens, int kdim, int dim, long 
     const int nAmax = (max_tokens - 1) / 2, nBmax = max_tokens / 2;
     if (nAmax > 128 || nBmax > 128) return tiled_geometry(max_tokens, kdim);
     g.n_kb = kdim / 64;
+    g.full_rows = ceil8(nBmax > 0 ? nBmax : 1);
     g.kb_a = (uint32_t)ceil8(nAmax > 0 ? nAmax : 1) * 128u;
     g.kb_b = (uint32_t)ceil8(nBmax > 0 ? nBmax : 1) * 128u;
     int cols = 32;
@@ -821,9 +838,9 @@ cudaError_t launch_image_tc(const ImageParams &p, const TcGeometry &g, cudaStrea
     const cuuint64_t rows_even = (cuuint64_t)((p.in.max_rows + 1) / 2), rows_odd = (cuuint64_t)(p.in.max_rows / 2);
     const char *keys = reinterpret_cast<const char *>(p.keys);
     CUtensorMap *const dsts[8] = {&maps.e32, &maps.o32, &maps.e8, &maps.o8, &maps.e256, &maps.o256, &maps.e128, &maps.o128};
-    for (int i = 0; i < (g.tiled ? 8 : 4); ++i) {
-        constexpr int kBox[4] = {32, 8, 256, 128};
-        const int odd = i & 1, box_rows = kBox[i >> 1];
+    const int box[4] = {32, 8, g.tiled ? 256 : g.full_rows, g.tiled ? 128 : 64};
+    for (int i = 0; i < 8; ++i) {
+        const int odd = i & 1, box_rows = box[i >> 1];
         cuuint64_t dims[2] = {(cuuint64_t)p.kdim, odd ? rows_odd : rows_even};
         cuuint64_t strides[1] = {(cuuint64_t)p.kdim * 2 * 2};   // every other row
         cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
