@@ -257,6 +257,20 @@ __device__ __forceinline__ F2 hidden_dot_exact_warp(const unsigned char *wt, int
     return f2_add_f(warp_sum_f2(acc), b1);
 }
 
+// The same by one thread, the weight row from global memory (units past the CTA's list).
+__device__ __noinline__ F2 hidden_dot_exact_thread(const __nv_bfloat16 *wg, const unsigned char *ut, int row, int dim,
+                                                   float b1) {
+    F2 acc = {0.0f, 0.0f};
+    for (int ch = 0; ch < dim / 8; ++ch) {
+        float wf[8], uf[8];
+        chunk_to_f(ldg16(wg + ch * 8), wf);
+        chunk_to_f(*reinterpret_cast<const uint4 *>(ut + u_tc_off(row, ch)), uf);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc = f2_add_f(acc, __fmul_rn(wf[e], uf[e]));
+    }
+    return f2_add_f(acc, b1);
+}
+
 // GELU of an exact pre-activation (float-float) rounded once to bf16, by one thread: with the
 // argument exact, the float GELU of its high part is within about a hundred float ulps of the
 // exact value (erfc's error, amplified by its argument for large |a|); only a unit closer than
@@ -320,7 +334,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
                              : "memory");
                 asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
             }
-            if (tid == 0) {
+            if (warp == 1 && elect_one()) {
                 const int nws = TS::w_stages(dim);
                 for (int q = 0; q < nws; ++q) {
                     mbar_init(smem_addr(&wbar[q]), 1);
@@ -482,7 +496,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
         if constexpr (kBf16) {
             const uint32_t tmem = tmem_base;
             const int nws = TS::w_stages(dim);
-            if (tid == 0)
+            if (warp == 1 && elect_one())
                 s_wfail = exit_tc_product<16>(&wmap, tmem, smem_addr(base), smem_addr(w_region), dim, nws, c0, wbar,
                                           wempty, &wdone, p.status)
                               ? 0
@@ -496,6 +510,8 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
             if (p.out_mode == 1) {
                 // ---- hidden layer: a = D + b1 straight from tensor memory, the weight ring intact ----
                 __shared__ float wn2[2][kExitCT], un[kExitBT];   // ||w_j||^2 in two halves; ||u||
+                __shared__ int s_flagged;
+                if (tid == 0) s_flagged = 0;
                 const bool resident = nws * 64 >= dim;           // every K-block in its own stage
                 {   // ||w_j||^2, two threads per row: from the ring (a row's 8 chunks in any order; rows
                     // past C and dims past dim are zero), else from global memory, 8 loads at a time
@@ -553,9 +569,19 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
                 // the bias addition and the float32 evaluation of a
                 const float a_rel = 0x1p-20f + (float)((dim + 15) / 16) * 0x1p-23f;
                 uint16_t *ho = reinterpret_cast<uint16_t *>(p.hidden_out);
-                uint16_t hb[4];
-                F2 ax[4];            // exact pre-activations of this thread's flagged units
-                unsigned fl = 0;     // its units near a rounding midpoint (bit i: sample sb + i)
+                // Units near a rounding midpoint go to a list of the CTA (sample slot * 128 + class), dealt out
+                // over its warps: they are a few percent of the units and uneven, and a warp that computed its
+                // own (up to 15 exact dot products against 5 on average) set the length of the phase.  The
+                // list lies in rows 8..15 of the u tile's K-blocks, which feed only unused columns.
+                auto flagged = [&](int k) {
+                    return reinterpret_cast<uint16_t *>(base + (size_t)(k >> 9) * 2048u + 1024u) + (k & 511);
+                };
+                const int list_cap = min(kExitBT * kExitCT, 512 * ((dim + 63) / 64));
+                auto unit_dot = [&](int sl, int cu, bool whole) {   // by the whole warp, or by one thread
+                    const __nv_bfloat16 *wg = reinterpret_cast<const __nv_bfloat16 *>(p.head.weight) + (size_t)(c0 + cu) * dim;
+                    return whole ? hidden_dot_exact_warp(resident ? w_region : nullptr, cu, wg, base, sl, dim, bias_s[cu])
+                                 : hidden_dot_exact_thread(wg, base, sl, dim, bias_s[cu]);
+                };
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int sl = sb + i;
@@ -566,34 +592,37 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
                     const float eg = 1.13f * ea + fabsf(g) * 0x1p-16f;
                     const float mid = __uint_as_float((__float_as_uint(g) & 0xFFFF0000u) | 0x8000u);
                     const bool exact = valid && !(isfinite(g) && fabsf(g - mid) > eg);
-                    hb[i] = __bfloat16_as_ushort(__float2bfloat16_rn(g));
-                    ax[i] = {0.0f, 0.0f};
-                    if (exact) fl |= 1u << i;
-                    // their exact dot products, one at a time by the whole warp
-                    for (unsigned mask = __ballot_sync(0xFFFFFFFFu, exact); mask; mask &= mask - 1) {
-                        const int src = __ffs(mask) - 1;
-                        const int scol = __shfl_sync(0xFFFFFFFFu, col, src);
-                        const F2 e = hidden_dot_exact_warp(
-                            resident ? w_region : nullptr, scol,
-                            reinterpret_cast<const __nv_bfloat16 *>(p.head.weight) + (size_t)(c0 + scol) * dim, base,
-                            sl, dim, bias_s[scol]);
-                        if (lane == src) ax[i] = e;
+                    uint16_t h = __bfloat16_as_ushort(__float2bfloat16_rn(g));
+                    bool later = false;
+                    if (exact) {
+                        const int k = atomicAdd(&s_flagged, 1);
+                        later = k < list_cap;
+                        if (later)
+                            *flagged(k) = (uint16_t)(sl * kExitCT + col);
+                        else
+                            h = gelu_exact_bf16(unit_dot(sl, col, false));
                     }
+                    if (valid && !later) ho[(size_t)(s0 + sl) * C + c0 + col] = h;
                 }
-                // their GELU, every thread its own (the double-precision fallback then runs once per
-                // unit, not once per lane of a warp)
-                for (unsigned m = fl; m; m &= m - 1) {
-                    const int i = __ffs(m) - 1;
-                    const F2 x = i == 0 ? ax[0] : i == 1 ? ax[1] : i == 2 ? ax[2] : ax[3];
-                    const uint16_t e = gelu_exact_bf16(x);
-                    hb[0] = i == 0 ? e : hb[0];
-                    hb[1] = i == 1 ? e : hb[1];
-                    hb[2] = i == 2 ? e : hb[2];
-                    hb[3] = i == 3 ? e : hb[3];
+                __syncthreads();
+                // their exact dot products, one at a time by a whole warp; their GELU, every lane its own (the
+                // double-precision fallback then runs once per unit, not once per lane)
+                const int n_fl = min(s_flagged, list_cap);
+                for (int k0 = warp; k0 < n_fl; k0 += 32 * (kExitThreads / 32)) {
+                    F2 mine = {0.0f, 0.0f};
+                    int unit = -1;
+                    for (int l = 0; l < 32; ++l) {
+                        const int k = k0 + l * (kExitThreads / 32);
+                        if (k >= n_fl) break;
+                        const int u = *flagged(k);
+                        const F2 e = unit_dot(u / kExitCT, u % kExitCT, true);
+                        if (lane == l) {
+                            mine = e;
+                            unit = u;
+                        }
+                    }
+                    if (unit >= 0) ho[(size_t)(s0 + unit / kExitCT) * C + c0 + unit % kExitCT] = gelu_exact_bf16(mine);
                 }
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (s0 + sb + i < B && c0 + col < C && !failed) ho[(size_t)(s0 + sb + i) * C + c0 + col] = hb[i];
             } else if (warp < 4 && !failed) {
                 // logits (+ bias) into shared memory over the ring: warp w < 4 reads the lanes
                 // (classes) 32w.. of D
@@ -810,7 +839,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    if (active && kBf16 && tid == 0) {
+    if (active && kBf16 && warp == 1 && elect_one()) {
         // the head's first weight chunks first: they depend on nothing and take longest to land
         const int nws = L::w_stages(dim);
         for (int q = 0; q < nws; ++q) {
@@ -960,7 +989,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
         if constexpr (kBf16) {
             // ---- D[128 classes][16 samples] = W_tile u^T on tcgen05 (exit_tc_product) ----------
             const uint32_t tmem = tmem_base;
-            if (tid == 0)
+            if (warp == 1 && elect_one())
                 s_wfail = exit_tc_product<16>(&wmap, tmem, smem_addr(base), smem_addr(w_region), dim, L::w_stages(dim), c0,
                                           wbar, wempty, &wdone, p.status)
                               ? 0
@@ -1156,7 +1185,7 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
                              : "memory");
                 asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
             }
-            if (tid == 32) {
+            if (warp == 1 && elect_one()) {
                 const int nws = L::w_stages(dim);
                 for (int q = 0; q < nws; ++q) {
                     mbar_init(smem_addr(&wbar[q]), 1);
@@ -1284,7 +1313,7 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
     if (active) {
         if constexpr (kBf16) {
             const uint32_t tmem = tmem_base;
-            if (tid == 32)
+            if (warp == 1 && elect_one())
                 s_wfail = exit_tc_product<BT>(&wmap, tmem, smem_addr(base), smem_addr(ring), dim, L::w_stages(dim), c0,
                                               wbar, wempty, &wdone, p.status)
                               ? 0
