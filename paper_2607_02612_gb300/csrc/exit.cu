@@ -386,10 +386,26 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
         // the row's chunk c as floats: from the tile, or from the float32 input rows
         const float *ur = p.in_mode == 2 && ok ? p.u_in + (size_t)s * dim : nullptr;
         const float *url = ur && p.u_in_lo ? p.u_in_lo + (size_t)s * dim : nullptr;   // float-float low parts
+        // rows of up to 512 dims are read once, into registers (the three passes below would each wait for L2)
+        constexpr int kHeld = 2;
+        const bool held = ur && nchunk <= 32 * kHeld;
+        float4 hv[kHeld][CH / 4], hl[kHeld][CH / 4];
+        if (held) {
+#pragma unroll
+            for (int q = 0; q < kHeld; ++q)
+#pragma unroll
+                for (int e = 0; e < CH / 4; ++e) {
+                    const int c = lane + 32 * q;
+                    hv[q][e] = c < nchunk ? *reinterpret_cast<const float4 *>(ur + c * CH + 4 * e) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    hl[q][e] = c < nchunk && url ? *reinterpret_cast<const float4 *>(url + c * CH + 4 * e)
+                                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+        }
         auto in_lo = [&](int c, float (&f)[CH]) {
 #pragma unroll
             for (int e = 0; e < CH; e += 4) {
-                const float4 v = url ? *reinterpret_cast<const float4 *>(url + c * CH + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const float4 v = held ? (c < 32 ? hl[0][e / 4] : hl[1][e / 4])
+                                      : url ? *reinterpret_cast<const float4 *>(url + c * CH + e) : make_float4(0.f, 0.f, 0.f, 0.f);
                 f[e] = v.x;
                 f[e + 1] = v.y;
                 f[e + 2] = v.z;
@@ -400,7 +416,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
             if (ur) {
 #pragma unroll
                 for (int e = 0; e < CH; e += 4) {
-                    const float4 v = *reinterpret_cast<const float4 *>(ur + c * CH + e);
+                    const float4 v = held ? (c < 32 ? hv[0][e / 4] : hv[1][e / 4]) : *reinterpret_cast<const float4 *>(ur + c * CH + e);
                     f[e] = v.x;
                     f[e + 1] = v.y;
                     f[e + 2] = v.z;
@@ -513,7 +529,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
                 __shared__ int s_flagged;
                 if (tid == 0) s_flagged = 0;
                 const bool resident = nws * 64 >= dim;           // every K-block in its own stage
-                {   // ||w_j||^2, two threads per row: from the ring (a row's 8 chunks in any order; rows
+                {   // ||w_j||^2, two threads per row: from the ring (a row's 8 chunks in any order, here one that keeps the banks apart; rows
                     // past C and dims past dim are zero), else from global memory, 8 loads at a time
                     const int r = tid & (kExitCT - 1), h = tid / kExitCT;
                     float acc = 0.0f;
@@ -523,7 +539,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
 #pragma unroll
                             for (int j2 = 0; j2 < 8; ++j2) {
                                 float f[8];
-                                chunk_to_f(*reinterpret_cast<const uint4 *>(row + 16 * j2), f);
+                                chunk_to_f(*reinterpret_cast<const uint4 *>(row + 16 * (j2 ^ (r & 7))), f);
 #pragma unroll
                                 for (int e = 0; e < 8; ++e) acc = fmaf(f[e], f[e], acc);
                             }
