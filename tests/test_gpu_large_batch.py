@@ -166,3 +166,15 @@ def test_bf16_merge_long_samples(counts, dim):
     r = np.minimum(rng.integers(20, 200, len(counts)), np.asarray(counts) // 2).astype(np.int32)
     rho = rng.uniform(0.3, 1.0, len(counts)).astype(np.float32)
     run_stage_and_compare(b, StageSpec(True, False, True, r=r, rho=rho), f"{counts}")
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("counts,dim,prune", [
+    ([197, 1, 2, 130], 768, True), ([90, 17, 33] * 25, 112, True), ([1024, 5], 16, True),
+    ([65, 3] * 200, 384, True), ([40, 1, 7] * 30, 1024, False)])
+def test_prune_and_compact_column_parts(dtype, counts, dim, prune):
+    """A sample's columns shared by several CTAs (few samples), and one CTA per sample (many)."""
+    b = make_batch(counts, dim, dtype, seed=len(counts), sizes="u1to4")
+    rng = np.random.default_rng(4)
+    rho = rng.uniform(0.2, 1.0, len(counts)).astype(np.float32) if prune else None
+    run_stage_and_compare(b, StageSpec(False, False, prune, rho=rho), f"{counts[:4]} x {len(counts)} d={dim}")
