@@ -321,6 +321,16 @@ __global__ void __launch_bounds__(kSelectThreads, 2) k_select(ImageParams p, int
 
 }  // namespace
 
+// The metadata without the padding between its arrays, from `base`: what the choice of the key chunk below
+// counts with.  The chunk is also the block of the squared norms' sums (image_f32.cu forms them the same
+// way), so it must not move with the layout.
+static size_t unpadded_meta(int n, size_t base) {
+    const size_t nA = (n - 1) / 2 > 0 ? (n - 1) / 2 : 1, nB = n / 2 > 0 ? n / 2 : 1;
+    size_t off = (base + 15) / 16 * 16 + 36 * nA + 12 * nB + 32 * (size_t)n + 8;
+    off = (off + 7) / 8 * 8 + 16 * (size_t)n + 160;
+    return (off + 15) / 16 * 16;
+}
+
 ImageGeometry image_geometry(int dtype, int max_tokens, int kdim, int do_merge) {
     ImageGeometry G{};
     const int eb = dtype == FUSION_BF16 ? 2 : 4;
@@ -329,18 +339,18 @@ ImageGeometry image_geometry(int dtype, int max_tokens, int kdim, int do_merge) 
     G.ra = rows_odd8(nA);
     G.rb = rows_odd8(nB);
     constexpr size_t kBudget = 227 * 1024 - 2048;   // leave room for static shared memory
-    const size_t meta = meta_layout(max_tokens, 0).total;
+    const size_t meta = unpadded_meta(max_tokens, 0);   // (the padding fits the room left above)
     if (!do_merge) {
         G.ok = meta <= kBudget;
-        G.smem = meta;
+        G.smem = meta_layout(max_tokens, 0).total;
         return G;
     }
-    const size_t full = meta_layout(max_tokens, stage_total(kdim / CH, G.ra, G.rb)).total;
-    if (full <= kBudget) {
+    const size_t full = stage_total(kdim / CH, G.ra, G.rb);
+    if (unpadded_meta(max_tokens, full) <= kBudget) {
         G.ok = 1;
         G.resident = 1;
         G.kc = kdim;
-        G.smem = full;
+        G.smem = meta_layout(max_tokens, full).total;
         return G;
     }
     const size_t per_dim = (size_t)(G.ra + G.rb) * eb;   // staged bytes per key dim

@@ -240,7 +240,11 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : TPW == 1 ? 1 : 2) k_merge_
                 }
                 __syncthreads();
             }
-            // cosine and row maximum with the lowest column on ties
+            // cosine and row maximum with the lowest column on ties: every tile leaves its 16 rows' maxima in
+            // the stages (all read by now), a thread per row takes the largest.  (64-bit maxima by shared-memory
+            // atomics, seven tiles on the same 16 rows, took up to 8 us.)
+            unsigned long long *tile_best = reinterpret_cast<unsigned long long *>(st0);
+            const int tile0 = pass * TPW * kW;
 #pragma unroll
             for (int w = 0; w < TPW; ++w) {
                 const int tile = (pass * TPW + w) * kW + warp;
@@ -265,11 +269,22 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : TPW == 1 ? 1 : 2) k_merge_
                     bk = o > bk ? o : bk;
                     o = __shfl_xor_sync(0xFFFFFFFFu, bk, 2);
                     bk = o > bk ? o : bk;
-                    if (t4 == 0 && row < na) atomicMax(m.best + a0 + row, bk);
+                    if (t4 == 0) tile_best[(tile - tile0) * 16 + g8 + 8 * i] = bk;   // 0 for rows past the CTA's share
                 }
             }
+            __syncthreads();
+            const int tile1 = min(tiles, tile0 + TPW * kW);
+            for (int a = tid; a < na; a += NT) {
+                const int t0 = (a >> 4) * NG;
+                unsigned long long o = m.best[a0 + a];
+                for (int t = max(t0, tile0); t < min(t0 + NG, tile1); ++t) {
+                    const unsigned long long b = tile_best[(t - tile0) * 16 + (a & 15)];
+                    o = b > o ? b : o;
+                }
+                m.best[a0 + a] = o;
+            }
+            __syncthreads();   // the next pass's copies overwrite the stages
         }
-        __syncthreads();
         if (CL > 1) {   // this CTA's row maxima to the others
             cg::cluster_group cl = cg::this_cluster();
             cl.sync();   // every CTA has initialised its maxima

@@ -138,17 +138,16 @@ __device__ __forceinline__ void issue_box(const TcMaps &maps, const Ring &R, con
     const uint32_t dst = smem_addr(sm + (half ? (size_t)R.rowsA * 128 : (size_t)0) + (size_t)st * R.kbs + (size_t)row0 * 128);
     tma_load_2d(dst, map, kb * 64, y + row0, smem_addr(&bar_full[st]));
 }
-// Every barrier a ring can use, from one thread at kernel entry: the fence that publishes the
-// initialisation waits for the thread's outstanding memory operations, so it runs before the
-// thread has issued any.
+// Every barrier a ring can use, from the lanes of one warp at kernel entry: the fence that publishes
+// the initialisation waits for a thread's outstanding memory operations, so it runs before the
+// warp has issued any.
 template <int NT>
 __device__ __forceinline__ void ring_barriers_init(unsigned long long *bar_full, unsigned long long *bar_empty,
                                                    unsigned long long *bar_done) {
-    for (int st = 0; st < kMaxStages; ++st) {
-        mbar_init(smem_addr(&bar_full[st]), 1);
-        mbar_init(smem_addr(&bar_empty[st]), 1 + NT / 32);
-    }
-    mbar_init(smem_addr(bar_done), 1);
+    const int lane = threadIdx.x & 31;
+    static_assert(kMaxStages == 16, "a full and an empty barrier per lane pair");
+    mbar_init(smem_addr(lane < 16 ? &bar_full[lane] : &bar_empty[lane - 16]), lane < 16 ? 1 : 1 + NT / 32);
+    if (lane == 0) mbar_init(smem_addr(bar_done), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -223,9 +222,9 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
         const CUtensorMap *mp = tid == 32 ? &maps.e32 : tid == 33 ? &maps.o32 : tid == 34 ? &maps.e8 : &maps.o8;
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(mp)) : "memory");
     }
-    // the ring's barriers, before this thread issues any memory operation (warp 0 issues the
+    // the ring's barriers, before this warp issues any memory operation (warp 0 issues the
     // tokens' loads after a CTA barrier: the fused plan's, or the one below)
-    if (tid == 36) ring_barriers_init<NT>(bar_full, bar_empty, &bar_done);
+    if (warp == 2) ring_barriers_init<NT>(bar_full, bar_empty, &bar_done);
     if (g.grouped && (tid == 38 || tid == 39))
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tid == 38 ? &maps.ge : &maps.go)) : "memory");
     if (tid == 0) s_fail = 0;   // visible after the barriers below, before any other write
@@ -237,7 +236,8 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
     // kernel's end; the exit mask is read after `griddepcontrol.wait` (without a programmatic
     // predecessor the wait returns at once)
     SampleInfo s;
-    if (!sample_begin<NT>(p, blockIdx.x, s, true)) {   // uniform over the CTA
+    const int part = g.parts > 1 ? (int)(blockIdx.x % (unsigned)g.parts) : 0;
+    if (!sample_begin<NT>(p, g.parts > 1 ? blockIdx.x / g.parts : blockIdx.x, s, true)) {   // uniform over the CTA
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         if (warp == 0)
@@ -432,7 +432,11 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
             ld.G = grouped ? gstride : 1024u;
             ld.K = grouped ? 1024u : kbs;
         }
-        finish_sample<__nv_bfloat16, NT>(p, s, m, ld);
+        if (finish_decide<NT>(p, s, m)) {
+            if (part == 0) write_index_outputs<NT>(p, s, m);
+            const int w = p.dim / 8;
+            write_rows<__nv_bfloat16, NT>(p, s, m, ld, w * part / g.parts, w * (part + 1) / g.parts);
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -479,7 +483,8 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");   // as in k_image_tc: the exit check's grid first
     SampleInfo s;
-    if (!sample_begin<kTiledThreads>(p, blockIdx.x, s)) {
+    const int part = g.parts > 1 ? (int)(blockIdx.x % (unsigned)g.parts) : 0;
+    if (!sample_begin<kTiledThreads>(p, g.parts > 1 ? blockIdx.x / g.parts : blockIdx.x, s)) {
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         if (warp == 0)
@@ -709,7 +714,11 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
     }
     if (s_fail == 0) {
         const GlobalLoader<__nv_bfloat16> gl{reinterpret_cast<const __nv_bfloat16 *>(p.x), (long long)s.start, p.dim};
-        finish_sample<__nv_bfloat16, kTiledThreads>(p, s, m, gl);
+        if (finish_decide<kTiledThreads>(p, s, m)) {
+            if (part == 0) write_index_outputs<kTiledThreads>(p, s, m);
+            const int w = p.dim / 8;
+            write_rows<__nv_bfloat16, kTiledThreads>(p, s, m, gl, w * part / g.parts, w * (part + 1) / g.parts);
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -830,8 +839,15 @@ TcGeometry image_tc_geometry(int dtype, int max_tokens, int kdim, int dim, long 
     return g;
 }
 
-cudaError_t launch_image_tc(const ImageParams &p, const TcGeometry &g, cudaStream_t s, bool pdl) {
+cudaError_t launch_image_tc(const ImageParams &p, const TcGeometry &geometry, cudaStream_t s, bool pdl) {
     if (p.in.max_batch == 0) return cudaSuccess;
+    // A small batch leaves SMs idle: up to four CTAs per sample, each making the sample's decisions (its
+    // keys come from L2 after the first) and writing a quarter of the columns; nothing is exchanged.  The
+    // gather and the means are 6 of the 24 us of one 197-token sample on its SM.
+    TcGeometry g = geometry;
+    const int slots = kSms * (g.tiled ? 1 : 2);
+    g.parts = 1;
+    while (g.parts < 4 && (long long)p.in.max_batch * (g.parts + 1) <= slots && p.dim / 8 / (g.parts + 1) >= 8) ++g.parts;
     EncodeTiledFn enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
     TcMaps maps{};
@@ -870,7 +886,7 @@ cudaError_t launch_image_tc(const ImageParams &p, const TcGeometry &g, cudaStrea
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(p.in.max_batch);
+    cfg.gridDim = dim3((unsigned)p.in.max_batch * (unsigned)g.parts);
     cfg.blockDim = dim3(g.tiled ? kTiledThreads : g.threads);
     cfg.dynamicSmemBytes = g.smem;
     cfg.stream = s;

@@ -166,6 +166,7 @@ struct TcGeometry {
     int ok;
     int tiled;         // halves beyond one tile: k_image_tc_tiled (M-tiles of 128 A rows, one CTA per SM)
     int threads;       // of k_image_tc
+    int parts;         // CTAs per sample, each a range of the output columns (set at the launch)
     int full_rows;     // rows of the largest TMA box of k_image_tc: half B of max_tokens tokens, rounded up to 8
     int grouped;       // samples that fit in shared memory load in 8-row groups of all K-blocks (one 3-D box
                        // per group) instead of through the ring

@@ -4,6 +4,8 @@
 // size-weighted means, pruning (Sec. III-E) and the gather into the compacted output.
 #pragma once
 
+#include <limits.h>
+
 #include "launch.h"
 
 namespace fz {
@@ -38,7 +40,8 @@ __host__ __device__ inline Meta meta_layout(int nmax, size_t base) {
     L.inv_b = off;  off += sizeof(float) * nB;
     L.match = off;  off += sizeof(int) * nA;
     L.sel = off;    off += sizeof(int) * nA;
-    L.mkey = off;   off += sizeof(int) * nA;
+    off = (off + 15) / 16 * 16;   // read four at a time, padded
+    L.mkey = off;   off += (sizeof(int) * nA + 15) / 16 * 16;
     L.mflag = off;  off += sizeof(int) * nmax;
     L.kflag = off;  off += sizeof(int) * nmax;
     L.opos = off;   off += sizeof(int) * (nmax + 1);
@@ -399,6 +402,7 @@ __device__ __forceinline__ void select_top_r(const SampleInfo &s, MetaPtrs &m) {
             m.sel[a] = rank < s.r_eff ? 1 : 0;
             if (rank < s.r_eff) m.mkey[rank] = (m.match[a] << kKeyShift) | a;
         }
+        if (tid < (-s.r_eff & 3)) m.mkey[s.r_eff + tid] = INT_MAX;   // above every key: pads the last group of four
     }
     __syncthreads();
 }
@@ -703,34 +707,48 @@ __device__ bool finish_decide(const ImageParams &p, const SampleInfo &s, MetaPtr
     for (int pos = tid; pos < N; pos += NT)
         m.mflag[pos] = (pos >= 2 && !(pos & 1) && m.sel[(pos - 2) / 2]) ? 0 : 1;
     if (R > 0) {
+        const int4 *k4 = reinterpret_cast<const int4 *>(m.mkey);
+        const int g4 = (R + 3) >> 2;
         for (int t = tid; t < R; t += NT) {
             const int key = m.mkey[t];
             int slot = 0;
-            for (int u = 0; u < R; ++u) slot += m.mkey[u] < key ? 1 : 0;
+#pragma unroll 4
+            for (int u = 0; u < g4; ++u) {
+                const int4 x = k4[u];
+                slot += (x.x < key ? 1 : 0) + (x.y < key ? 1 : 0) + (x.z < key ? 1 : 0) + (x.w < key ? 1 : 0);
+            }
             m.slist[slot] = key & ((1 << kKeyShift) - 1);
         }
-        for (int n = tid; n < nB; n += NT) {
-            int lt = 0, eq = 0;
-            for (int u = 0; u < R; ++u) {
-                const int b = m.mkey[u] >> kKeyShift;
-                lt += b < n ? 1 : 0;
-                eq += b == n ? 1 : 0;
+        for (int n = tid; n < nB; n += NT) {   // keys of B tokens below n, and up to n
+            const int k0 = n << kKeyShift, k1 = (n + 1) << kKeyShift;
+            int lt = 0, le = 0;
+#pragma unroll 4
+            for (int u = 0; u < g4; ++u) {
+                const int4 x = k4[u];
+                lt += (x.x < k0 ? 1 : 0) + (x.y < k0 ? 1 : 0) + (x.z < k0 ? 1 : 0) + (x.w < k0 ? 1 : 0);
+                le += (x.x < k1 ? 1 : 0) + (x.y < k1 ? 1 : 0) + (x.z < k1 ? 1 : 0) + (x.w < k1 ? 1 : 0);
             }
             m.scnt[n] = lt;
-            if (eq > 0) m.mlist[atomicAdd(&m.tmp[kMergedCount], 1)] = n;
+            if (le > lt) m.mlist[atomicAdd(&m.tmp[kMergedCount], 1)] = n;
         }
         if (tid == 0) m.scnt[nB] = R;
     }
     __syncthreads();
 
     // merged sizes and scores: float-float sums over the sources (exact for a few terms),
-    // rounded once; merged B tokens (mflag 2) also keep 1 / (sum of sizes) for the mean
-    for (int pos = tid; pos < N; pos += NT) {
-        if (!m.mflag[pos]) continue;
+    // rounded once; merged B tokens (mflag 2) also keep 1 / (sum of sizes) for the mean.  For
+    // pruning, the ordered merged score of every candidate; 0 marks a non-candidate (CLS or merged
+    // away), below every candidate's value
+    uint32_t *pv = reinterpret_cast<uint32_t *>(m.pk);
+    for (int pos = tid; pos < ((N + 3) & ~3); pos += NT) {
+        if (pos >= N || !m.mflag[pos]) {
+            pv[pos] = 0u;
+            continue;
+        }
         F2 sz = {m.tsize[pos], 0.0f};
         F2 sc = {m.tscore[pos], 0.0f};
         bool merged = false;
-        if (pos & 1) {
+        if (R > 0 && (pos & 1)) {
             const int n = (pos - 1) / 2;
             for (int q = m.scnt[n]; q < m.scnt[n + 1]; ++q) {
                 const int a = 2 + 2 * m.slist[q];
@@ -741,52 +759,58 @@ __device__ bool finish_decide(const ImageParams &p, const SampleInfo &s, MetaPtr
         }
         m.msize[pos] = sz.hi;
         m.mscore[pos] = sc.hi;
+        pv[pos] = pos > 0 ? max(ordered_bits(sc.hi), 1u) : 0u;
         if (merged) {
             const F2 inv = f2_div({1.0f, 0.0f}, sz);
             m.invd[pos] = make_float2(inv.hi, inv.lo);
             m.mflag[pos] = 2;
         }
-        if (p.scores && !isfinite(m.mscore[pos]) && pos > 0) raise_status(p.status, FUSION_DEV_NONFINITE);
+        if (p.scores && !isfinite(sc.hi) && pos > 0) raise_status(p.status, FUSION_DEV_NONFINITE);
     }
     __syncthreads();
 
-    // prune: CLS + the k highest merged scores, lowest position on ties
-    if (p.do_prune) {
-        bool nf = false;
-        const int k = keep_count(p.rho[s.id], N - R - 1, nf);
-        // the ordered merged score of every candidate; 0 marks a non-candidate (CLS or merged
-        // away), below every candidate's value (ordered values of floats are >= 1)
-        uint32_t *pv = reinterpret_cast<uint32_t *>(m.pk);
-        for (int pos = tid; pos < ((N + 3) & ~3); pos += NT)
-            pv[pos] = (pos > 0 && pos < N && m.mflag[pos]) ? max(ordered_bits(m.mscore[pos]), 1u) : 0u;
-        __syncthreads();
-        for (int pos = tid; pos < N; pos += NT) {
-            int keep = 0;
-            if (pos == 0) {
-                keep = 1;
-            } else if (m.mflag[pos]) {
-                // (CLS and merged-away tokens are 0, below every candidate)
-                keep = rank_of(pv, N, pos, pv[pos]) < k ? 1 : 0;
-            }
-            m.kflag[pos] = keep;
-            m.opos[pos] = keep;
+    // prune: CLS + the k highest merged scores, lowest position on ties (the plan has counted k from
+    // the keep ratio); else every token that was not merged away
+    const int k = s.out_n - 1;
+    unsigned *mask = reinterpret_cast<unsigned *>(m.tmp);   // [32]: kept tokens of positions 32 c ..
+    for (int p0 = 0; p0 < N; p0 += NT) {
+        const int pos = p0 + tid;
+        bool keep = false;
+        if (pos < N) {
+            keep = m.mflag[pos] != 0;
+            if (p.do_prune && keep && pos > 0) keep = rank_of(pv, N, pos, pv[pos]) < k;
+            m.kflag[pos] = keep ? 1 : 0;
         }
-    } else {
-        for (int pos = tid; pos < N; pos += NT) {
-            const int keep = m.mflag[pos] ? 1 : 0;
-            m.kflag[pos] = keep;
-            m.opos[pos] = keep;
-        }
+        const unsigned b = __ballot_sync(0xFFFFFFFFu, keep);
+        if ((tid & 31) == 0 && pos < N) mask[pos >> 5] = b;
     }
     __syncthreads();
-    const int total = block_scan_excl(m.opos, N, m.tmp);
+    // output position of every kept token (one barrier: every warp scans the masks itself), and the
+    // source of every output row; merged rows are stored complemented (negative)
+    static_assert(FUSION_MAX_TOKENS <= 32 * 32, "one mask per lane");
+    const int lane = tid & 31;
+    const unsigned own = 32 * lane < N ? mask[lane] : 0u;
+    int incl = __popc(own);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    for (int p0 = 0; p0 < N; p0 += NT) {
+        const int pos = p0 + tid, c = min(pos, N - 1) >> 5;
+        const int before = __shfl_sync(0xFFFFFFFFu, incl - __popc(own), c);   // c is the same for the whole warp
+        const unsigned b = __shfl_sync(0xFFFFFFFFu, own, c);
+        if (pos < N) {
+            const int o = before + __popc(b & ((1u << lane) - 1u));
+            m.opos[pos] = o;
+            if ((b >> lane) & 1u) m.srcpos[o] = m.mflag[pos] == 2 ? ~pos : pos;
+        }
+    }
     if (total != s.out_n) {   // the plan and the decisions disagree: a library bug
         if (tid == 0) raise_status(p.status, FUSION_DEV_INTERNAL);
         return false;
     }
-    // source of every output row; merged rows are stored complemented (negative)
-    for (int pos = tid; pos < N; pos += NT)
-        if (m.kflag[pos]) m.srcpos[m.opos[pos]] = m.mflag[pos] == 2 ? ~pos : pos;
     __syncthreads();
     return true;
 }
