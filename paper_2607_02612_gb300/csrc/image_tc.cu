@@ -483,8 +483,7 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");   // as in k_image_tc: the exit check's grid first
     SampleInfo s;
-    const int part = g.parts > 1 ? (int)(blockIdx.x % (unsigned)g.parts) : 0;
-    if (!sample_begin<kTiledThreads>(p, g.parts > 1 ? blockIdx.x / g.parts : blockIdx.x, s)) {
+    if (!sample_begin<kTiledThreads>(p, blockIdx.x, s)) {
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         if (warp == 0)
@@ -714,11 +713,7 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
     }
     if (s_fail == 0) {
         const GlobalLoader<__nv_bfloat16> gl{reinterpret_cast<const __nv_bfloat16 *>(p.x), (long long)s.start, p.dim};
-        if (finish_decide<kTiledThreads>(p, s, m)) {
-            if (part == 0) write_index_outputs<kTiledThreads>(p, s, m);
-            const int w = p.dim / 8;
-            write_rows<__nv_bfloat16, kTiledThreads>(p, s, m, gl, w * part / g.parts, w * (part + 1) / g.parts);
-        }
+        finish_sample<__nv_bfloat16, kTiledThreads>(p, s, m, gl);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -845,9 +840,9 @@ cudaError_t launch_image_tc(const ImageParams &p, const TcGeometry &geometry, cu
     // keys come from L2 after the first) and writing a quarter of the columns; nothing is exchanged.  The
     // gather and the means are 6 of the 24 us of one 197-token sample on its SM.
     TcGeometry g = geometry;
-    const int slots = kSms * (g.tiled ? 1 : 2);
     g.parts = 1;
-    while (g.parts < 4 && (long long)p.in.max_batch * (g.parts + 1) <= slots && p.dim / 8 / (g.parts + 1) >= 8) ++g.parts;
+    while (!g.tiled && g.parts < 4 && (long long)p.in.max_batch * (g.parts + 1) <= 2 * kSms && p.dim / 8 / (g.parts + 1) >= 8)
+        ++g.parts;
     EncodeTiledFn enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
     TcMaps maps{};
