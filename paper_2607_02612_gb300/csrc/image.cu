@@ -369,10 +369,10 @@ cudaError_t launch_image(int dtype, const ImageParams &p, size_t smem, cudaStrea
     if (p.in.max_batch == 0) return cudaSuccess;
     if (!p.do_merge) {
         // as many CTAs per sample as one wave of two per SM holds, each with at least 16 chunks (256 bytes)
-        // of a row
+        // of a row (a launch gate may stop a single CTA: its samples keep one)
         const int chunks = p.dim / (dtype == FUSION_BF16 ? 8 : 4);
         int parts = 1;
-        while (parts < 8 && (long long)p.in.max_batch * (parts + 1) <= 2 * 152 && chunks / (parts + 1) >= 16) ++parts;
+        while (!p.gate && parts < 8 && (long long)p.in.max_batch * (parts + 1) <= 2 * 152 && chunks / (parts + 1) >= 16) ++parts;
         auto kern = dtype == FUSION_BF16 ? k_select<__nv_bfloat16> : k_select<float>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

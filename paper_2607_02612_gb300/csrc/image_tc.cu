@@ -841,7 +841,8 @@ cudaError_t launch_image_tc(const ImageParams &p, const TcGeometry &geometry, cu
     // gather and the means are 6 of the 24 us of one 197-token sample on its SM.
     TcGeometry g = geometry;
     g.parts = 1;
-    while (!g.tiled && g.parts < 4 && (long long)p.in.max_batch * (g.parts + 1) <= 2 * kSms && p.dim / 8 / (g.parts + 1) >= 8)
+    // (a launch gate may stop a single CTA: its samples keep one)
+    while (!p.gate && !g.tiled && g.parts < 4 && (long long)p.in.max_batch * (g.parts + 1) <= 2 * kSms && p.dim / 8 / (g.parts + 1) >= 8)
         ++g.parts;
     EncodeTiledFn enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
