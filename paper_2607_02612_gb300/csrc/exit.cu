@@ -964,19 +964,14 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
                 const F2 rstd = f2_rsqrt(f2_add_f(var, p.head.eps));
                 if (gt == 0 && !(isfinite(mean.hi) && isfinite(var.hi))) raise_status(p.status, FUSION_DEV_NONFINITE);
                 for (int c = gt; c < nchunk; c += G * 32) {
-                    float f[CH], gf[CH], bf[CH];
-                    chunk_to_f(*reinterpret_cast<const uint4 *>(raw_chunk(j, c)), f);
-                    chunk_to_f(*reinterpret_cast<const uint4 *>(g_s + c * CH), gf);
-                    chunk_to_f(*reinterpret_cast<const uint4 *>(be_s + c * CH), bf);
                     uint4 outv;
                     if constexpr (kBf16) {
-                        uint32_t w4[4];
-    #pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            w4[q] = (uint32_t)ln_out_bf16(f[2 * q], mean, rstd, gf[2 * q], bf[2 * q]) |
-                                    ((uint32_t)ln_out_bf16(f[2 * q + 1], mean, rstd, gf[2 * q + 1], bf[2 * q + 1]) << 16);
-                        outv = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+                        outv = ln_chunk_bf16(raw_chunk(j, c), g_s + c * CH, be_s + c * CH, mean, rstd);
                     } else {
+                        float f[CH], gf[CH], bf[CH];
+                        chunk_to_f(*reinterpret_cast<const uint4 *>(raw_chunk(j, c)), f);
+                        chunk_to_f(*reinterpret_cast<const uint4 *>(g_s + c * CH), gf);
+                        chunk_to_f(*reinterpret_cast<const uint4 *>(be_s + c * CH), bf);
                         outv = make_uint4(__float_as_uint(ln_out_f32(f[0], mean, rstd, gf[0], bf[0])),
                                           __float_as_uint(ln_out_f32(f[1], mean, rstd, gf[1], bf[1])),
                                           __float_as_uint(ln_out_f32(f[2], mean, rstd, gf[2], bf[2])),
@@ -1101,7 +1096,10 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
 // samples x 64 classes, a lane two classes (24 shared-memory wavefronts per 128 FFMA at BT = 64; one
 // sample x 128 classes per warp, as k_exit_cl has it, takes 17 per 16).
 // Measured, tiles of 8 before -> now (cold caches): 8192 samples x 100 classes, d = 384, with the plan,
-// float32 173 -> 45 us and bf16 129 -> 30 us; 512 samples x 1000 classes, d = 768, bf16 34 -> 24 us.
+// float32 173 -> 44 us and bf16 129 -> 24 us; 512 samples x 1000 classes, d = 768, bf16 34 -> 20 us.
+// The LayerNorm is a third of that: sums on packed pairs, gamma and beta in shared memory, and the float-float
+// evaluation only where float32 does not settle an element (the chain of four such stages 383 -> 363 us in
+// bf16, 551 -> 541 in float32).
 // ---------------------------------------------------------------------------
 template <typename T, int BT>
 struct ExitRowsSmem {
@@ -1113,12 +1111,14 @@ struct ExitRowsSmem {
     static constexpr uint32_t w_stage = kTc ? kExitWStage : kExitCT * w_stride * 4u;
     static constexpr int lg_stride = kExitCT + 8;   // floats: the four samples of a warp 8 banks apart
     // u tile (bf16: K-blocks of [BT rows][128 bytes], swizzled; float32: [BT][dim + 4]) | weight ring (the
-    // logits tile [BT][lg_stride] afterwards) | bias | partials [BT][8] | rows, counts and bits [BT]
+    // logits tile [BT][lg_stride] afterwards) | bias | partials [BT][8] | gamma and beta
+    // (read per row and chunk: from global memory each read waited for L2) | rows, counts and bits [BT]
     static __host__ __device__ size_t u_bytes(int dim) {
         return kTc ? (size_t)((dim + 63) / 64) * BT * 128 : (size_t)BT * (dim + 4) * 4;
     }
     static __host__ __device__ size_t rest(int dim) {
-        return u_bytes(dim) + kExitCT * sizeof(float) + (size_t)BT * (8 * sizeof(float2) + 3 * sizeof(int)) + (kTc ? 1024 : 0);
+        return u_bytes(dim) + kExitCT * sizeof(float) + (size_t)BT * (8 * sizeof(float2) + 3 * sizeof(int)) + 2 * (size_t)dim * EB +
+               (kTc ? 1024 : 0);
     }
     static __host__ __device__ int w_stages(int dim) {
         if (!kTc) return kF32Stages;
@@ -1133,7 +1133,8 @@ struct ExitRowsSmem {
     }
     static __host__ __device__ size_t bias_off(int dim) { return u_bytes(dim) + ring_bytes(dim); }
     static __host__ __device__ size_t part_off(int dim) { return bias_off(dim) + kExitCT * sizeof(float); }
-    static __host__ __device__ size_t row_off(int dim) { return part_off(dim) + (size_t)BT * 8 * sizeof(float2); }
+    static __host__ __device__ size_t gb_off(int dim) { return part_off(dim) + (size_t)BT * 8 * sizeof(float2); }
+    static __host__ __device__ size_t row_off(int dim) { return gb_off(dim) + 2 * (size_t)dim * EB; }
     static __host__ __device__ size_t total(int dim) {
         return row_off(dim) + (size_t)BT * 3 * sizeof(int) + (kTc ? 1024 : 0);
     }
@@ -1179,6 +1180,7 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
     float *lg_s = reinterpret_cast<float *>(ring);   // [BT][kExitCT], after the product
     float *bias_s = reinterpret_cast<float *>(base + L::bias_off(dim));
     float2 *part_s = reinterpret_cast<float2 *>(base + L::part_off(dim));
+    uint4 *g_s = reinterpret_cast<uint4 *>(base + L::gb_off(dim)), *b_s = g_s + nchunk;   // gamma and beta
     int *row_s = reinterpret_cast<int *>(base + L::row_off(dim));   // CLS row of each sample, -1: none
     int *cnt_s = row_s + BT;     // the plan's counts: rows if the sample continues, then -1 where it exits
     int *bits_s = cnt_s + BT;    // and its status bits
@@ -1249,6 +1251,10 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
                     *reinterpret_cast<uint4 *>(uchunk(sl, c)) = make_uint4(0, 0, 0, 0);
             }
         }
+        for (int c = tid; c < nchunk; c += kExitThreads) {
+            cp_async16(g_s + c, reinterpret_cast<const T *>(p.head.gamma) + c * CH);
+            cp_async16(b_s + c, reinterpret_cast<const T *>(p.head.beta) + c * CH);
+        }
         cp_async_commit();
         const F2 rdim = f2_recip((float)dim);
         // lanes per row: a power of two, 4 (64 rows) .. 32 (8 rows or fewer)
@@ -1261,22 +1267,25 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
             const int j = j0 + tid / lpr, l = tid & (lpr - 1);
             const int sl = rank + j * ncl;
             const bool ok = j < nr && row_s[sl] >= 0;
-            float s1 = 0.0f, c1 = 0.0f, s2 = 0.0f, c2 = 0.0f, l2 = 0.0f;
+            // even and odd elements in the two lanes of packed sums: of x, of x^2 (rounded) and of what its
+            // rounding left (nothing for bf16, whose squares have 16 bits)
+            float2 s1 = make_float2(0.0f, 0.0f), c1 = s1, s2 = s1, c2 = s1, l2 = s1;
             if (ok) {
 #pragma unroll 1
                 for (int c = l; c < nchunk; c += lpr) {
                     float f[CH];
                     chunk_to_f(*reinterpret_cast<const uint4 *>(uchunk(sl, c)), f);
 #pragma unroll
-                    for (int e = 0; e < CH; ++e) {
-                        neu_add(s1, c1, f[e]);
-                        const F2 sq = two_prod(f[e], f[e]);
-                        neu_add(s2, c2, sq.hi);
-                        l2 = __fadd_rn(l2, sq.lo);
+                    for (int e = 0; e < CH; e += 2) {
+                        const float2 x = make_float2(f[e], f[e + 1]), sq = mul2(x, x);
+                        comp_add2(s1, c1, x);
+                        comp_add2(s2, c2, sq);
+                        if constexpr (!kBf16) l2 = add2(l2, fma2(x, x, make_float2(-sq.x, -sq.y)));
                     }
                 }
             }
-            F2 a1 = two_sum(s1, c1), a2 = f2_add_f(two_sum(s2, c2), l2);
+            F2 a1 = f2_add(two_sum(s1.x, c1.x), two_sum(s1.y, c1.y));
+            F2 a2 = f2_add_f(f2_add(two_sum(s2.x, c2.x), two_sum(s2.y, c2.y)), __fadd_rn(l2.x, l2.y));
 #pragma unroll 1
             for (int m = lpr >> 1; m >= 1; m >>= 1) {
                 a1 = f2_add(a1, f2_shfl_xor(a1, m));
@@ -1293,21 +1302,20 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
 #pragma unroll 1
             for (int c = l; c < nchunk; c += lpr) {
                 uint4 *dst = reinterpret_cast<uint4 *>(uchunk(sl, c));
-                float f[CH], gf[CH], bf[CH];
-                chunk_to_f(*dst, f);
-                chunk_to_f(ldg16(reinterpret_cast<const T *>(p.head.gamma) + c * CH), gf);
-                chunk_to_f(ldg16(reinterpret_cast<const T *>(p.head.beta) + c * CH), bf);
-                uint32_t w4[4];
+                uint4 o;
                 if constexpr (kBf16) {
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        w4[e] = (uint32_t)ln_out_bf16(f[2 * e], mean, rstd, gf[2 * e], bf[2 * e]) |
-                                ((uint32_t)ln_out_bf16(f[2 * e + 1], mean, rstd, gf[2 * e + 1], bf[2 * e + 1]) << 16);
+                    o = ln_chunk_bf16(reinterpret_cast<const __nv_bfloat16 *>(dst), reinterpret_cast<const __nv_bfloat16 *>(g_s + c),
+                                      reinterpret_cast<const __nv_bfloat16 *>(b_s + c), mean, rstd);
                 } else {
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) w4[e] = __float_as_uint(ln_out_f32(f[e], mean, rstd, gf[e], bf[e]));
+                    float f[CH], gf[CH], bf[CH];
+                    chunk_to_f(*dst, f);
+                    chunk_to_f(g_s[c], gf);
+                    chunk_to_f(b_s[c], bf);
+                    o = make_uint4(__float_as_uint(ln_out_f32(f[0], mean, rstd, gf[0], bf[0])),
+                                   __float_as_uint(ln_out_f32(f[1], mean, rstd, gf[1], bf[1])),
+                                   __float_as_uint(ln_out_f32(f[2], mean, rstd, gf[2], bf[2])),
+                                   __float_as_uint(ln_out_f32(f[3], mean, rstd, gf[3], bf[3])));
                 }
-                const uint4 o = make_uint4(w4[0], w4[1], w4[2], w4[3]);
                 *dst = o;
                 for (int r = 1; r < ncl; ++r) *cl.map_shared_rank(dst, rank + r < ncl ? rank + r : rank + r - ncl) = o;
             }

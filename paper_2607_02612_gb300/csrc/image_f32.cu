@@ -1,5 +1,5 @@
 // Per-sample merge -> prune -> gather for float32 tokens: the similarity on FFMA with the key dims
-// streamed through two cp.async stages, so that several CTAs share an SM (large batches of small
+// streamed through two to six cp.async stages, so that several CTAs share an SM (large batches of small
 // samples), and clusters of CTAs per sample (small batches of long ones).
 //
 // A cluster of CL CTAs owns a sample.  Each takes a run of 16-row strips of half A against all of half
@@ -14,9 +14,9 @@
 // Bound by the chain of latencies of one sample (loads, FFMA, decisions, gather) and, with enough
 // samples, by FFMA and L2.  The general kernel keeps a whole sample in shared memory (98 KB for 65
 // tokens of 384: two CTAs per SM) and gives 16 x 32 strips to warps, of which 65 tokens have two.
-// Measured, general kernel -> this one: 3277 of 8192 samples of 65 tokens, d = 384, continuing: 606 -> 269
+// Measured, general kernel -> this one: 3277 of 8192 samples of 65 tokens, d = 384, continuing: 606 -> 250
 // us (and 69 -> 39 us for the 210 that the fourth stage of that chain keeps); 8 samples of 197 tokens,
-// keys of their own, clusters of 8: 101 -> 55 us.  All with cold caches.
+// keys of their own, clusters of 8, the stage with its exit check: 117 -> 49 us.  All with cold caches.
 #include <cooperative_groups.h>
 
 #include "sample.cuh"
@@ -241,8 +241,8 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : TPW == 1 ? 1 : 2) k_merge_
                 __syncthreads();
             }
             // cosine and row maximum with the lowest column on ties: every tile leaves its 16 rows' maxima in
-            // the stages (all read by now), a thread per row takes the largest.  (64-bit maxima by shared-memory
-            // atomics, seven tiles on the same 16 rows, took up to 8 us.)
+            // the stages (all read by now), a thread per row takes the largest (no
+            // slower and no faster than 64-bit atomic maxima, and no entries to clear).
             unsigned long long *tile_best = reinterpret_cast<unsigned long long *>(st0);
             const int tile0 = pass * TPW * kW;
 #pragma unroll
@@ -346,7 +346,8 @@ F32Geometry image_f32_geometry(const ImageParams &p) {
     };
     g.small = small;
     // two CTAs per SM where 16 dims allow it; a batch that leaves SMs idle has each to itself, and more
-    // stages: 8 samples of 197 tokens, loop of six 64-dim stages: 12.4 us with two in flight, @S with all
+    // stages (a loop of six 64-dim stages took 12.4 of the kernel's 30 us with two in flight, most of it the
+    // wait for them)
     const bool alone = (long long)p.in.max_batch * g.cluster <= 152;
     const size_t most = 224 * 1024;
     for (size_t budget : {alone ? most : (size_t)110 * 1024, most})

@@ -1,15 +1,16 @@
 // Per-sample merge -> prune -> gather for bf16 tokens on the 5th-generation tensor
 // cores (tcgen05) with TMA, for samples of at most 257 tokens (|A|, |B| <= 128).
 //
-// One CTA of 256 threads per input sample.  The keys of half A (even positions) and
+// One CTA of 256 threads per input sample (128 threads for large batches of small samples; small
+// batches: up to four CTAs per sample, each a range of the output columns).  The keys of half A (even positions) and
 // half B (odd positions) arrive by TMA tensor loads in K-blocks of 64 dims, 128-byte
 // swizzled: K-block kb of a half is a [rows][128 B] tile, 16-byte chunk j of row t
-// stored at chunk position j ^ (t % 8).  Two tensor maps per parity of the global row
-// index (every other row of the token matrix) cover boxes of 32 and 8 rows, so any
-// half of any sample loads in whole 8-row groups.  The K-blocks stream through a ring
+// stored at chunk position j ^ (t % 8).  Tensor maps per parity of the global row index
+// (every other row of the token matrix) cover boxes of a whole half, 64, 32 and 8 rows, so any
+// half of any sample loads in whole 8-row groups and few copies.  The K-blocks stream through a ring
 // of stages (the whole sample stays resident when it fits).
 //
-// Thread 0 produces (TMA), thread 32 issues tcgen05.mma (M = 128 A rows, N = |B|
+// An elected lane of warp 0 produces (TMA), one of warp 1 issues tcgen05.mma (M = 128 A rows, N = |B|
 // rounded up to 16, K = 16 per instruction, f32 accumulation in tensor memory), and
 // every thread accumulates the squared norm of one A or B row from the same stages.
 // A stage is released when the MMAs that read it completed (tcgen05.commit) and all

@@ -178,3 +178,35 @@ def test_prune_and_compact_column_parts(dtype, counts, dim, prune):
     rng = np.random.default_rng(4)
     rho = rng.uniform(0.2, 1.0, len(counts)).astype(np.float32) if prune else None
     run_stage_and_compare(b, StageSpec(False, False, prune, rho=rho), f"{counts[:4]} x {len(counts)} d={dim}")
+
+
+@pytest.mark.parametrize("batch,dim", [(3, 128), (40, 272), (2440, 128), (9729, 80), (641, 272)])
+def test_layernorm_rounds_once(batch, dim):
+    """The exit check's LayerNorm in every tile size: with identity weights the logits are its bf16 rows,
+    each of which is the nearest bf16 value to the 64-bit one (beta cancels much of many elements).  The
+    slack is the float-float evaluation's relative error, 2^-40 of the terms."""
+    g = torch.Generator().manual_seed(batch)
+    x = (torch.randn((batch, dim), generator=g) * 3 + torch.randn((batch, 1), generator=g)).bfloat16()
+    gamma = (1 + 0.3 * torch.randn(dim, generator=g)).bfloat16()
+    beta = torch.randn(dim, generator=g).bfloat16()
+    eps = float(np.float32(1e-6))
+    xc = x.cuda()
+    b = runner.DeviceBatch("bf16", dim, batch, 1, batch, xc, xc, torch.ones(batch, device="cuda"), None,
+                           torch.arange(batch + 1, dtype=torch.int32, device="cuda"))
+    head = runner.HeadTensors(gamma.cuda(), beta.cuda(), eps, torch.eye(dim).bfloat16().cuda(), torch.zeros(dim).cuda(), 1e-6)
+    f = runner.Fusion(batch, dim)
+    o = f.exit_check(b, head)
+    assert int(f.status.item()) == 0 and bool(o["exit_mask"].all())
+    u = o["logits"].cpu()
+    xd = x.double()
+    d = xd - xd.mean(1, keepdim=True)
+    v = d / torch.sqrt((d * d).mean(1, keepdim=True) + eps) * gamma.double()
+    want = v + beta.double()
+    assert torch.equal(u, u.bfloat16().float())
+    err = (u.double() - want).abs()
+    slack = 2.0 ** -40 * (v.abs() + beta.double().abs())
+    bits = u.bfloat16().view(torch.int16)
+    for step in (-1, 1):
+        other = (bits + step).view(torch.bfloat16).double()
+        ok = (err <= (other - want).abs() + slack) | ~torch.isfinite(other)
+        assert bool(ok.all()), int((~ok).sum())
