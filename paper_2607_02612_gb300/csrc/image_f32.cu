@@ -16,7 +16,7 @@
 // tokens of 384: two CTAs per SM) and gives 16 x 32 strips to warps, of which 65 tokens have two.
 // Measured, general kernel -> this one: 3277 of 8192 samples of 65 tokens, d = 384, continuing: 606 -> 250
 // us (and 69 -> 39 us for the 210 that the fourth stage of that chain keeps); 8 samples of 197 tokens,
-// keys of their own, clusters of 8, the stage with its exit check: 117 -> 49 us.  All with cold caches.
+// keys of their own, clusters of 8, the stage with its exit check: 117 -> 47 us.  All with cold caches.
 #include <cooperative_groups.h>
 
 #include "sample.cuh"
@@ -51,7 +51,8 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : TPW == 1 ? 1 : 2) k_merge_
     SampleInfo s;
     if (!sample_begin<NT>(p, CL > 1 ? blockIdx.x / CL : blockIdx.x, s)) return;   // the same in every CTA of the cluster
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int kdim = p.kdim, kd = g.kd;
+    constexpr bool kSplit = NP > 0 && NT == 256;
+    const int kdim = p.kdim, kd = kSplit ? 64 : g.kd;
     const uint32_t rs = stage_row(kd);
     // this CTA's strips of half A
     const int strips = (s.nA + 15) / 16, per = (strips + CL - 1) / CL;
@@ -98,7 +99,16 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : TPW == 1 ? 1 : 2) k_merge_
     meta_init<NT>(p, s, m);
     __syncthreads();
     if (s.decide) {
-        const int g8 = lane >> 2, t4 = lane & 3;
+        // A thread's two rows and four columns of a tile.  kSplit (kd = 64): half of the warp sums the even
+        // 16-dim blocks, the other half the odd ones, of 4 rows x 4 columns per thread (8 shared-memory
+        // loads per 64 FFMA; 2 rows x 4 columns of every block take 12), and they swap the partial sums of
+        // each other's rows: every sum is formed from the same terms in the same order.  8 samples of 197
+        // tokens in clusters of 8, the stage: 49.1 -> 47.3 us.  Not with 128 threads, where the registers are
+        // needed for the CTAs of an SM: the chain of stages on 8192 samples 518 us instead of 516 at four CTAs,
+        // 554 instead of 537 at five.
+        const int h = lane >> 4, t4 = lane & 3;
+        const int g8 = kSplit ? ((lane >> 2) & 3) + 8 * h : lane >> 2;
+        constexpr int kRowStep = kSplit ? 4 : 8;
         float nlo[NP > 0 ? NP : 1], nhi[NP > 0 ? NP : 1];
 #pragma unroll
         for (int k = 0; k < (NP > 0 ? NP : 1); ++k) nlo[k] = nhi[k] = 0.0f;
@@ -123,6 +133,48 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : TPW == 1 ? 1 : 2) k_merge_
                     const int mt = tile / NG, ng = tile - mt * NG;
                     // rows past the halves read stale or unwritten shared memory inside the stage: their
                     // products are never used
+                    if constexpr (kSplit) {
+                        const unsigned char *rb = st + (uint32_t)(g.rows_a + ng * 16 + t4) * rs + h * 64;
+                        const unsigned char *own = st + (uint32_t)(mt * 16 + g8) * rs + h * 64;
+                        const unsigned char *oth = st + (uint32_t)(mt * 16 + (g8 ^ 8)) * rs + h * 64;
+#pragma unroll 1
+                        for (int k0 = 0; k0 < kw; k0 += 32) {
+                            const bool odd = k0 + 16 < kw;   // uniform: a second block
+                            float t[4][4] = {};
+                            if (h == 0 || odd) {
+#pragma unroll
+                                for (int kk = 0; kk < 16; kk += 4) {
+                                    const uint32_t o = (uint32_t)(k0 + kk) * 4;
+                                    float4 a[4];
+                                    a[0] = *reinterpret_cast<const float4 *>(own + o);
+                                    a[1] = *reinterpret_cast<const float4 *>(own + 4 * rs + o);
+                                    a[2] = *reinterpret_cast<const float4 *>(oth + o);
+                                    a[3] = *reinterpret_cast<const float4 *>(oth + 4 * rs + o);
+#pragma unroll
+                                    for (int e = 0; e < 4; ++e) {
+                                        const float4 b = *reinterpret_cast<const float4 *>(rb + (uint32_t)(4 * e) * rs + o);
+#pragma unroll
+                                        for (int i = 0; i < 4; ++i) {
+                                            t[i][e] = fmaf(a[i].x, b.x, t[i][e]);
+                                            t[i][e] = fmaf(a[i].y, b.y, t[i][e]);
+                                            t[i][e] = fmaf(a[i].z, b.z, t[i][e]);
+                                            t[i][e] = fmaf(a[i].w, b.w, t[i][e]);
+                                        }
+                                    }
+                                }
+                            }
+                            __syncwarp();
+#pragma unroll
+                            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    const float got = __shfl_xor_sync(0xFFFFFFFFu, t[i + 2][e], 16);
+                                    acc[w][i][e] += h ? got : t[i][e];
+                                    if (odd) acc[w][i][e] += h ? t[i][e] : got;
+                                }
+                        }
+                        continue;
+                    }
                     const unsigned char *ra = st + (uint32_t)(mt * 16 + g8) * rs;
                     const unsigned char *rb = st + (uint32_t)(g.rows_a + ng * 16 + t4) * rs;
 #pragma unroll 1
@@ -252,7 +304,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : TPW == 1 ? 1 : 2) k_merge_
                 const int mt = tile / NG, ng = tile - mt * NG;
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
-                    const int row = mt * 16 + g8 + 8 * i;
+                    const int row = mt * 16 + g8 + kRowStep * i;
                     unsigned long long bk = 0ull;
                     if (row < na) {
                         const float ia = m.inv_a[a0 + row];
@@ -269,7 +321,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 5 : TPW == 1 ? 1 : 2) k_merge_
                     bk = o > bk ? o : bk;
                     o = __shfl_xor_sync(0xFFFFFFFFu, bk, 2);
                     bk = o > bk ? o : bk;
-                    if (t4 == 0) tile_best[(tile - tile0) * 16 + g8 + 8 * i] = bk;   // 0 for rows past the CTA's share
+                    if (t4 == 0) tile_best[(tile - tile0) * 16 + g8 + kRowStep * i] = bk;   // 0 for rows past the CTA's share
                 }
             }
             __syncthreads();
