@@ -43,7 +43,7 @@ constexpr int kMaxStagesF32 = 6;
 // NT threads; TPW warp tiles held in registers per pass; NP > 0: squared norms summed from the stages,
 // NP rows per 16 threads (kd = 64, norm blocks of whole stages), else read again from global memory (L2).
 template <int NT, int TPW, int NP>
-__global__ void __launch_bounds__(NT, NT == 128 ? 5 : TPW == 1 ? 1 : 2) k_merge_f32(ImageParams p, F32Geometry g) {
+__global__ void __launch_bounds__(NT, NT == 128 ? 4 : TPW == 1 ? 1 : 2) k_merge_f32(ImageParams p, F32Geometry g) {
     extern __shared__ __align__(16) unsigned char sm[];
     constexpr int kW = NT / 32;
     const int CL = g.cluster;
