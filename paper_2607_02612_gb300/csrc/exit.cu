@@ -38,6 +38,7 @@ __device__ __forceinline__ void issue_w_chunk(const ExitParams &p, unsigned char
     constexpr int wchunks = KC / CH;
     const int kw = min(KC, dim - k0);
     const T *W = reinterpret_cast<const T *>(p.head.weight);
+#pragma unroll 1
     for (int it = tid; it < kExitCT * wchunks; it += kExitThreads) {
         const int row = it / wchunks, c = it - row * wchunks;
         T *dst = reinterpret_cast<T *>(stage_buf) + row * w_stride + c * CH;
@@ -104,6 +105,7 @@ __device__ __forceinline__ bool exit_tc_product(const CUtensorMap *wmap, uint32_
     bool okw = true;
     int waited = 0, issued = 0, loaded = nws;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
     for (int kc = 0; kc < nk; ++kc) {
         const int st = kc % nws;
         const uint32_t ph = (uint32_t)(kc / nws) & 1u;
@@ -114,6 +116,7 @@ __device__ __forceinline__ bool exit_tc_product(const CUtensorMap *wmap, uint32_
         waited = kc + 1;
         const uint32_t a0 = wr + (uint32_t)st * kExitWStage, b0 = ub + (uint32_t)kc * (NB * 128u);
         const int kw = min(64, dim - kc * 64);
+#pragma unroll 1
         for (int k = 0; k * 16 < kw; ++k)
             umma_bf16(tmem, sw128_desc(a0 + k * 32), sw128_desc(b0 + k * 32), exit_idesc(NB), (kc | k) ? 1u : 0u);
         umma_commit(smem_addr(&wempty[st]));
@@ -135,6 +138,7 @@ __device__ __forceinline__ bool exit_tc_product(const CUtensorMap *wmap, uint32_
         okw = mbar_wait(smem_addr(wdone), 0u);
     }
     if (!okw) {
+#pragma unroll 1
         for (int q = waited; q < loaded; ++q) (void)mbar_wait(smem_addr(&wbar[q % nws]), (uint32_t)(q / nws) & 1u);
         if (issued > 0) (void)mbar_wait(smem_addr(&wempty[(issued - 1) % nws]), (uint32_t)((issued - 1) / nws) & 1u);
         raise_status(status, FUSION_DEV_TIMEOUT);
@@ -165,6 +169,7 @@ __device__ __forceinline__ void exit_gemm(const ExitParams &p, const T *u_s, uns
     constexpr int KC = S::KC;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int u_stride = S::u_stride(dim);
+#pragma unroll 1
     for (int kc = 0; kc < n_k; ++kc) {
         const int k0 = kc * KC;
         const int kw = min(KC, dim - k0);
@@ -178,6 +183,7 @@ __device__ __forceinline__ void exit_gemm(const ExitParams &p, const T *u_s, uns
         const float *ur = reinterpret_cast<const float *>(u_s) + (size_t)warp * u_stride + k0;
         const float *ws = reinterpret_cast<const float *>(wbuf);
         float t[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 1
         for (int kk = 0; kk < kw; kk += 4) {
             const float4 uv = *reinterpret_cast<const float4 *>(ur + kk);
 #pragma unroll
@@ -217,6 +223,7 @@ __device__ __forceinline__ void exit_logits_f32(float *lg_s, const float *bias_s
 // which the last CTA of the sample tile writes the rows of the samples that exit.
 __device__ __forceinline__ void exit_stage_logits(const ExitParams &p, const float *lg_s, int s0, int c0, int B, int C) {
     if (!p.lg_tmp) return;
+#pragma unroll 1
     for (int it = threadIdx.x; it < kExitBT * kExitCT; it += kExitThreads) {
         const int sl = it / kExitCT, col = it - sl * kExitCT;
         if (s0 + sl < B && c0 + col < C) p.lg_tmp[(size_t)(s0 + sl) * C + c0 + col] = lg_s[it];
@@ -243,6 +250,7 @@ __device__ __forceinline__ F2 hidden_dot_exact_warp(const unsigned char *wt, int
                                                     const unsigned char *ut, int row, int dim, float b1) {
     const int lane = threadIdx.x & 31;
     F2 acc = {0.0f, 0.0f};
+#pragma unroll 1
     for (int c = lane * 8; c < dim; c += 256) {
         float wf[8], uf[8];
         const int ch = c >> 3;
@@ -261,6 +269,7 @@ __device__ __forceinline__ F2 hidden_dot_exact_warp(const unsigned char *wt, int
 __device__ __noinline__ F2 hidden_dot_exact_thread(const __nv_bfloat16 *wg, const unsigned char *ut, int row, int dim,
                                                    float b1) {
     F2 acc = {0.0f, 0.0f};
+#pragma unroll 1
     for (int ch = 0; ch < dim / 8; ++ch) {
         float wf[8], uf[8];
         chunk_to_f(ldg16(wg + ch * 8), wf);
@@ -336,12 +345,14 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
             }
             if (warp == 1 && elect_one()) {
                 const int nws = TS::w_stages(dim);
+#pragma unroll 1
                 for (int q = 0; q < nws; ++q) {
                     mbar_init(smem_addr(&wbar[q]), 1);
                     mbar_init(smem_addr(&wempty[q]), 1);
                 }
                 mbar_init(smem_addr(&wdone), 1);
                 asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+#pragma unroll 1
                 for (int q = 0; q < nws; ++q) {
                     mbar_expect_tx(smem_addr(&wbar[q]), kExitWStage);
                     tma_load_2d(smem_addr(w_region + (size_t)q * kExitWStage), &wmap, q * 64, c0, smem_addr(&wbar[q]));
@@ -354,6 +365,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
         // launched as a programmatic dependent of the kernel before it (the MLP head's layers):
         // the weights above are this call's own input; the rows below may be that kernel's output
         asm volatile("griddepcontrol.wait;" ::: "memory");
+#pragma unroll 1
         for (int it = tid; it < 16 * nchunk; it += kExitThreads) {
             const int sl = it / nchunk, c = it - sl * nchunk;
             const int s = s0 + sl;
@@ -428,6 +440,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
         };
         if (ok && !p.skip_ln) {
             float ss = 0.0f, sc = 0.0f, sl_lo = 0.0f;
+#pragma unroll 1
             for (int c = lane; c < nchunk; c += 32) {
                 float f[CH], fl[CH];
                 in_chunk(c, f);
@@ -443,6 +456,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
             const F2 mean = f2_mul(warp_sum_f2(url ? f2_add_f(two_sum(ss, sc), sl_lo) : two_sum(ss, sc)), rdim);
             ss = sc = 0.0f;
             float lo = 0.0f;
+#pragma unroll 1
             for (int c = lane; c < nchunk; c += 32) {
                 float f[CH], fl[CH];
                 in_chunk(c, f);
@@ -461,6 +475,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
             if (lane == 0 && !(isfinite(mean.hi) && isfinite(var.hi))) raise_status(p.status, FUSION_DEV_NONFINITE);
             const T *g = reinterpret_cast<const T *>(p.head.gamma);
             const T *bb = reinterpret_cast<const T *>(p.head.beta);
+#pragma unroll 1
             for (int c = lane; c < nchunk; c += 32) {
                 float f[CH], fl[CH], gf[CH], bf[CH];
                 in_chunk(c, f);
@@ -493,6 +508,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
                 }
             }
         } else if (!ok) {   // (skip_ln: the loaded rows stay as they are)
+#pragma unroll 1
             for (int c = lane; c < nchunk; c += 32) *reinterpret_cast<uint4 *>(uchunk(warp, c)) = make_uint4(0, 0, 0, 0);
         }
     }
@@ -534,6 +550,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
                     const int r = tid & (kExitCT - 1), h = tid / kExitCT;
                     float acc = 0.0f;
                     if (resident) {
+#pragma unroll 1
                         for (int q = h; q < nws; q += 2) {
                             const unsigned char *row = w_region + (size_t)q * kExitWStage + (size_t)r * 128;
 #pragma unroll
@@ -546,6 +563,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
                         }
                     } else if (c0 + r < C) {
                         const T *wr = reinterpret_cast<const T *>(p.head.weight) + (size_t)(c0 + r) * dim;
+#pragma unroll 1
                         for (int cb = h; cb < nchunk; cb += 16) {
                             uint4 v[8];
 #pragma unroll
@@ -564,6 +582,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
                 }
                 {   // ||u||^2 of each sample's row (warp -> sample slot)
                     float acc = 0.0f;
+#pragma unroll 1
                     for (int c = lane; c < nchunk; c += 32) {
                         float f[CH];
                         chunk_to_f(*reinterpret_cast<const uint4 *>(uchunk(warp, c)), f);
@@ -624,6 +643,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
                 // their exact dot products, one at a time by a whole warp; their GELU, every lane its own (the
                 // double-precision fallback then runs once per unit, not once per lane)
                 const int n_fl = min(s_flagged, list_cap);
+#pragma unroll 1
                 for (int k0 = warp; k0 < n_fl; k0 += 32 * (kExitThreads / 32)) {
                     F2 mine = {0.0f, 0.0f};
                     int unit = -1;
@@ -660,6 +680,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
             exit_logits_f32(lg_s, bias_s, acc, c0, C);
             __syncthreads();
             if (p.out_mode == 1) {   // hidden layer: GELU in float32
+#pragma unroll 1
                 for (int it = tid; it < kExitBT * kExitCT; it += kExitThreads) {
                     const int sl = it / kExitCT, col = it - sl * kExitCT;
                     const float a = lg_s[it];
@@ -704,6 +725,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
         if (s < B) {
             float m = -INFINITY;
             bool bad = false;
+#pragma unroll 1
             for (int q = lane; q < p.n_ctile; q += 32) {
                 const float2 pz = __ldcg(&p.partials[(size_t)s * p.n_ctile + q]);
                 m = fmaxf(m, pz.x);
@@ -713,6 +735,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
             for (int o = 16; o >= 1; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
             if (!__any_sync(0xFFFFFFFFu, bad)) {   // else a product timed out: no decision (status raised)
                 float z = 0.0f;
+#pragma unroll 1
                 for (int q = lane; q < p.n_ctile; q += 32) {
                     const float2 pz = __ldcg(&p.partials[(size_t)s * p.n_ctile + q]);
                     z += pz.y * expf(pz.x - m);
@@ -727,6 +750,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
                     if (!isfinite(m)) raise_status(p.status, FUSION_DEV_NONFINITE);
                 }
                 if (ex && p.logits && p.lg_tmp)   // logits only for the samples that exit
+#pragma unroll 1
                     for (int col = lane; col < p.head.classes; col += 32)
                         p.logits[(size_t)s * p.head.classes + col] =
                             __ldcg(&p.lg_tmp[(size_t)s * p.head.classes + col]);
@@ -858,12 +882,14 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
     if (active && kBf16 && warp == 1 && elect_one()) {
         // the head's first weight chunks first: they depend on nothing and take longest to land
         const int nws = L::w_stages(dim);
+#pragma unroll 1
         for (int q = 0; q < nws; ++q) {
             mbar_init(smem_addr(&wbar[q]), 1);
             mbar_init(smem_addr(&wempty[q]), 1);
         }
         mbar_init(smem_addr(&wdone), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+#pragma unroll 1
         for (int q = 0; q < nws; ++q) {
             mbar_expect_tx(smem_addr(&wbar[q]), kExitWStage);
             tma_load_2d(smem_addr(w_region + (size_t)q * kExitWStage), &wmap, q * 64, c0, smem_addr(&wbar[q]));
@@ -871,6 +897,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
     }
     if (active) {
         // own CLS rows, gamma and beta (group 0), then the bias
+#pragma unroll 1
         for (int it = tid; it < BT * nchunk; it += kExitThreads) {
             const int jj = it / nchunk, c = it - jj * nchunk;
             const int sli = rank + jj * ncl, si = s0 + sli;
@@ -887,6 +914,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
             else
                 *reinterpret_cast<uint4 *>(dst) = make_uint4(0, 0, 0, 0);
         }
+#pragma unroll 1
         for (int c = tid; c < 2 * nchunk; c += kExitThreads) {
             const bool isg = c < nchunk;
             const int cc = isg ? c : c - nchunk;
@@ -902,6 +930,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
         cp_async_commit();
         // padding rows 8..15 of the GEMM's A tile (float32; for bf16 they feed only the unused
         // columns 8..15 of the tensor-memory product)
+#pragma unroll 1
         for (int it = tid; !kBf16 && it < 8 * nchunk; it += kExitThreads) {
             const int r = 8 + it / nchunk, c = it % nchunk;
             *reinterpret_cast<uint4 *>(u_s + (size_t)r * u_stride + c * CH) = make_uint4(0, 0, 0, 0);
@@ -921,6 +950,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
         }
 
         // ---- LayerNorm, G warps per row: one pass of sum and sum of squares -----------
+#pragma unroll 1
         for (int jb = 0; jb < nrp; jb += ngr) {   // rounds of ngr rows (uniform trip count)
             const int j = jb + jw, sl = rank + j * ncl;
             const bool has_row = j < nrp && sl < BT;
@@ -930,6 +960,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
             const F2 rdim = f2_recip((float)dim);
             float s1 = 0.0f, c1 = 0.0f, s2 = 0.0f, c2 = 0.0f, l2 = 0.0f;
             if (ok) {
+#pragma unroll 1
                 for (int e = gt; e < dim; e += G * 32) {
                     const float v = to_float(raw_chunk(j, e / CH)[e % CH]);
                     neu_add(s1, c1, v);
@@ -963,6 +994,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
                 if (var.hi < 0.0f) var = {0.0f, 0.0f};
                 const F2 rstd = f2_rsqrt(f2_add_f(var, p.head.eps));
                 if (gt == 0 && !(isfinite(mean.hi) && isfinite(var.hi))) raise_status(p.status, FUSION_DEV_NONFINITE);
+#pragma unroll 1
                 for (int c = gt; c < nchunk; c += G * 32) {
                     uint4 outv;
                     if constexpr (kBf16) {
@@ -978,11 +1010,14 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
                                           __float_as_uint(ln_out_f32(f[3], mean, rstd, gf[3], bf[3])));
                     }
                     T *dst = kBf16 ? reinterpret_cast<T *>(base + u_tc_off(sl, c)) : u_s + (size_t)sl * u_stride + c * CH;
+#pragma unroll 1
                     for (int r = 0; r < ncl; ++r) *reinterpret_cast<uint4 *>(cl.map_shared_rank(dst, r)) = outv;
                 }
             } else if (has_row) {
+#pragma unroll 1
                 for (int c = gt; c < nchunk; c += G * 32) {
                     T *dst = kBf16 ? reinterpret_cast<T *>(base + u_tc_off(sl, c)) : u_s + (size_t)sl * u_stride + c * CH;
+#pragma unroll 1
                     for (int r = 0; r < ncl; ++r)
                         *reinterpret_cast<uint4 *>(cl.map_shared_rank(dst, r)) = make_uint4(0, 0, 0, 0);
                 }
@@ -1033,6 +1068,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
         // partial softmax of this class tile, warp -> sample slots warp, warp + 8, ...; to every
         // CTA of the cluster (a tile whose product timed out sends z = -1: no decision)
         const bool failed = s_wfail != 0;
+#pragma unroll 1
         for (int slw = warp; slw < BT; slw += kWarps) {
             const int sw = s0 + slw;
             float m = -INFINITY;
@@ -1053,11 +1089,13 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
     cl.sync();   // every CTA holds every partial of the tile's samples
     // Every CTA merges the partials in the same order (so all agree on every decision); the
     // owner writes the exit mask and c, every CTA its logits tile of the samples that exit.
+#pragma unroll 1
     for (int slw = warp; active && slw < BT; slw += kWarps) {
         const int sw = s0 + slw;
         if (sw >= B) continue;
         float m = -INFINITY;
         bool bad = false;
+#pragma unroll 1
         for (int q = lane; q < ncl; q += 32) {
             const float2 pz = part_s[slw * 8 + q];
             m = fmaxf(m, pz.x);
@@ -1067,6 +1105,7 @@ __global__ void __launch_bounds__(kExitThreads) k_exit_cl(const __grid_constant_
         for (int o = 16; o >= 1; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
         if (__any_sync(0xFFFFFFFFu, bad)) continue;   // a product timed out: no decision (status raised)
         float z = 0.0f;
+#pragma unroll 1
         for (int q = lane; q < ncl; q += 32) {
             const float2 pz = part_s[slw * 8 + q];
             z += pz.y * expf(pz.x - m);
@@ -1144,6 +1183,7 @@ struct ExitRowsSmem {
 template <typename S>
 __device__ __forceinline__ void issue_w_rows(const ExitParams &p, float *dst, int c0, int k0, int dim, int C) {
     constexpr int wch = S::KC / 4;
+#pragma unroll 1
     for (int it = threadIdx.x; it < kExitCT * wch; it += kExitThreads) {
         const int row = it / wch, c = it - row * wch;
         float *d = dst + row * S::w_stride + c * 4;
@@ -1205,21 +1245,25 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
             }
             if (warp == 1 && elect_one()) {
                 const int nws = L::w_stages(dim);
+#pragma unroll 1
                 for (int q = 0; q < nws; ++q) {
                     mbar_init(smem_addr(&wbar[q]), 1);
                     mbar_init(smem_addr(&wempty[q]), 1);
                 }
                 mbar_init(smem_addr(&wdone), 1);
                 asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+#pragma unroll 1
                 for (int q = 0; q < nws; ++q) {
                     mbar_expect_tx(smem_addr(&wbar[q]), kExitWStage);
                     tma_load_2d(smem_addr(ring + (size_t)q * kExitWStage), &wmap, q * 64, c0, smem_addr(&wbar[q]));
                 }
             }
         } else {
+#pragma unroll 1
             for (int q = 0; q < L::kF32Stages; ++q)
                 issue_w_rows<L>(p, reinterpret_cast<float *>(ring + q * L::w_stage), c0, q * L::KC, dim, C);
         }
+#pragma unroll 1
         for (int k = tid; k < BT; k += kExitThreads) {
             int row = -1, n = -1, bits = 0;
             if (s0 + k < B) {
@@ -1241,9 +1285,11 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
     if (active) {
         // ---- this CTA's rows (samples rank, rank + ncl, ... of the tile) into the u tile ------------
         const int nr = (BT - rank + ncl - 1) / ncl;
+#pragma unroll 1
         for (int j = warp; j < nr; j += kWarps) {
             const int sl = rank + j * ncl, row = row_s[sl];
             const T *src = reinterpret_cast<const T *>(p.x) + (long long)row * dim;
+#pragma unroll 1
             for (int c = lane; c < nchunk; c += 32) {
                 if (row >= 0)
                     cp_async16(uchunk(sl, c), src + c * CH);
@@ -1251,6 +1297,7 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
                     *reinterpret_cast<uint4 *>(uchunk(sl, c)) = make_uint4(0, 0, 0, 0);
             }
         }
+#pragma unroll 1
         for (int c = tid; c < nchunk; c += kExitThreads) {
             cp_async16(g_s + c, reinterpret_cast<const T *>(p.head.gamma) + c * CH);
             cp_async16(b_s + c, reinterpret_cast<const T *>(p.head.beta) + c * CH);
@@ -1263,6 +1310,7 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
         cp_async_wait_all();
         __syncthreads();
         // ---- LayerNorm in place, lpr lanes per row: one pass of sum and sum of squares ---------------
+#pragma unroll 1
         for (int j0 = 0; j0 < nr; j0 += kExitThreads / lpr) {
             const int j = j0 + tid / lpr, l = tid & (lpr - 1);
             const int sl = rank + j * ncl;
@@ -1317,14 +1365,18 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
                                    __float_as_uint(ln_out_f32(f[3], mean, rstd, gf[3], bf[3])));
                 }
                 *dst = o;
+#pragma unroll 1
                 for (int r = 1; r < ncl; ++r) *cl.map_shared_rank(dst, rank + r < ncl ? rank + r : rank + r - ncl) = o;
             }
         }
         // rows past the batch (or malformed): zero in the other CTAs too
+#pragma unroll 1
         for (int j = warp; ncl > 1 && j < nr; j += kWarps) {
             const int sl = rank + j * ncl;
             if (row_s[sl] >= 0) continue;
+#pragma unroll 1
             for (int c = lane; c < nchunk; c += 32)
+#pragma unroll 1
                 for (int r = 0; r < ncl; ++r)
                     *cl.map_shared_rank(reinterpret_cast<uint4 *>(uchunk(sl, c)), r) = make_uint4(0, 0, 0, 0);
         }
@@ -1348,6 +1400,7 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             if (s_wfail == 0) {   // D's lanes are classes; warps w and w + 4 share a quadrant's columns
                 const int cls = (warp & 3) * 32 + lane;
+#pragma unroll 1
                 for (int n0 = (warp >> 2) * 16; n0 < BT; n0 += 32) {
                     uint32_t v[16];
                     tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)n0, v);
@@ -1367,6 +1420,7 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
 #pragma unroll
             for (int i = 0; i < SP; ++i) acc[i][0] = acc[i][1] = 0.0f;
             const int n_k = (dim + L::KC - 1) / L::KC;
+#pragma unroll 1
             for (int kc = 0; kc < n_k; ++kc) {
                 asm volatile("cp.async.wait_group %0;\n" ::"n"(L::kF32Stages - 1) : "memory");
                 __syncthreads();
@@ -1374,6 +1428,7 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
                 const float *ws = reinterpret_cast<const float *>(stage) + (cb + lane) * L::w_stride;
                 const float *ur = reinterpret_cast<const float *>(base) + (size_t)sg * (dim + 4) + kc * L::KC;
                 const int kw = min(L::KC, dim - kc * L::KC);   // a multiple of 16
+#pragma unroll 1
                 for (int k0 = 0; k0 < kw; k0 += 16) {   // partial sums of 16 dims, as k_exit_cl
                     float t[SP][2];
 #pragma unroll
@@ -1422,6 +1477,7 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
     // tile whose product timed out sends z = -1: no decision)
     const bool failed = s_wfail != 0;
     const int l8 = lane & 7;
+#pragma unroll 1
     for (int k = tid >> 3; active && k < BT; k += kExitThreads / 8) {   // uniform per warp
         const float *l = lg_s + k * L::lg_stride + l8;
         float m = -INFINITY, zq[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -1441,6 +1497,7 @@ __global__ void __launch_bounds__(kExitThreads, 2) k_exit_rows(const __grid_cons
     cl.sync();   // every CTA holds every partial of the tile's samples
     // every CTA merges the partials in the same order; the owner writes the decision, every CTA its
     // logits tile of the samples that exit
+#pragma unroll 1
     for (int k = tid >> 3; active && k < BT; k += kExitThreads / 8) {
         const int sw = s0 + k;
         const float2 pz = l8 < ncl ? part_s[k * 8 + l8] : make_float2(-INFINITY, 0.0f);

@@ -71,6 +71,7 @@ __device__ void sim_argmax(const ImageParams &p, unsigned char *sm, size_t stage
     const int n_kchunk = (kdim + kc - 1) / kc;
     bool staged = false;
 
+#pragma unroll 1
     for (int pass = 0; pass < n_pass; ++pass) {
         float acc[kSPW][4][4];
 #pragma unroll
@@ -80,6 +81,7 @@ __device__ void sim_argmax(const ImageParams &p, unsigned char *sm, size_t stage
 #pragma unroll
                 for (int e = 0; e < 4; ++e) acc[a][q][e] = 0.0f;
 
+#pragma unroll 1
         for (int kci = 0; kci < n_kchunk; ++kci) {
             const int k0 = kci * kc;
             const int kw = min(kc, kdim - k0);
@@ -87,6 +89,7 @@ __device__ void sim_argmax(const ImageParams &p, unsigned char *sm, size_t stage
             if (!(p.resident && staged)) {
                 __syncthreads();   // previous readers of the staging area are done
                 const int total = (nA + nB) * nch;
+#pragma unroll 1
                 for (int it = tid; it < total; it += kImageThreads) {
                     const int tok = it / nch, c = it - tok * nch;
                     long long row;
@@ -107,12 +110,14 @@ __device__ void sim_argmax(const ImageParams &p, unsigned char *sm, size_t stage
                 staged = true;
                 if (pass == 0) {
                     // squared key norms, accumulated chunk by chunk (one warp per token)
+#pragma unroll 1
                     for (int tok = warp; tok < nA + nB; tok += kImageWarps) {
                         const bool isA = tok < nA;
                         const int tix = isA ? tok : tok - nA;
                         const unsigned char *base = isA ? regA : regB;
                         const int R = isA ? ra : rb;
                         float sq = 0.0f;
+#pragma unroll 1
                         for (int c = lane; c < nch; c += 32) {
                             float f[CH];
                             chunk_to_f(*reinterpret_cast<const uint4 *>(base + ((size_t)c * R + tix) * 16), f);
@@ -143,6 +148,7 @@ __device__ void sim_argmax(const ImageParams &p, unsigned char *sm, size_t stage
                 if constexpr (kBf16) {
                     const uint32_t baseA = smem_addr(regA), baseB = smem_addr(regB);
                     const int arow = mt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
+#pragma unroll 1
                     for (int kk = 0; kk < nch / 2; ++kk) {
                         uint32_t af[4];
                         const int achunk = 2 * kk + (lane >> 4);
@@ -168,6 +174,7 @@ __device__ void sim_argmax(const ImageParams &p, unsigned char *sm, size_t stage
                     }
                 } else {
                     const int r0 = mt * 16 + g;
+#pragma unroll 1
                     for (int c = 0; c < nch; ++c) {
                         const float4 a0 = *reinterpret_cast<const float4 *>(regA + ((size_t)c * ra + r0) * 16);
                         const float4 a1 = *reinterpret_cast<const float4 *>(regA + ((size_t)c * ra + r0 + 8) * 16);
@@ -205,6 +212,7 @@ __device__ void sim_argmax(const ImageParams &p, unsigned char *sm, size_t stage
 
         if (pass == 0) {
             __syncthreads();
+#pragma unroll 1
             for (int tok = tid; tok < nA + nB; tok += kImageThreads) {
                 float *ss = tok < nA ? ssA + tok : ssB + (tok - nA);
                 const float v = *ss;
@@ -276,7 +284,9 @@ __global__ void __launch_bounds__(kImageThreads, 1) k_image(ImageParams p) {
     const size_t stage_b = stage_a_bytes(stage_chunks, p.ra), stage = stage_total(stage_chunks, p.ra, p.rb);
     MetaPtrs m(sm, meta_layout(p.in.max_tokens, stage));
     meta_init<kImageThreads>(p, s, m);
+#pragma unroll 1
     for (int a = tid; a < s.nA; a += kImageThreads) m.inv_a[a] = 0.0f;
+#pragma unroll 1
     for (int n = tid; n < s.nB; n += kImageThreads) m.inv_b[n] = 0.0f;
     __syncthreads();
 

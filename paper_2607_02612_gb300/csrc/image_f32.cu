@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : TPW == 1 ? 1 : 2) k_merge_
     };
     // a pass begins with S stages in flight; every stage is one commit group, empty past the last
     auto start = [&] {
+#pragma unroll 1
         for (int q = 0; q < S; ++q) {
             if (q < n_stage) issue(q);
             else cp_async_commit();
@@ -112,6 +113,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : TPW == 1 ? 1 : 2) k_merge_
         float nlo[NP > 0 ? NP : 1], nhi[NP > 0 ? NP : 1];
 #pragma unroll
         for (int k = 0; k < (NP > 0 ? NP : 1); ++k) nlo[k] = nhi[k] = 0.0f;
+#pragma unroll 1
         for (int pass = 0; sim && pass < n_pass; ++pass) {
             if (pass > 0) start();
             float acc[TPW][2][4];
@@ -121,6 +123,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : TPW == 1 ? 1 : 2) k_merge_
                 for (int i = 0; i < 2; ++i)
 #pragma unroll
                     for (int e = 0; e < 4; ++e) acc[w][i][e] = 0.0f;
+#pragma unroll 1
             for (int q = 0; q < n_stage; ++q) {
                 wait_stage(S);
                 __syncthreads();
@@ -251,10 +254,12 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : TPW == 1 ? 1 : 2) k_merge_
                     else m.inv_b[row - na] = inv;
                 };
                 if constexpr (NP > 0) {
+#pragma unroll 1
                     for (int row = tid; row < rows; row += NT)   // after the last stage's barrier
                         put(row, row < na ? m.inv_a[a0 + row] : m.inv_b[row - na]);
                 } else {
                     // four rows at a time, so that their loads are in flight together
+#pragma unroll 1
                     for (int row0 = warp; row0 < rows; row0 += 4 * kW) {
                         const float4 *src[4];
                         float v[4];
@@ -265,6 +270,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : TPW == 1 ? 1 : 2) k_merge_
                                 keys + (long long)(s.start + (row < na ? 2 + 2 * tok : 1 + 2 * tok)) * kdim);
                             v[u] = 0.0f;
                         }
+#pragma unroll 1
                         for (int k0 = 0; k0 < kdim; k0 += p.kc) {
                             const int nch = min(p.kc, kdim - k0) / 4;
                             float sq[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -326,9 +332,11 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : TPW == 1 ? 1 : 2) k_merge_
             }
             __syncthreads();
             const int tile1 = min(tiles, tile0 + TPW * kW);
+#pragma unroll 1
             for (int a = tid; a < na; a += NT) {
                 const int t0 = (a >> 4) * NG;
                 unsigned long long o = m.best[a0 + a];
+#pragma unroll 1
                 for (int t = max(t0, tile0); t < min(t0 + NG, tile1); ++t) {
                     const unsigned long long b = tile_best[(t - tile0) * 16 + (a & 15)];
                     o = b > o ? b : o;
@@ -340,6 +348,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : TPW == 1 ? 1 : 2) k_merge_
         if (CL > 1) {   // this CTA's row maxima to the others
             cg::cluster_group cl = cg::this_cluster();
             cl.sync();   // every CTA has initialised its maxima
+#pragma unroll 1
             for (int t = tid; t < na * (CL - 1); t += NT) {
                 const int k = t / na, a = a0 + t - k * na;
                 *cl.map_shared_rank(m.best + a, k < rank ? k : k + 1) = m.best[a];

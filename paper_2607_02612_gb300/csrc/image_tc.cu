@@ -160,6 +160,7 @@ __device__ __forceinline__ void ring_start(const TcMaps &maps, const Ring &R, co
     __syncwarp();
     const int S0 = min(R.S, nkb);
     if (lane < S0) mbar_expect_tx(smem_addr(&bar_full[lane]), R.kbs);
+#pragma unroll 1
     for (int t = lane; t < S0 * R.per_kb; t += 32)
         issue_box(maps, R, g, start, nA, nB, sm, bar_full, t / R.per_kb, t % R.per_kb);
 }
@@ -177,6 +178,7 @@ __device__ __forceinline__ void group_start(const TcMaps &maps, const Ring &R, i
     if (lane == 0) mbar_expect_tx(smem_addr(&bar_full[0]), (uint32_t)(GA + GB) * gstride);
     const bool oddA = (start + 2) & 1, oddB = (start + 1) & 1;
     const int yA = (start + 2) >> 1, yB = (start + 1) >> 1;
+#pragma unroll 1
     for (int b = lane; b < GA + GB; b += 32) {
         const bool isB = b >= GA;
         const int q = isB ? b - GA : b;
@@ -189,11 +191,13 @@ __device__ __forceinline__ void group_start(const TcMaps &maps, const Ring &R, i
 // group; waited for in meta_init_rest).
 template <int NT>
 __device__ __forceinline__ void prefetch_own(const ImageParams &p, int start, int N, const MetaPtrs &m, uint4 *cls) {
+#pragma unroll 1
     for (int pos = threadIdx.x; pos < N; pos += NT) {
         cp_async4(&m.tsize[pos], p.sizes + start + pos);
         if (p.scores) cp_async4(&m.tscore[pos], p.scores + start + pos);
     }
     const uint4 *row = reinterpret_cast<const uint4 *>(reinterpret_cast<const __nv_bfloat16 *>(p.x) + (long long)start * p.dim);
+#pragma unroll 1
     for (int c = threadIdx.x; c < p.dim / 8; c += NT) cp_async16(&cls[c], row + c);
     cp_async_commit();
 }
@@ -255,6 +259,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
     unsigned char *regB = sm + (size_t)R.rowsA * 128;  // stage st, half B: regB + st * kbs (ring layout)
     auto produce = [&](int kb) {   // a whole K-block from one thread
         mbar_expect_tx(smem_addr(&bar_full[kb % S]), kbs);
+#pragma unroll 1
         for (int b = 0; b < R.per_kb; ++b) issue_box(maps, R, g, s.start, s.nA, s.nB, sm, bar_full, kb, b);
     };
 
@@ -295,6 +300,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
             } else if (warp == 1 && elect_one()) {
                 const uint32_t a0 = smem_addr(sm), b0 = smem_addr(gB);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
                 for (int kb = 0; kb < nkb; ++kb)
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
@@ -303,6 +309,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
                 umma_commit(smem_addr(&bar_done));
             }
         }
+#pragma unroll 1
         for (int kb = 0; kb < (grouped ? 0 : nkb); ++kb) {
             const int st = kb % S;
             const uint32_t par = (uint32_t)(kb / S) & 1u;
@@ -349,6 +356,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
                 const unsigned char *base = grouped ? (rA ? sm : gB) + (size_t)(rr >> 3) * gstride + (rr & 7) * 128
                                                     : (rA ? regA : regB) + (size_t)rr * 128;
                 const uint32_t kstep = grouped ? 1024u : kbs;   // bytes from one K-block of the row to the next
+#pragma unroll 1
                 for (int c = part; c < nkb * 8; c += kT)
                     neumaier_add(ss, sc, chunk_sq(*reinterpret_cast<const uint4 *>(
                                              base + (size_t)(c >> 3) * kstep + (((c & 7) ^ (rr & 7)) << 4))));
@@ -389,6 +397,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
             // so a strict comparison keeps the first of equal values (and -0 equals +0)
             float bv = -INFINITY;
             int bi = -1;
+#pragma unroll 1
             for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
                 uint32_t v[16];
                 tmem_ld16(lane_addr + (uint32_t)c0, v);
@@ -742,6 +751,7 @@ TcGeometry tiled_geometry(int max_tokens, int kdim) {
     // the largest stage and the furthest read from its start over all samples of at most max_tokens: with
     // one M-tile less a pass has more columns
     size_t per_stage = 0, reach = 0;
+#pragma unroll 1
     for (int nM = 1; nM <= (nAmax + 127) / 128; ++nM) {
         const int nblk = std::min(256, 512 / nM & ~15);
         const size_t a = (size_t)ceil8(std::min(nAmax, nM * 128)) * 128;
@@ -865,6 +875,7 @@ cudaError_t launch_image_tc(const ImageParams &p, const TcGeometry &geometry, cu
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
+#pragma unroll 1
     for (int odd = 0; odd < 2 && g.grouped; ++odd) {   // (64 dims, row, K-block), box 8 rows x all K-blocks
         cuuint64_t dims[3] = {64, odd ? rows_odd : rows_even, (cuuint64_t)(p.kdim / 64)};
         cuuint64_t strides[2] = {(cuuint64_t)p.kdim * 2 * 2, 128};

@@ -91,6 +91,7 @@ __device__ inline void plan_scan(const PlanArgs &a, int B) {
     __syncthreads();
     const int tiles = B > 0 ? (B + a.pt - 1) / a.pt : 0;
     int base_s = 0, base_r = 0;
+#pragma unroll 1
     for (int t0 = 0; t0 < tiles; t0 += blockDim.x) {
         int4 v = make_int4(0, 0, 0, 0);
         if (t0 + t < tiles) v = __ldcg(a.agg + t0 + t);
@@ -110,6 +111,7 @@ __device__ inline void plan_scan(const PlanArgs &a, int B) {
         }
         __syncthreads();
         int ps = base_s, pr = base_r, ts = 0, tr = 0;
+#pragma unroll 1
         for (int k = 0; k < nw; ++k) {
             if (k < w) {
                 ps += wsum[0][k];
