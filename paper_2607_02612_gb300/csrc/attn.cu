@@ -27,7 +27,8 @@
 // tokens); two CTAs (four warpgroups) per SM hide each other's waits for the products.  The forms before
 // it, one CTA per (head, sample) with block-wide barriers between load, product, softmax and product,
 // idled in them, and samples past 256 tokens formed S twice (a pass for the maximum).  256 samples of
-// 100 to 197 tokens x 6 heads: 62 -> 43 us; 128 of 577 x 16 heads: 769 -> 317 us (0.55 PFLOP/s).
+// 100 to 197 tokens x 6 heads: 62 -> 43 us; 128 of 577 x 16 heads: 769 -> 307 us (0.57 PFLOP/s; 317 with
+// the loops over key blocks and rows unrolled by the compiler).
 // Measured and not taken: halves of 32 keys with two S buffers (495 us at 577 tokens: twice the barriers),
 // a first pass for the maximum with two S buffers (440), the shift allowed to lag by 2^8 (309).
 //
@@ -192,8 +193,11 @@ __global__ void __launch_bounds__(NWG * 160, NWG == 2 ? 2 : 3)
         mbar_expect_tx(smem_addr(b), (uint32_t)cnt * 128u);
         if (cnt == 128) return tma_load_2d(smem_addr(dst), &maps.b128, x, y0, smem_addr(b));
         int r = 0;
+#pragma unroll 1
         for (; r + 64 <= cnt; r += 64) tma_load_2d(smem_addr(dst + r * 128), &maps.b64, x, y0 + r, smem_addr(b));
+#pragma unroll 1
         for (; r + 32 <= cnt; r += 32) tma_load_2d(smem_addr(dst + r * 128), &maps.b32, x, y0 + r, smem_addr(b));
+#pragma unroll 1
         for (; r < cnt; r += 8) tma_load_2d(smem_addr(dst + r * 128), &maps.b8, x, y0 + r, smem_addr(b));
     };
     auto block_rows = [&](int j) { return (min(kKeyBlock, n_u - j * kKeyBlock) + 7) & ~7; };
@@ -220,8 +224,10 @@ __global__ void __launch_bounds__(NWG * 160, NWG == 2 ? 2 : 3)
     if (warp == NWG * 4) {   // the first blocks at once (the second issuing warp allocates meanwhile)
         const int n0 = min((n_u + kKeyBlock - 1) / kKeyBlock, ns);
         if (elect_one()) {
+#pragma unroll 1
             for (int j = 0; j < n0; ++j) {
                 load_k(j, j);
+#pragma unroll 1
                 for (int w = 0; j == 0 && w < nw; ++w) load_q(w);
                 load_v(j, j);
             }
@@ -236,6 +242,7 @@ __global__ void __launch_bounds__(NWG * 160, NWG == 2 ? 2 : 3)
     }
     if (warp < NWG * 4) {   // log2 of the key sizes meanwhile, four loads of a thread in flight
         float lmax = -INFINITY, lmin = INFINITY;
+#pragma unroll 1
         for (int j0 = tid; j0 < nb * kKeyBlock; j0 += NWG * 512) {
             float sz[4];
 #pragma unroll
@@ -289,6 +296,7 @@ __global__ void __launch_bounds__(NWG * 160, NWG == 2 ? 2 : 3)
         bool ok = warp_wait(smem_addr(&bar.q[w]), 0);
         RingPos kp, vp, rf;   // stages of block j + 1's K, of block j's V, and of the block to refill next
         int next = min(nb_u, ns);
+#pragma unroll 1
         for (int j = -1; ok && j < nb_u; ++j) {
             const int cnt = min(kKeyBlock, n_u - j * kKeyBlock), np = (cnt + 15) & ~15;
             if (j >= 0) {
@@ -296,6 +304,7 @@ __global__ void __launch_bounds__(NWG * 160, NWG == 2 ? 2 : 3)
                 if (ok && cnt < np) {
                     // V rows past the sample (another sample's rows or stale memory) read as zero in P V (both
                     // tiles' warps write these zeros)
+#pragma unroll 1
                     for (int c = lane; c < (np - cnt) * 8; c += 32)
                         reinterpret_cast<uint4 *>(Vr + vp.st * kKeyBytes + (size_t)cnt * 128)[c] = make_uint4(0u, 0u, 0u, 0u);
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
@@ -349,6 +358,7 @@ __global__ void __launch_bounds__(NWG * 160, NWG == 2 ? 2 : 3)
         float m = 0.0f, mraw = -INFINITY;        // the shift; the largest S so far
         float2 lsum = make_float2(0.0f, 0.0f);   // even and odd keys
         bool ok = true;
+#pragma unroll 1
         for (int j = 0; ok && j < nb; ++j) {
             ok = warp_wait(smem_addr(&bar.s[w]), (uint32_t)j & 1u);   // S of block j, and O up to the block before
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -441,10 +451,12 @@ __global__ void __launch_bounds__(NWG * 160, NWG == 2 ? 2 : 3)
     if (s_fail != 0 && warp == NWG * 4) {   // let everything this CTA started finish before it leaves
         if (lane == 0) {
             raise_status(p.status, FUSION_DEV_TIMEOUT);
+#pragma unroll 1
             for (int j = max(0, s_kv - ns); j < s_kv; ++j) {
                 (void)mbar_wait(smem_addr(&bar.k[j % ns]), (uint32_t)(j / ns) & 1u);
                 (void)mbar_wait(smem_addr(&bar.v[j % ns]), (uint32_t)(j / ns) & 1u);
             }
+#pragma unroll 1
             for (int w = 0; w < nw; ++w) (void)mbar_wait(smem_addr(&bar.q[w]), 0);
         }
         __syncwarp();
