@@ -173,9 +173,11 @@ int fusion_set_launch_gate(const int32_t *flag, int64_t polls);
  * Bytes of scratch device memory every call needs for a batch bound of
  * max_batch samples and an exit head of `classes` classes (pass the largest
  * head used with this workspace; 1 when no exit check is run).  The workspace
- * must be zero-filled before its first use; every call leaves it zero-filled
- * again when its kernels complete, so it can be reused on the same stream
- * without clearing.  Calls that overlap on the device must not share one.
+ * must be zero-filled before its first use.  What must be zero when a call begins are the
+ * counters at its start (the first 256 KB, whatever the bounds), and every call leaves them zero
+ * when its kernels complete; the rest holds whatever the last call left there.  So it can be reused
+ * on the same stream without clearing, by calls of any bounds that it is large enough for.  Calls that
+ * overlap on the device must not share one.
  */
 size_t fusion_workspace_size(int32_t max_batch, int32_t classes);
 
@@ -225,8 +227,8 @@ int fusion_exit_check(int dtype, fusion_ragged in, const void *x, int32_t dim,
 
 /*
  * Scratch bytes of fusion_exit_check_mlp for max_batch samples, token width dim and
- * the head's hidden width and classes; zero-filled before its first use, left
- * zero-filled by every call (as fusion_workspace_size).
+ * the head's hidden width and classes; zero-filled before its first use, reusable without
+ * clearing (as fusion_workspace_size).
  */
 size_t fusion_exit_mlp_workspace_size(int32_t max_batch, int32_t dim, int32_t hidden, int32_t classes);
 
@@ -259,8 +261,8 @@ int fusion_exit_check_mlp(int dtype, fusion_ragged in, const void *x, int32_t di
  * an allocation would stall).  This call takes the same inputs and outputs as
  * fusion_exit_check but no workspace: its scratch lives in a 1 MiB device array
  * inside the library, present on every GPU that loads the library until the
- * process exits.  A batch bound and class count whose scratch exceeds 1 MiB (see
- * fusion_workspace_size) is rejected with FUSION_ERR_WORKSPACE before anything is
+ * process exits.  A batch bound and class count whose scratch (that of
+ * fusion_workspace_size, with only this call's counters) exceeds 1 MiB is rejected with FUSION_ERR_WORKSPACE before anything is
  * enqueued.  Every call looks up the array's device address in the current context
  * (a host-side query); the first call on a device may load the library's device code
  * there, so make that first call before any stream capture.  Calls allocate nothing
@@ -405,7 +407,8 @@ int fusion_stage(int dtype, int flags, fusion_ragged in, const void *x, int32_t 
  * Bytes of scratch of fusion_stage_mlp with both FUSION_STAGE_MERGE and FUSION_STAGE_EXIT:
  * the MLP head's scratch (fusion_exit_mlp_workspace_size) and room for the merged batch
  * (max_rows token rows of dim elements at 4 bytes each, their sizes, scores and input rows,
- * and max_batch + 1 offsets).  Zero-filled before its first use, left zero-filled by every call.
+ * and max_batch + 1 offsets).  Zero-filled before its first use, reusable without clearing (as
+ * fusion_workspace_size).
  */
 size_t fusion_stage_mlp_workspace_size(int32_t max_batch, int64_t max_rows, int32_t dim, int32_t hidden,
                                        int32_t classes);
@@ -421,7 +424,7 @@ size_t fusion_stage_mlp_workspace_size(int32_t max_batch, int64_t max_rows, int3
  * in.max_batch, in.max_rows, dim, head.hidden, head.classes) bytes with both merging and the
  * exit check, fusion_exit_mlp_workspace_size(in.max_batch, dim, head.hidden, head.classes)
  * with the exit check alone, else fusion_workspace_size(in.max_batch, 1); zero-filled before
- * first use and left so.
+ * its first use.
  * Errors: those of fusion_stage and fusion_exit_check_mlp.
  */
 int fusion_stage_mlp(int dtype, int flags, fusion_ragged in, const void *x, int32_t dim,

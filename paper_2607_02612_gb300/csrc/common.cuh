@@ -42,16 +42,20 @@ constexpr int kImageThreads = 512;
 constexpr int kImageWarps = kImageThreads / 32;
 
 // Workspace layout (bytes from the workspace base; every block 256-aligned).
-// The plan's counts and the plan come first, so their offsets depend on max_batch
-// only; the exit counters and partial softmax sums follow, then the logits tiles of
+// The counters that must be zero when a call begins come first, in a block whose size depends on
+// nothing: calls of other batch bounds and class counts on the same workspace put their data behind it,
+// wherever their bounds place it, so no call finds another's leftovers in a counter.  The plan's counts
+// and the plan follow, then the partial softmax sums and the logits tiles of
 // the general exit kernel (heads of more than kExitClMaxTiles class tiles only: its
 // CTAs cannot wait for one another, so the last CTA of a sample tile copies the rows
-// of the samples that exit from there).
+// of the samples that exit from there).  None of that needs to be zero.
 constexpr int kExitClMaxTiles = 8;   // class tiles of the cluster exit kernel (portable cluster size)
+// The plan's counter, then one per sample tile of the general exit kernel, whose grid has at most 65535.
+constexpr int kWsCounters = 1 << 16;
 struct WsLayout {
+    size_t counters;   // int[kWsCounters], zero between calls
     size_t slot;       // int[max_batch]: output rows of every input sample (the plan's counts)
     size_t plan;       // int[4]: batch valid, survivor count
-    size_t counters;   // int[n_btile + 1], zero between calls
     size_t partials;   // float2[n_btile * kExitBT * n_ctile]; after the exit check the plan's tile totals
     size_t lg;         // float[n_btile * kExitBT][classes] (empty for heads of <= kExitClMaxTiles tiles)
     size_t total;
@@ -65,12 +69,12 @@ __host__ __device__ inline WsLayout ws_layout(int max_batch, int classes) {
     const int nbt = ceil_div(max_batch > 0 ? max_batch : 1, kExitBT);
     const int nct = ceil_div(classes > 0 ? classes : 1, kExitCT);
     size_t off = 0;
+    L.counters = off;
+    off += align256(sizeof(int) * (size_t)kWsCounters);
     L.slot = off;
     off += align256(sizeof(int) * (size_t)(max_batch > 0 ? max_batch : 1));
     L.plan = off;
     off += align256(sizeof(int) * 4);
-    L.counters = off;
-    off += align256(sizeof(int) * (size_t)(nbt + 1));
     L.partials = off;
     off += align256(sizeof(float) * 2 * (size_t)nbt * kExitBT * (size_t)nct);
     L.lg = off;

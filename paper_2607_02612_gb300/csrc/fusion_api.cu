@@ -58,7 +58,7 @@ Head dev(const fusion_exit_head &h) {
 struct Ws {
     int *cnt;
     int *plan;
-    int *counters;
+    int *plan_counter, *counters;   // zero between calls
     float2 *partials;
     float *lg;   // logits tiles of the general exit kernel (NULL for heads it does not run)
 };
@@ -67,16 +67,16 @@ Ws carve(void *ws, int32_t max_batch, int32_t classes) {
     const WsLayout L = ws_layout(max_batch, classes);
     unsigned char *b = static_cast<unsigned char *>(ws);
     return Ws{reinterpret_cast<int *>(b + L.slot), reinterpret_cast<int *>(b + L.plan),
-              reinterpret_cast<int *>(b + L.counters), reinterpret_cast<float2 *>(b + L.partials),
+              reinterpret_cast<int *>(b + L.counters), reinterpret_cast<int *>(b + L.counters) + 1, reinterpret_cast<float2 *>(b + L.partials),
               L.total > L.lg ? reinterpret_cast<float *>(b + L.lg) : nullptr};
 }
 
 // The plan's scratch for batches above the fused plan's bound.
-void plan_scratch(PlanArgs &pa, const Ws &w, int32_t max_batch) {
+void plan_scratch(PlanArgs &pa, const Ws &w) {
     pa.cnt = w.cnt;
     pa.plan = w.plan;
     pa.agg = reinterpret_cast<int4 *>(w.partials);
-    pa.counter = w.counters + ceil_div(max_batch > 0 ? max_batch : 1, kExitBT);
+    pa.counter = w.plan_counter;
     pa.pt = kPlanTile;
 }
 
@@ -243,7 +243,7 @@ int fusion_merge(int dtype, fusion_ragged in, const void *x, int32_t dim, const 
     pa.merge = 1;
     pa.r = r;
     pa.offsets_out = offsets_out;
-    plan_scratch(pa, w, in.max_batch);
+    plan_scratch(pa, w);
     pa.status = dev_status;
     record(ev.start, s);
     if (!fuse_plan(in)) FZ_TRY(cuda_rc(launch_plan(pa, s)));
@@ -310,7 +310,7 @@ int fusion_prune(int dtype, fusion_ragged in, const void *x, int32_t dim, const 
     pa.prune = 1;
     pa.rho = rho;
     pa.offsets_out = offsets_out;
-    plan_scratch(pa, w, in.max_batch);
+    plan_scratch(pa, w);
     pa.status = dev_status;
     const ProfileEvents ev = take_profile();
     record(ev.start, s);
@@ -348,7 +348,7 @@ int fusion_compact(int dtype, fusion_ragged in, const void *x, int32_t dim, cons
     pa.offsets_out = offsets_out;
     pa.ids_out = ids_out;
     pa.batch_out = batch_out;
-    plan_scratch(pa, w, in.max_batch);
+    plan_scratch(pa, w);
     pa.status = dev_status;
     const ProfileEvents ev = take_profile();
     record(ev.start, s);
@@ -646,7 +646,7 @@ int stage_impl(int dtype, int flags, const fusion_ragged &in, const void *x, int
     pa.offsets_out = offsets_out;
     pa.ids_out = ids_out;
     pa.batch_out = batch_out;
-    plan_scratch(pa, w, in.max_batch);
+    plan_scratch(pa, w);
     pa.status = dev_status;
     if (do_exit && mlp && do_merge) {
         // The MLP head reads the merged tokens (Sec. III-B): merge into the workspace, the exit

@@ -17,7 +17,7 @@ struct ExitParams {
     uint8_t *exit_mask;
     float *logits;
     float *max_prob;
-    int *counters;   // workspace: [n_btile + 1], zero on entry, zero on exit
+    int *counters;   // workspace: [n_btile], zero on entry, zero on exit
     float2 *partials;
     float *lg_tmp;   // workspace [n_btile * kExitBT][classes]: logits tiles of the general kernel (its
                      // last CTA per sample tile writes the rows of the samples that exit); NULL when

@@ -53,8 +53,12 @@ extern "C" int fusion_exit_check_noalloc(int dtype, fusion_ragged in, const void
     if (!aligned16(head.ln_gamma) || !aligned16(head.ln_beta) || !aligned16(head.weight))
         return FUSION_ERR_INVALID_ARG;
     if (head.classes < 1) return FUSION_ERR_SHAPE;
+    // the workspace's data, then the counters of this call's tiles (cleared below, so they need no fixed place)
     const WsLayout L = ws_layout(in.max_batch, head.classes);
-    if (L.total > kNoAllocScratchBytes) return FUSION_ERR_WORKSPACE;
+    const size_t counters = L.total - L.slot;
+    const int n_btile = ceil_div(in.max_batch > 0 ? in.max_batch : 1, kExitBT);
+    const size_t counter_bytes = sizeof(int) * ((size_t)n_btile + 1);
+    if (counters + align256(counter_bytes) > kNoAllocScratchBytes) return FUSION_ERR_WORKSPACE;
 
     unsigned char *base = nullptr;
     const int rc = scratch_on_current_device(&base);
@@ -69,15 +73,15 @@ extern "C" int fusion_exit_check_noalloc(int dtype, fusion_ragged in, const void
     e.exit_mask = exit_mask;
     e.logits = logits;
     e.max_prob = max_prob;
-    e.counters = reinterpret_cast<int *>(base + L.counters);
-    e.partials = reinterpret_cast<float2 *>(base + L.partials);
-    e.lg_tmp = (logits && L.total > L.lg) ? reinterpret_cast<float *>(base + L.lg) : nullptr;
+    e.counters = reinterpret_cast<int *>(base + counters);
+    e.partials = reinterpret_cast<float2 *>(base + (L.partials - L.slot));
+    e.lg_tmp = (logits && L.total > L.lg) ? reinterpret_cast<float *>(base + (L.lg - L.slot)) : nullptr;
     e.n_ctile = ceil_div(head.classes, kExitCT);
-    e.n_btile = ceil_div(in.max_batch > 0 ? in.max_batch : 1, kExitBT);
+    e.n_btile = n_btile;
     e.do_plan = 0;
     e.status = dev_status;
     // the completion counters must start at zero; everything else is written before it is read
-    if (cudaMemsetAsync(e.counters, 0, sizeof(int) * (size_t)(e.n_btile + 1), s) != cudaSuccess)
+    if (cudaMemsetAsync(e.counters, 0, counter_bytes, s) != cudaSuccess)
         return FUSION_ERR_CUDA;
     return launch_exit(dtype, e, s) == cudaSuccess ? FUSION_OK : FUSION_ERR_CUDA;
 }
