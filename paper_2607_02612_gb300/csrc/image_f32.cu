@@ -392,16 +392,49 @@ constexpr int kSmallTokens = 65;   // four 16 x 16 tiles: four warps, one tile e
 F32Geometry image_f32_geometry(const ImageParams &p) {
     F32Geometry g{};
     const int nA = (p.in.max_tokens - 1) / 2, nB = p.in.max_tokens / 2;
-    const bool small = p.in.max_tokens <= kSmallTokens;
-    const int strips = ceil_div(nA > 0 ? nA : 1, 16);
-    // the most CTAs per sample (portable cluster sizes) that one wave of two CTAs per SM holds, while
-    // every CTA has a strip; a gate may stop a single CTA, which a cluster cannot
-    g.cluster = 1;
-    while (!p.gate && g.cluster < 8 && g.cluster * 2 <= strips + 1 &&
-           (long long)p.in.max_batch * g.cluster * 2 <= 2 * 152)
-        g.cluster *= 2;
+    const int N = p.in.max_tokens, B = p.in.max_batch;
+    const bool small = N <= kSmallTokens;
+    const int strips = ceil_div(nA > 0 ? nA : 1, 16), cols = ceil_div(nB > 0 ? nB : 1, 16);
+    // CTAs per sample (portable cluster sizes), each with a strip at least; a gate may stop a single CTA, which a
+    // cluster cannot.  A cluster lies in one GPC: 15 clusters of 8, 36 of 4 or 76 of 2 have an SM per CTA at once,
+    // twice as many share SMs (cudaOccupancyMaxActiveClusters), and one more begins a second wave (76 samples of
+    // 100 tokens, d = 384, in clusters of 4 82 us, of 2 50).
+    auto fits = [&](int cl, int most) { return !p.gate && cl <= strips + 1 && B <= most; };
+    // With an SM each they are the fastest form measured, except that pairs have half of the general kernel's
+    // threads per SM for the decisions, which long samples with narrow keys spend their time on (76 samples of 300
+    // tokens, d = 48: 64 us, general kernel 51).
+    const bool narrow = p.kdim < 192, one_tile = N <= kSmallTokens + 1;
+    // Two per SM gain less: where the similarity is nearly all of the time (60 samples of 197 tokens, d = 192:
+    // clusters of 4 59 us, of 2 68; 100 tokens 48 and 36; past 600 tokens the stages are 16 dims: 700 tokens, d =
+    // 384, 627 and 502), in pairs where a pass's 64 tiles are three quarters used (100 samples, d = 384: 577 tokens
+    // 566 us, general kernel 620; 257 tokens 141 and 126) ...
+    const int pair_tiles = ceil_div(strips, 2) * cols;
+    const bool full = 4 * pair_tiles >= 3 * 64 * ceil_div(pair_tiles, 64);
+    const bool four = N > 150 && N <= 600, two = four && !narrow && full;
+    // ... and in a call with an exit check, whose samples that leave free the SMs (half of the batch continuing:
+    // 20 samples of 197 tokens, d = 384, clusters of 8 52 us, of 4 77; 100 of 100 tokens pairs 51 us, general kernel
+    // 62; everyone continuing 73 and 60 of the 77 that the call took before either), up to where the whole batch
+    // would be slower than the general kernel and the exit check before were.
+    const bool exits = p.plan_args.exit_mask != nullptr;
+    const bool exit8 = exits && !(narrow && N > 150), exit4 = exits && !(narrow && N > 600);
+    const bool exit2 = exits && !one_tile && N <= 600 && (N <= 129 ? p.kdim < 768 : N <= 197 || (!narrow && full));
+    g.cluster = fits(8, exit8 ? 30 : 15) ? 8
+                : fits(4, four || exit4 ? 72 : 36) ? 4
+                : fits(2, two || exit2 ? 152 : narrow && N > 150 ? 0 : 76) ? 2
+                : 1;
+    // One CTA per sample with more than eight tiles: 256 threads against the general kernel's 512, but two CTAs
+    // per SM where that has one.  In a wave of at most 152 samples each CTA is alone and slower (300 tokens,
+    // d = 384: 354 us, general kernel 203); between 153 and 304 it needs one wave instead of two (197 tokens,
+    // d = 384, 200 samples: 180 us, general kernel 202), from 305 to 456 two against three (340 samples 333,
+    // 289); past that the waves even out (608 samples of 100 tokens, d = 384: 159, 175) until the long samples'
+    // decisions take over (257 tokens, d = 192, half of 608 continuing: 215, 191).  How many continue is known here
+    // only without an exit check and without a device count; else 153 to 456 samples may leave one wave, which
+    // costs nothing up to 80 tokens and d = 384 (100 of 200 samples: 73 us, at the start's general kernel 72).
+    const bool known = !p.in.batch && !p.plan_args.exit_mask;
+    const bool few_waves = (known && B <= 2 * 152) || (N <= 80 && p.kdim <= 384);
+    if (g.cluster == 1 && !one_tile && !(N <= 197 && B > 152 && (B > 3 * 152 || few_waves))) return g;
     g.rows_a = ceil_div(strips, g.cluster) * 16;
-    g.rows_b = ceil_div(nB > 0 ? nB : 1, 16) * 16;
+    g.rows_b = cols * 16;
     auto need = [&](int kd, int S) {
         return meta_layout(p.in.max_tokens, (size_t)S * (g.rows_a + g.rows_b) * stage_row(kd)).total;
     };
@@ -409,7 +442,7 @@ F32Geometry image_f32_geometry(const ImageParams &p) {
     // two CTAs per SM where 16 dims allow it; a batch that leaves SMs idle has each to itself, and more
     // stages (a loop of six 64-dim stages took 12.4 of the kernel's 30 us with two in flight, most of it the
     // wait for them)
-    const bool alone = (long long)p.in.max_batch * g.cluster <= 152;
+    const bool alone = B <= (g.cluster == 4 ? 36 : 152 / g.cluster);
     const size_t most = 224 * 1024;
     for (size_t budget : {alone ? most : (size_t)110 * 1024, most})
         for (int kd = 64; kd >= 16; kd /= 2) {
