@@ -759,12 +759,14 @@ TcGeometry tiled_geometry(int max_tokens, int kdim) {
         reach = std::max({reach, (size_t)nM * 16384, a + (size_t)std::min(nblk, npad_max) * 128});
     }
     // one CTA per SM: all of its shared memory, the metadata at the end; at least two stages (shorter
-    // samples of the call have more, from their own sizes)
+    // samples of the call have more, from their own sizes): up to 962 tokens (64 samples of 960 tokens, d =
+    // 384: 140 us, on the general kernel 699).  The stages end where the metadata begin: copies write whole
+    // stages, and what a product reads past them feeds only unused rows and columns.
     const size_t usable = (227 * 1024 - 6144 - 1024) / 1024 * 1024;   // static shared memory, alignment
     const size_t meta = meta_layout(max_tokens, 0).total;
-    if (2 * per_stage + 2048 + meta > usable || per_stage + reach > usable) return TcGeometry{};
+    if (2 * per_stage + meta > usable || per_stage + reach > usable) return TcGeometry{};
     g.meta_base = (uint32_t)((usable - meta) / 16 * 16);
-    g.stage_region = g.meta_base - 2048;
+    g.stage_region = g.meta_base;
     g.stages = (int)(g.stage_region / per_stage);
     g.usable = (uint32_t)usable;
     g.smem = g.usable + 1024;

@@ -159,7 +159,8 @@ def test_bf16_merge_small_ctas(counts, dim, keys, kdim):
     ([513, 514, 512, 258], 64),              # two M-tiles of 128 rows exactly, one row over, three
     ([577, 640, 641, 130], 192),             # three M-tiles: passes of 160 columns, the last ones ragged
     ([769, 770, 771, 300], 64),              # four M-tiles: passes of 128
-    ([900, 860], 128), ([1024, 3], 64)])     # the longest samples, and those the general kernel takes
+    ([900, 860], 128), ([1024, 3], 64),      # the longest samples, and those the general kernel takes
+    ([962, 947, 3, 300], 320)])              # two stages next to the metadata, refilled in turn
 def test_bf16_merge_long_samples(counts, dim):
     b = make_batch(counts, dim, "bf16", seed=len(counts), sizes="u1to4")
     rng = np.random.default_rng(3)

@@ -78,3 +78,10 @@ def test_float32_merges_leave_the_general_kernel_only_where_measured_faster(rout
     got = routes([("F", *q) for q in expected])
     for (q, want), (ok, cluster) in zip(expected.items(), got):
         assert (cluster if ok else 0) == want, q
+
+
+def test_long_bf16_merges_stay_on_the_tensor_cores(routes):
+    """Every length past one tile up to 962 tokens (two stages and the metadata fill an SM's shared memory)."""
+    lengths = range(258, 963)
+    for n, (ok, tiled, _) in zip(lengths, routes([("T", n, 384, 64, 0) for n in lengths])):
+        assert ok and tiled, n
