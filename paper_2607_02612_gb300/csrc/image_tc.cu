@@ -796,8 +796,14 @@ TcGeometry image_tc_geometry(int dtype, int max_tokens, int kdim, int dim, long 
     // four K-block stages, as many per SM as fit (the samples' chains of latencies overlap; a sample that does
     // not stay in shared memory is gathered from L2).  8192 samples of 9 to 65 tokens, d = 384, four stages
     // that keep 40 % each, per-sample kernels 452 -> 318 us; at 304 samples a CTA of 256 threads finishes its
-    // sample sooner and every sample has one at once.
-    if (max_batch > 2 * kSms && max_tokens <= 129) {
+    // sample sooner and every sample has one at once.  Where a sample's rows pass 68 KB, the few
+    // samples past 304 may start as short ones end (305 samples of 2 to 65 tokens, d = 1024, merged: 256 threads 42
+    // us, 128 46; 340 of them 53, 47; 305 of 2 to 33 tokens 33, 35).  Three CTAs per SM (100 tokens from d = 384)
+    // do not halve the waves: they serve one wave of their own, up to 456 samples, and, with narrower rows, the
+    // batches with a plan kernel (100 tokens, d = 384, merged, 256 / 128 threads: 400 samples 48 / 36 us, 500 52 /
+    // 58, 608 54 / 62, 1100 93 / 87; d = 768: 500 samples 72 / 96).
+    constexpr int kWave = 2 * kSms;
+    if (max_batch > kWave && max_tokens <= 129) {
         auto small = [&](int S) {
             const size_t meta_base = (size_t)S * per_stage;
             return std::max(meta_layout(max_tokens, meta_base).total + (size_t)dim * 2, (size_t)(S - 1) * per_stage + reach);
@@ -806,6 +812,10 @@ TcGeometry image_tc_geometry(int dtype, int max_tokens, int kdim, int dim, long 
         for (int per_sm = 4; per_sm >= 3; --per_sm) {
             // 228 KB per SM, 1 KB of it reserved per CTA, 1 KB of alignment slack and the static arrays
             if (small(S) + 1024 + 1536 + 1024 > (size_t)228 * 1024 / per_sm) continue;
+            const bool past_wave = max_batch > kWave + kWave / 16;
+            if (per_sm == 4 ? 2 * dim * max_tokens > 68 * 1024 && !past_wave
+                            : !past_wave || (max_batch > 3 * kSms && (max_batch <= kFusedPlanMaxBatch || dim > 384)))
+                break;
             g.threads = 128;
             g.stages = S;
             g.stage_region = (uint32_t)(S * per_stage);

@@ -85,3 +85,16 @@ def test_long_bf16_merges_stay_on_the_tensor_cores(routes):
     lengths = range(258, 963)
     for n, (ok, tiled, _) in zip(lengths, routes([("T", n, 384, 64, 0) for n in lengths])):
         assert ok and tiled, n
+
+
+def test_small_bf16_ctas_only_where_measured_faster(routes):
+    """Threads of a CTA over (tokens, width, batch bound): four CTAs per SM, three, or too much shared memory."""
+    expected = {
+        (65, 384, 304): 256, (65, 384, 305): 128, (100, 192, 305): 128, (65, 768, 323): 256, (65, 768, 324): 128,
+        (33, 1024, 305): 128, (17, 1024, 8192): 128,
+        (100, 384, 323): 256, (100, 384, 324): 128, (100, 384, 456): 128, (100, 384, 457): 256, (100, 384, 1024): 256,
+        (100, 384, 1025): 128, (100, 768, 456): 128, (100, 768, 1025): 256, (129, 192, 500): 256, (129, 192, 2500): 128,
+        (129, 64, 500): 128, (129, 384, 2500): 256, (130, 64, 2500): 256, (197, 384, 2500): 256,
+    }
+    for (q, want), (ok, _, threads) in zip(expected.items(), routes([("T", *q, 0) for q in expected])):
+        assert ok and threads == want, q
