@@ -355,7 +355,9 @@ __global__ void __launch_bounds__(NWG * 160, NWG == 2 ? 2 : 3)
         }
         const bool sized = lszmax != 0.0f || lszmin != 0.0f;
         constexpr float kScale2 = 0.18033688011112042f;   // log2(e) / sqrt(64)
-        float m = 0.0f, mraw = -INFINITY;        // the shift; the largest S so far
+        // the shift; the largest S so far, at least the lowest finite value: a row whose first blocks are -inf
+        // (infinite inputs, an overflowing product) has probabilities of zero there, not of -inf - (-inf)
+        float m = 0.0f, mraw = -3.402823466e38f;
         float2 lsum = make_float2(0.0f, 0.0f);   // even and odd keys
         bool ok = true;
 #pragma unroll 1

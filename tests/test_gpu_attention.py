@@ -118,6 +118,19 @@ def test_attention_vit_l_shapes():
     assert st == 0
 
 
+@pytest.mark.parametrize("n,low", [(65, 0), (130, 0), (130, 1), (200, 1), (577, 0), (577, 4)])
+def test_attention_blocks_of_minus_infinity(n, low):
+    """The logits of one block of 64 keys are below every float (the dot product -1.2e39 overflows to -inf): its keys
+    have probability 0, wherever the block lies, also where it is the first one that a row meets."""
+    offsets, qkv, sz = _case([n], 2, 67)
+    f = bf16_bits_to_f32(qkv)
+    for h in range(2):
+        f[:, h * DH] = -4.0                                      # dim 0 of every query
+        f[64 * low:64 * (low + 1), (2 + h) * DH] = 3e38          # and of the block's keys
+    st = _check(offsets, f32_to_bf16_bits(f), 2, sz, f"-inf block {low} of {n}")
+    assert st == 0
+
+
 def test_attention_malformed():
     offsets, qkv, sz = _case([10, 20, 30], 2, 64)
     bad = offsets.copy()
