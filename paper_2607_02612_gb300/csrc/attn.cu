@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(NWG * 160, NWG == 2 ? 2 : 3)
                 lsz[j] = l;
                 if (j < n) {
                     lmax = fmaxf(lmax, l);
-                    lmin = fminf(lmin, l);
+                    lmin = fminf(lmin, l == l ? l : -1.0f);   // (a NaN is a size too: not ignored as the minimum would)
                 }
             }
         }

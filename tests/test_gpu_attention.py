@@ -131,6 +131,18 @@ def test_attention_blocks_of_minus_infinity(n, low):
     assert st == 0
 
 
+def test_attention_nan_size_shows():
+    """A token size that is not a number reaches every row of its sample, whatever the other sizes are, and no row of
+    another sample."""
+    offsets, qkv, _ = _case([70, 33], 2, 68)
+    for other in (1.0, 2.0):
+        sz = np.full(103, other, np.float32)
+        sz[66] = np.nan
+        g, st = _run(offsets, qkv, 2, sz)
+        f = bf16_bits_to_f32(g)
+        assert st == 0 and np.isnan(f[:70]).all() and np.isfinite(f[70:]).all(), other
+
+
 def test_attention_malformed():
     offsets, qkv, sz = _case([10, 20, 30], 2, 64)
     bad = offsets.copy()
