@@ -463,8 +463,9 @@ __global__ void __launch_bounds__(NWG * 160, NWG == 2 ? 2 : 3)
         }
         __syncwarp();
     }
-    if (s_fail != 0) {   // uniform: each issuing thread drains its own products
-        if (warp >= NWG * 4 && warp - NWG * 4 < nw && lane == 0) {
+    if (s_fail != 0) {   // uniform: each issuing thread drains its own products (a commit covers only those, and
+                         // the election picks the same lane every time)
+        if (warp >= NWG * 4 && warp - NWG * 4 < nw && elect_one()) {
             umma_commit(smem_addr(&bar.drain[warp - NWG * 4]));
             (void)mbar_wait(smem_addr(&bar.drain[warp - NWG * 4]), 0);
         }

@@ -712,7 +712,7 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
                 for (int q = max(0, issued - S); q < issued; ++q)
                     (void)mbar_wait(smem_addr(&bar_full[q % S]), (uint32_t)(q / S) & 1u);
             }
-            if (tid == 32) {
+            if (warp == 1 && elect_one()) {   // the lane that issued the products: a commit covers only its own
                 umma_commit(smem_addr(&bar_drain));
                 (void)mbar_wait(smem_addr(&bar_drain), 0u);
             }
