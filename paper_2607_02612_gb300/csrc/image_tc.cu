@@ -144,11 +144,11 @@ __device__ __forceinline__ void issue_box(const TcMaps &maps, const Ring &R, con
 // warp has issued any.
 template <int NT>
 __device__ __forceinline__ void ring_barriers_init(unsigned long long *bar_full, unsigned long long *bar_empty,
-                                                   unsigned long long *bar_done) {
+                                                   unsigned long long *bar_done, unsigned long long *bar_drain) {
     const int lane = threadIdx.x & 31;
     static_assert(kMaxStages == 16, "a full and an empty barrier per lane pair");
     mbar_init(smem_addr(lane < 16 ? &bar_full[lane] : &bar_empty[lane - 16]), lane < 16 ? 1 : 1 + NT / 32);
-    if (lane == 0) mbar_init(smem_addr(bar_done), 1);
+    if (lane < 2) mbar_init(smem_addr(lane == 0 ? bar_done : bar_drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
     k_image_tc(const __grid_constant__ TcMaps maps, ImageParams p, TcGeometry g) {
     extern __shared__ unsigned char sm_raw[];
     unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ __align__(8) unsigned long long bar_full[kMaxStages], bar_empty[kMaxStages], bar_done;
+    __shared__ __align__(8) unsigned long long bar_full[kMaxStages], bar_empty[kMaxStages], bar_done, bar_drain;
     __shared__ uint32_t tmem_base;
     __shared__ int s_fail;
     __shared__ unsigned long long half_best[NT == 256 ? 128 : 1];
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
     }
     // the ring's barriers, before this warp issues any memory operation (warp 0 issues the
     // tokens' loads after a CTA barrier: the fused plan's, or the one below)
-    if (warp == 2) ring_barriers_init<NT>(bar_full, bar_empty, &bar_done);
+    if (warp == 2) ring_barriers_init<NT>(bar_full, bar_empty, &bar_done, &bar_drain);
     if (g.grouped && (tid == 38 || tid == 39))
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tid == 38 ? &maps.ge : &maps.go)) : "memory");
     if (tid == 0) s_fail = 0;   // visible after the barriers below, before any other write
@@ -293,11 +293,14 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
         const int row = isA ? tid : tid - splitA;
         const bool has_row = !resident && row < (isA ? s.nA : s.nB);
         float ss = 0.0f, sc = 0.0f;
+        // A lane whose wait gave up goes on through the loop without waiting, because the others meet it there (an
+        // election, a warp barrier); it only does nothing that needs what it waited for.  (A vote after every wait
+        // instead: long samples 136 -> 140 us, four stages of 8192 images 298 -> 302.)
         bool ok = true;
+        int issued = grouped ? 1 : min(S, nkb);   // stages whose copies were issued (the count of warp 0's elected lane)
         if (grouped) {   // everything behind one barrier; all products at once
-            if (!mbar_wait(smem_addr(&bar_full[0]), 0u)) {
-                ok = false;
-            } else if (warp == 1 && elect_one()) {
+            ok = mbar_wait(smem_addr(&bar_full[0]), 0u);
+            if (warp == 1 && elect_one() && ok) {
                 const uint32_t a0 = smem_addr(sm), b0 = smem_addr(gB);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
@@ -313,11 +316,8 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
         for (int kb = 0; kb < (grouped ? 0 : nkb); ++kb) {
             const int st = kb % S;
             const uint32_t par = (uint32_t)(kb / S) & 1u;
-            if (!mbar_wait(smem_addr(&bar_full[st]), par)) {
-                ok = false;
-                break;
-            }
-            if (warp == 1 && elect_one()) {
+            ok = ok && mbar_wait(smem_addr(&bar_full[st]), par);
+            if (warp == 1 && elect_one() && ok) {
                 const uint32_t a0 = smem_addr(regA + (size_t)st * kbs), b0 = smem_addr(regB + (size_t)st * kbs);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
@@ -335,9 +335,11 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_addr(&bar_empty[st]));
             if (warp == 0 && kb + S < nkb) {   // refill this stage once everyone is done with it
-                ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_addr(&bar_empty[st]), par));
-                if (!ok) break;
-                if (elect_one()) produce(kb + S);
+                ok = ok && mbar_wait(smem_addr(&bar_empty[st]), par);
+                if (elect_one() && ok) {
+                    produce(kb + S);
+                    ++issued;
+                }
                 __syncwarp();
             }
         }
@@ -425,7 +427,18 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : 2)
                 m.best[r] = bk;
             }
         } else {
-            if (tid == 0) raise_status(p.status, FUSION_DEV_TIMEOUT);
+            // a wait gave up: let the copies and products in flight land (bounded) before the
+            // shared and tensor memory are released
+            if (warp == 0 && elect_one()) {
+                raise_status(p.status, FUSION_DEV_TIMEOUT);
+#pragma unroll 1
+                for (int q = max(0, issued - S); q < issued; ++q)
+                    (void)mbar_wait(smem_addr(&bar_full[q % S]), (uint32_t)(q / S) & 1u);
+            }
+            if (warp == 1 && elect_one()) {   // the lane that issued the products: a commit covers only its own
+                umma_commit(smem_addr(&bar_drain));
+                (void)mbar_wait(smem_addr(&bar_drain), 0u);
+            }
         }
         __syncthreads();
         if (s_fail == 0) select_top_r<NT>(s, m);
@@ -503,7 +516,7 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
     }
     const bool dec = s.decide;
     const int nkb = g.n_kb;
-    int issued = 0;   // stages issued (thread 0's count; warp 0 issues the first ones)
+    int issued = 0;   // stages issued (the count of warp 0's elected lane; the warp issues the first ones)
     const int nM = max(1, (s.nA + 127) >> 7);       // M-tiles of half A
     const int rowsA = (s.nA + 7) & ~7;
     const int npad = (s.nB + 15) & ~15;             // columns of the product
@@ -601,12 +614,9 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
                 const int q = ps * nkb + kb;
                 const int st = q % S;
                 const uint32_t par = (uint32_t)(q / S) & 1u;
-                if (!mbar_wait(smem_addr(&bar_full[st]), par)) {
-                    ok = false;
-                    break;
-                }
+                ok = ok && mbar_wait(smem_addr(&bar_full[st]), par);   // (as in k_image_tc)
                 const unsigned char *stA = sm + (size_t)st * kbs, *stB = stA + aBytes;
-                if (warp == 1 && elect_one()) {
+                if (warp == 1 && elect_one() && ok) {
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(cols >> 3) << 17) | (8u << 24);
                     for (int mt = 0; mt < nM; ++mt) {
@@ -634,11 +644,12 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_addr(&bar_empty[st]));
                 if (warp == 0 && q + S < nq) {   // refill this stage (possibly with the next pass's K-block)
-                    ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_addr(&bar_empty[st]), par));
-                    if (!ok) break;
-                    if (elect_one()) produce(q + S);
+                    ok = ok && mbar_wait(smem_addr(&bar_empty[st]), par);
+                    if (elect_one() && ok) {
+                        produce(q + S);
+                        ++issued;
+                    }
                     __syncwarp();
-                    ++issued;
                 }
             }
             if (!ok) atomicOr(&s_fail, 1);
@@ -707,7 +718,7 @@ __global__ void __launch_bounds__(kTiledThreads, 1)
         if (s_fail != 0) {
             // a wait gave up: let the copies and products in flight land (bounded) before the
             // shared and tensor memory are released
-            if (tid == 0) {
+            if (warp == 0 && elect_one()) {
                 raise_status(p.status, FUSION_DEV_TIMEOUT);
                 for (int q = max(0, issued - S); q < issued; ++q)
                     (void)mbar_wait(smem_addr(&bar_full[q % S]), (uint32_t)(q / S) & 1u);

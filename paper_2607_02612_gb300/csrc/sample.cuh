@@ -137,6 +137,7 @@ __device__ __forceinline__ int cancel_empty(const ImageParams &p, int n_live) {
                 : "memory");
             if (!mbar_wait(ba, n & 1)) {
                 raise_status(p.status, FUSION_DEV_TIMEOUT);
+                (void)mbar_wait(ba, n & 1);   // the reply is still to be written here
                 break;
             }
             uint32_t ok, x;
