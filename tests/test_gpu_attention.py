@@ -75,8 +75,8 @@ def _check(offsets, qkv, H, sizes, label, nb=None, **kw):
 
 @pytest.mark.parametrize("sizes", [True, False])
 def test_attention_tile_boundaries(sizes):
-    """Sample lengths on both sides of every boundary of the resident-sample kernel: 8-row TMA boxes,
-    16-key MMA granularity, 64-key K-blocks, the 128-row query tile, the 256-token bound."""
+    """Sample lengths on both sides of the kernel's boundaries: 8-row TMA boxes, 16-key MMA granularity,
+    64-key blocks, the 128-row query tile, the ring's four blocks, two query tiles."""
     Ns = [1, 2, 7, 8, 9, 15, 16, 17, 63, 64, 65, 127, 128, 129, 130, 191, 192, 200, 255, 256]
     offsets, qkv, sz = _case(Ns, 3, 61, lead=3, tail=5)
     st = _check(offsets, qkv, 3, sz if sizes else None, f"boundaries sizes={sizes}")
@@ -103,8 +103,8 @@ def test_attention_large_logits_and_count():
 
 @pytest.mark.parametrize("sizes", [True, False])
 def test_attention_long_samples(sizes):
-    """Samples past 256 tokens stream key blocks of 128 (the ViT-L/16@384 length, 577, and the
-    1024-token bound), mixed with short ones in the same call and around the block edges."""
+    """Samples past 256 tokens take several pairs of query tiles and refill the ring of key blocks (the
+    ViT-L/16@384 length, 577, and the 1024-token bound), mixed with short ones in the same call."""
     Ns = [577, 1, 300, 129, 1024, 256, 257, 385, 640]
     offsets, qkv, sz = _case(Ns, 2, 65, lead=2, tail=3)
     st = _check(offsets, qkv, 2, sz if sizes else None, f"long samples sizes={sizes}")
@@ -115,6 +115,31 @@ def test_attention_vit_l_shapes():
     """ViT-L/16@384: 16 heads of 64, 577 tokens, a few images."""
     offsets, qkv, sz = _case([577, 577, 400], 16, 66)
     st = _check(offsets, qkv, 16, sz, "ViT-L 16 heads")
+    assert st == 0
+
+
+@pytest.mark.parametrize("sizes", [True, False])
+@pytest.mark.parametrize("longest", [1, 16, 64, 65, 128, 129, 192, 193])
+def test_attention_call_maximum(longest, sizes):
+    """The call's maximum picks the form: one query tile per CTA up to 128 tokens, two beyond, and a ring of as many
+    key blocks as the longest sample has, up to four.  Ragged samples up to it."""
+    Ns = [longest] + [max(1, longest - d) for d in (1, 7, 8, 15, 16, 63, 64, 100)] + [1, longest]
+    offsets, qkv, sz = _case(Ns, 3, longest, lead=2, tail=4)
+    st = _check(offsets, qkv, 3, sz if sizes else None, f"maximum {longest} sizes={sizes}")
+    assert st == 0
+
+
+@pytest.mark.parametrize("n", [129, 257, 577])
+def test_attention_rising_maxima(n):
+    """Logits that rise from key block to key block (by about 24 each): the rows of O and their sums are rescaled by
+    large factors at every block, and end with the last block's keys."""
+    offsets, qkv, sz = _case([n, n], 2, n)
+    f = bf16_bits_to_f32(qkv)
+    block = np.concatenate([np.arange(n), np.arange(n)]) // 64
+    for h in range(2):
+        f[:, h * DH] = 16.0
+        f[:, (2 + h) * DH] = 12.0 * block
+    st = _check(offsets, f32_to_bf16_bits(f), 2, sz, f"rising {n}")
     assert st == 0
 
 
@@ -154,6 +179,6 @@ def test_attention_malformed():
     g, st = _run(long, qkv2, 2, None, max_tokens=256)
     assert st & fz.FUSION_DEV_BAD_OFFSETS
     assert (g[10:300] == SENTINEL).all()
-    g, st = _run(long, qkv2, 2, None, max_tokens=280)   # the key-block kernel checks the same
+    g, st = _run(long, qkv2, 2, None, max_tokens=280)   # past one pair of query tiles
     assert st & fz.FUSION_DEV_BAD_OFFSETS
     assert (g[10:300] == SENTINEL).all()

@@ -1,6 +1,7 @@
 """The float32 merged mean's division step (sample.cuh, mean_of for float), restated in exact rational
 arithmetic with one rounding per operation: the quotient it returns is the correctly rounded one, ties
-included."""
+included.  This is the arithmetic alone, for divisors that are floats; test_gpu_mean_rounding.py holds the kernel's
+output to it."""
 from fractions import Fraction
 
 import numpy as np
