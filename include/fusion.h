@@ -90,7 +90,8 @@ extern "C" {
 #define FUSION_MAX_TOKENS 1024
 #define FUSION_MAX_DIM 1024
 /* batches of at most this many samples run their plan (validation, output offsets)
-   inside the per-sample kernel; larger ones launch a plan kernel first */
+   inside the per-sample kernel; larger ones have it made before, by the linear exit
+   check (heads of up to 1024 classes) or a plan kernel */
 #define FUSION_FUSED_PLAN_MAX_BATCH 1024
 
 /* Size-aware attention (fusion_attention): head width and the longest sample. */

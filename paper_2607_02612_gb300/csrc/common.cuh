@@ -54,7 +54,7 @@ constexpr int kExitClMaxTiles = 8;   // class tiles of the cluster exit kernel (
 constexpr int kWsCounters = 1 << 16;
 struct WsLayout {
     size_t counters;   // int[kWsCounters], zero between calls
-    size_t slot;       // int[max_batch]: output rows of every input sample (the plan's counts)
+    size_t cnt;        // int[max_batch]: output rows of every input sample (the plan's counts)
     size_t plan;       // int[4]: batch valid, survivor count
     size_t partials;   // float2[n_btile * kExitBT * n_ctile]; after the exit check the plan's tile totals
     size_t lg;         // float[n_btile * kExitBT][classes] (empty for heads of <= kExitClMaxTiles tiles)
@@ -71,7 +71,7 @@ __host__ __device__ inline WsLayout ws_layout(int max_batch, int classes) {
     size_t off = 0;
     L.counters = off;
     off += align256(sizeof(int) * (size_t)kWsCounters);
-    L.slot = off;
+    L.cnt = off;
     off += align256(sizeof(int) * (size_t)(max_batch > 0 ? max_batch : 1));
     L.plan = off;
     off += align256(sizeof(int) * 4);
@@ -272,49 +272,6 @@ __device__ __forceinline__ uint16_t f2_to_bf16_bits(F2 v) {
         if (away || (!toward && (up & 1u))) up += 1;
     }
     return (uint16_t)up;
-}
-
-// ---------------------------------------------------------------------------
-// block-wide exclusive scan of v[0..n) in shared memory, in chunks of 2 * blockDim.x
-// elements (one chunk for n <= 2 * blockDim.x).  All threads must call; tmp needs 33 ints.
-// Returns the total.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ int block_scan_excl(int *v, int n, int *tmp) {
-    const int t = threadIdx.x;
-    const int lane = t & 31, w = t >> 5, nw = (blockDim.x + 31) >> 5;
-    int base = 0;
-    for (int c0 = 0; c0 < n; c0 += 2 * (int)blockDim.x) {
-        const int i0 = c0 + 2 * t, i1 = i0 + 1;
-        const int a = (i0 < n) ? v[i0] : 0;
-        const int b = (i1 < n) ? v[i1] : 0;
-        const int s = a + b;
-        int incl = s;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (lane == 31) tmp[w] = incl;
-        __syncthreads();
-        if (w == 0) {
-            const int x = (lane < nw) ? tmp[lane] : 0;
-            int ix = x;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xFFFFFFFFu, ix, o);
-                if (lane >= o) ix += y;
-            }
-            if (lane < nw) tmp[lane] = ix - x;
-            if (lane == 31) tmp[32] = ix;
-        }
-        __syncthreads();
-        const int excl = base + tmp[w] + incl - s;
-        if (i0 < n) v[i0] = excl;
-        if (i1 < n) v[i1] = excl + a;
-        base += tmp[32];
-        __syncthreads();
-    }
-    return base;
 }
 
 // ceil(rho * P) with rho taken exactly, clamped to [0, P]; NaN keeps nothing; NaN and

@@ -398,7 +398,8 @@ __global__ void __launch_bounds__(kExitThreads) k_exit(const __grid_constant__ C
         // the row's chunk c as floats: from the tile, or from the float32 input rows
         const float *ur = p.in_mode == 2 && ok ? p.u_in + (size_t)s * dim : nullptr;
         const float *url = ur && p.u_in_lo ? p.u_in_lo + (size_t)s * dim : nullptr;   // float-float low parts
-        // rows of up to 512 dims are read once, into registers (the three passes below would each wait for L2)
+        // rows of up to 64 chunks (512 dims in bf16, 256 in float32) are read once, into registers (the three passes
+        // below would each wait for L2)
         constexpr int kHeld = 2;
         const bool held = ur && nchunk <= 32 * kHeld;
         float4 hv[kHeld][CH / 4], hl[kHeld][CH / 4];
@@ -1662,7 +1663,7 @@ size_t exit_rows_smem(int dtype, int bt, int dim) {
 
 // The linear head's samples per cluster: 8 (k_exit_cl, several warps per LayerNorm row) while the
 // class tiles of all sample tiles fit one wave of two CTAs per SM, else the smallest of 16, 32 and 64
-// (k_exit_rows, one warp per row) whose tiles do, 64 for the largest batches: a larger tile reads the
+// (k_exit_rows, up to 32 lanes per row) whose tiles do, 64 for the largest batches: a larger tile reads the
 // weights for more samples (8192 samples x 100 classes at d = 384 read them 1024 times in tiles of 8),
 // a smaller one has more CTAs to spread.  The plan's tiles are at least 32.  0: the general kernel.
 int exit_samples_per_tile(int dtype, const ExitParams &p, bool plan) {

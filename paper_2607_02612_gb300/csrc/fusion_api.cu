@@ -56,7 +56,7 @@ Head dev(const fusion_exit_head &h) {
 }
 
 struct Ws {
-    int *cnt;
+    int *cnt;        // the plan's counts
     int *plan;
     int *plan_counter, *counters;   // zero between calls
     float2 *partials;
@@ -66,7 +66,7 @@ struct Ws {
 Ws carve(void *ws, int32_t max_batch, int32_t classes) {
     const WsLayout L = ws_layout(max_batch, classes);
     unsigned char *b = static_cast<unsigned char *>(ws);
-    return Ws{reinterpret_cast<int *>(b + L.slot), reinterpret_cast<int *>(b + L.plan),
+    return Ws{reinterpret_cast<int *>(b + L.cnt), reinterpret_cast<int *>(b + L.plan),
               reinterpret_cast<int *>(b + L.counters), reinterpret_cast<int *>(b + L.counters) + 1, reinterpret_cast<float2 *>(b + L.partials),
               L.total > L.lg ? reinterpret_cast<float *>(b + L.lg) : nullptr};
 }
@@ -168,7 +168,7 @@ cudaError_t launch_sample_kernel(int dtype, const ImageParams &p, const ImageGeo
         const TcGeometry T = image_tc_geometry(dtype, p.in.max_tokens, p.kdim, p.dim, p.in.max_rows, 1, kTcSmemBudgetKb,
                                                p.in.max_batch);
         if (T.ok) return launch_image_tc(p, T, s, pdl);
-        if (dtype == FUSION_F32) {   // the general kernel for samples whose stages do not fit
+        if (dtype == FUSION_F32) {   // the general kernel for samples whose stages do not fit, or that it serves sooner
             const F32Geometry F = image_f32_geometry(p);
             if (F.ok) return launch_image_f32(p, F, s);
         }

@@ -1,8 +1,9 @@
 // Per-sample merge (Sec. III-C) -> prune (Sec. III-E) -> gather into the
 // compacted output batch, for whatever the float32 merge kernel (image_f32.cu) and the tcgen05 one
-// (image_tc.cu) do not take: bf16 keys whose width is not a multiple of 64, the longest samples; and,
-// in a kernel of its own below, pruning or compaction without merging.  One CTA per input sample; a sample that exited (or is
-// beyond the device batch count) returns at once.
+// (image_tc.cu) do not take: bf16 keys whose width is not a multiple of 64, the longest samples, the float32
+// batches past 66 tokens that it serves sooner; and, in a kernel of its own below, pruning or compaction
+// without merging.  One CTA per input sample; a sample that exited (or is beyond the device batch count)
+// returns at once.
 //
 // Merge decisions.  The keys of half A (even positions) and half B (odd
 // positions) are staged in shared memory in a chunk-major layout: the 16-byte

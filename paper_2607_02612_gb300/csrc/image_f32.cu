@@ -12,8 +12,9 @@
 // sums of 16 dims, squared norms per block of `kc` dims with chunk c of a block in lane c % 32.
 //
 // Bound by the chain of latencies of one sample (loads, FFMA, decisions, gather) and, with enough
-// samples, by FFMA and L2.  The general kernel keeps a whole sample in shared memory (98 KB for 65
-// tokens of 384: two CTAs per SM) and gives 16 x 32 strips to warps, of which 65 tokens have two.
+// samples, by FFMA and L2.  The general kernel keeps a whole sample in shared memory where it can, has one CTA
+// of 512 threads per SM (its 128 registers) and gives 16 x 32 strips to warps, of which 65 tokens have two.  It stays
+// the faster one for many batches of longer samples (image_f32_geometry has the rule).
 // Measured, general kernel -> this one: 3277 of 8192 samples of 65 tokens, d = 384, continuing: 606 -> 219
 // us (and 69 -> 29 us for the 210 that the fourth stage of that chain keeps); 8 samples of 197 tokens,
 // keys of their own, clusters of 8, the stage with its exit check: 117 -> 45 us.  All with cold caches.

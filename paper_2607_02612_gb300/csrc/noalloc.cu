@@ -55,7 +55,7 @@ extern "C" int fusion_exit_check_noalloc(int dtype, fusion_ragged in, const void
     if (head.classes < 1) return FUSION_ERR_SHAPE;
     // the workspace's data, then the counters of this call's tiles (cleared below, so they need no fixed place)
     const WsLayout L = ws_layout(in.max_batch, head.classes);
-    const size_t counters = L.total - L.slot;
+    const size_t counters = L.total - L.cnt;
     const int n_btile = ceil_div(in.max_batch > 0 ? in.max_batch : 1, kExitBT);
     const size_t counter_bytes = sizeof(int) * ((size_t)n_btile + 1);
     if (counters + align256(counter_bytes) > kNoAllocScratchBytes) return FUSION_ERR_WORKSPACE;
@@ -74,8 +74,8 @@ extern "C" int fusion_exit_check_noalloc(int dtype, fusion_ragged in, const void
     e.logits = logits;
     e.max_prob = max_prob;
     e.counters = reinterpret_cast<int *>(base + counters);
-    e.partials = reinterpret_cast<float2 *>(base + (L.partials - L.slot));
-    e.lg_tmp = (logits && L.total > L.lg) ? reinterpret_cast<float *>(base + (L.lg - L.slot)) : nullptr;
+    e.partials = reinterpret_cast<float2 *>(base + (L.partials - L.cnt));
+    e.lg_tmp = (logits && L.total > L.lg) ? reinterpret_cast<float *>(base + (L.lg - L.cnt)) : nullptr;
     e.n_ctile = ceil_div(head.classes, kExitCT);
     e.n_btile = n_btile;
     e.do_plan = 0;

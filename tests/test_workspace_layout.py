@@ -12,7 +12,7 @@ PROGRAM = r"""
 int main(int argc, char **argv) {
     for (int k = 1; k + 1 < argc; k += 2) {
         const fz::WsLayout L = fz::ws_layout(atoi(argv[k]), atoi(argv[k + 1]));
-        const size_t at[5] = {L.slot, L.plan, L.partials, L.lg, L.total};
+        const size_t at[5] = {L.cnt, L.plan, L.partials, L.lg, L.total};
         size_t end = L.total;   // of the counters: where the next block begins
         for (size_t v : at)
             if (v > L.counters && v < end) end = v;
