@@ -310,24 +310,23 @@ __global__ void __launch_bounds__(kImageThreads, 1) k_image(ImageParams p) {
 // CTAs without exchanging anything: each repeats the decisions (ranks of the scores, a scan) and writes a
 // range of columns; the first one writes the index outputs.  Bound by DRAM once enough chunks are in
 // flight: 2048 per CTA, two CTAs per SM.  77 samples of 120 to 197 tokens, d = 768, float32:
-// 27.5 us with one CTA of 512 threads per sample (half the SMs, 12 rounds of loads) -> 22.5 us.
+// 27.5 us with one CTA of 512 threads per sample (half the SMs, 12 rounds of loads) -> 22.5 us.  Past 224 tokens the
+// ranks (tokens squared) need the threads while SMs are free: CTAs of 512 threads, one per SM.
 // ---------------------------------------------------------------------------
-constexpr int kSelectThreads = 256;
-
-template <typename T>
-__global__ void __launch_bounds__(kSelectThreads, 2) k_select(ImageParams p, int parts) {
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) k_select(ImageParams p, int parts) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int part = (int)(blockIdx.x % (unsigned)parts);
     SampleInfo s;
-    if (!sample_begin<kSelectThreads>(p, (int)(blockIdx.x / (unsigned)parts), s)) return;
+    if (!sample_begin<NT>(p, (int)(blockIdx.x / (unsigned)parts), s)) return;
     MetaPtrs m(sm, meta_layout(p.in.max_tokens, 0));
-    meta_init<kSelectThreads>(p, s, m);
+    meta_init<NT>(p, s, m);
     __syncthreads();
-    if (!finish_decide<kSelectThreads>(p, s, m)) return;
-    if (part == 0) write_index_outputs<kSelectThreads>(p, s, m);
+    if (!finish_decide<NT>(p, s, m)) return;
+    if (part == 0) write_index_outputs<NT>(p, s, m);
     const GlobalLoader<T> ld{reinterpret_cast<const T *>(p.x), (long long)s.start, p.dim};
     const int w = p.dim / Elem<T>::kPerChunk;
-    write_rows<T, kSelectThreads>(p, s, m, ld, w * part / parts, w * (part + 1) / parts);
+    write_rows<T, NT>(p, s, m, ld, w * part / parts, w * (part + 1) / parts);
 }
 
 }  // namespace
@@ -379,15 +378,20 @@ ImageGeometry image_geometry(int dtype, int max_tokens, int kdim, int do_merge) 
 cudaError_t launch_image(int dtype, const ImageParams &p, size_t smem, cudaStream_t s) {
     if (p.in.max_batch == 0) return cudaSuccess;
     if (!p.do_merge) {
-        // as many CTAs per sample as one wave of two per SM holds, each with at least 16 chunks (256 bytes)
-        // of a row (a launch gate may stop a single CTA: its samples keep one)
-        const int chunks = p.dim / (dtype == FUSION_BF16 ? 8 : 4);
+        // as many CTAs per sample as one wave holds, each with at least 16 chunks (256 bytes) of a row (a launch
+        // gate may stop a single CTA: its samples keep one).  Long samples of up to 152: CTAs of 512 threads, one per
+        // SM (40 samples, d = 192, float32: 800 tokens 41 us with CTAs of 256, 30 of 512; 400 tokens 27, 23), but
+        // three of 256 rather than one of 512 where that would gather wide rows alone (77 of 400 tokens, d = 1024: 55
+        // us, 62).
+        const int chunks = p.dim / (dtype == FUSION_BF16 ? 8 : 4), B = p.in.max_batch;
+        const bool wide = p.in.max_tokens > 224 && B <= 152 && !(p.in.max_tokens <= 600 && chunks >= 96 && B > 76 && B <= 101);
         int parts = 1;
-        while (!p.gate && parts < 8 && (long long)p.in.max_batch * (parts + 1) <= 2 * 152 && chunks / (parts + 1) >= 16) ++parts;
-        auto kern = dtype == FUSION_BF16 ? k_select<__nv_bfloat16> : k_select<float>;
+        while (!p.gate && parts < 8 && (long long)B * (parts + 1) <= (wide ? 152 : 2 * 152) && chunks / (parts + 1) >= 16) ++parts;
+        auto kern = dtype == FUSION_BF16 ? (wide ? k_select<__nv_bfloat16, 512> : k_select<__nv_bfloat16, 256>)
+                                         : (wide ? k_select<float, 512> : k_select<float, 256>);
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        kern<<<(unsigned)p.in.max_batch * (unsigned)parts, kSelectThreads, smem, s>>>(p, parts);
+        kern<<<(unsigned)B * (unsigned)parts, wide ? 512 : 256, smem, s>>>(p, parts);
         return cudaGetLastError();
     }
     const dim3 grid(p.in.max_batch);

@@ -172,7 +172,8 @@ def test_bf16_merge_long_samples(counts, dim):
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("counts,dim,prune", [
     ([197, 1, 2, 130], 768, True), ([90, 17, 33] * 25, 112, True), ([1024, 5], 16, True),
-    ([65, 3] * 200, 384, True), ([40, 1, 7] * 30, 1024, False)])
+    ([65, 3] * 200, 384, True), ([40, 1, 7] * 30, 1024, False),
+    ([600, 5], 768, True), ([300, 225, 2] * 40, 64, True), ([260, 1, 450] * 30, 1024, True)])   # 512 threads, 512, 256
 def test_prune_and_compact_column_parts(dtype, counts, dim, prune):
     """A sample's columns shared by several CTAs (few samples), and one CTA per sample (many)."""
     b = make_batch(counts, dim, dtype, seed=len(counts), sizes="u1to4")
