@@ -402,8 +402,8 @@ F32Geometry image_f32_geometry(const ImageParams &p) {
     // 100 tokens, d = 384, in clusters of 4 82 us, of 2 50).
     auto fits = [&](int cl, int most) { return !p.gate && cl <= strips + 1 && B <= most; };
     // With an SM each they are the fastest form measured, except that pairs have half of the general kernel's
-    // threads per SM for the decisions, which long samples with narrow keys spend their time on (76 samples of 300
-    // tokens, d = 48: 64 us, general kernel 51).
+    // threads per SM for the decisions, which samples with narrow keys spend their time on once a warp has more than
+    // a tile (76 samples of 300 tokens, d = 48: 64 us, general kernel 51).
     const bool narrow = p.kdim < 192, one_tile = N <= kSmallTokens + 1;
     // Two per SM gain less: where the similarity is nearly all of the time (60 samples of 197 tokens, d = 192:
     // clusters of 4 59 us, of 2 68; 100 tokens 48 and 36; past 600 tokens the stages are 16 dims: 700 tokens, d =
@@ -415,13 +415,13 @@ F32Geometry image_f32_geometry(const ImageParams &p) {
     // ... and in a call with an exit check, whose samples that leave free the SMs (half of the batch continuing:
     // 20 samples of 197 tokens, d = 384, clusters of 8 52 us, of 4 77; 100 of 100 tokens pairs 51 us, general kernel
     // 62; everyone continuing 73 and 60 of the 77 that the call took before either), up to where the whole batch
-    // would be slower than the general kernel and the exit check before were.
-    const bool exits = p.plan_args.exit_mask != nullptr;
-    const bool exit8 = exits && !(narrow && N > 150), exit4 = exits && !(narrow && N > 600);
-    const bool exit2 = exits && !one_tile && N <= 600 && (N <= 129 ? p.kdim < 768 : N <= 197 || (!narrow && full));
-    g.cluster = fits(8, exit8 ? 30 : 15) ? 8
-                : fits(4, four || exit4 ? 72 : 36) ? 4
-                : fits(2, two || exit2 ? 152 : narrow && N > 150 ? 0 : 76) ? 2
+    // would be slower than the general kernel and the exit check before were (64 samples of 65 to 130 tokens, d = 48:
+    // clusters of 4 40 us, 36 before).
+    const bool exits = p.plan_args.exit_mask != nullptr && !narrow;
+    const bool exit2 = exits && !one_tile && N <= 600 && (N <= 129 ? p.kdim < 768 : N <= 197 || full);
+    g.cluster = fits(8, exits ? 30 : 15) ? 8
+                : fits(4, four || exits ? 72 : 36) ? 4
+                : fits(2, two || exit2 ? 152 : narrow && pair_tiles > 8 ? 0 : 76) ? 2
                 : 1;
     // One CTA per sample with more than eight tiles: 256 threads against the general kernel's 512, but two CTAs
     // per SM where that has one.  In a wave of at most 152 samples each CTA is alone and slower (300 tokens,
@@ -432,7 +432,7 @@ F32Geometry image_f32_geometry(const ImageParams &p) {
     // only without an exit check and without a device count; else 153 to 456 samples may leave one wave, which
     // costs nothing up to 80 tokens and d = 384 (100 of 200 samples: 73 us, at the start's general kernel 72).
     const bool known = !p.in.batch && !p.plan_args.exit_mask;
-    const bool few_waves = (known && B <= 2 * 152) || (N <= 80 && p.kdim <= 384);
+    const bool few_waves = (known && B <= 2 * 152) || (N <= 80 && !narrow && p.kdim <= 384);
     if (g.cluster == 1 && !one_tile && !(N <= 197 && B > 152 && (B > 3 * 152 || few_waves))) return g;
     g.rows_a = ceil_div(strips, g.cluster) * 16;
     g.rows_b = cols * 16;

@@ -67,10 +67,10 @@ def test_float32_merges_leave_the_general_kernel_only_where_measured_faster(rout
         (80, 1024, 77, 0): 0, (129, 768, 152, 0): 0, (257, 384, 100, 0): 0, (400, 192, 100, 0): 0, (577, 48, 100, 0): 0,
         (800, 192, 100, 0): 0, (100, 1024, 153, 0): 0, (300, 384, 200, 0): 0, (197, 384, 304, 0): 0, (80, 384, 200, 0): 1,
         (80, 768, 200, 0): 0, (80, 384, 400, 0): 1, (100, 384, 457, 0): 1, (197, 192, 2000, 0): 1, (257, 192, 608, 0): 0,
-        (577, 48, 608, 0): 0,
+        (577, 48, 608, 0): 0, (129, 48, 64, 0): 2, (130, 48, 64, 0): 0, (80, 80, 153, 0): 0, (80, 192, 153, 0): 1,
         # without
         (197, 384, 15, 1): 8, (197, 384, 16, 1): 4, (100, 768, 36, 1): 4, (100, 768, 37, 1): 2, (197, 192, 37, 1): 4,
-        (577, 192, 72, 1): 4, (700, 384, 37, 1): 2, (150, 384, 76, 1): 2, (300, 48, 76, 1): 0, (150, 48, 76, 1): 2,
+        (577, 192, 72, 1): 4, (700, 384, 37, 1): 2, (150, 384, 76, 1): 2, (300, 48, 76, 1): 0, (129, 48, 76, 1): 2,
         (80, 48, 77, 1): 0, (100, 384, 100, 1): 0, (197, 192, 152, 1): 0, (577, 384, 100, 1): 2, (300, 192, 77, 1): 2,
         (257, 192, 77, 1): 0, (100, 384, 200, 1): 1, (197, 384, 304, 1): 1, (197, 384, 400, 1): 0, (257, 192, 200, 1): 0,
         (700, 192, 305, 1): 0,
