@@ -416,9 +416,9 @@ F32Geometry image_f32_geometry(const ImageParams &p) {
     // 20 samples of 197 tokens, d = 384, clusters of 8 52 us, of 4 77; 100 of 100 tokens pairs 51 us, general kernel
     // 62; everyone continuing 73 and 60 of the 77 that the call took before either), up to where the whole batch
     // would be slower than the general kernel and the exit check before were (64 samples of 65 to 130 tokens, d = 48:
-    // clusters of 4 40 us, 36 before).
+    // clusters of 4 40 us, 36 before; 152 of 50 to 100 tokens, d = 384, merge and exit check, pairs 70 us, 66 before).
     const bool exits = p.plan_args.exit_mask != nullptr && !narrow;
-    const bool exit2 = exits && !one_tile && N <= 600 && (N <= 129 ? p.kdim < 768 : N <= 197 || full);
+    const bool exit2 = exits && !one_tile && N <= 600 && (N <= 129 ? p.kdim < 768 && B <= 114 : N <= 197 || full);
     g.cluster = fits(8, exits ? 30 : 15) ? 8
                 : fits(4, four || exits ? 72 : 36) ? 4
                 : fits(2, two || exit2 ? 152 : narrow && pair_tiles > 8 ? 0 : 76) ? 2

@@ -63,7 +63,7 @@ def test_float32_merges_leave_the_general_kernel_only_where_measured_faster(rout
         (197, 384, 15, 0): 8, (197, 384, 16, 0): 8, (197, 768, 30, 0): 8, (300, 192, 31, 0): 4, (300, 48, 19, 0): 4,
         (100, 768, 37, 0): 4, (100, 768, 72, 0): 4, (100, 768, 73, 0): 2, (150, 384, 76, 0): 2, (577, 192, 72, 0): 4,
         (577, 192, 73, 0): 2, (700, 384, 60, 0): 4, (700, 384, 76, 0): 2, (257, 48, 73, 0): 0, (700, 48, 60, 0): 0,
-        (100, 384, 77, 0): 2, (197, 384, 152, 0): 2, (577, 384, 100, 0): 2, (300, 384, 152, 0): 2, (150, 1024, 100, 0): 2,
+        (100, 384, 77, 0): 2, (100, 384, 114, 0): 2, (100, 384, 115, 0): 0, (197, 384, 152, 0): 2, (577, 384, 100, 0): 2, (300, 384, 152, 0): 2, (150, 1024, 100, 0): 2,
         (80, 1024, 77, 0): 0, (129, 768, 152, 0): 0, (257, 384, 100, 0): 0, (400, 192, 100, 0): 0, (577, 48, 100, 0): 0,
         (800, 192, 100, 0): 0, (100, 1024, 153, 0): 0, (300, 384, 200, 0): 0, (197, 384, 304, 0): 0, (80, 384, 200, 0): 1,
         (80, 768, 200, 0): 0, (80, 384, 400, 0): 1, (100, 384, 457, 0): 1, (197, 192, 2000, 0): 1, (257, 192, 608, 0): 0,
