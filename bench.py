@@ -103,7 +103,7 @@ def peaks():
 # includes.  The recorded DRAM traffic stays valid while none of these changes.
 IMAGE_TC_SOURCES = ("paper_2607_02612_gb300/csrc/image_tc.cu", "paper_2607_02612_gb300/csrc/sample.cuh",
                     "paper_2607_02612_gb300/csrc/launch.h", "paper_2607_02612_gb300/csrc/plan.cuh",
-                    "paper_2607_02612_gb300/csrc/common.cuh", "include/fusion.h")
+                    "paper_2607_02612_gb300/csrc/tc.cuh", "paper_2607_02612_gb300/csrc/common.cuh", "include/fusion.h")
 
 
 def source_hash() -> str:
